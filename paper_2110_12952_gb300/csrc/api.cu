@@ -140,7 +140,7 @@ extern "C" int fractal_create(int k, int s, int r, int dim, const int32_t *offse
         delete f;
         return cuda_fail(e, "fractal_create: no usable CUDA device");
     }
-    f->tile_levels_user = cached_tile_levels(f, &f->stages_user);
+    apply_tuned(f);
     *out = f;
     return FR_OK;
 }
@@ -223,7 +223,7 @@ extern "C" int fractal_create_mixed(int s, int r, int dim, const int32_t *ks, co
         return cuda_fail(e, "fractal_create_mixed: no usable CUDA device");
     }
     D.mix = f->d_mix;
-    f->tile_levels_user = cached_tile_levels(f, &f->stages_user);
+    apply_tuned(f);
     *out = f;
     return FR_OK;
 }
@@ -237,6 +237,7 @@ extern "C" int fractal_destroy(fractal_t *f)
     cudaDeviceSynchronize();
     free_step_plan(f->plan);
     free_tb_plan(f->tb);
+    free_slice_plan(f->slice);
     fr_paper_aux_free(f);
     free_bb_plan(f->bb);
     cudaFree(f->scratch);
@@ -269,6 +270,7 @@ extern "C" int fractal_set_tile_levels(fractal_t *f, int levels)
         return fail(FR_EINVAL, "fractal_set_tile_levels: levels must be -1 or in [0, r]");
     if (levels != f->tile_levels_user && f->server_refs.load() > 0)
         return fail(FR_EBUSY, "fractal_set_tile_levels: a server still holds requests on this handle");
+    f->sliced_tuned = false;
     if (levels != f->tile_levels_user) {
         f->tile_levels_user = levels;
         cudaDeviceSynchronize();
@@ -285,6 +287,7 @@ extern "C" int fractal_set_pipeline_stages(fractal_t *f, int stages)
         return fail(FR_EINVAL, "fractal_set_pipeline_stages: stages must be -1 or in [2, 4]");
     if (stages != f->stages_user && f->server_refs.load() > 0)
         return fail(FR_EBUSY, "fractal_set_pipeline_stages: a server still holds requests on this handle");
+    f->sliced_tuned = false;
     if (stages != f->stages_user) {
         f->stages_user = stages;
         cudaDeviceSynchronize();
@@ -380,7 +383,14 @@ extern "C" int fractal_step(fractal_t *f, const uint8_t *in, uint8_t *out, int64
         }
         return FR_OK;
     }
-    int rc = ensure_step_plan(f);
+    int rc;
+    if (((f->tile_levels_user < 0 && f->stages_user < 0) || f->sliced_tuned) && !f->test_extra_tx) {
+        // (a tile depth or stage count set by the caller asks for the tile kernels)
+        bool done = false;
+        rc = try_slice_step(f, in, out, steps, birth, survive, st, &done);
+        if (rc || done) return rc;
+    }
+    rc = ensure_step_plan(f);
     if (rc) return rc;
     if (steps > 1 && bit3_plan(f)) return launch_bit3_generations(f, in, out, steps, birth, survive, st);
     if (steps > 1) {

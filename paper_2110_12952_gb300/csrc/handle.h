@@ -9,6 +9,7 @@
 #include <vector>
 
 #include "internal.cuh"
+#include "slice.h"
 
 namespace fr {
 
@@ -141,6 +142,8 @@ struct fractal {
     int tb_gens = 0;                 // temporal blocking: generations per pass (0 = off)
     int tb_levels_user = -1;         // its tile depth (-1 = automatic)
     fr::TbPlan tb;
+    fr::SlicePlan slice;             // the bit-sliced step of 2D fractals
+    bool sliced_tuned = false;       // the autotuner found it faster than the tile depth it set
     void *paper_aux = nullptr;       // the paper's approaches (paper_kernels.cu): geometry and scratch
     // a different transition table per level (fractal_create_mixed); then
     // `offsets` holds the levels' tables one after the other
@@ -203,7 +206,7 @@ int launch_copy_normalise(const uint8_t *in, uint8_t *out, int64_t n, int num_sm
 int preload_copy_kernel();
 int ensure_status(fractal *f);
 int take_status(fractal *f);
-int cached_tile_levels(const fractal *f, int *stages);
+void apply_tuned(fractal *f);   // the autotuner's choice for this fractal, if it has made one
 int autotune_step(fractal *f, const uint8_t *in, uint8_t *out, uint32_t birth, uint32_t survive,
                   cudaStream_t st, int *best);
 

@@ -1,0 +1,1304 @@
+// slice.cu -- the bit-sliced compact step of 2D fractals (Sec. 3 stencil
+// procedure on 32 tiles at a time).
+//
+// A tile is a level-L subtree (k^L cells, contiguous in omega).  All tiles
+// have the same local neighbour structure: cell l of a tile has, for each
+// Moore direction, either no neighbour at all, a fixed local cell of the same
+// tile, or a fixed local cell of the neighbouring tile in a fixed direction.
+// So 32 tiles are packed into words, bit t of word l being cell l of tile
+// 32 g + t, and one generation of a word is: load the words of its member
+// neighbours (at most 8, addresses from a table that is the same for every
+// group), add them bit-sliced, apply the rule as logic.  Cells off the
+// fractal take no storage, no loads and no operations.
+//
+// The cells of neighbouring tiles that touch a tile (its halo: 8 for the
+// triangle, 4 x 81 + 4 for the carpet's 81 x 81 tiles) travel as bit strings:
+// with every state goes, per tile, a word for each run of at most 32 border
+// cells (its exports).  Lane t of a warp loads the export of tile 32 g + t's
+// neighbour, and a 32 x 32 bit transposition across the warp turns the lanes'
+// words into the halo cells' words; the exports of the new state are made by
+// the same transposition from its words.
+//
+// Bytes become bits first, in omega order (16 consecutive bytes per thread and
+// load, a nibble per word by a carry-free multiply), so that everything that
+// is not aligned happens in bits: lane t takes 32 cells of tile t out of the
+// bit string with one funnel shift, and a 32 x 32 bit transposition across
+// the warp (five shuffle stages) leaves lane p with cell p of 32 tiles.  The
+// way back is the same in reverse.
+#include <cuda_runtime.h>
+#include <stdint.h>
+
+#include <string.h>
+
+#include <algorithm>
+#include <vector>
+
+#include "handle.h"
+#include "step.h"
+#include "tma.cuh"
+
+namespace fr {
+
+constexpr int kSliceBlock = 256;   // threads per block of the streaming kernels
+constexpr int kSliceAhead = 2;     // halo words per warp loaded ahead of their group
+constexpr int kSliceBatch = 2;     // 16-byte units per thread and batch copied to shared memory ahead
+constexpr int kSliceRounds = 32;   // resident kernel: most 32-cell chunks per warp
+
+struct SliceArgs {
+    int64_t NT, NG;
+    int KL, KLp, NC, NJ, XW, H;
+    int64_t ex;             // word offset of a state's exports behind its cells
+    int BP;                 // packing: words between tiles' bit strings when a tile is 2^bsh words, else 0
+    int bsh;                // (30: another number)
+    uint32_t lane_bits;     // packing: bits between tiles' bit strings
+    int RP;                 // unpacking: words between tiles' bit strings (odd)
+    int AW, A_zero;         // words of one group's array, index of its 32 zero words
+    DivU32 kdiv;            // division by KL
+    uint32_t mb[9], ms[9];  // rule: all ones where a dead / live cell with c live neighbours becomes live
+    const uint4 *tab;
+    const uint32_t *jobs;   // halo words: export word | direction << 8
+    const uint16_t *xlist;  // [XW][32]: cells of the export words
+    const uint2 *cells;     // [H] halo cells: cell of the neighbouring tile, word index | direction << 16
+    const int32_t *nbr;
+    uint32_t *bar;
+    int *status;
+};
+
+// Transpose of a 32 x 32 bit matrix held as a row per lane: afterwards bit t
+// of lane p is what bit p of lane t was.  Five exchanges of halves: of 16 and
+// 8 bits by byte permutes, of 4, 2 and 1 by a rotation and a bit select.
+struct Transpose32 {
+    uint32_t sel16, sel8, keep[3], rot[3];
+    __device__ __forceinline__ Transpose32(int lane)
+    {
+        sel16 = (lane & 16) ? 0x3276u : 0x5410u;
+        sel8 = (lane & 8) ? 0x3715u : 0x6240u;
+#pragma unroll
+        for (int i = 0; i < 3; ++i) {
+            const int s = 4 >> i;
+            const uint32_t lowm = s == 4 ? 0x0f0f0f0fu : s == 2 ? 0x33333333u : 0x55555555u;
+            const bool low = (lane & s) == 0;
+            keep[i] = low ? lowm : ~lowm;
+            rot[i] = low ? s : 32 - s;
+        }
+    }
+    __device__ __forceinline__ uint32_t operator()(uint32_t x) const
+    {
+        x = __byte_perm(x, __shfl_xor_sync(0xffffffffu, x, 16), sel16);
+        x = __byte_perm(x, __shfl_xor_sync(0xffffffffu, x, 8), sel8);
+#pragma unroll
+        for (int i = 0; i < 3; ++i) {
+            const uint32_t y = __shfl_xor_sync(0xffffffffu, x, 4 >> i);
+            x = (x & keep[i]) | (__funnelshift_l(y, y, rot[i]) & ~keep[i]);
+        }
+        return x;
+    }
+};
+
+__device__ __forceinline__ uint32_t sl_xor3(uint32_t a, uint32_t b, uint32_t c) { return a ^ b ^ c; }
+__device__ __forceinline__ uint32_t sl_maj3(uint32_t a, uint32_t b, uint32_t c) { return (a & b) | (c & (a | b)); }
+__device__ __forceinline__ uint32_t sl_mux(uint32_t s, uint32_t a, uint32_t b) { return (s & a) | (~s & b); }
+
+// Next state of 32 cells from their neighbours' words n[0..D-1] (absent ones
+// zero): bit-sliced count, then the rule.
+template <int D, bool LIFE>
+__device__ __forceinline__ uint32_t slice_rule(const SliceArgs &a, const uint32_t *n, uint32_t alive)
+{
+    uint32_t t0, t1, t2, t3 = 0u;
+    if constexpr (D == 4) {
+        const uint32_t s = sl_xor3(n[0], n[1], n[2]), c = sl_maj3(n[0], n[1], n[2]);
+        const uint32_t k = s & n[3];
+        t0 = s ^ n[3];
+        t1 = c ^ k;
+        t2 = c & k;
+    } else {
+        const uint32_t s0 = sl_xor3(n[0], n[1], n[2]), c0 = sl_maj3(n[0], n[1], n[2]);
+        const uint32_t s1 = sl_xor3(n[3], n[4], n[5]), c1 = sl_maj3(n[3], n[4], n[5]);
+        if constexpr (D == 6) {
+            const uint32_t k = s0 & s1;
+            t0 = s0 ^ s1;
+            t1 = sl_xor3(c0, c1, k);
+            t2 = sl_maj3(c0, c1, k);
+        } else if constexpr (D == 7) {
+            const uint32_t k = sl_maj3(s0, s1, n[6]);
+            t0 = sl_xor3(s0, s1, n[6]);
+            t1 = sl_xor3(c0, c1, k);
+            t2 = sl_maj3(c0, c1, k);
+        } else {
+            const uint32_t s2 = n[6] ^ n[7], c2 = n[6] & n[7];
+            const uint32_t k = sl_maj3(s0, s1, s2);
+            t0 = sl_xor3(s0, s1, s2);
+            const uint32_t u = sl_xor3(c0, c1, c2), v = sl_maj3(c0, c1, c2);
+            t1 = u ^ k;
+            const uint32_t w = u & k;
+            t2 = v ^ w;
+            t3 = v & w;
+        }
+    }
+    if constexpr (LIFE) return t1 & ~t2 & (t0 | alive);   // B3/S23 (a count of 8 has t1 = 0)
+    uint32_t b = sl_mux(t2, sl_mux(t1, sl_mux(t0, a.mb[7], a.mb[6]), sl_mux(t0, a.mb[5], a.mb[4])),
+                        sl_mux(t1, sl_mux(t0, a.mb[3], a.mb[2]), sl_mux(t0, a.mb[1], a.mb[0])));
+    uint32_t s = sl_mux(t2, sl_mux(t1, sl_mux(t0, a.ms[7], a.ms[6]), sl_mux(t0, a.ms[5], a.ms[4])),
+                        sl_mux(t1, sl_mux(t0, a.ms[3], a.ms[2]), sl_mux(t0, a.ms[1], a.ms[0])));
+    if constexpr (D == 8) {
+        b = sl_mux(t3, a.mb[8], b);
+        s = sl_mux(t3, a.ms[8], s);
+    }
+    return sl_mux(alive, s, b);
+}
+
+// ---------------------------------------------------------------- pack
+
+// 16 cells (bytes of any nonzero value) -> 16 bits.
+__device__ __forceinline__ uint32_t slice_bits16(uint4 v)
+{
+    if ((v.x | v.y | v.z | v.w) & 0xfefefefeu) {   // bytes other than 0 and 1
+        v.x = (((v.x & 0x7f7f7f7fu) + 0x7f7f7f7fu) | v.x) >> 7 & 0x01010101u;
+        v.y = (((v.y & 0x7f7f7f7fu) + 0x7f7f7f7fu) | v.y) >> 7 & 0x01010101u;
+        v.z = (((v.z & 0x7f7f7f7fu) + 0x7f7f7f7fu) | v.z) >> 7 & 0x01010101u;
+        v.w = (((v.w & 0x7f7f7f7fu) + 0x7f7f7f7fu) | v.w) >> 7 & 0x01010101u;
+    }
+    // the four 0/1 bytes of a word land in the product's top nibble
+    uint32_t x = (v.w * 0x10204080u) >> 28;
+    x = __funnelshift_l(v.z * 0x10204080u, x, 4);
+    x = __funnelshift_l(v.y * 0x10204080u, x, 4);
+    return __funnelshift_l(v.x * 0x10204080u, x, 4);
+}
+
+// The exports of a group from its words N: lane i takes cell i of an export
+// word, lane t gets tile t's bits.
+__device__ __forceinline__ void slice_export(const SliceArgs &a, const Transpose32 &tr, const uint32_t *N, uint32_t *ex,
+                                             int warp, int nw, int lane)
+{
+    for (int x = warp; x < a.XW; x += nw) ex[32 * x + lane] = tr(N[__ldg(a.xlist + 32 * x + lane)]);
+}
+
+// Words of a group's bit string in shared memory (one to spare for the funnel shifts).
+__device__ __forceinline__ int slice_string_words(const SliceArgs &a) { return a.BP ? 32 * a.BP : a.KLp + 1; }
+
+// Half word i of a group's bit string.  A tile of 2^bsh words (bsh = 30:
+// other tiles) takes one word more, so that the 32 tiles' rows fall into
+// different banks.
+__device__ __forceinline__ void slice_put16(const SliceArgs &a, uint32_t *B, int i, uint32_t x)
+{
+    reinterpret_cast<uint16_t *>(B)[i + 2 * (i >> (a.bsh + 1))] = (uint16_t)x;
+}
+
+// Units of 16 bytes from `from` on (of a buffer that is not 16-byte aligned:
+// all of them), byte by byte.
+__device__ __forceinline__ void slice_odd_units(const SliceArgs &a, const uint8_t *__restrict__ src, int bytes, int from,
+                                                uint32_t *B, int tid, int nth)
+{
+    for (int i = from + tid; 16 * i < bytes; i += nth) {
+        uint32_t x = 0;
+        for (int j = 0; j < 16 && 16 * i + j < bytes; ++j) x |= (uint32_t)(src[16 * i + j] != 0) << j;
+        slice_put16(a, B, i, x);
+    }
+}
+
+// The bytes of group g as a bit string in omega order, by nth threads.
+__device__ __forceinline__ void slice_bytes_to_string(const SliceArgs &a, const uint8_t *__restrict__ in, int64_t g,
+                                                      uint32_t *B, int tid, int nth)
+{
+    const int bytes = (int)min((int64_t)32, a.NT - 32 * g) * a.KL;
+    const uint8_t *src = in + 32 * g * a.KL;
+    const int whole = ((uintptr_t)in & 15) == 0 ? bytes / 16 : 0;
+#pragma unroll 4
+    for (int i = tid; i < whole; i += nth)
+        slice_put16(a, B, i, slice_bits16(__ldcs(reinterpret_cast<const uint4 *>(src) + i)));
+    slice_odd_units(a, src, bytes, whole, B, tid, nth);
+}
+
+// The same for blocks that walk the groups: every thread copies the 16-byte
+// units it will convert into its own slots of shared memory, two batches
+// ahead and across group boundaries, and waits for its own copies only.
+struct SliceRing {
+    uint8_t *slot;       // this thread's first slot of batch buffer 0
+    int64_t g;           // the batch to be copied next: its group, first unit, the group's units
+    int first, whole, buf;
+    static constexpr int kUnits = kSliceBatch * kSliceBlock;   // per batch
+    __device__ __forceinline__ int units(const SliceArgs &a, const uint8_t *in, int64_t gq) const
+    {
+        if (gq >= a.NG || ((uintptr_t)in & 15)) return 0;
+        return (int)min((int64_t)32, a.NT - 32 * gq) * a.KL / 16;
+    }
+    __device__ __forceinline__ void issue(const SliceArgs &a, const uint8_t *__restrict__ in, int b)
+    {
+        const int n = whole - first - (int)threadIdx.x;   // units left from this thread's first on
+        if (n > 0) {
+            const uint8_t *src = in + 32 * g * a.KL + 16 * (int64_t)(first + (int)threadIdx.x);
+            const uint32_t dst = smem_addr(slot) + 16 * kUnits * b;
+#pragma unroll
+            for (int k = 0; k < kSliceBatch; ++k)
+                if (kSliceBlock * k < n)
+                    asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(dst + 16 * kSliceBlock * k),
+                                 "l"(src + 16 * kSliceBlock * k)
+                                 : "memory");
+        }
+        asm volatile("cp.async.commit_group;" ::: "memory");
+        first += kUnits;
+        if (first >= whole) {
+            g += gridDim.x;
+            first = 0;
+            whole = units(a, in, g);
+        }
+    }
+    __device__ __forceinline__ void start(const SliceArgs &a, const uint8_t *__restrict__ in, void *ring)
+    {
+        slot = (uint8_t *)ring + 16 * threadIdx.x;
+        g = blockIdx.x;
+        first = 0;
+        whole = units(a, in, g);
+        buf = 0;
+        issue(a, in, 0);
+        issue(a, in, 1);
+    }
+    // the bit string of group gc (the groups in the order of the walk)
+    __device__ __forceinline__ void string(const SliceArgs &a, const uint8_t *__restrict__ in, int64_t gc, uint32_t *B)
+    {
+        const int n = units(a, in, gc);
+        for (int f = 0; f < n; f += kUnits, buf ^= 1) {
+            asm volatile("cp.async.wait_group 1;" ::: "memory");
+            const uint4 *p = reinterpret_cast<const uint4 *>(slot) + kUnits * buf;
+            const int left = n - f - (int)threadIdx.x;
+#pragma unroll
+            for (int k = 0; k < kSliceBatch; ++k)
+                if (kSliceBlock * k < left)
+                    slice_put16(a, B, f + (int)threadIdx.x + kSliceBlock * k, slice_bits16(p[kSliceBlock * k]));
+            issue(a, in, buf);
+        }
+        const int bytes = (int)min((int64_t)32, a.NT - 32 * gc) * a.KL;
+        slice_odd_units(a, in + 32 * gc * a.KL, bytes, n, B, threadIdx.x, kSliceBlock);
+    }
+};
+
+// Chunk c of the string, transposed: lane p gets cell 32 c + p of the tiles.
+__device__ __forceinline__ uint32_t slice_string_chunk(const SliceArgs &a, const Transpose32 &tr, const uint32_t *B, int c,
+                                                       int nt, int lane)
+{
+    const uint32_t b = (uint32_t)lane * a.lane_bits + 32u * (uint32_t)c;
+    const uint32_t *wp = B + (b >> 5);
+    const uint32_t x = __funnelshift_r(wp[0], wp[1], b & 31u);
+    return tr(lane < nt ? x : 0u);
+}
+
+// Bytes -> packed state: blocks walk the groups.  The cells of a group are
+// contiguous in omega (32 k^L bytes, a multiple of 32 from the buffer's
+// start); their bits go to shared memory in that order, and each warp then
+// takes 32 cells of 32 tiles at a time through the transposition.  Bound by
+// issue slots and the latency of its loads (carpet r = 10, 1.07e9 cells:
+// 0.20 ms, 5.9 TB/s read and written).
+__global__ void __launch_bounds__(kSliceBlock, 5)
+slice_pack_kernel(SliceArgs a, const uint8_t *__restrict__ in, uint32_t *__restrict__ bits)
+{
+    extern __shared__ __align__(16) uint32_t smem[];
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = blockDim.x >> 5;
+    const Transpose32 tr(lane);
+    SliceRing ring;
+    ring.start(a, in, smem);
+    uint32_t *N = smem + 8 * kSliceBatch * kSliceBlock;   // the packed words
+    uint32_t *B = N + a.KLp;
+    for (int64_t g = blockIdx.x; g < a.NG; g += gridDim.x) {
+        const int nt = (int)min((int64_t)32, a.NT - 32 * g);
+        ring.string(a, in, g, B);
+        __syncthreads();
+        uint32_t *dst = bits + g * a.KLp;
+#pragma unroll 2
+        for (int c = warp; c < a.NC; c += nw) {
+            const uint32_t x = slice_string_chunk(a, tr, B, c, nt, lane);
+            dst[32 * c + lane] = x;
+            N[32 * c + lane] = x;
+        }
+        __syncthreads();
+        slice_export(a, tr, N, bits + a.ex + g * a.XW * 32, warp, nw, lane);
+    }
+}
+
+// ---------------------------------------------------------------- step
+
+// Tile 32 g + lane's neighbour for halo word j, and the export word it sends.
+__device__ __forceinline__ int32_t slice_nbr(const SliceArgs &a, int64_t g, uint32_t job, int lane)
+{
+    return __ldg(a.nbr + (g * 8 + (job >> 8)) * 32 + lane);
+}
+__device__ __forceinline__ uint32_t slice_import(const SliceArgs &a, const uint32_t *ex, int32_t Q, uint32_t job)
+{
+    // (the exports may have been written by other blocks of this launch: loads go to L2)
+    return Q < 0 ? 0u : __ldcg(ex + ((int64_t)(Q >> 5) * a.XW + (job & 0xffu)) * 32 + (Q & 31));
+}
+
+// The group's words into shared memory, asynchronously.
+__device__ __forceinline__ void slice_load(const SliceArgs &a, uint32_t *A, const uint32_t *sg)
+{
+    for (int i = threadIdx.x; i < a.KLp / 4; i += blockDim.x)
+        asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(smem_addr(A + 4 * i)), "l"(sg + 4 * i) : "memory");
+    asm volatile("cp.async.commit_group;" ::: "memory");
+}
+
+// All blocks of the launch have arrived `n` times (n = 1, 2, ...): bounded.
+__device__ __forceinline__ bool slice_grid_barrier(const SliceArgs &a, uint32_t n)
+{
+    __syncthreads();
+    bool ok = true;
+    if (threadIdx.x == 0) {
+        __threadfence();
+        atomicAdd(a.bar, 1u);
+        const uint32_t want = n * gridDim.x;
+        ok = false;
+        for (uint32_t i = 0; i < kWaitLimit; ++i) {
+            uint32_t v;
+            asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(v) : "l"(a.bar) : "memory");
+            if ((int32_t)(v - want) >= 0) {
+                ok = true;
+                break;
+            }
+        }
+        if (!ok) atomicExch(a.status, FR_ETIMEOUT);
+        __threadfence();
+    }
+    return __syncthreads_or(!ok) == 0;
+}
+
+// 32 cells of a group from cell o of its omega order on, from the tiles' bit
+// strings (rows of RP words; bits past a tile's k^L cells are not defined).
+__device__ __forceinline__ uint32_t slice_take32(const SliceArgs &a, const uint32_t *R, uint32_t o, uint32_t nt)
+{
+    uint32_t t = divu(a.kdiv, o), l = o - t * (uint32_t)a.KL;
+    const uint32_t *p = R + t * (uint32_t)a.RP + (l >> 5);
+    uint32_t x = __funnelshift_r(p[0], p[1], l & 31u);
+    uint32_t have = (uint32_t)a.KL - l;   // cells of this tile from here on
+    while (have < 32u && ++t < nt) {
+        x = (x & ((1u << have) - 1u)) | R[t * (uint32_t)a.RP] << have;
+        have += (uint32_t)a.KL;
+    }
+    return x;
+}
+
+// Byte J of x, a nibble -> 4 bytes of 0/1: the byte alone, a carry-free
+// multiply, a mask.
+template <int J>
+__device__ __forceinline__ uint32_t slice_nib(uint32_t x)
+{
+    return (__byte_perm(x, 0u, 0x4440 | J) * 0x00204081u) & 0x01010101u;
+}
+
+// The group's new bytes from the tiles' bit strings: 32 cells per thread.
+__device__ __forceinline__ void slice_string_to_bytes(const SliceArgs &a, const uint32_t *R, uint8_t *__restrict__ out,
+                                                      int64_t g, int tid, int nth)
+{
+    const int nt = (int)min((int64_t)32, a.NT - 32 * g);
+    const int bytes = nt * a.KL;
+    uint8_t *ob = out + 32 * g * a.KL;
+    const int whole = ((uintptr_t)out & 15) == 0 ? bytes / 16 : 0;   // 16-byte units
+    const int lane = tid & 31;
+    // a warp's 32 x 32 cells; the lanes pass halves on so that consecutive
+    // lanes store consecutive 16 bytes
+#pragma unroll 2
+    for (int i = tid - lane; 2 * i < whole; i += nth) {
+        uint32_t x = 0u;
+        if (2 * (i + lane) < whole) x = slice_take32(a, R, 32u * (uint32_t)(i + lane), (uint32_t)nt);
+#pragma unroll
+        for (int h = 0; h < 2; ++h) {
+            const uint32_t y = __shfl_sync(0xffffffffu, x, 16 * h + (lane >> 1)) >> (16 * (lane & 1));
+            const int u = 2 * i + 32 * h + lane;
+            const uint32_t e = y & 0x0f0fu, o = (y >> 4) & 0x0f0fu;
+            if (u < whole)
+                __stcs(reinterpret_cast<uint4 *>(ob) + u,
+                       make_uint4(slice_nib<0>(e), slice_nib<0>(o), slice_nib<1>(e), slice_nib<1>(o)));
+        }
+    }
+    for (int i = 16 * whole + tid; i < bytes; i += nth) {
+        const uint32_t t = divu(a.kdiv, (uint32_t)i), l = (uint32_t)i - t * (uint32_t)a.KL;
+        ob[i] = (uint8_t)((R[t * (uint32_t)a.RP + (l >> 5)] >> (l & 31u)) & 1u);
+    }
+}
+
+// Next state of cells 32 c .. 32 c + 31 of a group's tiles from its words A.
+template <int D, bool LIFE>
+__device__ __forceinline__ uint32_t slice_next(const SliceArgs &a, const uint4 tab, const uint32_t *A, int c, int lane)
+{
+    const uint32_t r[4] = {tab.x, tab.y, tab.z, tab.w};
+    uint32_t n[8];
+#pragma unroll
+    for (int k = 0; k < D; ++k)
+        n[k] = *reinterpret_cast<const uint32_t *>(reinterpret_cast<const uint8_t *>(A) +
+                                                   ((k & 1) ? r[k / 2] >> 16 : r[k / 2] & 0xffffu));
+    return slice_rule<D, LIFE>(a, n, A[32 * c + lane]);
+}
+
+// `gens` generations of a packed state, blocks walking the groups; between
+// generations the launch's blocks meet at a grid barrier (a cooperative
+// launch when there is more than one block).  BYTES: one generation whose
+// results leave as bytes.
+template <int D, bool LIFE, bool BYTES>
+__global__ void __launch_bounds__(kSliceBlock, LIFE ? 5 : 4)
+slice_step_kernel(SliceArgs a, const uint32_t *src, uint32_t *dst, uint8_t *__restrict__ out, int gens)
+{
+    extern __shared__ __align__(16) uint32_t smem[];
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, nw = blockDim.x >> 5;
+    const Transpose32 tr(lane);
+    uint32_t *N = smem + 2 * a.AW;   // the new words; BYTES: the results' bit strings
+    uint32_t *R = N;
+    if (tid < 64) smem[(tid >> 5) * a.AW + a.A_zero + lane] = 0u;   // the words of absent neighbours
+    uint32_t job[kSliceAhead];
+#pragma unroll
+    for (int i = 0; i < kSliceAhead; ++i) job[i] = warp + i * nw < a.NJ ? __ldg(a.jobs + warp + i * nw) : 0u;
+    uint32_t buf = 0;
+    for (int gen = 0; gen < gens; ++gen) {
+        uint32_t e[kSliceAhead];   // halo words of the next group, loaded ahead
+        if (blockIdx.x < a.NG) {
+            slice_load(a, smem + buf * a.AW, src + (int64_t)blockIdx.x * a.KLp);
+#pragma unroll
+            for (int i = 0; i < kSliceAhead; ++i)
+                e[i] = warp + i * nw < a.NJ ? slice_import(a, src + a.ex, slice_nbr(a, blockIdx.x, job[i], lane), job[i]) : 0u;
+        }
+        for (int64_t g = blockIdx.x; g < a.NG; g += gridDim.x, buf ^= 1) {
+            uint32_t *A = smem + buf * a.AW;
+            const int64_t gn = g + gridDim.x;
+#pragma unroll
+            for (int i = 0; i < kSliceAhead; ++i)
+                if (warp + i * nw < a.NJ) A[a.KLp + 32 * (warp + i * nw) + lane] = tr(e[i]);
+            for (int j = warp + kSliceAhead * nw; j < a.NJ; j += nw) {
+                const uint32_t jb = __ldg(a.jobs + j);
+                A[a.KLp + 32 * j + lane] = tr(slice_import(a, src + a.ex, slice_nbr(a, g, jb, lane), jb));
+            }
+            asm volatile("cp.async.wait_all;" ::: "memory");
+            __syncthreads();
+            int32_t Q[kSliceAhead];
+            if (gn < a.NG) {
+                slice_load(a, smem + (buf ^ 1) * a.AW, src + gn * a.KLp);
+#pragma unroll
+                for (int i = 0; i < kSliceAhead; ++i) Q[i] = warp + i * nw < a.NJ ? slice_nbr(a, gn, job[i], lane) : -1;
+            }
+            uint32_t *dg = BYTES ? nullptr : dst + g * a.KLp;
+#pragma unroll 2
+            for (int c = warp; c < a.NC; c += nw) {
+                const uint32_t w = slice_next<D, LIFE>(a, __ldg(a.tab + 32 * c + lane), A, c, lane);
+                if (BYTES) {
+                    R[lane * a.RP + c] = tr(w);
+                } else {
+                    dg[32 * c + lane] = w;
+                    N[32 * c + lane] = w;
+                }
+            }
+            if (gn < a.NG) {
+#pragma unroll
+                for (int i = 0; i < kSliceAhead; ++i) e[i] = slice_import(a, src + a.ex, Q[i], job[i]);
+            }
+            __syncthreads();
+            if (BYTES) {
+                slice_string_to_bytes(a, R, out, g, tid, blockDim.x);
+            } else {
+                slice_export(a, tr, N, dst + a.ex + g * a.XW * 32, warp, nw, lane);
+            }
+        }
+        if (!BYTES && gen + 1 < gens) {
+            if (gridDim.x > 1) {
+                if (!slice_grid_barrier(a, (uint32_t)gen + 1u)) break;
+            } else {
+                __syncthreads();
+            }
+            const uint32_t *t = src;
+            src = dst;
+            dst = const_cast<uint32_t *>(t);
+        }
+    }
+    if (!BYTES && gens > 1 && gridDim.x > 1 && tid == 0) {
+        // the last block to leave resets the barrier for the next launch
+        if (atomicAdd(a.bar + 1, 1u) == gridDim.x - 1) {
+            a.bar[0] = 0u;
+            a.bar[1] = 0u;
+            __threadfence();
+        }
+    }
+}
+
+// One generation from bytes to bytes in one pass, for fractals whose tiles
+// have a halo of at most 32 cells (the triangle 8, the Vicsek fractal 4):
+// those cells are read as bytes from the neighbouring tiles (lane t follows
+// tile 32 g + t, a ballot makes the word), the rest as in the two-pass
+// kernels.  The bit strings of the old and of the new state share a place.
+// Issue-bound (60 % of the slots, HBM at 79 %): triangle r = 20 in 1.31 ms
+// against 1.49 ms of the tap kernel and 1.45 ms of the two-pass kernels.
+// Tiles of 2187 cells: with 729 it took 1.57 ms (a group's fixed work, about
+// 1600 instructions, per fewer cells), with 6561 1.72 ms (the neighbour table
+// no longer stays near the SM).
+template <int D, bool LIFE>
+__global__ void __launch_bounds__(kSliceBlock, LIFE ? 5 : 4)
+slice_single_kernel(SliceArgs a, const uint8_t *__restrict__ in, uint8_t *__restrict__ out)
+{
+    extern __shared__ __align__(16) uint32_t smem[];
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, nw = blockDim.x >> 5;
+    const Transpose32 tr(lane);
+    SliceRing ring;
+    ring.start(a, in, smem);
+    uint32_t *A = smem + 8 * kSliceBatch * kSliceBlock, *B = A + a.AW;
+    if (tid < 32) A[a.A_zero + tid] = 0u;   // the words of absent neighbours
+    // this warp's first halo cell of the next group, loaded ahead
+    const uint2 h0 = warp < a.H ? __ldg(a.cells + warp) : make_uint2(0u, 0u);
+    uint32_t hv = 0u;
+    auto halo = [&](int64_t g, uint2 h) -> uint32_t {
+        const int32_t Q = __ldg(a.nbr + (g * 8 + (h.y >> 16)) * 32 + lane);
+        return Q < 0 ? 0u : (uint32_t)__ldg(in + (int64_t)Q * a.KL + h.x);
+    };
+    if (warp < a.H && blockIdx.x < a.NG) hv = halo(blockIdx.x, h0);
+    for (int64_t g = blockIdx.x; g < a.NG; g += gridDim.x) {
+        const int nt = (int)min((int64_t)32, a.NT - 32 * g);
+        const int64_t gn = g + gridDim.x;
+        ring.string(a, in, g, B);
+        if (warp < a.H) {
+            const uint32_t b = __ballot_sync(0xffffffffu, hv != 0u);
+            if (lane == 0) A[h0.y & 0xffffu] = b;
+            if (gn < a.NG) hv = halo(gn, h0);
+        }
+        for (int h = warp + nw; h < a.H; h += nw) {
+            const uint2 e = __ldg(a.cells + h);
+            const uint32_t b = __ballot_sync(0xffffffffu, halo(g, e) != 0u);
+            if (lane == 0) A[e.y & 0xffffu] = b;
+        }
+        __syncthreads();
+#pragma unroll 2
+        for (int c = warp; c < a.NC; c += nw) A[32 * c + lane] = slice_string_chunk(a, tr, B, c, nt, lane);
+        __syncthreads();
+#pragma unroll 2
+        for (int c = warp; c < a.NC; c += nw)
+            B[lane * a.RP + c] = tr(slice_next<D, LIFE>(a, __ldg(a.tab + 32 * c + lane), A, c, lane));
+        __syncthreads();
+        slice_string_to_bytes(a, B, out, g, tid, blockDim.x);
+        __syncthreads();
+    }
+}
+
+// States whose packed words fit in the SMs' shared memory together: one
+// launch packs the bytes, runs all generations and writes the bytes.  A block
+// owns fixed groups, whose words stay in shared memory and are replaced in
+// place (the new words wait in registers until the block has read the old
+// ones; the groups' bit strings of the first and the last step take the same
+// place); only the exports go through memory (ex0 / ex1 in turn), with a grid
+// barrier per generation.  The neighbour table, the export lists and the
+// places of the tiles' halo words in the exports are kept in shared memory as
+// well: with so much of it in use little is left of L1.  ONE: a single block;
+// its exports stay in shared memory too.  Bound by issue slots and, for small
+// states, by the barrier and the chain of latencies around it.  Microseconds
+// per generation, byte-wise tile kernels -> here: triangle r = 8 6.1 -> 0.5,
+// r = 16 23 -> 6.3, carpet r = 9 96 -> 14, H-fractal r = 9 107 -> 8.
+
+// A block's items (item j of its group q, n per group) dealt to its warps, a
+// run of `rounds` items each; past the last item a warp repeats it.
+struct SliceWalk {
+    int q, j, n, groups;
+    __device__ __forceinline__ SliceWalk(int n_, int groups_, int first) : q(first / n_), j(first % n_), n(n_), groups(groups_)
+    {
+        clamp();
+    }
+    __device__ __forceinline__ void clamp()
+    {
+        if (q >= groups) {
+            q = groups - 1;
+            j = n - 1;
+        }
+    }
+    __device__ __forceinline__ void next()
+    {
+        if (++j == n) {
+            j = 0;
+            ++q;
+            clamp();
+        }
+    }
+};
+
+template <int D, bool LIFE, bool ONE, int ROUNDS>
+__global__ void __launch_bounds__(1024, 1)
+slice_resident_kernel(SliceArgs a, const uint8_t *__restrict__ in, uint8_t *__restrict__ out, uint32_t *ex0, uint32_t *ex1,
+                      int per_block, int64_t steps)
+{
+    extern __shared__ __align__(16) uint32_t smem[];
+    const int tid = threadIdx.x, nth = blockDim.x, lane = tid & 31, warp = tid >> 5, nw = nth >> 5;
+    const Transpose32 tr(lane);
+    uint4 *tab = reinterpret_cast<uint4 *>(smem);
+    uint32_t *exs = smem + 4 * a.KLp;   // ONE: both export buffers
+    const int exw = ONE ? (int)a.NG * a.XW * 32 : 0;
+    uint16_t *xlist = reinterpret_cast<uint16_t *>(exs + 2 * exw);
+    int32_t *from = reinterpret_cast<int32_t *>(exs + 2 * exw + a.XW * 16);
+    uint32_t *A0 = exs + 2 * exw + a.XW * 16 + per_block * a.NJ * 32;
+    if (ONE) {
+        ex0 = exs;
+        ex1 = exs + exw;
+    }
+    const int64_t g0 = blockIdx.x, gs = gridDim.x;
+    const int mine = (int)min((int64_t)per_block, (a.NG - g0 + gs - 1) / gs);   // this block's groups
+    const int rounds = (mine * a.NC + nw - 1) / nw;
+    for (int i = tid; i < a.KLp; i += nth) tab[i] = __ldg(a.tab + i);
+    for (int i = tid; i < a.XW * 32; i += nth) xlist[i] = __ldg(a.xlist + i);
+    for (int x = warp; x < mine * a.NJ; x += nw) {
+        const int q = x / a.NJ;
+        const uint32_t jb = __ldg(a.jobs + (x - q * a.NJ));
+        const int32_t Q = slice_nbr(a, g0 + q * gs, jb, lane);
+        from[x * 32 + lane] = Q < 0 ? -1 : ((Q >> 5) * a.XW + (int)(jb & 0xffu)) * 32 + (Q & 31);
+    }
+    for (int q = 0; q < mine; ++q) slice_bytes_to_string(a, in, g0 + q * gs, A0 + q * a.AW, tid, nth);
+    __syncthreads();
+    uint32_t w[ROUNDS];
+    const SliceWalk chunk0(a.NC, mine, warp * rounds);
+    {
+        SliceWalk k = chunk0;
+        const int nt_last = (int)(a.NT - 32 * (a.NG - 1));   // tiles of the last group, the last one of its block
+        const int short_q = (g0 + (mine - 1) * gs == a.NG - 1) ? mine - 1 : -1;
+#pragma unroll
+        for (int i = 0; i < ROUNDS; ++i)
+            if (i < rounds) {
+                w[i] = slice_string_chunk(a, tr, A0 + k.q * a.AW, k.j, k.q == short_q ? nt_last : 32, lane);
+                k.next();
+            }
+    }
+    __syncthreads();
+    for (int q = warp; q < mine; q += nw) A0[q * a.AW + a.A_zero + lane] = 0u;   // the words of absent neighbours
+    auto put_words = [&]() {
+        SliceWalk k = chunk0;
+#pragma unroll
+        for (int i = 0; i < ROUNDS; ++i)
+            if (i < rounds) {
+                A0[k.q * a.AW + 32 * k.j + lane] = w[i];
+                k.next();
+            }
+    };
+    const int ex_rounds = (mine * a.XW + nw - 1) / nw, im_rounds = (mine * a.NJ + nw - 1) / nw;
+    const SliceWalk ex_walk0(max(a.XW, 1), mine, warp * ex_rounds), im_walk0(max(a.NJ, 1), mine, warp * im_rounds);
+    auto put_exports = [&](uint32_t *ex) {
+        SliceWalk k = ex_walk0;
+        for (int i = 0; i < ex_rounds; ++i, k.next()) {
+            const uint32_t v = tr(A0[k.q * a.AW + xlist[32 * k.j + lane]]);
+            if (ONE) ex[(k.q * a.XW + k.j) * 32 + lane] = v;
+            else __stcg(ex + ((g0 + k.q * gs) * a.XW + k.j) * 32 + lane, v);
+        }
+    };
+    put_words();
+    __syncthreads();
+    put_exports(ex0);
+    for (int64_t gen = 1; gen <= steps; ++gen) {
+        // everybody's exports of the state before this generation are there
+        if (ONE) __syncthreads();
+        else if (!slice_grid_barrier(a, (uint32_t)gen)) break;
+        const uint32_t *ei = (gen & 1) ? ex0 : ex1;
+        {
+            SliceWalk k = im_walk0;
+#pragma unroll 2
+            for (int i = 0; i < im_rounds; ++i, k.next()) {
+                const int at = from[(k.q * a.NJ + k.j) * 32 + lane];
+                uint32_t e = 0u;
+                if (at >= 0) e = ONE ? ei[at] : __ldcg(ei + at);
+                A0[k.q * a.AW + a.KLp + 32 * k.j + lane] = tr(e);
+            }
+        }
+        __syncthreads();
+        {
+            SliceWalk k = chunk0;
+#pragma unroll
+            for (int i = 0; i < ROUNDS; ++i)
+                if (i < rounds) {
+                    w[i] = slice_next<D, LIFE>(a, tab[32 * k.j + lane], A0 + k.q * a.AW, k.j, lane);
+                    k.next();
+                }
+        }
+        __syncthreads();
+        if (gen < steps) {
+            put_words();
+            __syncthreads();
+            put_exports((gen & 1) ? ex1 : ex0);
+        }
+    }
+    {
+        SliceWalk k = chunk0;
+#pragma unroll
+        for (int i = 0; i < ROUNDS; ++i)
+            if (i < rounds) {
+                A0[k.q * a.AW + lane * a.RP + k.j] = tr(w[i]);
+                k.next();
+            }
+    }
+    __syncthreads();
+    for (int q = 0; q < mine; ++q) slice_string_to_bytes(a, A0 + q * a.AW, out, g0 + q * gs, tid, nth);
+    if (!ONE && tid == 0) {
+        // the last block to leave resets the barrier for the next launch
+        if (atomicAdd(a.bar + 1, 1u) == gridDim.x - 1) {
+            a.bar[0] = 0u;
+            a.bar[1] = 0u;
+            __threadfence();
+        }
+    }
+}
+
+// Neighbours of every tile, a row of 32 lanes per group and direction
+// (tiles past the last have none), from rows of 8 per tile.
+__global__ void slice_nbr_kernel(FracDev F, int64_t NT, int64_t NG, int coarse_levels, int32_t coarse_side, int32_t *__restrict__ out)
+{
+    for (int64_t T = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; T < 32 * NG; T += (int64_t)gridDim.x * blockDim.x) {
+        int32_t c[3] = {0, 0, 0};
+        if (T < NT) lambda64(F, (uint64_t)T, coarse_levels, c);
+        for (int d = 0; d < 8; ++d) {
+            const int q = d < 4 ? d : d + 1;
+            const int32_t x = c[0] + q % 3 - 1, y = c[1] + q / 3 - 1;
+            int64_t v = -1;
+            if (T < NT && x >= 0 && x < coarse_side && y >= 0 && y < coarse_side) v = nu_levels(F, x, y, 0, coarse_levels);
+            out[((T >> 5) * 8 + d) * 32 + (T & 31)] = (int32_t)v;
+        }
+    }
+}
+
+// ---------------------------------------------------------------- plan
+
+static int64_t pw(int64_t b, int e)
+{
+    int64_t v = 1;
+    for (int i = 0; i < e; ++i) v *= b;
+    return v;
+}
+
+// Neighbours of the cells of an m-level box: entry [l][d9] (d9 = (dx + 1) +
+// 3 (dy + 1)) is the neighbour's number in the box that holds it | that box's
+// direction << 24 (4: the same box), or -1 where the fractal has none.
+using SliceNbrs = std::vector<int32_t>;
+
+// One level more: level 0 digits move as `first` says, and where they leave
+// their block the rest moves as it does with m - 1 levels.
+static SliceNbrs slice_deepen(const SliceNbrs &first, const SliceNbrs &rest, int k)
+{
+    const size_t n = rest.size() / 9;
+    SliceNbrs out(n * k * 9);
+    for (size_t r = 0; r < n; ++r)
+        for (int j = 0; j < k; ++j)
+            for (int d = 0; d < 9; ++d) {
+                const int32_t a = first[(size_t)j * 9 + d];
+                int32_t v = -1;
+                if (a >= 0) {
+                    const int32_t b = (a >> 24) == 4 ? (int32_t)r | 4 << 24 : rest[r * 9 + (a >> 24)];
+                    if (b >= 0) v = ((b & 0xffffff) * k + (a & 0xffffff)) | (b & ~0xffffff);
+                }
+                out[(r * k + j) * 9 + d] = v;
+            }
+    return out;
+}
+
+// The neighbours in a single block of s x s digits.
+static SliceNbrs slice_first(const fractal *f)
+{
+    SliceNbrs out((size_t)f->k * 9, -1);
+    for (int j = 0; j < f->k; ++j)
+        for (int d = 0; d < 9; ++d) {
+            int q[2] = {f->offsets[(size_t)2 * j] + d % 3 - 1, f->offsets[(size_t)2 * j + 1] + d / 3 - 1}, b[2];
+            for (int i = 0; i < 2; ++i) {
+                b[i] = q[i] < 0 ? -1 : (q[i] >= f->s ? 1 : 0);
+                q[i] -= b[i] * f->s;
+            }
+            const int h = f->dev.hinv[q[0] + f->s * q[1]];
+            if (h >= 0) out[(size_t)j * 9 + d] = h | ((b[0] + 1) + 3 * (b[1] + 1)) << 24;
+        }
+    return out;
+}
+
+struct SliceTables {
+    int KL = 0, H = 0, D = 0;
+    int zero = 0;                   // the first of 32 zero words in a group's array
+    SliceNbrs nb;
+    std::vector<int32_t> hidx;      // [9][KL]: word of a halo cell (by its box's direction), -1 = none
+    std::vector<uint32_t> jobs;     // halo words: export word | direction slot << 8
+    std::vector<uint16_t> xlist;    // [XW][32] cells of the export words
+    std::vector<uint32_t> cells;    // halo cells: cell of the neighbouring tile, word index | direction slot << 16
+    int XW() const { return (int)xlist.size() / 32; }
+};
+
+static SliceTables slice_tables(SliceNbrs &&nbrs)
+{
+    SliceTables t;
+    t.nb = std::move(nbrs);
+    t.KL = (int)(t.nb.size() / 9);
+    const int KL = t.KL, KLp = (KL + 31) / 32 * 32;
+    t.hidx.assign((size_t)9 * KL, -1);
+    for (int l = 0; l < KL; ++l) {
+        int n = 0;
+        for (int d = 0; d < 9; ++d) {
+            const int32_t v = d == 4 ? -1 : t.nb[(size_t)l * 9 + d];
+            if (v < 0) continue;
+            ++n;
+            if ((v >> 24) != 4) t.hidx[(size_t)(v >> 24) * KL + (v & 0xffffff)] = 0;
+        }
+        t.D = std::max(t.D, n);
+    }
+    // export words: the directions with the most border cells first, their
+    // cells in runs of 32; a run whose cells all lie in an earlier word uses
+    // that one (a corner cell is in its sides' words)
+    std::vector<int> cells[9];
+    int order[8] = {0, 1, 2, 3, 5, 6, 7, 8};
+    for (int d : order)
+        for (int l = 0; l < KL; ++l)
+            if (t.hidx[(size_t)d * KL + l] >= 0) cells[d].push_back(l);
+    std::stable_sort(order, order + 8, [&](int x, int y) { return cells[x].size() > cells[y].size(); });
+    std::vector<std::vector<int>> words;
+    for (int d : order)
+        for (size_t i = 0; i < cells[d].size(); i += 32) {
+            const std::vector<int> run(cells[d].begin() + i, cells[d].begin() + std::min(i + 32, cells[d].size()));
+            int w = -1;
+            for (int x = 0; x < (int)words.size() && w < 0; ++x)
+                if (std::includes(words[x].begin(), words[x].end(), run.begin(), run.end())) w = x;
+            if (w < 0) {
+                w = (int)words.size();
+                words.push_back(run);
+            }
+            const uint32_t slot = (uint32_t)(d < 4 ? d : d - 1);
+            for (int l : run) {
+                const int at = KLp + 32 * (int)t.jobs.size() +
+                               (int)(std::lower_bound(words[w].begin(), words[w].end(), l) - words[w].begin());
+                t.hidx[(size_t)d * KL + l] = at;
+                t.cells.push_back((uint32_t)l);
+                t.cells.push_back((uint32_t)at | slot << 16);
+            }
+            t.jobs.push_back((uint32_t)w | slot << 8);
+            t.H += (int)run.size();
+        }
+    for (const auto &w : words)
+        for (int i = 0; i < 32; ++i) t.xlist.push_back((uint16_t)w[std::min<size_t>(i, w.size() - 1)]);
+    t.zero = KLp + std::max(32 * (int)t.jobs.size(), 64);
+    return t;
+}
+
+// The neighbour table [KLp][8] (byte offsets): the 32 cells of a chunk are
+// added by 32 lanes, one neighbour per lane and load, and the order of a
+// cell's neighbours is free; each goes to the load that has the fewest words
+// in its bank so far (triangle: 9.4 -> 6.0 shared-memory wavefronts per chunk,
+// carpet 14.6 -> 8.6).  The loads a cell has no neighbour for read a zero word
+// from the emptiest bank.
+static void slice_neighbour_table(const SliceTables &t, int D, uint16_t *tab)
+{
+    const int KLp = (t.KL + 31) / 32 * 32, all = (1 << D) - 1;
+    std::vector<uint8_t> loaded((size_t)t.zero + 32, 0);   // per word: the loads of this chunk that read it
+    for (int c = 0; c < KLp; c += 32) {
+        // [bank][x]: the loads that read x words of the bank, as a bit set
+        uint8_t with[32][33] = {};
+        int v[32][8], put[32][8], n[32];
+        for (int b = 0; b < 32; ++b) with[b][0] = (uint8_t)all;
+        for (int i = 0; i < 32; ++i) {
+            n[i] = 0;
+            for (int d = 0; d < 9 && c + i < t.KL; ++d) {
+                const int32_t a = d == 4 ? -1 : t.nb[(size_t)(c + i) * 9 + d];
+                if (a < 0) continue;
+                v[i][n[i]++] = (a >> 24) == 4 ? a & 0xffffff : t.hidx[(size_t)(a >> 24) * t.KL + (a & 0xffffff)];
+            }
+        }
+        for (int want = D; want >= 1; --want)   // cells with the most neighbours first
+            for (int i = 0; i < 32; ++i) {
+                if (n[i] != want) continue;
+                int open = all;
+                for (int e = 0; e < n[i]; ++e) {
+                    const int w = v[i][e], b = w & 31;
+                    int pick = open & loaded[w];
+                    if (!pick) {
+                        int x = 0;
+                        while (!(pick = open & with[b][x])) ++x;
+                        pick &= -pick;
+                        with[b][x] &= (uint8_t)~pick;
+                        with[b][x + 1] |= (uint8_t)pick;
+                        loaded[w] |= (uint8_t)pick;
+                    }
+                    pick &= -pick;
+                    open &= ~pick;
+                    int k = 0;
+                    while (!((pick >> k) & 1)) ++k;
+                    put[i][e] = k;
+                }
+            }
+        for (int i = 0; i < 32; ++i)
+            for (int e = 0; e < n[i]; ++e) loaded[v[i][e]] = 0;
+        for (int k = 0; k < D; ++k) {
+            int z = 0, least = 33;
+            for (int b = 0; b < 32; ++b) {
+                int x = 0;
+                while (!((with[(t.zero + b) & 31][x] >> k) & 1)) ++x;
+                if (x < least) {
+                    least = x;
+                    z = b;
+                }
+            }
+            for (int i = 0; i < 32; ++i) tab[(size_t)(c + i) * 8 + k] = (uint16_t)(4 * (t.zero + z));
+        }
+        for (int k = D; k < 8; ++k)
+            for (int i = 0; i < 32; ++i) tab[(size_t)(c + i) * 8 + k] = (uint16_t)(4 * t.zero);
+        for (int i = 0; i < 32; ++i)
+            for (int e = 0; e < n[i]; ++e) tab[(size_t)(c + i) * 8 + put[i][e]] = (uint16_t)(4 * v[i][e]);
+    }
+}
+
+void free_slice_plan(SlicePlan &p)
+{
+    cudaFree(p.arena);
+    cudaFree(p.bits[0]);
+    cudaFree(p.bits[1]);
+    p = SlicePlan();
+}
+
+using StepFn = void (*)(SliceArgs, const uint32_t *, uint32_t *, uint8_t *, int);
+
+template <int D>
+static StepFn step_fn_d(bool life, bool bytes)
+{
+    if (bytes) return life ? slice_step_kernel<D, true, true> : slice_step_kernel<D, false, true>;
+    return life ? slice_step_kernel<D, true, false> : slice_step_kernel<D, false, false>;
+}
+
+static StepFn step_fn(int D, bool life, bool bytes)
+{
+    switch (D) {
+        case 4: return step_fn_d<4>(life, bytes);
+        case 6: return step_fn_d<6>(life, bytes);
+        case 7: return step_fn_d<7>(life, bytes);
+        default: return step_fn_d<8>(life, bytes);
+    }
+}
+
+using SingleFn = void (*)(SliceArgs, const uint8_t *, uint8_t *);
+
+static SingleFn single_fn(int D, bool life)
+{
+    switch (D) {
+        case 4: return life ? slice_single_kernel<4, true> : slice_single_kernel<4, false>;
+        case 6: return life ? slice_single_kernel<6, true> : slice_single_kernel<6, false>;
+        case 7: return life ? slice_single_kernel<7, true> : slice_single_kernel<7, false>;
+        default: return life ? slice_single_kernel<8, true> : slice_single_kernel<8, false>;
+    }
+}
+
+using ResidentFn = void (*)(SliceArgs, const uint8_t *, uint8_t *, uint32_t *, uint32_t *, int, int64_t);
+
+// rounds: 32-cell chunks per warp
+template <int D, bool ONE>
+static ResidentFn resident_fn_d(bool life, int rounds)
+{
+    if (rounds <= 1) return life ? slice_resident_kernel<D, true, ONE, 1> : slice_resident_kernel<D, false, ONE, 1>;
+    if (ONE || rounds <= 8) return life ? slice_resident_kernel<D, true, ONE, 8> : slice_resident_kernel<D, false, ONE, 8>;
+    if (rounds <= 20) return life ? slice_resident_kernel<D, true, false, 20> : slice_resident_kernel<D, false, false, 20>;
+    return life ? slice_resident_kernel<D, true, false, kSliceRounds> : slice_resident_kernel<D, false, false, kSliceRounds>;
+}
+
+static ResidentFn resident_fn(const SlicePlan &s, bool life)
+{
+    const bool one = s.grid_resident == 1;
+    switch (s.geo.D) {
+        case 4: return one ? resident_fn_d<4, true>(life, s.rounds) : resident_fn_d<4, false>(life, s.rounds);
+        case 6: return one ? resident_fn_d<6, true>(life, s.rounds) : resident_fn_d<6, false>(life, s.rounds);
+        case 7: return one ? resident_fn_d<7, true>(life, s.rounds) : resident_fn_d<7, false>(life, s.rounds);
+        default: return one ? resident_fn_d<8, true>(life, s.rounds) : resident_fn_d<8, false>(life, s.rounds);
+    }
+}
+
+static bool slice_fractal_ok(const fractal *f) { return f->dim == 2 && !f->mixed && f->k >= 2 && f->r >= 1; }
+
+// Geometry of the tables of one tile depth.
+static SliceGeo slice_geo(const fractal *f, int L, const SliceTables &t)
+{
+    SliceGeo p;
+    p.L = L;
+    p.KL = t.KL;
+    p.NC = (t.KL + 31) / 32;
+    p.KLp = 32 * p.NC;
+    p.NJ = (int)t.jobs.size();
+    p.XW = t.XW();
+    p.H = t.H;
+    p.D = t.D <= 4 ? 4 : (t.D <= 6 ? 6 : t.D);
+    p.NT = pw(f->k, f->r - L);
+    p.NG = (p.NT + 31) / 32;
+    p.AW = p.KLp + std::max(32 * p.NJ, 64) + 32;   // at least a group's bit strings
+    // tiles of 2, 4, 8, ... words: the rows of 32 lanes would share banks
+    p.BP = p.KL >= 64 && (p.KL & (p.KL - 1)) == 0 ? p.KL / 32 + 1 : 0;
+    p.RP = (p.NC + 1) | 1;
+    return p;
+}
+static int string_words(const SliceGeo &p) { return p.BP ? 32 * p.BP : p.KLp + 1; }
+
+constexpr int kSliceMaxKL = 4096;
+constexpr int kSliceWave = 760;
+constexpr int kSliceSmem = 220 * 1024;   // resident kernel: shared memory per block
+
+// Blocks, groups per block and threads of the resident kernel, and its
+// estimated cycles per generation; false when the state does not fit.
+static bool slice_resident_shape(const SliceGeo &p, int num_sms, SlicePlan *s, double *cost)
+{
+    // one block where that takes no more than 8 chunks per warp, else as many as there are SMs
+    for (int64_t grid : {(int64_t)1, std::min<int64_t>(num_sms, p.NG)}) {
+        const int64_t per = (p.NG + grid - 1) / grid, chunks = per * p.NC;
+        const int64_t rounds = (chunks + 31) / 32;
+        if (rounds > (grid == 1 ? 8 : kSliceRounds)) continue;
+        const int64_t exw = grid == 1 ? 2 * p.NG * p.XW * 32 : 0;
+        const int64_t smem = 4 * (4 * p.KLp + exw + 16 * p.XW + per * (32 * p.NJ + p.AW));
+        if (smem > kSliceSmem) continue;
+        // `n` warp-sized items of `instr` instructions: at least a chain of
+        // latencies per round, else the SM's issue rate
+        auto cycles = [](double n, double instr) {
+            return std::ceil(n / 32) * std::max(170.0, std::min(n, 32.0) * instr / 2.8);
+        };
+        const double c = (grid > 1 ? 3000 : 100) + cycles((double)chunks, 55) + cycles((double)per * p.NJ, 35) +
+                         cycles((double)per * p.XW, 35);
+        if (s->resident && c >= *cost) continue;
+        *cost = c;
+        s->resident = true;
+        s->per_block = (int)per;
+        s->grid_resident = (int)grid;
+        s->smem_resident = (int)smem;
+        s->rounds = (int)rounds;
+        s->block_resident = (int)std::min<int64_t>(1024, std::max<int64_t>(128, (chunks + 3) / 4 * 128));
+    }
+    return s->resident;
+}
+
+// Tables for the tile depth that costs least per generation: the resident
+// kernel's where the state fits in shared memory, else the streaming one's (a
+// group of 32 tiles adds its cells' neighbours, about 45 instructions per 32
+// cells, makes and takes its halo words, about 30 each, and pays its loops
+// and barriers, about 400; kSliceWave groups run at a time).
+static int slice_levels(const fractal *f, SlicePlan *plan, SliceTables *tables)
+{
+    int best = 0;
+    double cost = 0;
+    const SliceNbrs first = slice_first(f);
+    SliceNbrs nbrs = first;
+    for (int L = 1; L <= f->r && pw(f->k, L) <= kSliceMaxKL; ++L) {
+        if (L > 1) nbrs = slice_deepen(first, nbrs, f->k);
+        if ((double)pw(f->k, f->r - L) >= 2147483648.0) continue;
+        SliceTables t = slice_tables(SliceNbrs(nbrs));
+        const SliceGeo p = slice_geo(f, L, t);
+        if (p.AW * 4 > 65535 || p.XW > 255) continue;
+        SlicePlan s;
+        double c;
+        if (!slice_resident_shape(p, f->num_sms, &s, &c)) {
+            const int64_t waves = (p.NG + kSliceWave - 1) / kSliceWave;
+            c = (double)waves * (p.NC * 45 + 30.0 * (p.NJ + p.XW) + 400);
+        }
+        if (best && plan->resident && !s.resident) continue;
+        if (!best || (s.resident && !plan->resident) || c < cost) {
+            best = L;
+            cost = c;
+            *plan = s;
+            plan->geo = p;
+            *tables = std::move(t);
+        }
+    }
+    return best;
+}
+
+static int build_slice_plan(fractal *f, cudaStream_t st)
+{
+    SliceTables t;
+    SlicePlan s;
+    if (slice_levels(f, &s, &t) < 1) return FR_EINVAL;
+    SliceGeo &p = s.geo;
+    const int ring = 32 * kSliceBatch * kSliceBlock;
+    s.smem_pack = ring + 4 * (string_words(p) + p.KLp);
+    s.smem_single = ring + 4 * (p.AW + std::max(string_words(p), 32 * p.RP + 1));
+    s.smem_step = 4 * (2 * p.AW + p.KLp);
+    s.smem_bytes = 4 * (2 * p.AW + 32 * p.RP + 1);
+    // one allocation: the tables (copied from the host in one piece), the
+    // grid barrier's zeros, the neighbouring tiles and the resident exports
+    size_t off = 0;
+    auto take = [&](size_t bytes) {
+        const size_t at = off;
+        off += (bytes + 255) / 256 * 256;
+        return at;
+    };
+    const size_t o_tab = take((size_t)p.KLp * 16), o_jobs = take(t.jobs.size() * 4), o_xl = take(t.xlist.size() * 2),
+                 o_cells = take(t.cells.size() * 4), o_bar = take(8), host = off;
+    const size_t o_nbr = take((size_t)p.NG * 256 * sizeof(int32_t)),
+                 exb = s.resident ? (size_t)p.NG * p.XW * 128 : 0, o_ex0 = take(exb), o_ex1 = take(exb);
+    std::vector<uint8_t> img(host, 0);
+    slice_neighbour_table(t, p.D, reinterpret_cast<uint16_t *>(img.data() + o_tab));
+    memcpy(img.data() + o_jobs, t.jobs.data(), t.jobs.size() * 4);
+    memcpy(img.data() + o_xl, t.xlist.data(), t.xlist.size() * 2);
+    memcpy(img.data() + o_cells, t.cells.data(), t.cells.size() * 4);
+    cudaError_t e = cudaMalloc(&s.arena, off);
+    if (e == cudaSuccess) e = cudaMemcpyAsync(s.arena, img.data(), host, cudaMemcpyHostToDevice, st);
+    p.tab = reinterpret_cast<uint4 *>(s.arena + o_tab);
+    p.jobs = reinterpret_cast<uint32_t *>(s.arena + o_jobs);
+    p.xlist = reinterpret_cast<uint16_t *>(s.arena + o_xl);
+    p.cells = reinterpret_cast<uint2 *>(s.arena + o_cells);
+    s.bar = reinterpret_cast<uint32_t *>(s.arena + o_bar);
+    p.nbr = reinterpret_cast<int32_t *>(s.arena + o_nbr);
+    s.ex[0] = reinterpret_cast<uint32_t *>(s.arena + o_ex0);
+    s.ex[1] = reinterpret_cast<uint32_t *>(s.arena + o_ex1);
+    if (e == cudaSuccess) {
+        const int64_t blocks = std::min<int64_t>((32 * p.NG + 255) / 256, (int64_t)f->num_sms * 16);
+        slice_nbr_kernel<<<(unsigned)blocks, 256, 0, st>>>(f->dev, p.NT, p.NG, f->r - p.L, (int32_t)pw(f->s, f->r - p.L), p.nbr);
+        e = cudaGetLastError();
+        if (e == cudaSuccess) e = cudaStreamSynchronize(st);   // the tables serve calls on any stream from here on
+    }
+    // shared memory and grids
+    int per_sm = 0;
+    if (s.resident) {
+        for (int life = 0; life < 2 && e == cudaSuccess; ++life) {
+            ResidentFn fn = resident_fn(s, life);
+            e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, kSliceSmem);
+            if (e == cudaSuccess)
+                e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, fn, s.block_resident, s.smem_resident);
+            if (e == cudaSuccess && per_sm < 1) e = cudaErrorInvalidConfiguration;
+        }
+    }
+    {
+        const int most = 100 * 1024;
+        if (std::max(std::max(s.smem_pack, s.smem_single), std::max(s.smem_step, s.smem_bytes)) > most) e = cudaErrorInvalidConfiguration;
+        if (e == cudaSuccess) e = cudaFuncSetAttribute(slice_pack_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, most);
+        if (e == cudaSuccess) e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, slice_pack_kernel, kSliceBlock, s.smem_pack);
+        for (int life = 0; life < 2 && p.H <= 32 && e == cudaSuccess; ++life) {
+            int n = 0;
+            e = cudaFuncSetAttribute(single_fn(p.D, life), cudaFuncAttributeMaxDynamicSharedMemorySize, most);
+            if (e == cudaSuccess)
+                e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, single_fn(p.D, life), kSliceBlock, s.smem_single);
+            s.grid_single[life] = (int)std::min<int64_t>((int64_t)n * f->num_sms, p.NG);
+        }
+        s.grid_pack = (int)std::min<int64_t>((int64_t)std::max(per_sm, 1) * f->num_sms, p.NG);
+        for (int life = 0; life < 2 && e == cudaSuccess; ++life)
+            for (int bytes = 0; bytes < 2 && e == cudaSuccess; ++bytes) {
+                StepFn fn = step_fn(p.D, life, bytes);
+                e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, most);
+                if (e == cudaSuccess)
+                    e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, fn, kSliceBlock, bytes ? s.smem_bytes : s.smem_step);
+                if (e == cudaSuccess && per_sm < 1) e = cudaErrorInvalidConfiguration;
+                (bytes ? s.grid_bytes : s.grid_step)[life] = (int)std::min<int64_t>((int64_t)per_sm * f->num_sms, p.NG);
+            }
+    }
+    if (e != cudaSuccess) {
+        cudaGetLastError();
+        free_slice_plan(s);
+        return e == cudaErrorMemoryAllocation ? FR_ENOMEM : FR_ECUDA;
+    }
+    s.state = 1;
+    f->slice = s;
+    return FR_OK;
+}
+
+// One packed-state buffer of the streaming kernels, allocated when first needed.
+static bool slice_buffer(fractal *f, int i)
+{
+    SlicePlan &s = f->slice;
+    if (s.bits[i]) return true;
+    if (cudaMalloc(&s.bits[i], (size_t)s.geo.NG * (s.geo.KLp + 32 * s.geo.XW) * sizeof(uint32_t)) == cudaSuccess) return true;
+    cudaGetLastError();
+    s.bits[i] = nullptr;
+    return false;
+}
+
+// Whether `steps` generations run in the resident kernel.  A single
+// generation of a state with many groups is faster as two streaming launches.
+static bool slice_use_resident(const SlicePlan &s, int64_t steps, int num_sms)
+{
+    return s.resident && (steps > 1 || s.geo.NG <= num_sms);
+}
+
+int try_slice_step(fractal *f, const uint8_t *in, uint8_t *out, int64_t steps, uint32_t birth, uint32_t survive,
+                   cudaStream_t st, bool *done)
+{
+    *done = false;
+    if (!slice_fractal_ok(f) || steps < 1) return FR_OK;
+    SlicePlan &s = f->slice;
+    if (s.state < 0) return FR_OK;
+    // how the call will run: in one resident or single-pass launch, or with packed states between launches
+    bool res = false, packed = false;
+    auto choose = [&]() {
+        res = slice_use_resident(s, steps, f->num_sms);
+        packed = !res && !(steps == 1 && s.grid_single[0] > 0);
+    };
+    choose();
+    if (s.state == 0 || (packed && (!s.bits[0] || (steps > 1 && !s.bits[1])))) {
+        // nothing is allocated under capture: the tile kernels run there as before
+        cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
+        if (cudaStreamIsCapturing(st, &cs) != cudaSuccess || cs != cudaStreamCaptureStatusNone) {
+            cudaGetLastError();
+            return FR_OK;
+        }
+        int rc = ensure_status(f);
+        if (rc) return rc;
+        if (s.state == 0 && build_slice_plan(f, st) != FR_OK) {
+            s.state = -1;
+            return FR_OK;
+        }
+        choose();
+        if (packed && (!slice_buffer(f, 0) || (steps > 1 && !slice_buffer(f, 1)))) return FR_OK;
+    }
+    const SliceGeo &p = s.geo;
+    SliceArgs a;
+    a.NT = p.NT;
+    a.NG = p.NG;
+    a.KL = p.KL;
+    a.KLp = p.KLp;
+    a.NC = p.NC;
+    a.NJ = p.NJ;
+    a.BP = p.BP;
+    a.RP = p.RP;
+    a.AW = p.AW;
+    a.A_zero = p.AW - 32;
+    a.XW = p.XW;
+    a.ex = p.NG * p.KLp;
+    a.kdiv = make_div((uint32_t)p.KL);
+    a.bsh = 30;
+    if (p.BP)
+        for (a.bsh = 0; (32 << a.bsh) < p.KL;) ++a.bsh;
+    a.lane_bits = p.BP ? 32u * (uint32_t)p.BP : (uint32_t)p.KL;
+    for (int c = 0; c < 9; ++c) {
+        a.mb[c] = (birth >> c) & 1u ? 0xffffffffu : 0u;
+        a.ms[c] = (survive >> c) & 1u ? 0xffffffffu : 0u;
+    }
+    a.tab = p.tab;
+    a.jobs = p.jobs;
+    a.xlist = p.xlist;
+    a.cells = p.cells;
+    a.H = p.H;
+    a.nbr = p.nbr;
+    a.bar = s.bar;
+    a.status = f->status;
+    const bool life = (birth & 0x1ffu) == 0x8u && (survive & 0x1ffu) == 0xcu;
+    if (res) {
+        ResidentFn fn = resident_fn(s, life);
+        uint32_t *e0 = s.ex[0], *e1 = s.ex[1];
+        int per_block = s.per_block;
+        void *args[] = {&a, &in, &out, &e0, &e1, &per_block, &steps};
+        if (s.grid_resident > 1)
+            FR_CUDA(cudaLaunchCooperativeKernel((const void *)fn, dim3(s.grid_resident), dim3(s.block_resident), args,
+                                                s.smem_resident, st));
+        else
+            FR_CUDA(cudaLaunchKernel((const void *)fn, dim3(1), dim3(s.block_resident), args, s.smem_resident, st));
+        *done = true;
+        return FR_OK;
+    }
+    if (!packed) {
+        single_fn(p.D, life)<<<s.grid_single[life], kSliceBlock, s.smem_single, st>>>(a, in, out);
+        FR_CUDA(cudaGetLastError());
+        *done = true;
+        return FR_OK;
+    }
+    slice_pack_kernel<<<s.grid_pack, kSliceBlock, s.smem_pack, st>>>(a, in, s.bits[0]);
+    FR_CUDA(cudaGetLastError());
+    *done = true;
+    int64_t left = steps - 1;   // generations before the one that writes bytes
+    int cur = 0;
+    StepFn fn = step_fn(p.D, life, false);
+    while (left > 0) {
+        int gens = (int)std::min<int64_t>(left, 1 << 20);
+        const uint32_t *src = s.bits[cur];
+        uint32_t *dst = s.bits[cur ^ 1];
+        uint8_t *none = nullptr;
+        void *args[] = {&a, &src, &dst, &none, &gens};
+        if (s.grid_step[life] > 1 && gens > 1)
+            FR_CUDA(cudaLaunchCooperativeKernel((const void *)fn, dim3(s.grid_step[life]), dim3(kSliceBlock), args, s.smem_step, st));
+        else
+            FR_CUDA(cudaLaunchKernel((const void *)fn, dim3(s.grid_step[life]), dim3(kSliceBlock), args, s.smem_step, st));
+        left -= gens;
+        if (gens & 1) cur ^= 1;
+    }
+    {
+        StepFn fb = step_fn(p.D, life, true);
+        const uint32_t *src = s.bits[cur];
+        uint32_t *none = nullptr;
+        int one = 1;
+        void *args[] = {&a, &src, &none, &out, &one};
+        FR_CUDA(cudaLaunchKernel((const void *)fb, dim3(s.grid_bytes[life]), dim3(kSliceBlock), args, s.smem_bytes, st));
+    }
+    return FR_OK;
+}
+
+}  // namespace fr

@@ -1,0 +1,55 @@
+// slice.h -- the bit-sliced step of 2D fractals (slice.cu): plan and entry
+// points (internal; not part of the ABI).
+#pragma once
+
+#include <cuda_runtime.h>
+#include <stdint.h>
+
+#include "internal.cuh"
+
+struct fractal;
+
+namespace fr {
+
+// Tiles of k^L cells (level-L subtrees) in groups of 32: bit t of word
+// (g, slot) of a packed state is cell `slot` of tile 32 g + t.  Every tile
+// has the same neighbour structure, so one word operation advances the same
+// cell of 32 tiles.
+struct SliceGeo {
+    int L = 0;
+    int KL = 0, KLp = 0;      // cells per tile; the same rounded up to 32 (words per group)
+    int NC = 0;               // 32-cell chunks per tile
+    int64_t NT = 0, NG = 0;   // tiles, groups of 32
+    int H = 0;                // halo cells per tile
+    int D = 0;                // neighbours per cell the kernel adds (the largest degree, as 4, 6, 7 or 8)
+    int NJ = 0, XW = 0;       // halo words a tile takes, export words it gives (at most 32 cells each)
+    int BP = 0, RP = 0, AW = 0;   // shared-memory geometry (SliceArgs)
+    uint4 *tab = nullptr;        // per cell: byte offsets (8 x uint16) of its neighbours' words in a group's word array
+    uint32_t *jobs = nullptr;    // [NJ]: export word | direction << 8
+    uint16_t *xlist = nullptr;   // [XW][32]: cells of the export words
+    uint2 *cells = nullptr;      // [H]: cell of the neighbouring tile, its word in a group's array | direction << 16
+    int32_t *nbr = nullptr;      // [NG][8][32]: neighbouring tile of each tile of a group by direction, -1 = none
+};
+
+struct SlicePlan {
+    int state = 0;            // 0: not planned yet, 1: planned, -1: not possible for this fractal
+    SliceGeo geo;
+    bool resident = false;    // the packed state stays in shared memory: one launch for all generations
+    int per_block = 0, rounds = 0, block_resident = 0, grid_resident = 0, smem_resident = 0;
+    int smem_pack = 0, smem_step = 0, smem_bytes = 0, smem_single = 0;
+    int grid_pack = 0, grid_step[2] = {0, 0}, grid_bytes[2] = {0, 0}, grid_single[2] = {0, 0};   // [1]: with the constant rule
+    uint32_t *bits[2] = {nullptr, nullptr};   // packed states: NG x KLp words, then the exports, NG x XW x 32
+    uint8_t *arena = nullptr;                 // the tables, and:
+    uint32_t *ex[2] = {nullptr, nullptr};     // resident kernel: the exports alone
+    uint32_t *bar = nullptr;                  // grid barrier: arrivals, exits
+};
+
+void free_slice_plan(SlicePlan &p);
+
+// `steps` >= 1 generations from bytes to bytes; *done = false (and nothing
+// launched) when the fractal, the handle's settings or the memory at hand
+// rule the sliced step out.
+int try_slice_step(fractal *f, const uint8_t *in, uint8_t *out, int64_t steps, uint32_t birth, uint32_t survive,
+                   cudaStream_t st, bool *done);
+
+}  // namespace fr

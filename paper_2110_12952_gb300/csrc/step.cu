@@ -969,6 +969,17 @@ __global__ void nbr_table_kernel(FracDev F, int64_t NT, int coarse_levels, int32
     }
 }
 
+// Fills the table of the NT tiles' neighbours (coarse_levels levels above them).
+int launch_nbr_table(const fractal *f, int64_t NT, int coarse_levels, int nbrw, int32_t *table)
+{
+    const int64_t g = std::min<int64_t>((NT + 255) / 256, (int64_t)f->num_sms * 16);
+    nbr_table_kernel<<<(int)std::max<int64_t>(g, 1), 256>>>(f->dev, NT, coarse_levels, (int32_t)ipow(f->s, coarse_levels),
+                                                            nbrw, table);
+    FR_CUDA(cudaGetLastError());
+    FR_CUDA(cudaDeviceSynchronize());
+    return FR_OK;
+}
+
 template <int DIM, int MODE, bool MULTI>
 __global__ void step_tma_kernel(FracDev F, StepArgs a, const uint8_t *__restrict__ in,
                                 uint8_t *__restrict__ out);
@@ -1256,12 +1267,10 @@ int ensure_step_plan(fractal *f)
         free_step_plan(p);
         return cuda_fail(e, "fractal_step: neighbour table allocation");
     }
-    {
-        int64_t g = std::min<int64_t>((p.NT + 255) / 256, (int64_t)f->num_sms * 16);
-        nbr_table_kernel<<<(int)std::max<int64_t>(g, 1), 256>>>(
-            f->dev, p.NT, p.coarse_levels, (int32_t)ipow(f->s, p.coarse_levels), p.nbrw, p.nbr);
-        FR_CUDA(cudaGetLastError());
-        FR_CUDA(cudaDeviceSynchronize());
+    rc = launch_nbr_table(f, p.NT, p.coarse_levels, p.nbrw, p.nbr);
+    if (rc) {
+        free_step_plan(p);
+        return rc;
     }
     if (p.mode == kModeBit3) rc = configure_bit3(p, f->num_sms);
     else if (dim == 3) rc = p.mode == kModeBox3 ? configure<3, kModeBox3>(p, f->num_sms) : configure<3, kModeCell>(p, f->num_sms);
@@ -2828,12 +2837,10 @@ int ensure_tb_plan(fractal *f)
         free_tb_plan(p);
         return cuda_fail(e, "temporal blocking: neighbour table allocation");
     }
-    {
-        const int64_t g = std::min<int64_t>((p.NT + 255) / 256, (int64_t)f->num_sms * 16);
-        nbr_table_kernel<<<(int)std::max<int64_t>(g, 1), 256>>>(f->dev, p.NT, f->r - L,
-                                                                (int32_t)ipow(f->s, f->r - L), 8, p.nbr);
-        FR_CUDA(cudaGetLastError());
-        FR_CUDA(cudaDeviceSynchronize());
+    rc = launch_nbr_table(f, p.NT, f->r - L, 8, p.nbr);
+    if (rc) {
+        free_tb_plan(p);
+        return rc;
     }
     auto kfn = P == 0 ? step_tb_kernel<0, false> : step_tb_kernel<1, false>;
     auto kfl = P == 0 ? step_tb_kernel<0, true> : step_tb_kernel<1, true>;
@@ -2893,7 +2900,11 @@ int launch_tb_once(fractal *f, const uint8_t *in, uint8_t *out, int gens, uint32
 // ---------------------------------------------------------------- autotune
 
 static std::mutex g_tune_mu;
-static std::map<std::string, std::pair<int, int>> g_tune_cache;  // fractal + device -> (tile levels, stages)
+struct Tuned {
+    int levels, stages;
+    bool sliced;   // the bit-sliced step was faster than every tile depth
+};
+static std::map<std::string, Tuned> g_tune_cache;  // by fractal and device
 
 static std::string tune_key(const fractal *f)
 {
@@ -2910,22 +2921,27 @@ static std::string tune_key(const fractal *f)
     return key;
 }
 
-int cached_tile_levels(const fractal *f, int *stages)
+void apply_tuned(fractal *f)
 {
     std::lock_guard<std::mutex> lk(g_tune_mu);
     auto it = g_tune_cache.find(tune_key(f));
-    if (stages) *stages = it == g_tune_cache.end() ? -1 : it->second.second;
-    return it == g_tune_cache.end() ? -1 : it->second.first;
+    if (it == g_tune_cache.end()) return;
+    f->tile_levels_user = it->second.levels;
+    f->stages_user = it->second.stages;
+    f->sliced_tuned = it->second.sliced;
 }
 
 // Times the candidate plans on the caller's buffers and keeps the fastest:
 // the tile depths (the deepest that fit in shared memory and the three
-// below), each with 2, 3 and 4 input pipeline stages.
+// below), each with 2, 3 and 4 input pipeline stages, and the bit-sliced step
+// (which keeps its own tile depth: the fastest tile kernel's is reported and
+// serves the calls that need tile kernels).
 int autotune_step(fractal *f, const uint8_t *in, uint8_t *out, uint32_t birth, uint32_t survive,
                   cudaStream_t st, int *best_out)
 {
     int lmax = 0;
     f->stages_user = -1;
+    f->sliced_tuned = false;
     for (int L = 0; L <= f->r; ++L) {
         if (plan_layout(f, L).total > 200 * 1024) break;
         lmax = L;
@@ -2935,6 +2951,16 @@ int autotune_step(fractal *f, const uint8_t *in, uint8_t *out, uint32_t birth, u
     cudaEvent_t e0, e1;
     FR_CUDA(cudaEventCreate(&e0));
     FR_CUDA(cudaEventCreate(&e1));
+    // average time of three calls after two
+    auto time_calls = [&](auto call, float *ms) -> bool {
+        int rc = FR_OK;
+        for (int w = 0; w < 2 && !rc; ++w) rc = call();
+        if (!rc) rc = (cudaEventRecord(e0, st) == cudaSuccess) ? FR_OK : FR_ECUDA;
+        for (int w = 0; w < 3 && !rc; ++w) rc = call();
+        if (!rc) rc = (cudaEventRecord(e1, st) == cudaSuccess) ? FR_OK : FR_ECUDA;
+        if (!rc) rc = (cudaEventSynchronize(e1) == cudaSuccess) ? FR_OK : FR_ECUDA;
+        return !rc && cudaEventElapsedTime(ms, e0, e1) == cudaSuccess;
+    };
     for (int L = lmax; L >= 0 && L >= lmax - 3; --L) {
         if (cells_above(f, L) >= ((int64_t)1 << 31)) break;
         for (int ns = 2; ns <= 4; ++ns) {
@@ -2943,19 +2969,26 @@ int autotune_step(fractal *f, const uint8_t *in, uint8_t *out, uint32_t birth, u
             if (plan_layout(f, L).total > 200 * 1024) continue;
             if (ensure_step_plan(f) != FR_OK) continue;
             if (f->plan.mode == kModeBit3 && ns > 2) continue;   // it has no input stages
-            int rc = FR_OK;
-            for (int w = 0; w < 2 && !rc; ++w) rc = launch_step_once(f, in, out, birth, survive, st);
-            if (!rc) rc = (cudaEventRecord(e0, st) == cudaSuccess) ? FR_OK : FR_ECUDA;
-            for (int w = 0; w < 3 && !rc; ++w) rc = launch_step_once(f, in, out, birth, survive, st);
-            if (!rc) rc = (cudaEventRecord(e1, st) == cudaSuccess) ? FR_OK : FR_ECUDA;
-            if (!rc) rc = (cudaEventSynchronize(e1) == cudaSuccess) ? FR_OK : FR_ECUDA;
             float ms = 0.f;
-            if (!rc && cudaEventElapsedTime(&ms, e0, e1) == cudaSuccess && (best < 0 || ms < best_ms)) {
+            if (time_calls([&]() { return launch_step_once(f, in, out, birth, survive, st); }, &ms) &&
+                (best < 0 || ms < best_ms)) {
                 best = L;
                 best_st = ns;
                 best_ms = ms;
             }
         }
+    }
+    bool sliced = false;
+    {
+        float ms = 0.f;
+        if (best >= 0 && time_calls(
+                             [&]() {
+                                 bool done = false;
+                                 const int rc = try_slice_step(f, in, out, 1, birth, survive, st, &done);
+                                 return rc ? rc : (done ? FR_OK : FR_EINVAL);
+                             },
+                             &ms))
+            sliced = ms < best_ms;
     }
     cudaEventDestroy(e0);
     cudaEventDestroy(e1);
@@ -2967,11 +3000,12 @@ int autotune_step(fractal *f, const uint8_t *in, uint8_t *out, uint32_t birth, u
     }
     f->tile_levels_user = best;
     f->stages_user = best_st;
+    f->sliced_tuned = sliced;
     int rc = ensure_step_plan(f);
     if (rc) return rc;
     {
         std::lock_guard<std::mutex> lk(g_tune_mu);
-        g_tune_cache[tune_key(f)] = std::make_pair(best, best_st);
+        g_tune_cache[tune_key(f)] = Tuned{best, best_st, sliced};
     }
     if (best_out) *best_out = best;
     return take_status(f);

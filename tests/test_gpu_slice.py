@@ -1,0 +1,96 @@
+"""The bit-sliced step of 2D fractals (slice.cu) against the oracle, at the
+sizes where its tiles, groups of 32 tiles, 32-cell chunks and 16-byte units
+end: fewer tiles than a group, a last group that is not full, tiles that are
+and are not whole words, one and many generations per call, rules beyond
+B3/S23, buffers that are not 16-byte aligned and bytes other than 0 and 1."""
+import numpy as np
+import pytest
+import torch
+
+import oracle
+from paper_2110_12952_gb300 import workloads as W
+
+pytestmark = pytest.mark.gpu
+
+RULES = [W.LIFE_B3S23, W.rule_masks([3, 6], [2, 3]), W.rule_masks([1, 8], [0, 1, 2, 5, 8])]
+CASES = [("triangle", r) for r in (1, 2, 3, 5, 8, 11, 13)] + [("triangle_mirrored", 10), ("carpet", 1), ("carpet", 2),
+         ("carpet", 5), ("carpet", 6), ("vicsek", 2), ("vicsek", 6), ("vicsek", 8), ("h_fractal", 3), ("h_fractal", 6),
+         ("x_fractal", 7), ("chandelier", 4), ("chandelier", 8), ("candy", 2), ("candy", 5), ("empty_bottles", 6),
+         ("full_square", 3), ("full_square", 9), ("cantor_set", 5), ("cantor_set", 15)]
+
+
+def pair(fam, r):
+    from paper_2110_12952_gb300 import Fractal
+    return Fractal.from_family(fam, r), oracle.Fractal(fam.k, fam.s, r, fam.dim, fam.table())
+
+
+@pytest.mark.parametrize("name,r", CASES)
+def test_slice_step_matches_oracle(name, r):
+    fam = W.FAMILIES[name]
+    g, o = pair(fam, r)
+    x = o.init_bernoulli(11 + r, 0.45)
+    x[::7] *= 201   # any nonzero byte is alive
+    for i, (rule, steps) in enumerate(zip(RULES * 2, (1, 2, 3, 1, 5, 8))):
+        off = (0, 0, 3, 16, 9, 0)[i]
+        src = torch.empty(g.cells + 64, dtype=torch.uint8, device="cuda")[off:off + g.cells]
+        whole = torch.full((g.cells + 64,), 77, dtype=torch.uint8, device="cuda")
+        dst = whole[64 - off - i:64 - off - i + g.cells] if i else whole[:g.cells]
+        src.copy_(torch.from_numpy(x))
+        g.step(src, out=dst, steps=steps, rule=rule)
+        want = o.step(x, rule=oracle.Rule(*rule), steps=steps)
+        assert np.array_equal(dst.cpu().numpy(), want), (name, r, rule, steps, off)
+        assert int((whole == 77).sum()) == 64          # nothing written around the result
+        assert np.array_equal(src.cpu().numpy(), x)
+    g.check()
+    g.close()
+
+
+def test_slice_step_under_capture():
+    # a captured call replays with new contents of the same buffers; a handle that has not run yet captures too
+    fam = W.CARPET
+    for warm in (True, False):
+        g, o = pair(fam, 5)
+        x = torch.empty(g.cells, dtype=torch.uint8, device="cuda")
+        y = torch.empty_like(x)
+        z = torch.empty_like(x)
+        if warm:
+            g.step(x, out=y, steps=4)
+            g.step(x, out=z, steps=1)
+        else:
+            assert g.tile_levels >= 0   # builds the tile kernels' tables only
+        torch.cuda.synchronize()
+        graph = torch.cuda.CUDAGraph()
+        with torch.cuda.graph(graph):
+            g.step(x, out=z, steps=1)
+            if warm:
+                g.step(x, out=y, steps=4)
+        for seed in (3, 4):
+            v = o.init_bernoulli(seed, 0.5)
+            x.copy_(torch.from_numpy(v))
+            graph.replay()
+            torch.cuda.synchronize()
+            assert np.array_equal(z.cpu().numpy(), o.step(v, steps=1))
+            if warm:
+                assert np.array_equal(y.cpu().numpy(), o.step(v, steps=4))
+        del graph
+        g.close()
+
+
+@pytest.mark.parametrize("name,r", [("triangle", 17), ("vicsek", 12), ("h_fractal", 10)])
+def test_streamed_states_match_single_generations(name, r):
+    # states too large for the resident kernel keep their packed words in memory between launches; one call of
+    # several generations equals as many calls of one, and those the tile kernels'
+    from paper_2110_12952_gb300 import Fractal
+    fam = W.FAMILIES[name]
+    g, tiles = Fractal.from_family(fam, r), Fractal.from_family(fam, r)
+    tiles.tile_levels = tiles.tile_levels   # an explicit depth: the tile kernels
+    x = g.init_bernoulli(5, 0.4)
+    ref, one = x, x
+    for steps in (1, 2, 3):
+        ref = tiles.step(ref, steps=1)
+        one = g.step(one, steps=1)
+        assert torch.equal(one, ref)
+        assert torch.equal(g.step(x, steps=steps), ref), steps
+    g.check()
+    g.close()
+    tiles.close()

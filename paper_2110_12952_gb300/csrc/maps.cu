@@ -2,10 +2,18 @@
 // the paper's multi-dimensional compact coordinate (Eqs. 6-8), compact <->
 // box views, and the seeded Bernoulli initial state.
 //
-// All of it is integer work decoded digit by digit on the CUDA cores with
-// multiply-high division by the constants s and k.
+// Large arrays go through tables of several levels at once: lambda and nu are
+// sums over the levels, so a table over the digits of m levels (built by each
+// block in shared memory) replaces m digit steps by one look-up, and the
+// triangle's 20 levels by three or four.  The digit loops they replace read
+// the transition tables from constant memory at a different address per lane,
+// which the hardware serialises (one pass per distinct address); they remain
+// for short arrays, where building a table would cost more, and for fractals
+// with a different table per level.
 #include <cuda_runtime.h>
 #include <stdint.h>
+
+#include <algorithm>
 
 #include "handle.h"
 
@@ -30,6 +38,334 @@ __global__ void lambda_kernel(FracDev F, const int64_t *__restrict__ omega, int6
         if (w >= 0 && w < cells) lambda64(F, (uint64_t)w, F.r, p);
         for (int i = 0; i < F.dim; ++i) coords[e * F.dim + i] = p[i];
     }
+}
+
+// Unsigned division of x < 2^63 by a constant (DivU32's method with 64 bits).
+struct DivU64 {
+    uint64_t m;
+    uint32_t sh;
+};
+
+static DivU64 make_div64(uint64_t d)
+{
+    uint32_t l = 1;
+    while ((1ull << l) < d) ++l;
+    // ceil(2^(63 + l) / d), below 2^64 because d > 2^(l - 1)
+    const unsigned __int128 num = (unsigned __int128)1 << (63 + l);
+    return DivU64{(uint64_t)((num + d - 1) / d), l - 1};
+}
+
+constexpr int kMapTable = 4096;     // most entries of a table
+constexpr int kMapGroups = 16;      // most groups of levels
+constexpr int kMapBlock = 512;
+constexpr int kMapBlocksPerSM = 4;
+constexpr int64_t kMapLong = 1 << 16;   // arrays from here on go through tables
+
+// lambda through tables: entry i holds the coordinates of i over m levels
+// (16 bits each in 2D, 10 in 3D); omega's base-k^m digits pick the entries.
+struct LambdaTab {
+    int m, groups, n;        // levels per group, groups, entries (k^m)
+    int m_last, n_last;      // the same of the last group, whose table follows (n_last = n: the same table)
+    int last;                // where the last group's table starts
+    int wide;                // groups before which the number may reach 2^31
+    uint32_t scale[kMapGroups];   // s^(m g)
+    DivU64 div64;            // by k^m
+    DivU32 div32;
+};
+
+template <int DIM>
+__device__ __forceinline__ void lambda_table(const FracDev &F, const LambdaTab &L, uint32_t *tab)
+{
+    const int all = L.n + (L.n_last == L.n ? 0 : L.n_last);
+    for (int i = threadIdx.x; i < all; i += blockDim.x) {
+        int32_t p[3];
+        lambda32(F, (uint32_t)(i < L.n ? i : i - L.n), i < L.n ? L.m : L.m_last, p);
+        tab[i] = DIM == 2 ? (uint32_t)p[0] | (uint32_t)p[1] << 16
+                          : (uint32_t)p[0] | (uint32_t)p[1] << 10 | (uint32_t)p[2] << 20;
+    }
+}
+
+template <int DIM>
+__device__ __forceinline__ void lambda_lookup(const LambdaTab &L, const uint32_t *tab, uint64_t w, int32_t *p)
+{
+    uint32_t x = 0, y = 0, z = 0, v = (uint32_t)w;
+    // (the loop is unrolled and left at a group count that is the same for all)
+#pragma unroll
+    for (int g = 0; g < kMapGroups; ++g) {
+        if (g == L.groups) break;
+        uint32_t q;
+        if (g < L.wide) {   // the number may still reach 2^31
+            w = __umul64hi(w, L.div64.m) >> L.div64.sh;
+            q = (uint32_t)w;
+        } else {
+            q = divu(L.div32, v);
+        }
+        const uint32_t e = tab[v - q * (uint32_t)L.n + (g == L.groups - 1 ? L.last : 0)];
+        v = q;
+        if (DIM == 2) {
+            x += L.scale[g] * (e & 0xffffu);
+            y += L.scale[g] * (e >> 16);
+        } else {
+            x += L.scale[g] * (e & 0x3ffu);
+            y += L.scale[g] * ((e >> 10) & 0x3ffu);
+            z += L.scale[g] * (e >> 20);
+        }
+    }
+    p[0] = (int32_t)x;
+    p[1] = (int32_t)y;
+    if (DIM == 3) p[2] = (int32_t)z;
+}
+
+// 2^25 points of the triangle at r = 20: 1447 us with the digit loop (its
+// constant loads serialised), 155 us here (3.4 TB/s; issue slots and latency)
+template <int DIM, bool VEC>
+__global__ void __launch_bounds__(kMapBlock) lambda_tab_kernel(FracDev F, LambdaTab L, const int64_t *__restrict__ omega,
+                                                               int64_t count, int64_t cells, int32_t *__restrict__ coords)
+{
+    __shared__ uint32_t tab[2 * kMapTable];
+    lambda_table<DIM>(F, L, tab);
+    __syncthreads();
+    const int64_t step = (int64_t)gridDim.x * blockDim.x, t0 = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
+    if (VEC) {
+        // two points per 16-byte load; their coordinates as 16 bytes (2D)
+        const int64_t pairs = count / 2;
+#pragma unroll 4
+        for (int64_t e = t0; e < pairs; e += step) {
+            const longlong2 w = __ldcs(reinterpret_cast<const longlong2 *>(omega) + e);
+            int32_t p[2 * DIM];
+#pragma unroll
+            for (int h = 0; h < 2; ++h) {
+                const int64_t v = h ? w.y : w.x;
+                const bool ok = v >= 0 && v < cells;
+                lambda_lookup<DIM>(L, tab, ok ? (uint64_t)v : 0u, p + DIM * h);
+                for (int i = 0; i < DIM; ++i) p[DIM * h + i] = ok ? p[DIM * h + i] : -1;
+            }
+            if (DIM == 2) __stcs(reinterpret_cast<int4 *>(coords) + e, make_int4(p[0], p[1], p[2], p[3]));
+            else
+                for (int i = 0; i < 3; ++i) __stcs(reinterpret_cast<int2 *>(coords) + 3 * e + i, make_int2(p[2 * i], p[2 * i + 1]));
+        }
+    }
+    for (int64_t e = (VEC ? count / 2 * 2 : 0) + t0; e < count; e += step) {
+        const int64_t v = omega[e];
+        int32_t p[3] = {-1, -1, -1};
+        if (v >= 0 && v < cells) lambda_lookup<DIM>(L, tab, (uint64_t)v, p);
+        for (int i = 0; i < DIM; ++i) coords[e * DIM + i] = p[i];
+    }
+}
+
+// nu through tables: entry x + s^m (y + s^m z) holds the replica digits of m
+// levels as a number (base k), or -1 where some level's digits are no
+// replica.  With COMPACT it holds the compact coordinate of the m levels
+// instead (m a multiple of the dimension, so that every group starts at the
+// first axis), 16 bits per component in 2D, 10 in 3D.
+struct NuTab {
+    int m, groups, n;        // levels per group, groups, entries (s^(m dim))
+    int m_last, n_last;      // the same of the last group, whose table follows (n_last = n: the same table)
+    int last;                // where the last group's table starts
+    uint32_t sm;             // s^m
+    int shift;               // log2 of s^m, or -1
+    DivU32 div;              // by s^m
+    int64_t scale[kMapGroups];   // k^(m g); compact coordinate: k^(m g / dim)
+};
+
+template <int DIM, bool COMPACT>
+__device__ __forceinline__ void nu_table(const FracDev &F, const NuTab &N, uint32_t *tab)
+{
+    const int all = N.n + (N.n_last == N.n ? 0 : N.n_last);
+    for (int i = threadIdx.x; i < all; i += blockDim.x) {
+        // (the last group's digits run over s^m_last only, but are laid out
+        // like the others': entries in between are never read)
+        uint32_t c[3] = {0, 0, 0}, v = (uint32_t)(i < N.n ? i : i - N.n);
+        const int m = i < N.n ? N.m : N.m_last;
+        for (int a = 0; a < DIM; ++a) {
+            const uint32_t q = divu(N.div, v);
+            c[a] = v - q * N.sm;
+            v = q;
+        }
+        uint32_t acc[3] = {0, 0, 0}, w = 1;
+        bool ok = true;
+        for (int mu = 0; mu < m; ++mu) {
+            uint32_t t = 0, base = 1;
+            for (int a = 0; a < DIM; ++a) {
+                const uint32_t q = divu(F.sdiv, c[a]);
+                t += (c[a] - q * F.s) * base;
+                base *= F.s;
+                c[a] = q;
+            }
+            const int h = F.hinv[t];
+            ok = ok && h >= 0;
+            const int axis = COMPACT ? mu % DIM : 0;
+            acc[axis] += (uint32_t)h * w;
+            if (!COMPACT || axis == DIM - 1) w *= F.k;
+        }
+        tab[i] = !ok ? 0xffffffffu
+                     : (!COMPACT ? acc[0] : (DIM == 2 ? acc[0] | acc[1] << 16 : acc[0] | acc[1] << 10 | acc[2] << 20));
+    }
+}
+
+// POW2: s^m is a power of two.
+template <int DIM, bool COMPACT, bool POW2>
+__device__ __forceinline__ void nu_lookup(const NuTab &N, const uint32_t *tab, int32_t side, const int32_t *c, int64_t *out)
+{
+    constexpr int NC = COMPACT ? DIM : 1;
+    uint32_t v[3] = {(uint32_t)c[0], (uint32_t)c[1], DIM == 3 ? (uint32_t)c[2] : 0u};
+    // (a negative coordinate is a large unsigned one)
+    bool ok = v[0] < (uint32_t)side && v[1] < (uint32_t)side && v[2] < (uint32_t)side;
+#pragma unroll
+    for (int a = 0; a < DIM; ++a) v[a] = ok ? v[a] : 0u;
+    int64_t acc[3] = {0, 0, 0};
+#pragma unroll
+    for (int g = 0; g < kMapGroups; ++g) {
+        if (g == N.groups) break;
+        uint32_t i = g == N.groups - 1 ? (uint32_t)N.last : 0u, w = 1;
+#pragma unroll
+        for (int a = 0; a < DIM; ++a) {
+            const uint32_t q = POW2 ? v[a] >> N.shift : divu(N.div, v[a]);
+            const uint32_t d = POW2 ? v[a] & (N.sm - 1u) : v[a] - q * N.sm;
+            i += POW2 ? d << (a * N.shift) : d * w;
+            w *= N.sm;
+            v[a] = q;
+        }
+        const uint32_t e = tab[i];
+        ok = ok && e != 0xffffffffu;
+        if (!COMPACT) acc[0] += N.scale[g] * (int64_t)e;
+        else if (DIM == 2) {
+            acc[0] += N.scale[g] * (int64_t)(e & 0xffffu);
+            acc[1] += N.scale[g] * (int64_t)(e >> 16);
+        } else {
+            acc[0] += N.scale[g] * (int64_t)(e & 0x3ffu);
+            acc[1] += N.scale[g] * (int64_t)((e >> 10) & 0x3ffu);
+            acc[2] += N.scale[g] * (int64_t)(e >> 20);
+        }
+    }
+    for (int i = 0; i < NC; ++i) out[i] = ok ? acc[i] : -1;
+}
+
+// 2^25 points of the triangle at r = 20: nu 957 -> 145 us, compact coordinate
+// 1094 -> 185 us
+template <int DIM, bool COMPACT, bool VEC, bool POW2>
+__global__ void __launch_bounds__(kMapBlock) nu_tab_kernel(FracDev F, NuTab N, int32_t side, const int32_t *__restrict__ coords,
+                                                           int64_t count, int64_t *__restrict__ out)
+{
+    constexpr int NC = COMPACT ? DIM : 1;
+    __shared__ uint32_t tab[2 * kMapTable];
+    nu_table<DIM, COMPACT>(F, N, tab);
+    __syncthreads();
+    const int64_t step = (int64_t)gridDim.x * blockDim.x, t0 = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
+    if (VEC) {
+        // 2D: two points per 16-byte load
+        const int64_t pairs = count / 2;
+#pragma unroll 4
+        for (int64_t e = t0; e < pairs; e += step) {
+            const int4 v = __ldcs(reinterpret_cast<const int4 *>(coords) + e);
+            const int32_t c[4] = {v.x, v.y, v.z, v.w};
+            int64_t r[2 * NC];
+            nu_lookup<2, COMPACT, POW2>(N, tab, side, c, r);
+            nu_lookup<2, COMPACT, POW2>(N, tab, side, c + 2, r + NC);
+            for (int i = 0; i < NC; ++i)
+                __stcs(reinterpret_cast<longlong2 *>(out) + NC * e + i, make_longlong2(r[2 * i], r[2 * i + 1]));
+        }
+    }
+    for (int64_t e = (VEC ? count / 2 * 2 : 0) + t0; e < count; e += step) {
+        int32_t c[3] = {0, 0, 0};
+        for (int i = 0; i < DIM; ++i) c[i] = coords[e * DIM + i];
+        int64_t r[3];
+        nu_lookup<DIM, COMPACT, POW2>(N, tab, side, c, r);
+        for (int i = 0; i < NC; ++i) out[e * NC + i] = r[i];
+    }
+}
+
+static bool lambda_tab(const fractal *f, LambdaTab *L)
+{
+    if (f->mixed || f->k < 2 || f->r < 1) return false;
+    const int64_t most = f->dim == 2 ? 65536 : 1024;
+    int64_t n = f->k, sm = f->s;
+    int m = 1;
+    while (m < f->r && n * f->k <= kMapTable && sm * f->s <= most) {
+        n *= f->k;
+        sm *= f->s;
+        ++m;
+    }
+    const int groups = (f->r + m - 1) / m, m_last = f->r - m * (groups - 1);
+    int64_t n_last = 1;
+    for (int i = 0; i < m_last; ++i) n_last *= f->k;
+    if (groups > kMapGroups) return false;
+    L->m = m;
+    L->groups = groups;
+    L->n = (int)n;
+    L->m_last = m_last;
+    L->n_last = (int)n_last;
+    L->last = n_last == n ? 0 : (int)n;
+    L->wide = 0;
+    for (int64_t c = f->cells - 1; c >> 31; c /= n) ++L->wide;
+    uint32_t scale = 1;
+    for (int g = 0; g < kMapGroups; ++g, scale *= (uint32_t)sm) L->scale[g] = scale;
+    L->div64 = make_div64((uint64_t)n);
+    L->div32 = make_div((uint32_t)n);
+    return true;
+}
+
+static bool nu_tab(const fractal *f, bool compact, NuTab *N)
+{
+    if (f->mixed || f->r < 1) return false;
+    const int unit = compact ? f->dim : 1;
+    int64_t block = 1, sm1 = 1, k1 = 1;   // entries, side and members of `unit` levels
+    for (int i = 0; i < unit; ++i) {
+        sm1 *= f->s;
+        k1 *= f->k;
+    }
+    for (int i = 0; i < f->dim; ++i) block *= sm1;
+    if (block > kMapTable) return false;
+    // components are stored in 16 or 10 bits, nu in 31
+    const int64_t most = !compact ? (int64_t)1 << 31 : (f->dim == 2 ? 65535 : 1024);
+    const int64_t kc1 = compact ? f->k : k1;   // growth of a component per `unit` levels
+    int64_t n = block, sm = sm1, kc = kc1;
+    int m = unit;
+    if (kc > most) return false;
+    while (m < f->r && n * block <= kMapTable && kc * kc1 <= most) {
+        n *= block;
+        sm *= sm1;
+        kc *= kc1;
+        m += unit;
+    }
+    const int groups = (f->r + m - 1) / m, m_last = f->r - m * (groups - 1);
+    // the last group's largest index + 1: its coordinates stay below s^m_last, in steps of s^m
+    int64_t sl = 1, n_last = 0, row = 1;
+    for (int i = 0; i < m_last; ++i) sl *= f->s;
+    for (int i = 0; i < f->dim; ++i, row *= sm) n_last += (sl - 1) * row;
+    if (groups > kMapGroups) return false;
+    N->m = m;
+    N->groups = groups;
+    N->n = (int)n;
+    N->m_last = m_last;
+    N->n_last = m_last == m ? (int)n : (int)n_last + 1;
+    N->last = m_last == m ? 0 : (int)n;
+    N->sm = (uint32_t)sm;
+    N->shift = -1;
+    if ((sm & (sm - 1)) == 0)
+        for (N->shift = 0; (1ll << N->shift) < sm;) ++N->shift;
+    N->div = make_div((uint32_t)sm);
+    uint64_t scale = 1;   // (past the last group it may wrap: never read)
+    for (int g = 0; g < kMapGroups; ++g, scale *= (uint64_t)kc) N->scale[g] = (int64_t)scale;
+    return true;
+}
+
+static int map_grid(const fractal *f, int64_t count)
+{
+    return (int)std::min<int64_t>((int64_t)f->num_sms * kMapBlocksPerSM, (count + kMapBlock - 1) / kMapBlock);
+}
+
+template <bool COMPACT>
+static int launch_nu_tab(const fractal *f, const NuTab &N, const int32_t *coords, int64_t count, int64_t *out, cudaStream_t st)
+{
+    const bool vec = f->dim == 2 && ((uintptr_t)coords & 15) == 0 && ((uintptr_t)out & 15) == 0;
+    const int grid = map_grid(f, count), side = (int32_t)f->side;
+    if (f->dim == 3) nu_tab_kernel<3, COMPACT, false, false><<<grid, kMapBlock, 0, st>>>(f->dev, N, side, coords, count, out);
+    else if (vec && N.shift >= 0) nu_tab_kernel<2, COMPACT, true, true><<<grid, kMapBlock, 0, st>>>(f->dev, N, side, coords, count, out);
+    else if (vec) nu_tab_kernel<2, COMPACT, true, false><<<grid, kMapBlock, 0, st>>>(f->dev, N, side, coords, count, out);
+    else nu_tab_kernel<2, COMPACT, false, false><<<grid, kMapBlock, 0, st>>>(f->dev, N, side, coords, count, out);
+    FR_CUDA(cudaGetLastError());
+    return FR_OK;
 }
 
 __device__ __forceinline__ bool in_box(const FracDev &F, int32_t side, const int32_t *c)
@@ -173,6 +509,52 @@ __global__ void gather_kernel(FracDev F, int64_t cells, int64_t side,
     }
 }
 
+// Compact <-> box by tiles of m levels (k^m <= kMapTable cells): the place of
+// a tile's cells relative to the tile's own is the same for all tiles, so each
+// block builds that table once in shared memory and walks runs of up to 32
+// tiles, whose places its first warp computes with lambda.  A cell then costs one
+// table look-up; what bounds it is the byte-wise access to the box (rows of a
+// few cells).  Menger r = 6: scatter
+// 1140 -> 273 us (and 57 us of memset), gather 1148 -> 88 us.
+template <bool SCATTER>
+__global__ void __launch_bounds__(256) box_tiles_kernel(FracDev F, int64_t NT, int m, int KL, DivU32 kldiv, int run, uint32_t side,
+                                                        const uint8_t *__restrict__ src, uint8_t *__restrict__ dst)
+{
+    __shared__ uint32_t tab[kMapTable];
+    __shared__ int64_t place[32];
+    for (int l = threadIdx.x; l < KL; l += blockDim.x) {
+        int32_t p[3];
+        lambda32(F, (uint32_t)l, m, p);
+        tab[l] = (uint32_t)p[0] + side * ((uint32_t)p[1] + side * (uint32_t)p[2]);
+    }
+    int64_t sm = 1;
+    for (int i = 0; i < m; ++i) sm *= F.s;
+    for (int64_t t0 = run * (int64_t)blockIdx.x; t0 < NT; t0 += run * (int64_t)gridDim.x) {
+        const int nt = (int)min((int64_t)run, NT - t0);
+        __syncthreads();
+        if ((int)threadIdx.x < nt) {
+            int32_t p[3];
+            lambda64(F, (uint64_t)(t0 + threadIdx.x), F.r - m, p);
+            place[threadIdx.x] = sm * (p[0] + (int64_t)side * (p[1] + (int64_t)side * p[2]));
+        }
+        __syncthreads();
+        const int64_t w0 = t0 * KL;
+        if (SCATTER) {   // tile by tile: the stores to a tile's rows stay close together
+            for (int t = 0; t < nt; ++t) {
+                uint8_t *b = dst + place[t];
+#pragma unroll 4
+                for (int l = threadIdx.x; l < KL; l += 256) b[tab[l]] = src[w0 + (int64_t)t * KL + l] != 0;
+            }
+        } else {
+#pragma unroll 4
+            for (int i = threadIdx.x; i < nt * KL; i += 256) {
+                const int t = (int)divu(kldiv, (uint32_t)i);
+                dst[w0 + i] = src[place[t] + tab[i - t * KL]] != 0;
+            }
+        }
+    }
+}
+
 __global__ void copy_normalise_kernel(const uint8_t *__restrict__ in, uint8_t *__restrict__ out,
                                       int64_t n)
 {
@@ -202,6 +584,35 @@ int preload_copy_kernel()
 
 using namespace fr;
 
+// Whether the views go by tiles, and the tile depth: the deepest with at most
+// kMapTable cells whose places fit in 32 bits, and with four tiles per SM
+// where the state has as many (of 128 cells or more).
+static int box_tile_levels(const fractal *f)
+{
+    if (f->mixed || f->k < 2 || f->cells < kMapLong) return 0;
+    int m = 0;
+    int64_t kl = f->k, sm = f->s;
+    for (; m < f->r && kl <= kMapTable; ++m, kl *= f->k, sm *= f->s) {
+        const double most = (double)(sm - 1) * (1.0 + (double)f->side + (f->dim == 3 ? (double)f->side * f->side : 0.0));
+        if (most >= 4294967296.0 || (kl / f->k >= 128 && f->cells / kl < 4 * f->num_sms)) break;
+    }
+    return m;
+}
+
+template <bool SCATTER>
+static int launch_box_tiles(const fractal *f, int m, const uint8_t *src, uint8_t *dst, cudaStream_t st)
+{
+    int64_t KL = 1;
+    for (int i = 0; i < m; ++i) KL *= f->k;
+    const int64_t NT = f->cells / KL;
+    const int64_t blocks = (int64_t)f->num_sms * 8;
+    const int run = (int)std::max<int64_t>(1, std::min<int64_t>(32, NT / blocks));
+    const int grid = (int)std::min<int64_t>((NT + run - 1) / run, blocks);
+    box_tiles_kernel<SCATTER><<<grid, 256, 0, st>>>(f->dev, NT, m, (int)KL, make_div((uint32_t)KL), run, (uint32_t)f->side, src, dst);
+    FR_CUDA(cudaGetLastError());
+    return FR_OK;
+}
+
 static int fail_null(const char *what)
 {
     set_error(FR_EINVAL, std::string(what) + ": NULL argument");
@@ -214,6 +625,18 @@ extern "C" int fractal_lambda(const fractal_t *f, const int64_t *omega, int64_t 
     if (!f || (count > 0 && (!omega || !coords))) return fail_null("fractal_lambda");
     if (count < 0) return fail_null("fractal_lambda (count < 0)");
     if (count == 0) return FR_OK;
+    LambdaTab L;
+    if (count >= kMapLong && lambda_tab(f, &L)) {
+        const bool vec = ((uintptr_t)omega & 15) == 0 && ((uintptr_t)coords & 15) == 0;
+        const int grid = map_grid(f, count);
+        cudaStream_t st = (cudaStream_t)stream;
+        if (f->dim == 3 && vec) lambda_tab_kernel<3, true><<<grid, kMapBlock, 0, st>>>(f->dev, L, omega, count, f->cells, coords);
+        else if (f->dim == 3) lambda_tab_kernel<3, false><<<grid, kMapBlock, 0, st>>>(f->dev, L, omega, count, f->cells, coords);
+        else if (vec) lambda_tab_kernel<2, true><<<grid, kMapBlock, 0, st>>>(f->dev, L, omega, count, f->cells, coords);
+        else lambda_tab_kernel<2, false><<<grid, kMapBlock, 0, st>>>(f->dev, L, omega, count, f->cells, coords);
+        FR_CUDA(cudaGetLastError());
+        return FR_OK;
+    }
     lambda_kernel<<<grid_for(count, 256, f->num_sms), 256, 0, (cudaStream_t)stream>>>(
         f->dev, omega, count, f->cells, coords);
     FR_CUDA(cudaGetLastError());
@@ -226,6 +649,8 @@ extern "C" int fractal_nu(const fractal_t *f, const int32_t *coords, int64_t cou
     if (!f || (count > 0 && (!omega || !coords))) return fail_null("fractal_nu");
     if (count < 0) return fail_null("fractal_nu (count < 0)");
     if (count == 0) return FR_OK;
+    NuTab N;
+    if (count >= kMapLong && nu_tab(f, false, &N)) return launch_nu_tab<false>(f, N, coords, count, omega, (cudaStream_t)stream);
     nu_kernel<<<grid_for(count, 256, f->num_sms), 256, 0, (cudaStream_t)stream>>>(
         f->dev, (int32_t)f->side, coords, count, omega);
     FR_CUDA(cudaGetLastError());
@@ -238,6 +663,8 @@ extern "C" int fractal_nu2d(const fractal_t *f, const int32_t *coords, int64_t c
     if (!f || (count > 0 && (!out || !coords))) return fail_null("fractal_nu2d");
     if (count < 0) return fail_null("fractal_nu2d (count < 0)");
     if (count == 0) return FR_OK;
+    NuTab N;
+    if (count >= kMapLong && nu_tab(f, true, &N)) return launch_nu_tab<true>(f, N, coords, count, out, (cudaStream_t)stream);
     nu2d_kernel<<<grid_for(count, 256, f->num_sms), 256, 0, (cudaStream_t)stream>>>(
         f->dev, (int32_t)f->side, coords, count, out);
     FR_CUDA(cudaGetLastError());
@@ -269,6 +696,7 @@ extern "C" int fractal_scatter_to_box(const fractal_t *f, const uint8_t *compact
     }
     cudaStream_t st = (cudaStream_t)stream;
     FR_CUDA(cudaMemsetAsync(box, 0, (size_t)f->box_cells, st));
+    if (const int m = box_tile_levels(f)) return launch_box_tiles<true>(f, m, compact, box, st);
     scatter_kernel<<<grid_for(f->cells, 256, f->num_sms), 256, 0, st>>>(
         f->dev, f->cells, f->side, compact, box);
     FR_CUDA(cudaGetLastError());
@@ -279,6 +707,7 @@ extern "C" int fractal_gather_from_box(const fractal_t *f, const uint8_t *box, u
                                        void *stream)
 {
     if (!f || !compact || !box) return fail_null("fractal_gather_from_box");
+    if (const int m = box_tile_levels(f)) return launch_box_tiles<false>(f, m, box, compact, (cudaStream_t)stream);
     gather_kernel<<<grid_for(f->cells, 256, f->num_sms), 256, 0, (cudaStream_t)stream>>>(
         f->dev, f->cells, f->side, box, compact);
     FR_CUDA(cudaGetLastError());

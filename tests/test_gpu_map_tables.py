@@ -1,0 +1,73 @@
+"""The maps and the box views through tables (maps.cu) against the oracle:
+arrays long enough for the tables, levels that do and do not divide into whole
+groups, fractals whose first digit tuple is and is not a replica, indices
+beyond 2^31, points off the fractal and outside the box, odd counts, and
+buffers that are only aligned to their type."""
+import numpy as np
+import pytest
+import torch
+
+import oracle
+from paper_2110_12952_gb300 import workloads as W
+
+pytestmark = pytest.mark.gpu
+
+N = 66001   # from 2^16 points on the maps use tables
+CASES = [("triangle", 1), ("triangle", 7), ("triangle", 13), ("triangle", 20), ("carpet", 3), ("carpet", 9), ("vicsek", 4),
+         ("vicsek", 12), ("menger", 2), ("menger", 5), ("menger", 7), ("candy", 7), ("x_fractal", 11), ("full_square", 15),
+         ("cantor_set", 19)]
+
+
+@pytest.mark.parametrize("name,r", CASES)
+@pytest.mark.parametrize("skew", [0, 1])
+def test_long_map_arrays(name, r, skew):
+    from paper_2110_12952_gb300 import Fractal
+    fam = W.FAMILIES[name]
+    g, o = Fractal.from_family(fam, r), oracle.Fractal(fam.k, fam.s, r, fam.dim, fam.table())
+    rng = np.random.default_rng(r)
+    w = rng.integers(0, o.cells, N, dtype=np.int64)
+    w[:4] = (0, o.cells - 1, -1, o.cells)
+    buf = torch.empty(N + skew, dtype=torch.int64, device="cuda")[skew:]
+    buf.copy_(torch.from_numpy(w))
+    out = torch.empty((N + skew) * fam.dim, dtype=torch.int32, device="cuda")[skew * fam.dim:].view(N, fam.dim)
+    lam = g.lam(buf, out=out).cpu().numpy()
+    want = np.full((N, fam.dim), -1, dtype=np.int64)
+    ok = (w >= 0) & (w < o.cells)
+    want[ok] = o.lam(w[ok])
+    assert np.array_equal(lam, want)
+    # the points' neighbours, random points and points outside
+    c = lam.copy()
+    c[ok] += rng.integers(-1, 2, (int(ok.sum()), fam.dim), dtype=np.int32)
+    c[5:9] = (-1, 0, o.side, 2**31 - 1)[:1]
+    c[9:200] = rng.integers(0, o.side, (191, fam.dim))
+    c[200:204, 0] = (-(2**31), -5, o.side - 1, o.side)
+    cb = torch.empty((N + skew) * fam.dim, dtype=torch.int32, device="cuda")[skew * fam.dim:].view(N, fam.dim)
+    cb.copy_(torch.from_numpy(c))
+    nu = torch.empty(N + skew, dtype=torch.int64, device="cuda")[skew:]
+    n2 = torch.empty((N + skew) * fam.dim, dtype=torch.int64, device="cuda")[skew * fam.dim:].view(N, fam.dim)
+    assert np.array_equal(g.nu(cb, out=nu).cpu().numpy(), o.nu(c))
+    assert np.array_equal(g.nu2d(cb, out=n2).cpu().numpy(), o.nu2d(c))
+    g.close()
+
+
+@pytest.mark.parametrize("name,r", [("triangle", 11), ("triangle", 12), ("carpet", 6), ("vicsek", 7), ("menger", 4), ("candy", 5),
+                                    ("full_square", 8)])
+def test_box_views_by_tiles(name, r):
+    from paper_2110_12952_gb300 import Fractal
+    fam = W.FAMILIES[name]
+    g, o = Fractal.from_family(fam, r), oracle.Fractal(fam.k, fam.s, r, fam.dim, fam.table())
+    x = o.init_bernoulli(3, 0.5)
+    x[::5] *= 9
+    idx = o.lam(np.arange(o.cells)) @ (o.side ** np.arange(fam.dim))
+    for off in (0, 3):
+        src = torch.empty(o.cells + off, dtype=torch.uint8, device="cuda")[off:]
+        src.copy_(torch.from_numpy(x))
+        box = torch.full((o.box_cells + off,), 5, dtype=torch.uint8, device="cuda")[off:]
+        g.scatter(src, out=box)
+        want = np.zeros(o.box_cells, dtype=np.uint8)
+        want[idx] = x != 0
+        assert np.array_equal(box.cpu().numpy(), want)
+        box += 2 * box   # members alive: 3
+        back = torch.full((o.cells + off,), 5, dtype=torch.uint8, device="cuda")[off:]
+        assert np.array_equal(g.gather(box, out=back).cpu().numpy(), (x != 0).astype(np.uint8))
+    g.close()

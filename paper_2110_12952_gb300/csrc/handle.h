@@ -174,6 +174,7 @@ inline int64_t cells_above(const fractal *f, int L)
 }
 
 int ensure_step_plan(fractal *f);
+int rows_preset_of(const fractal *f);   // 0: the carpet, 1: the Vicsek fractal (preset offsets), -1: another
 int ensure_tb_plan(fractal *f);
 void fr_paper_aux_free(fractal *f);
 void free_tb_plan(TbPlan &p);

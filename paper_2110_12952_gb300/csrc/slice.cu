@@ -42,6 +42,7 @@ namespace fr {
 constexpr int kSliceBlock = 256;   // threads per block of the streaming kernels
 constexpr int kSliceAhead = 2;     // halo words per warp loaded ahead of their group
 constexpr int kSliceBatch = 2;     // 16-byte units per thread and batch copied to shared memory ahead
+constexpr int kSliceSingleHalo = 32;   // most halo cells of a tile for the single-pass kernel
 constexpr int kSliceRounds = 32;   // resident kernel: most 32-cell chunks per warp
 
 struct SliceArgs {
@@ -1144,7 +1145,7 @@ static int build_slice_plan(fractal *f, cudaStream_t st)
         if (std::max(std::max(s.smem_pack, s.smem_single), std::max(s.smem_step, s.smem_bytes)) > most) e = cudaErrorInvalidConfiguration;
         if (e == cudaSuccess) e = cudaFuncSetAttribute(slice_pack_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, most);
         if (e == cudaSuccess) e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, slice_pack_kernel, kSliceBlock, s.smem_pack);
-        for (int life = 0; life < 2 && p.H <= 32 && e == cudaSuccess; ++life) {
+        for (int life = 0; life < 2 && p.H <= kSliceSingleHalo && e == cudaSuccess; ++life) {
             int n = 0;
             e = cudaFuncSetAttribute(single_fn(p.D, life), cudaFuncAttributeMaxDynamicSharedMemorySize, most);
             if (e == cudaSuccess)
@@ -1183,10 +1184,27 @@ static bool slice_buffer(fractal *f, int i)
     return false;
 }
 
+// Whether a single generation is faster in the tile kernels (one launch, no
+// packing).  Measured per launch in a graph, tiles -> sliced: single pass
+// (few halo cells) triangle r = 10 4.6 -> 10 us, r = 12 4.8 -> 3.3, r = 15
+// 10.4 -> 9.6; others H-fractal r = 7 (0.8 million cells) 6.4 -> 6.5, r = 8
+// 18 -> 8.3; carpet r = 7 (2.1 million) 5.7 -> 6.3, r = 8 19 -> 15; Vicsek
+// r = 11 21.5 -> 22, r = 12 96 -> 101.
+// (halo_cells < 0: not known yet; only what holds for any)
+static bool slice_one_generation_by_tiles(const fractal *f, int halo_cells)
+{
+    const int preset = rows_preset_of(f);
+    if (preset == 1 || f->cells < (1 << 17)) return true;
+    if (halo_cells < 0) return false;
+    if (halo_cells <= kSliceSingleHalo) return false;
+    return f->cells < (preset == 0 ? 4 << 20 : 1 << 20);
+}
+
 // Whether `steps` generations run in the resident kernel.  A single
-// generation of a state with many groups is faster as two streaming launches.
+// generation of a state with many groups is faster as streaming launches.
 static bool slice_use_resident(const SlicePlan &s, int64_t steps, int num_sms)
 {
+    if (steps == 1 && s.geo.H <= kSliceSingleHalo) return false;
     return s.resident && (steps > 1 || s.geo.NG <= num_sms);
 }
 
@@ -1197,6 +1215,7 @@ int try_slice_step(fractal *f, const uint8_t *in, uint8_t *out, int64_t steps, u
     if (!slice_fractal_ok(f) || steps < 1) return FR_OK;
     SlicePlan &s = f->slice;
     if (s.state < 0) return FR_OK;
+    if (steps == 1 && slice_one_generation_by_tiles(f, s.state > 0 ? s.geo.H : -1)) return FR_OK;
     // how the call will run: in one resident or single-pass launch, or with packed states between launches
     bool res = false, packed = false;
     auto choose = [&]() {
@@ -1217,6 +1236,7 @@ int try_slice_step(fractal *f, const uint8_t *in, uint8_t *out, int64_t steps, u
             s.state = -1;
             return FR_OK;
         }
+        if (steps == 1 && slice_one_generation_by_tiles(f, s.geo.H)) return FR_OK;
         choose();
         if (packed && (!slice_buffer(f, 0) || (steps > 1 && !slice_buffer(f, 1)))) return FR_OK;
     }

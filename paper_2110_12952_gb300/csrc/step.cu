@@ -519,7 +519,7 @@ static TapTables tap_tables(const fractal *f, int L)
 }
 
 // ---- rows mode: the carpet and the Vicsek fractal (see rows_layout.h)
-static int rows_preset_of(const fractal *f)
+int rows_preset_of(const fractal *f)
 {
     if (f->mixed || f->dim != 2 || f->s != 3) return -1;
     auto same = [&](int k, const int *ox, const int *oy) {

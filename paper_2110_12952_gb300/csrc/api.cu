@@ -243,6 +243,7 @@ extern "C" int fractal_destroy(fractal_t *f)
     cudaFree(f->scratch);
     cudaFree(f->b3_state[0]);
     cudaFree(f->b3_state[1]);
+    for (uint32_t *w : f->bb_words) cudaFree(w);
     cudaFree(f->bb_scratch);
     cudaFree(f->host_io[0]);
     cudaFree(f->host_io[1]);
@@ -444,6 +445,11 @@ extern "C" int fractal_bb_step(fractal_t *f, const uint8_t *in, uint8_t *out, in
         // zero generations: the masked, normalised box (no births; every
         // live member survives whatever its count)
         return launch_bb_once(f, in, out, 0u, 0xffffffffu, st);
+    }
+    {
+        bool done = false;
+        rc = try_bb_packed(f, in, out, steps, birth, survive, st, &done);
+        if (rc || done) return rc;
     }
     if (steps > 1) {
         rc = ensure_buffer(&f->bb_scratch, f->box_cells, "fractal_bb_step: scratch allocation");

@@ -134,6 +134,7 @@ struct fractal {
     fr::BBPlan bb;
     uint8_t *scratch = nullptr;      // k^r bytes, ping-pong for steps > 1
     uint32_t *b3_state[2] = {nullptr, nullptr};  // bit3 plans, steps > 1: bit-packed tile states (ping-pong)
+    uint32_t *bb_words[3] = {nullptr, nullptr, nullptr};   // box steps: membership and packed boxes (ping-pong)
     uint8_t *bb_scratch = nullptr;   // n^dim bytes, ping-pong for BB steps > 1
     uint8_t *host_io[2] = {nullptr, nullptr};  // device buffers of run_host
     fr::HostPipe pipe;                          // run_host's chunked pipeline
@@ -201,6 +202,10 @@ int launch_bit3_generations(fractal *f, const uint8_t *in, uint8_t *out, int64_t
 // of the same buffer, which holds readable_cells cells), into `out`.
 int launch_step_tiles(fractal *f, const uint8_t *in, uint8_t *out, const int32_t *nbr, int64_t ntiles,
                       int64_t readable_cells, uint32_t birth, uint32_t survive, cudaStream_t st);
+// `steps` generations with the box packed into bits between them; *done =
+// false (nothing launched) where the row kernels serve the call.
+int try_bb_packed(fractal *f, const uint8_t *in, uint8_t *out, int64_t steps, uint32_t birth, uint32_t survive,
+                  cudaStream_t st, bool *done);
 int launch_bb_once(fractal *f, const uint8_t *in, uint8_t *out, uint32_t birth,
                    uint32_t survive, cudaStream_t st);
 int launch_copy_normalise(const uint8_t *in, uint8_t *out, int64_t n, int num_sms, cudaStream_t st);

@@ -1,0 +1,45 @@
+"""Box generations through packed words (bb.cu) against the oracle: sides that
+are and are not whole words, rows that start at any byte, one and several
+words per row, bytes other than 0 and 1 on and off the fractal, the two rules
+with a closed form and others, one and several generations."""
+import numpy as np
+import pytest
+import torch
+
+import oracle
+from paper_2110_12952_gb300 import workloads as W
+
+pytestmark = pytest.mark.gpu
+
+CASES = [("triangle", 5), ("triangle", 6), ("triangle", 9), ("full_square", 5), ("full_square", 10), ("carpet", 4), ("carpet", 5),
+         ("carpet", 6), ("vicsek", 7), ("candy", 3), ("candy", 5), ("menger", 4), ("menger", 5)]
+
+
+@pytest.mark.parametrize("name,r", CASES)
+def test_box_generations_match_oracle(name, r):
+    from paper_2110_12952_gb300 import Fractal
+    fam = W.FAMILIES[name]
+    g, o = Fractal.from_family(fam, r), oracle.Fractal(fam.k, fam.s, r, fam.dim, fam.table())
+    rng = np.random.default_rng(r)
+    x = (rng.random(o.box_cells) < 0.45).astype(np.uint8) * rng.integers(1, 256, o.box_cells).astype(np.uint8)
+    rules = [W.MENGER_B5S45, W.rule_masks([4], [3, 4, 5, 26])] if fam.dim == 3 else [W.LIFE_B3S23, W.rule_masks([2, 8], [0, 1, 2, 3, 8])]
+    src = torch.from_numpy(x).cuda()
+    for rule, steps in zip(rules * 2, (1, 2, 3, 2)):
+        whole = torch.full((o.box_cells + 64,), 77, dtype=torch.uint8, device="cuda")
+        g.bb_step(src, out=whole[:o.box_cells], steps=steps, rule=rule)
+        want = o.bb_step(x, rule=oracle.Rule(*rule), steps=steps)
+        assert np.array_equal(whole[:o.box_cells].cpu().numpy(), want), (name, r, rule, steps)
+        assert int((whole[o.box_cells:] == 77).sum()) == 64
+    assert torch.equal(src.cpu(), torch.from_numpy(x))
+    g.close()
+
+
+def test_long_box_rows():
+    # rows longer than a packing tile (16384 cells) and than a block's words: the full square at side 32768 against
+    # single generations of the row kernel
+    from paper_2110_12952_gb300 import Fractal
+    g = Fractal.from_family(W.FULL_SQUARE, 15)
+    x = torch.empty(g.box_cells, dtype=torch.uint8, device="cuda").bernoulli_(0.4)
+    one = g.bb_step(g.bb_step(x, steps=1), steps=1)
+    assert torch.equal(g.bb_step(x, steps=2), one)
+    g.close()

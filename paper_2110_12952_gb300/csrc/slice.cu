@@ -31,6 +31,8 @@
 #include <string.h>
 
 #include <algorithm>
+#include <cmath>
+#include <new>
 #include <vector>
 
 #include "handle.h"
@@ -42,8 +44,21 @@ namespace fr {
 constexpr int kSliceBlock = 256;   // threads per block of the streaming kernels
 constexpr int kSliceAhead = 2;     // halo words per warp loaded ahead of their group
 constexpr int kSliceBatch = 2;     // 16-byte units per thread and batch copied to shared memory ahead
+constexpr int kSliceSmem = 220 * 1024;   // resident kernel: shared memory per block
+constexpr int64_t kSliceBatchCells = 60000000;   // batches: most cells of an instance
 constexpr int kSliceSingleHalo = 32;   // most halo cells of a tile for the single-pass kernel
 constexpr int kSliceRounds = 32;   // resident kernel: most 32-cell chunks per warp
+
+// One group of a batch: its bytes, its tiles and where its instance lies
+// among the launch's groups.
+struct SliceGroup {
+    const uint8_t *in;
+    uint8_t *out;
+    int32_t nt;                 // tiles (at most 32)
+    int32_t tile0, levels, side;   // first tile in its instance; the instance's levels above the tiles, and its side in tiles
+    int32_t group0;             // the instance's first group
+    int32_t steps;              // generations; groups come in order of decreasing steps
+};
 
 struct SliceArgs {
     int64_t NT, NG;
@@ -54,13 +69,14 @@ struct SliceArgs {
     uint32_t lane_bits;     // packing: bits between tiles' bit strings
     int RP;                 // unpacking: words between tiles' bit strings (odd)
     int AW, A_zero;         // words of one group's array, index of its 32 zero words
-    DivU32 kdiv;            // division by KL
+    DivU32 kdiv, cdiv, jdiv, xdiv;   // division by KL, NC, NJ and XW
     uint32_t mb[9], ms[9];  // rule: all ones where a dead / live cell with c live neighbours becomes live
     const uint4 *tab;
     const uint32_t *jobs;   // halo words: export word | direction << 8
     const uint16_t *xlist;  // [XW][32]: cells of the export words
     const uint2 *cells;     // [H] halo cells: cell of the neighbouring tile, word index | direction << 16
     const int32_t *nbr;
+    const SliceGroup *groups;   // batches: [NG], else null
     uint32_t *bar;
     int *status;
 };
@@ -197,13 +213,12 @@ __device__ __forceinline__ void slice_odd_units(const SliceArgs &a, const uint8_
     }
 }
 
-// The bytes of group g as a bit string in omega order, by nth threads.
-__device__ __forceinline__ void slice_bytes_to_string(const SliceArgs &a, const uint8_t *__restrict__ in, int64_t g,
-                                                      uint32_t *B, int tid, int nth)
+// The bytes of a group of nt tiles as a bit string in omega order, by nth threads.
+__device__ __forceinline__ void slice_bytes_to_string(const SliceArgs &a, const uint8_t *__restrict__ src, int nt, uint32_t *B,
+                                                      int tid, int nth)
 {
-    const int bytes = (int)min((int64_t)32, a.NT - 32 * g) * a.KL;
-    const uint8_t *src = in + 32 * g * a.KL;
-    const int whole = ((uintptr_t)in & 15) == 0 ? bytes / 16 : 0;
+    const int bytes = nt * a.KL;
+    const int whole = ((uintptr_t)src & 15) == 0 ? bytes / 16 : 0;
 #pragma unroll 4
     for (int i = tid; i < whole; i += nth)
         slice_put16(a, B, i, slice_bits16(__ldcs(reinterpret_cast<const uint4 *>(src) + i)));
@@ -383,14 +398,12 @@ __device__ __forceinline__ uint32_t slice_nib(uint32_t x)
     return (__byte_perm(x, 0u, 0x4440 | J) * 0x00204081u) & 0x01010101u;
 }
 
-// The group's new bytes from the tiles' bit strings: 32 cells per thread.
-__device__ __forceinline__ void slice_string_to_bytes(const SliceArgs &a, const uint32_t *R, uint8_t *__restrict__ out,
-                                                      int64_t g, int tid, int nth)
+// The new bytes of a group of nt tiles from the tiles' bit strings: 32 cells per thread.
+__device__ __forceinline__ void slice_string_to_bytes(const SliceArgs &a, const uint32_t *R, uint8_t *__restrict__ ob, int nt,
+                                                      int tid, int nth)
 {
-    const int nt = (int)min((int64_t)32, a.NT - 32 * g);
     const int bytes = nt * a.KL;
-    uint8_t *ob = out + 32 * g * a.KL;
-    const int whole = ((uintptr_t)out & 15) == 0 ? bytes / 16 : 0;   // 16-byte units
+    const int whole = ((uintptr_t)ob & 15) == 0 ? bytes / 16 : 0;   // 16-byte units
     const int lane = tid & 31;
     // a warp's 32 x 32 cells; the lanes pass halves on so that consecutive
     // lanes store consecutive 16 bytes
@@ -488,7 +501,7 @@ slice_step_kernel(SliceArgs a, const uint32_t *src, uint32_t *dst, uint8_t *__re
             }
             __syncthreads();
             if (BYTES) {
-                slice_string_to_bytes(a, R, out, g, tid, blockDim.x);
+                slice_string_to_bytes(a, R, out + 32 * g * a.KL, (int)min((int64_t)32, a.NT - 32 * g), tid, blockDim.x);
             } else {
                 slice_export(a, tr, N, dst + a.ex + g * a.XW * 32, warp, nw, lane);
             }
@@ -565,7 +578,7 @@ slice_single_kernel(SliceArgs a, const uint8_t *__restrict__ in, uint8_t *__rest
         for (int c = warp; c < a.NC; c += nw)
             B[lane * a.RP + c] = tr(slice_next<D, LIFE>(a, __ldg(a.tab + 32 * c + lane), A, c, lane));
         __syncthreads();
-        slice_string_to_bytes(a, B, out, g, tid, blockDim.x);
+        slice_string_to_bytes(a, B, out + 32 * g * a.KL, nt, tid, blockDim.x);
         __syncthreads();
     }
 }
@@ -588,8 +601,10 @@ slice_single_kernel(SliceArgs a, const uint8_t *__restrict__ in, uint8_t *__rest
 // run of `rounds` items each; past the last item a warp repeats it.
 struct SliceWalk {
     int q, j, n, groups;
-    __device__ __forceinline__ SliceWalk(int n_, int groups_, int first) : q(first / n_), j(first % n_), n(n_), groups(groups_)
+    __device__ __forceinline__ SliceWalk(int n_, const DivU32 &ndiv, int groups_, int first)
+        : q(n_ > 1 ? (int)divu(ndiv, (uint32_t)first) : first), n(n_), groups(groups_)
     {
+        j = first - q * n;
         clamp();
     }
     __device__ __forceinline__ void clamp()
@@ -609,7 +624,7 @@ struct SliceWalk {
     }
 };
 
-template <int D, bool LIFE, bool ONE, int ROUNDS>
+template <int D, bool LIFE, bool ONE, int ROUNDS, bool BATCH>
 __global__ void __launch_bounds__(1024, 1)
 slice_resident_kernel(SliceArgs a, const uint8_t *__restrict__ in, uint8_t *__restrict__ out, uint32_t *ex0, uint32_t *ex1,
                       int per_block, int64_t steps)
@@ -622,7 +637,8 @@ slice_resident_kernel(SliceArgs a, const uint8_t *__restrict__ in, uint8_t *__re
     const int exw = ONE ? (int)a.NG * a.XW * 32 : 0;
     uint16_t *xlist = reinterpret_cast<uint16_t *>(exs + 2 * exw);
     int32_t *from = reinterpret_cast<int32_t *>(exs + 2 * exw + a.XW * 16);
-    uint32_t *A0 = exs + 2 * exw + a.XW * 16 + per_block * a.NJ * 32;
+    int32_t *left = from + per_block * a.NJ * 32;   // generations of the block's groups, decreasing
+    uint32_t *A0 = reinterpret_cast<uint32_t *>(left + per_block);
     if (ONE) {
         ex0 = exs;
         ex1 = exs + exw;
@@ -638,54 +654,84 @@ slice_resident_kernel(SliceArgs a, const uint8_t *__restrict__ in, uint8_t *__re
         const int32_t Q = slice_nbr(a, g0 + q * gs, jb, lane);
         from[x * 32 + lane] = Q < 0 ? -1 : ((Q >> 5) * a.XW + (int)(jb & 0xffu)) * 32 + (Q & 31);
     }
-    for (int q = 0; q < mine; ++q) slice_bytes_to_string(a, in, g0 + q * gs, A0 + q * a.AW, tid, nth);
+    auto tiles = [&](int64_t g) { return BATCH ? a.groups[g].nt : (int)min((int64_t)32, a.NT - 32 * g); };
+    if (BATCH)
+        for (int q = tid; q < mine; q += nth) left[q] = a.groups[g0 + q * gs].steps;
+    for (int q = 0; q < mine; ++q) {
+        const int64_t g = g0 + q * gs;
+        slice_bytes_to_string(a, BATCH ? a.groups[g].in : in + 32 * g * a.KL, tiles(g), A0 + q * a.AW, tid, nth);
+    }
     __syncthreads();
     uint32_t w[ROUNDS];
-    const SliceWalk chunk0(a.NC, mine, warp * rounds);
     {
-        SliceWalk k = chunk0;
-        const int nt_last = (int)(a.NT - 32 * (a.NG - 1));   // tiles of the last group, the last one of its block
-        const int short_q = (g0 + (mine - 1) * gs == a.NG - 1) ? mine - 1 : -1;
+        // (bits of tiles past a group's last are never read by others)
+        SliceWalk k(a.NC, a.cdiv, mine, warp * rounds);
 #pragma unroll
         for (int i = 0; i < ROUNDS; ++i)
             if (i < rounds) {
-                w[i] = slice_string_chunk(a, tr, A0 + k.q * a.AW, k.j, k.q == short_q ? nt_last : 32, lane);
+                w[i] = slice_string_chunk(a, tr, A0 + k.q * a.AW, k.j, 32, lane);
                 k.next();
             }
     }
     __syncthreads();
     for (int q = warp; q < mine; q += nw) A0[q * a.AW + a.A_zero + lane] = 0u;   // the words of absent neighbours
-    auto put_words = [&]() {
-        SliceWalk k = chunk0;
+    // groups with generations left (the first ones; all of them unless BATCH) and the rounds their items take
+    int active = mine, now = rounds, im_n = (mine * a.NJ + nw - 1) / nw, ex_n = (mine * a.XW + nw - 1) / nw;
+    const SliceWalk chunks0(a.NC, a.cdiv, mine, warp * rounds), im0(max(a.NJ, 1), a.jdiv, mine, warp * im_n),
+        ex0w(max(a.XW, 1), a.xdiv, mine, warp * ex_n);
+    auto chunk_walk = [&]() { return BATCH ? SliceWalk(a.NC, a.cdiv, active, warp * now) : chunks0; };
+    // the new words of the first `groups` groups
+    auto put_words = [&](int groups) {
+        SliceWalk k = chunk_walk();
 #pragma unroll
         for (int i = 0; i < ROUNDS; ++i)
-            if (i < rounds) {
-                A0[k.q * a.AW + 32 * k.j + lane] = w[i];
+            if (i < now) {
+                if (!BATCH || k.q < groups) A0[k.q * a.AW + 32 * k.j + lane] = w[i];
                 k.next();
             }
     };
-    const int ex_rounds = (mine * a.XW + nw - 1) / nw, im_rounds = (mine * a.NJ + nw - 1) / nw;
-    const SliceWalk ex_walk0(max(a.XW, 1), mine, warp * ex_rounds), im_walk0(max(a.NJ, 1), mine, warp * im_rounds);
-    auto put_exports = [&](uint32_t *ex) {
-        SliceWalk k = ex_walk0;
-        for (int i = 0; i < ex_rounds; ++i, k.next()) {
+    // the bit strings of the groups from `from` on
+    auto put_strings = [&](int first) {
+        SliceWalk k = chunk_walk();
+#pragma unroll
+        for (int i = 0; i < ROUNDS; ++i)
+            if (i < now) {
+                if (!BATCH || k.q >= first) A0[k.q * a.AW + lane * a.RP + k.j] = tr(w[i]);
+                k.next();
+            }
+    };
+    auto put_exports = [&](int groups, uint32_t *ex) {
+        if (BATCH && groups == 0) return;
+        if (BATCH && groups != active) ex_n = (groups * a.XW + nw - 1) / nw;
+        SliceWalk k = BATCH ? SliceWalk(max(a.XW, 1), a.xdiv, groups, warp * ex_n) : ex0w;
+        for (int i = 0; i < ex_n; ++i, k.next()) {
             const uint32_t v = tr(A0[k.q * a.AW + xlist[32 * k.j + lane]]);
             if (ONE) ex[(k.q * a.XW + k.j) * 32 + lane] = v;
             else __stcg(ex + ((g0 + k.q * gs) * a.XW + k.j) * 32 + lane, v);
         }
     };
-    put_words();
+    auto put_bytes = [&](int first, int end) {
+        for (int q = first; q < end; ++q) {
+            const int64_t g = g0 + q * gs;
+            slice_string_to_bytes(a, A0 + q * a.AW, BATCH ? a.groups[g].out : out + 32 * g * a.KL, tiles(g), tid, nth);
+        }
+    };
+    put_words(mine);
     __syncthreads();
-    put_exports(ex0);
+    put_exports(mine, ex0);
     for (int64_t gen = 1; gen <= steps; ++gen) {
         // everybody's exports of the state before this generation are there
         if (ONE) __syncthreads();
         else if (!slice_grid_barrier(a, (uint32_t)gen)) break;
+        if (BATCH && active == 0) continue;
+        int going = active;   // groups with more generations after this one
+        if (BATCH)
+            while (going > 0 && left[going - 1] == gen) --going;
         const uint32_t *ei = (gen & 1) ? ex0 : ex1;
         {
-            SliceWalk k = im_walk0;
+            SliceWalk k = BATCH ? SliceWalk(max(a.NJ, 1), a.jdiv, active, warp * im_n) : im0;
 #pragma unroll 2
-            for (int i = 0; i < im_rounds; ++i, k.next()) {
+            for (int i = 0; i < im_n; ++i, k.next()) {
                 const int at = from[(k.q * a.NJ + k.j) * 32 + lane];
                 uint32_t e = 0u;
                 if (at >= 0) e = ONE ? ei[at] : __ldcg(ei + at);
@@ -694,32 +740,40 @@ slice_resident_kernel(SliceArgs a, const uint8_t *__restrict__ in, uint8_t *__re
         }
         __syncthreads();
         {
-            SliceWalk k = chunk0;
+            SliceWalk k = chunk_walk();
 #pragma unroll
             for (int i = 0; i < ROUNDS; ++i)
-                if (i < rounds) {
+                if (i < now) {
                     w[i] = slice_next<D, LIFE>(a, tab[32 * k.j + lane], A0 + k.q * a.AW, k.j, lane);
                     k.next();
                 }
         }
         __syncthreads();
-        if (gen < steps) {
-            put_words();
+        if (BATCH ? going > 0 : gen < steps) {
+            put_words(going);
+            if (!BATCH) {
+                __syncthreads();
+                put_exports(mine, (gen & 1) ? ex1 : ex0);
+            }
+        }
+        if (BATCH) {
+            if (going < active) put_strings(going);   // the last generation of some groups
             __syncthreads();
-            put_exports((gen & 1) ? ex1 : ex0);
+            put_exports(going, (gen & 1) ? ex1 : ex0);
+            if (going < active) {
+                put_bytes(going, active);
+                active = going;
+                now = (active * a.NC + nw - 1) / nw;
+                im_n = (active * a.NJ + nw - 1) / nw;
+                ex_n = (active * a.XW + nw - 1) / nw;
+            }
         }
     }
-    {
-        SliceWalk k = chunk0;
-#pragma unroll
-        for (int i = 0; i < ROUNDS; ++i)
-            if (i < rounds) {
-                A0[k.q * a.AW + lane * a.RP + k.j] = tr(w[i]);
-                k.next();
-            }
+    if (!BATCH) {
+        put_strings(0);
+        __syncthreads();
+        put_bytes(0, mine);
     }
-    __syncthreads();
-    for (int q = 0; q < mine; ++q) slice_string_to_bytes(a, A0 + q * a.AW, out, g0 + q * gs, tid, nth);
     if (!ONE && tid == 0) {
         // the last block to leave resets the barrier for the next launch
         if (atomicAdd(a.bar + 1, 1u) == gridDim.x - 1) {
@@ -732,17 +786,28 @@ slice_resident_kernel(SliceArgs a, const uint8_t *__restrict__ in, uint8_t *__re
 
 // Neighbours of every tile, a row of 32 lanes per group and direction
 // (tiles past the last have none), from rows of 8 per tile.
-__global__ void slice_nbr_kernel(FracDev F, int64_t NT, int64_t NG, int coarse_levels, int32_t coarse_side, int32_t *__restrict__ out)
+__global__ void slice_nbr_kernel(FracDev F, int64_t NT, int64_t NG, int coarse_levels, int32_t coarse_side,
+                                 const SliceGroup *__restrict__ groups, int32_t *__restrict__ out)
 {
-    for (int64_t T = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; T < 32 * NG; T += (int64_t)gridDim.x * blockDim.x) {
+    for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < 32 * NG; i += (int64_t)gridDim.x * blockDim.x) {
+        int64_t T = i, base = 0;
+        bool live = T < NT;
+        if (groups) {   // a batch: the tile's place in its instance, whose tiles start at group group0
+            const SliceGroup s = groups[i >> 5];
+            live = (i & 31) < s.nt;
+            T = s.tile0 + (i & 31);
+            base = 32 * (int64_t)s.group0;
+            coarse_levels = s.levels;
+            coarse_side = s.side;
+        }
         int32_t c[3] = {0, 0, 0};
-        if (T < NT) lambda64(F, (uint64_t)T, coarse_levels, c);
+        if (live) lambda64(F, (uint64_t)T, coarse_levels, c);
         for (int d = 0; d < 8; ++d) {
             const int q = d < 4 ? d : d + 1;
             const int32_t x = c[0] + q % 3 - 1, y = c[1] + q / 3 - 1;
             int64_t v = -1;
-            if (T < NT && x >= 0 && x < coarse_side && y >= 0 && y < coarse_side) v = nu_levels(F, x, y, 0, coarse_levels);
-            out[((T >> 5) * 8 + d) * 32 + (T & 31)] = (int32_t)v;
+            if (live && x >= 0 && x < coarse_side && y >= 0 && y < coarse_side) v = nu_levels(F, x, y, 0, coarse_levels);
+            out[((i >> 5) * 8 + d) * 32 + (i & 31)] = v < 0 ? -1 : (int32_t)(base + v);
         }
     }
 }
@@ -971,27 +1036,57 @@ static SingleFn single_fn(int D, bool life)
 using ResidentFn = void (*)(SliceArgs, const uint8_t *, uint8_t *, uint32_t *, uint32_t *, int, int64_t);
 
 // rounds: 32-cell chunks per warp
-template <int D, bool ONE>
-static ResidentFn resident_fn_d(bool life, int rounds)
+template <int D, bool LIFE>
+static ResidentFn resident_fn_d(const SlicePlan &s)
 {
-    if (rounds <= 1) return life ? slice_resident_kernel<D, true, ONE, 1> : slice_resident_kernel<D, false, ONE, 1>;
-    if (ONE || rounds <= 8) return life ? slice_resident_kernel<D, true, ONE, 8> : slice_resident_kernel<D, false, ONE, 8>;
-    if (rounds <= 20) return life ? slice_resident_kernel<D, true, false, 20> : slice_resident_kernel<D, false, false, 20>;
-    return life ? slice_resident_kernel<D, true, false, kSliceRounds> : slice_resident_kernel<D, false, false, kSliceRounds>;
+    if (s.groups) return s.rounds <= 8 ? slice_resident_kernel<D, LIFE, false, 8, true> : slice_resident_kernel<D, LIFE, false, kSliceRounds, true>;
+    if (s.grid_resident == 1)
+        return s.rounds <= 1 ? slice_resident_kernel<D, LIFE, true, 1, false> : slice_resident_kernel<D, LIFE, true, 8, false>;
+    if (s.rounds <= 8) return slice_resident_kernel<D, LIFE, false, 8, false>;
+    if (s.rounds <= 20) return slice_resident_kernel<D, LIFE, false, 20, false>;
+    return slice_resident_kernel<D, LIFE, false, kSliceRounds, false>;
 }
 
 static ResidentFn resident_fn(const SlicePlan &s, bool life)
 {
-    const bool one = s.grid_resident == 1;
     switch (s.geo.D) {
-        case 4: return one ? resident_fn_d<4, true>(life, s.rounds) : resident_fn_d<4, false>(life, s.rounds);
-        case 6: return one ? resident_fn_d<6, true>(life, s.rounds) : resident_fn_d<6, false>(life, s.rounds);
-        case 7: return one ? resident_fn_d<7, true>(life, s.rounds) : resident_fn_d<7, false>(life, s.rounds);
-        default: return one ? resident_fn_d<8, true>(life, s.rounds) : resident_fn_d<8, false>(life, s.rounds);
+        case 4: return life ? resident_fn_d<4, true>(s) : resident_fn_d<4, false>(s);
+        case 6: return life ? resident_fn_d<6, true>(s) : resident_fn_d<6, false>(s);
+        case 7: return life ? resident_fn_d<7, true>(s) : resident_fn_d<7, false>(s);
+        default: return life ? resident_fn_d<8, true>(s) : resident_fn_d<8, false>(s);
     }
 }
 
 static bool slice_fractal_ok(const fractal *f) { return f->dim == 2 && !f->mixed && f->k >= 2 && f->r >= 1; }
+
+// The resident kernels of the plan may use its shared memory, a block per SM.
+static cudaError_t resident_ready(const SlicePlan &s)
+{
+    cudaError_t e = cudaSuccess;
+    for (int life = 0; life < 2 && e == cudaSuccess; ++life) {
+        ResidentFn fn = resident_fn(s, life);
+        int per_sm = 0;
+        e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, kSliceSmem);
+        if (e == cudaSuccess)
+            e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, fn, s.block_resident, s.smem_resident);
+        if (e == cudaSuccess && per_sm < 1) e = cudaErrorInvalidConfiguration;
+    }
+    return e;
+}
+
+static int launch_resident(const SlicePlan &s, const SliceArgs &a, bool life, const uint8_t *in, uint8_t *out, int64_t steps,
+                           cudaStream_t st)
+{
+    ResidentFn fn = resident_fn(s, life);
+    uint32_t *e0 = s.ex[0], *e1 = s.ex[1];
+    int per_block = s.per_block;
+    void *args[] = {(void *)&a, &in, &out, &e0, &e1, &per_block, &steps};
+    if (s.grid_resident > 1)
+        FR_CUDA(cudaLaunchCooperativeKernel((const void *)fn, dim3(s.grid_resident), dim3(s.block_resident), args, s.smem_resident, st));
+    else
+        FR_CUDA(cudaLaunchKernel((const void *)fn, dim3(1), dim3(s.block_resident), args, s.smem_resident, st));
+    return FR_OK;
+}
 
 // Geometry of the tables of one tile depth.
 static SliceGeo slice_geo(const fractal *f, int L, const SliceTables &t)
@@ -1017,19 +1112,19 @@ static int string_words(const SliceGeo &p) { return p.BP ? 32 * p.BP : p.KLp + 1
 
 constexpr int kSliceMaxKL = 4096;
 constexpr int kSliceWave = 760;
-constexpr int kSliceSmem = 220 * 1024;   // resident kernel: shared memory per block
 
 // Blocks, groups per block and threads of the resident kernel, and its
 // estimated cycles per generation; false when the state does not fit.
-static bool slice_resident_shape(const SliceGeo &p, int num_sms, SlicePlan *s, double *cost)
+static bool slice_resident_shape(const SliceGeo &p, int num_sms, bool batch, SlicePlan *s, double *cost)
 {
     // one block where that takes no more than 8 chunks per warp, else as many as there are SMs
     for (int64_t grid : {(int64_t)1, std::min<int64_t>(num_sms, p.NG)}) {
+        if (grid == 1 && batch && p.NG > 1) continue;   // (batches: no kernel for a single block's exports)
         const int64_t per = (p.NG + grid - 1) / grid, chunks = per * p.NC;
         const int64_t rounds = (chunks + 31) / 32;
         if (rounds > (grid == 1 ? 8 : kSliceRounds)) continue;
         const int64_t exw = grid == 1 ? 2 * p.NG * p.XW * 32 : 0;
-        const int64_t smem = 4 * (4 * p.KLp + exw + 16 * p.XW + per * (32 * p.NJ + p.AW));
+        const int64_t smem = 4 * (4 * p.KLp + exw + 16 * p.XW + per * (32 * p.NJ + 1 + p.AW));
         if (smem > kSliceSmem) continue;
         // `n` warp-sized items of `instr` instructions: at least a chain of
         // latencies per round, else the SM's issue rate
@@ -1069,7 +1164,7 @@ static int slice_levels(const fractal *f, SlicePlan *plan, SliceTables *tables)
         if (p.AW * 4 > 65535 || p.XW > 255) continue;
         SlicePlan s;
         double c;
-        if (!slice_resident_shape(p, f->num_sms, &s, &c)) {
+        if (!slice_resident_shape(p, f->num_sms, false, &s, &c)) {
             const int64_t waves = (p.NG + kSliceWave - 1) / kSliceWave;
             c = (double)waves * (p.NC * 45 + 30.0 * (p.NJ + p.XW) + 400);
         }
@@ -1085,6 +1180,41 @@ static int slice_levels(const fractal *f, SlicePlan *plan, SliceTables *tables)
     return best;
 }
 
+// One allocation: the tables (copied from the host in one piece), the grid
+// barrier's zeros, the neighbouring tiles and the resident exports.
+static cudaError_t slice_upload(SliceGeo &p, const SliceTables &t, SlicePlan &s, const std::vector<SliceGroup> &groups,
+                                cudaStream_t st)
+{
+    size_t off = 0;
+    auto take = [&](size_t bytes) {
+        const size_t at = off;
+        off += (bytes + 255) / 256 * 256;
+        return at;
+    };
+    const size_t o_tab = take((size_t)p.KLp * 16), o_jobs = take(t.jobs.size() * 4), o_xl = take(t.xlist.size() * 2),
+                 o_cells = take(t.cells.size() * 4), o_bar = take(8), o_groups = take(groups.size() * sizeof(SliceGroup)), host = off;
+    const size_t o_nbr = take((size_t)p.NG * 256 * sizeof(int32_t)),
+                 exb = s.resident ? (size_t)p.NG * p.XW * 128 : 0, o_ex0 = take(exb), o_ex1 = take(exb);
+    std::vector<uint8_t> img(host, 0);
+    slice_neighbour_table(t, p.D, reinterpret_cast<uint16_t *>(img.data() + o_tab));
+    memcpy(img.data() + o_jobs, t.jobs.data(), t.jobs.size() * 4);
+    memcpy(img.data() + o_xl, t.xlist.data(), t.xlist.size() * 2);
+    memcpy(img.data() + o_cells, t.cells.data(), t.cells.size() * 4);
+    if (!groups.empty()) memcpy(img.data() + o_groups, groups.data(), groups.size() * sizeof(SliceGroup));
+    cudaError_t e = cudaMalloc(&s.arena, off);
+    if (e == cudaSuccess) e = cudaMemcpyAsync(s.arena, img.data(), host, cudaMemcpyHostToDevice, st);
+    p.tab = reinterpret_cast<uint4 *>(s.arena + o_tab);
+    p.jobs = reinterpret_cast<uint32_t *>(s.arena + o_jobs);
+    p.xlist = reinterpret_cast<uint16_t *>(s.arena + o_xl);
+    p.cells = reinterpret_cast<uint2 *>(s.arena + o_cells);
+    p.nbr = reinterpret_cast<int32_t *>(s.arena + o_nbr);
+    s.bar = reinterpret_cast<uint32_t *>(s.arena + o_bar);
+    s.groups = groups.empty() ? nullptr : s.arena + o_groups;
+    s.ex[0] = reinterpret_cast<uint32_t *>(s.arena + o_ex0);
+    s.ex[1] = reinterpret_cast<uint32_t *>(s.arena + o_ex1);
+    return e;
+}
+
 static int build_slice_plan(fractal *f, cudaStream_t st)
 {
     SliceTables t;
@@ -1096,50 +1226,16 @@ static int build_slice_plan(fractal *f, cudaStream_t st)
     s.smem_single = ring + 4 * (p.AW + std::max(string_words(p), 32 * p.RP + 1));
     s.smem_step = 4 * (2 * p.AW + p.KLp);
     s.smem_bytes = 4 * (2 * p.AW + 32 * p.RP + 1);
-    // one allocation: the tables (copied from the host in one piece), the
-    // grid barrier's zeros, the neighbouring tiles and the resident exports
-    size_t off = 0;
-    auto take = [&](size_t bytes) {
-        const size_t at = off;
-        off += (bytes + 255) / 256 * 256;
-        return at;
-    };
-    const size_t o_tab = take((size_t)p.KLp * 16), o_jobs = take(t.jobs.size() * 4), o_xl = take(t.xlist.size() * 2),
-                 o_cells = take(t.cells.size() * 4), o_bar = take(8), host = off;
-    const size_t o_nbr = take((size_t)p.NG * 256 * sizeof(int32_t)),
-                 exb = s.resident ? (size_t)p.NG * p.XW * 128 : 0, o_ex0 = take(exb), o_ex1 = take(exb);
-    std::vector<uint8_t> img(host, 0);
-    slice_neighbour_table(t, p.D, reinterpret_cast<uint16_t *>(img.data() + o_tab));
-    memcpy(img.data() + o_jobs, t.jobs.data(), t.jobs.size() * 4);
-    memcpy(img.data() + o_xl, t.xlist.data(), t.xlist.size() * 2);
-    memcpy(img.data() + o_cells, t.cells.data(), t.cells.size() * 4);
-    cudaError_t e = cudaMalloc(&s.arena, off);
-    if (e == cudaSuccess) e = cudaMemcpyAsync(s.arena, img.data(), host, cudaMemcpyHostToDevice, st);
-    p.tab = reinterpret_cast<uint4 *>(s.arena + o_tab);
-    p.jobs = reinterpret_cast<uint32_t *>(s.arena + o_jobs);
-    p.xlist = reinterpret_cast<uint16_t *>(s.arena + o_xl);
-    p.cells = reinterpret_cast<uint2 *>(s.arena + o_cells);
-    s.bar = reinterpret_cast<uint32_t *>(s.arena + o_bar);
-    p.nbr = reinterpret_cast<int32_t *>(s.arena + o_nbr);
-    s.ex[0] = reinterpret_cast<uint32_t *>(s.arena + o_ex0);
-    s.ex[1] = reinterpret_cast<uint32_t *>(s.arena + o_ex1);
+    cudaError_t e = slice_upload(p, t, s, {}, st);
     if (e == cudaSuccess) {
         const int64_t blocks = std::min<int64_t>((32 * p.NG + 255) / 256, (int64_t)f->num_sms * 16);
-        slice_nbr_kernel<<<(unsigned)blocks, 256, 0, st>>>(f->dev, p.NT, p.NG, f->r - p.L, (int32_t)pw(f->s, f->r - p.L), p.nbr);
+        slice_nbr_kernel<<<(unsigned)blocks, 256, 0, st>>>(f->dev, p.NT, p.NG, f->r - p.L, (int32_t)pw(f->s, f->r - p.L), nullptr, p.nbr);
         e = cudaGetLastError();
         if (e == cudaSuccess) e = cudaStreamSynchronize(st);   // the tables serve calls on any stream from here on
     }
     // shared memory and grids
     int per_sm = 0;
-    if (s.resident) {
-        for (int life = 0; life < 2 && e == cudaSuccess; ++life) {
-            ResidentFn fn = resident_fn(s, life);
-            e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, kSliceSmem);
-            if (e == cudaSuccess)
-                e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, fn, s.block_resident, s.smem_resident);
-            if (e == cudaSuccess && per_sm < 1) e = cudaErrorInvalidConfiguration;
-        }
-    }
+    if (s.resident && e == cudaSuccess) e = resident_ready(s);
     {
         const int most = 100 * 1024;
         if (std::max(std::max(s.smem_pack, s.smem_single), std::max(s.smem_step, s.smem_bytes)) > most) e = cudaErrorInvalidConfiguration;
@@ -1208,6 +1304,45 @@ static bool slice_use_resident(const SlicePlan &s, int64_t steps, int num_sms)
     return s.resident && (steps > 1 || s.geo.NG <= num_sms);
 }
 
+static SliceArgs slice_args(const SliceGeo &p, uint32_t birth, uint32_t survive, uint32_t *bar, int *status)
+{
+    SliceArgs a;
+    a.NT = p.NT;
+    a.NG = p.NG;
+    a.KL = p.KL;
+    a.KLp = p.KLp;
+    a.NC = p.NC;
+    a.NJ = p.NJ;
+    a.BP = p.BP;
+    a.RP = p.RP;
+    a.AW = p.AW;
+    a.A_zero = p.AW - 32;
+    a.XW = p.XW;
+    a.ex = p.NG * p.KLp;
+    a.kdiv = make_div((uint32_t)p.KL);
+    a.cdiv = make_div((uint32_t)std::max(2, p.NC));
+    a.jdiv = make_div((uint32_t)std::max(2, p.NJ));
+    a.xdiv = make_div((uint32_t)std::max(2, p.XW));
+    a.bsh = 30;
+    if (p.BP)
+        for (a.bsh = 0; (32 << a.bsh) < p.KL;) ++a.bsh;
+    a.lane_bits = p.BP ? 32u * (uint32_t)p.BP : (uint32_t)p.KL;
+    for (int c = 0; c < 9; ++c) {
+        a.mb[c] = (birth >> c) & 1u ? 0xffffffffu : 0u;
+        a.ms[c] = (survive >> c) & 1u ? 0xffffffffu : 0u;
+    }
+    a.tab = p.tab;
+    a.jobs = p.jobs;
+    a.xlist = p.xlist;
+    a.cells = p.cells;
+    a.H = p.H;
+    a.nbr = p.nbr;
+    a.groups = nullptr;
+    a.bar = bar;
+    a.status = status;
+    return a;
+}
+
 int try_slice_step(fractal *f, const uint8_t *in, uint8_t *out, int64_t steps, uint32_t birth, uint32_t survive,
                    cudaStream_t st, bool *done)
 {
@@ -1241,47 +1376,11 @@ int try_slice_step(fractal *f, const uint8_t *in, uint8_t *out, int64_t steps, u
         if (packed && (!slice_buffer(f, 0) || (steps > 1 && !slice_buffer(f, 1)))) return FR_OK;
     }
     const SliceGeo &p = s.geo;
-    SliceArgs a;
-    a.NT = p.NT;
-    a.NG = p.NG;
-    a.KL = p.KL;
-    a.KLp = p.KLp;
-    a.NC = p.NC;
-    a.NJ = p.NJ;
-    a.BP = p.BP;
-    a.RP = p.RP;
-    a.AW = p.AW;
-    a.A_zero = p.AW - 32;
-    a.XW = p.XW;
-    a.ex = p.NG * p.KLp;
-    a.kdiv = make_div((uint32_t)p.KL);
-    a.bsh = 30;
-    if (p.BP)
-        for (a.bsh = 0; (32 << a.bsh) < p.KL;) ++a.bsh;
-    a.lane_bits = p.BP ? 32u * (uint32_t)p.BP : (uint32_t)p.KL;
-    for (int c = 0; c < 9; ++c) {
-        a.mb[c] = (birth >> c) & 1u ? 0xffffffffu : 0u;
-        a.ms[c] = (survive >> c) & 1u ? 0xffffffffu : 0u;
-    }
-    a.tab = p.tab;
-    a.jobs = p.jobs;
-    a.xlist = p.xlist;
-    a.cells = p.cells;
-    a.H = p.H;
-    a.nbr = p.nbr;
-    a.bar = s.bar;
-    a.status = f->status;
+    const SliceArgs a = slice_args(p, birth, survive, s.bar, f->status);
     const bool life = (birth & 0x1ffu) == 0x8u && (survive & 0x1ffu) == 0xcu;
     if (res) {
-        ResidentFn fn = resident_fn(s, life);
-        uint32_t *e0 = s.ex[0], *e1 = s.ex[1];
-        int per_block = s.per_block;
-        void *args[] = {&a, &in, &out, &e0, &e1, &per_block, &steps};
-        if (s.grid_resident > 1)
-            FR_CUDA(cudaLaunchCooperativeKernel((const void *)fn, dim3(s.grid_resident), dim3(s.block_resident), args,
-                                                s.smem_resident, st));
-        else
-            FR_CUDA(cudaLaunchKernel((const void *)fn, dim3(1), dim3(s.block_resident), args, s.smem_resident, st));
+        const int rc = launch_resident(s, a, life, in, out, steps, st);
+        if (rc) return rc;
         *done = true;
         return FR_OK;
     }
@@ -1302,7 +1401,7 @@ int try_slice_step(fractal *f, const uint8_t *in, uint8_t *out, int64_t steps, u
         const uint32_t *src = s.bits[cur];
         uint32_t *dst = s.bits[cur ^ 1];
         uint8_t *none = nullptr;
-        void *args[] = {&a, &src, &dst, &none, &gens};
+        void *args[] = {(void *)&a, &src, &dst, &none, &gens};
         if (s.grid_step[life] > 1 && gens > 1)
             FR_CUDA(cudaLaunchCooperativeKernel((const void *)fn, dim3(s.grid_step[life]), dim3(kSliceBlock), args, s.smem_step, st));
         else
@@ -1315,9 +1414,181 @@ int try_slice_step(fractal *f, const uint8_t *in, uint8_t *out, int64_t steps, u
         const uint32_t *src = s.bits[cur];
         uint32_t *none = nullptr;
         int one = 1;
-        void *args[] = {&a, &src, &none, &out, &one};
+        void *args[] = {(void *)&a, &src, &none, &out, &one};
         FR_CUDA(cudaLaunchKernel((const void *)fb, dim3(s.grid_bytes[life]), dim3(kSliceBlock), args, s.smem_bytes, st));
     }
+    return FR_OK;
+}
+
+// ---------------------------------------------------------------- batches
+
+// Many instances of one fractal in resident launches: their groups stand in
+// one list (an instance starts a group of its own; the neighbour table keeps
+// them apart) and run as if they were one state.  Instances of few
+// generations come last in every block's share and drop out on the way.
+// Instances whose packed words do not fit the SMs' shared memory together run
+// in several launches, one after the other, each through all of its
+// generations; levels below a launch's tile depth have launches of their own.
+struct SliceBatch {
+    struct Launch {
+        SlicePlan plan;
+        SliceArgs args;
+        bool life;
+        int64_t steps;
+    };
+    std::vector<Launch> launches;
+};
+
+void free_slice_batch(SliceBatch *b)
+{
+    if (!b) return;
+    for (auto &l : b->launches) free_slice_plan(l.plan);
+    delete b;
+}
+
+int slice_batch_launches(const SliceBatch *b) { return (int)b->launches.size(); }
+
+int run_slice_batch(const SliceBatch *b, cudaStream_t st)
+{
+    for (const auto &l : b->launches) {
+        const int rc = launch_resident(l.plan, l.args, l.life, nullptr, nullptr, l.steps, st);
+        if (rc) return rc;
+    }
+    return FR_OK;
+}
+
+bool slice_batch_takes(const fractal *f, int64_t steps)
+{
+    return slice_fractal_ok(f) && steps >= 2 && steps < (1 << 30) && f->cells <= kSliceBatchCells &&
+           ((f->tile_levels_user < 0 && f->stages_user < 0) || f->sliced_tuned);
+}
+
+// Groups that fit one launch at this tile depth (0: none), and its cycles per generation.
+static int64_t slice_batch_fit(SliceGeo p, int num_sms, int64_t groups, double *cost)
+{
+    for (int n = 1; n <= 256; ++n) {
+        p.NG = (groups + n - 1) / n;
+        SlicePlan s;
+        double c = 0;
+        if (slice_resident_shape(p, num_sms, true, &s, &c)) {
+            *cost = n * c;
+            return p.NG;
+        }
+    }
+    return 0;
+}
+
+int build_slice_batch(const std::vector<SliceBatchItem> &items, uint32_t birth, uint32_t survive, cudaStream_t st, SliceBatch **out)
+{
+    *out = nullptr;
+    fractal *rep = items[0].f;
+    int rc = ensure_status(rep);
+    if (rc) return rc;
+    int rmax = 0;
+    for (const auto &i : items) rmax = std::max(rmax, i.f->r);
+    // tables by tile depth
+    std::vector<SliceTables> tabs(1);
+    std::vector<SliceGeo> geos(1);
+    const SliceNbrs first = slice_first(rep);
+    SliceNbrs nbrs = first;
+    for (int L = 1; L <= rmax && pw(rep->k, L) <= kSliceMaxKL; ++L) {
+        if (L > 1) nbrs = slice_deepen(first, nbrs, rep->k);
+        tabs.push_back(slice_tables(SliceNbrs(nbrs)));
+        geos.push_back(slice_geo(rep, L, tabs.back()));
+    }
+    const int lmax = (int)tabs.size() - 1;
+    auto groups_of = [&](const SliceBatchItem &i, int L) { return (pw(rep->k, i.f->r - L) + 31) / 32; };
+    // best[b]: tile depth and cost of all instances of fewer than b levels
+    struct Choice { int L = 0; int64_t cap = 0; double cost = 0; };
+    std::vector<Choice> best(rmax + 2);
+    for (int b = 2; b <= rmax + 1; ++b) {
+        bool any = false;
+        for (const auto &i : items) any = any || i.f->r < b;
+        if (!any) continue;
+        Choice pick;
+        for (int L = 1; L <= std::min(lmax, b - 1); ++L) {
+            if (geos[L].AW * 4 > 65535 || geos[L].XW > 255) continue;
+            int64_t groups = 0, largest = 0;
+            for (const auto &i : items)
+                if (i.f->r < b && i.f->r >= L) {
+                    groups += groups_of(i, L);
+                    largest = std::max(largest, groups_of(i, L));
+                }
+            double c = 0;
+            int64_t cap = 0;
+            if (groups) {
+                cap = slice_batch_fit(geos[L], rep->num_sms, groups, &c);
+                if (cap < largest) {   // as few launches as the largest instance allows
+                    double one = 0;
+                    cap = slice_batch_fit(geos[L], rep->num_sms, largest, &one);
+                    if (cap < largest) continue;
+                    c = one * std::ceil((double)groups / (double)cap);
+                }
+            }
+            bool rest = false;
+            for (const auto &i : items) rest = rest || i.f->r < L;
+            if (rest && best[L].L == 0) continue;
+            c += rest ? best[L].cost : 0.0;
+            if (pick.L == 0 || c < pick.cost) {
+                pick.L = L;
+                pick.cap = cap;
+                pick.cost = c;
+            }
+        }
+        best[b] = pick;
+    }
+    if (best[rmax + 1].L == 0) return FR_EINVAL;
+    SliceBatch *batch = new (std::nothrow) SliceBatch();
+    if (!batch) return FR_ENOMEM;
+    const bool life = (birth & 0x1ffu) == 0x8u && (survive & 0x1ffu) == 0xcu;
+    for (int b = rmax + 1; b > 1 && best[b].L > 0; b = best[b].L) {
+        const int L = best[b].L;
+        std::vector<const SliceBatchItem *> in;
+        for (const auto &i : items)
+            if (i.f->r < b && i.f->r >= L) in.push_back(&i);
+        std::stable_sort(in.begin(), in.end(), [](const SliceBatchItem *x, const SliceBatchItem *y) { return x->steps > y->steps; });
+        for (size_t i0 = 0; i0 < in.size();) {
+            std::vector<SliceGroup> groups;
+            size_t i = i0;
+            for (; i < in.size() && (i == i0 || (int64_t)groups.size() + groups_of(*in[i], L) <= best[b].cap); ++i) {
+                const SliceBatchItem &it = *in[i];
+                const int64_t NT = pw(rep->k, it.f->r - L), n = groups_of(it, L);
+                const int32_t g0 = (int32_t)groups.size(), levels = it.f->r - L, side = (int32_t)pw(rep->s, it.f->r - L);
+                for (int64_t g = 0; g < n; ++g)
+                    groups.push_back(SliceGroup{it.in + 32 * g * geos[L].KL, it.out + 32 * g * geos[L].KL,
+                                                (int32_t)std::min<int64_t>(32, NT - 32 * g), (int32_t)(32 * g), levels, side, g0,
+                                                (int32_t)it.steps});
+            }
+            batch->launches.emplace_back();
+            SliceBatch::Launch &l = batch->launches.back();
+            l.life = life;
+            l.steps = in[i0]->steps;
+            l.plan.geo = geos[L];
+            SliceGeo &p = l.plan.geo;
+            p.NG = (int64_t)groups.size();
+            p.NT = 32 * p.NG;
+            double c = 0;
+            cudaError_t e = slice_resident_shape(p, rep->num_sms, true, &l.plan, &c) ? cudaSuccess : cudaErrorInvalidConfiguration;
+            if (e == cudaSuccess) e = slice_upload(p, tabs[L], l.plan, groups, st);
+            if (e == cudaSuccess) {
+                const int64_t blocks = std::min<int64_t>((32 * p.NG + 255) / 256, (int64_t)rep->num_sms * 16);
+                slice_nbr_kernel<<<(unsigned)blocks, 256, 0, st>>>(rep->dev, p.NT, p.NG, 0, 1,
+                                                                   reinterpret_cast<const SliceGroup *>(l.plan.groups), p.nbr);
+                e = cudaGetLastError();
+                if (e == cudaSuccess) e = cudaStreamSynchronize(st);
+            }
+            if (e == cudaSuccess) e = resident_ready(l.plan);
+            if (e != cudaSuccess) {
+                cudaGetLastError();
+                free_slice_batch(batch);
+                return e == cudaErrorMemoryAllocation ? FR_ENOMEM : FR_ECUDA;
+            }
+            l.args = slice_args(p, birth, survive, l.plan.bar, rep->status);
+            l.args.groups = reinterpret_cast<const SliceGroup *>(l.plan.groups);
+            i0 = i;
+        }
+    }
+    *out = batch;
     return FR_OK;
 }
 

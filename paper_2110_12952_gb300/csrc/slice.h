@@ -5,6 +5,8 @@
 #include <cuda_runtime.h>
 #include <stdint.h>
 
+#include <vector>
+
 #include "internal.cuh"
 
 struct fractal;
@@ -40,6 +42,7 @@ struct SlicePlan {
     int grid_pack = 0, grid_step[2] = {0, 0}, grid_bytes[2] = {0, 0}, grid_single[2] = {0, 0};   // [1]: with the constant rule
     uint32_t *bits[2] = {nullptr, nullptr};   // packed states: NG x KLp words, then the exports, NG x XW x 32
     uint8_t *arena = nullptr;                 // the tables, and:
+    uint8_t *groups = nullptr;                // batches: the groups (SliceGroup)
     uint32_t *ex[2] = {nullptr, nullptr};     // resident kernel: the exports alone
     uint32_t *bar = nullptr;                  // grid barrier: arrivals, exits
 };
@@ -51,5 +54,20 @@ void free_slice_plan(SlicePlan &p);
 // rule the sliced step out.
 int try_slice_step(fractal *f, const uint8_t *in, uint8_t *out, int64_t steps, uint32_t birth, uint32_t survive,
                    cudaStream_t st, bool *done);
+
+// Batches: the instances that may go through sliced launches, their launches
+// (all items of one fractal table and one rule), and running them.
+struct SliceBatchItem {
+    fractal *f;
+    const uint8_t *in;
+    uint8_t *out;
+    int64_t steps;
+};
+struct SliceBatch;
+bool slice_batch_takes(const fractal *f, int64_t steps);
+int build_slice_batch(const std::vector<SliceBatchItem> &items, uint32_t birth, uint32_t survive, cudaStream_t st, SliceBatch **out);
+int run_slice_batch(const SliceBatch *b, cudaStream_t st);
+int slice_batch_launches(const SliceBatch *b);
+void free_slice_batch(SliceBatch *b);
 
 }  // namespace fr

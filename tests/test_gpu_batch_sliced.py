@@ -1,0 +1,57 @@
+"""Batches through sliced launches (slice.cu) against the oracle: levels below
+and above the launches' tile depth, single and several launches per fractal,
+uneven generation counts, two rules, unaligned buffers, instances next to each
+other in memory, and instances that the tile kernels keep."""
+import numpy as np
+import pytest
+import torch
+
+import oracle
+from paper_2110_12952_gb300 import workloads as W
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.mark.parametrize("seed,even", [(1, True), (2, False), (3, False)])
+def test_uneven_sliced_batches(seed, even):
+    from paper_2110_12952_gb300 import Batch, Fractal
+    rng = np.random.default_rng(seed)
+    levels = {"triangle": (1, 12), "carpet": (1, 6), "vicsek": (2, 8), "h_fractal": (3, 5), "menger": (3, 3)}
+    specs = []
+    for i in range(70):
+        name = list(levels)[int(rng.integers(0, len(levels)))]
+        lo, hi = levels[name]
+        steps = 7 if even else int(rng.integers(0, 25))
+        rule = W.default_rule(W.FAMILIES[name]) if i % 5 else (W.rule_masks([2], [1, 2, 3]) if name != "menger" else W.MENGER_B5S45)
+        specs.append((W.FAMILIES[name], int(rng.integers(lo, hi + 1)), steps, rule, int(rng.integers(0, 3))))
+    handles, batch, bufs = {}, Batch(), []
+    total = sum(f.k ** r + 40 for f, r, _, _, _ in specs)
+    src = torch.zeros(total, dtype=torch.uint8, device="cuda")
+    dst = torch.full((total,), 77, dtype=torch.uint8, device="cuda")
+    pos = 0
+    for i, (fam, r, steps, rule, skew) in enumerate(specs):
+        if (fam.name, r) not in handles:
+            handles[fam.name, r] = (Fractal.from_family(fam, r), oracle.Fractal(fam.k, fam.s, r, fam.dim, fam.table()))
+        g, o = handles[fam.name, r]
+        pos = (pos + 15) // 16 * 16 + skew
+        x, y = src[pos:pos + g.cells], dst[pos:pos + g.cells]
+        x.copy_(torch.from_numpy(o.init_bernoulli(i, 0.45)))
+        batch.add(g, x, y, steps, rule=rule)
+        bufs.append((pos, g.cells))
+        pos += g.cells
+    for rep in range(2):
+        batch.run()
+        torch.cuda.synchronize()
+        got = dst.cpu().numpy().copy()
+        for i, ((fam, r, steps, rule, _), (p, n)) in enumerate(zip(specs, bufs)):
+            o = handles[fam.name, r][1]
+            want = o.step(o.init_bernoulli(i + 1000 * rep, 0.45), rule=oracle.Rule(*rule), steps=steps)
+            assert np.array_equal(got[p:p + n], want), (fam.name, r, steps, i)
+            got[p:p + n] = 77
+        assert (got == 77).all()    # nothing written between the instances
+        for i, ((fam, r, _, _, _), (p, n)) in enumerate(zip(specs, bufs)):
+            src[p:p + n].copy_(torch.from_numpy(handles[fam.name, r][1].init_bernoulli(i + 1000, 0.45)))
+    batch.close()
+    for g, _ in handles.values():
+        g.check()
+        g.close()

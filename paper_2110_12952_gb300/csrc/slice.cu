@@ -1,5 +1,5 @@
-// slice.cu -- the bit-sliced compact step of 2D fractals (Sec. 3 stencil
-// procedure on 32 tiles at a time).
+// slice.cu -- the bit-sliced compact step (Sec. 3 stencil procedure on 32
+// tiles at a time).
 //
 // A tile is a level-L subtree (k^L cells, contiguous in omega).  All tiles
 // have the same local neighbour structure: cell l of a tile has, for each
@@ -42,6 +42,7 @@
 namespace fr {
 
 constexpr int kSliceBlock = 256;   // threads per block of the streaming kernels
+constexpr int kSliceBlock3 = 512;  // the same in 3D, where a group is larger (Menger: 8000 words and 3700 halo words)
 constexpr int kSliceAhead = 2;     // halo words per warp loaded ahead of their group
 constexpr int kSliceBatch = 2;     // 16-byte units per thread and batch copied to shared memory ahead
 constexpr int kSliceSmem = 220 * 1024;   // resident kernel: shared memory per block
@@ -63,6 +64,8 @@ struct SliceGroup {
 struct SliceArgs {
     int64_t NT, NG;
     int KL, KLp, NC, NJ, XW, H;
+    int ND;                 // directions: 8, or 26 in 3D
+    uint32_t birth, survive;
     int64_t ex;             // word offset of a state's exports behind its cells
     int BP;                 // packing: words between tiles' bit strings when a tile is 2^bsh words, else 0
     int bsh;                // (30: another number)
@@ -115,6 +118,45 @@ struct Transpose32 {
 __device__ __forceinline__ uint32_t sl_xor3(uint32_t a, uint32_t b, uint32_t c) { return a ^ b ^ c; }
 __device__ __forceinline__ uint32_t sl_maj3(uint32_t a, uint32_t b, uint32_t c) { return (a & b) | (c & (a | b)); }
 __device__ __forceinline__ uint32_t sl_mux(uint32_t s, uint32_t a, uint32_t b) { return (s & a) | (~s & b); }
+
+// N bits of one weight added: their sum's low bit, and the carries.
+template <int N>
+__device__ __forceinline__ uint32_t sl_reduce(const uint32_t *x, uint32_t *carry)
+{
+    uint32_t s = x[0];
+    int c = 0;
+#pragma unroll
+    for (int i = 1; i + 1 < N; i += 2) {
+        carry[c++] = sl_maj3(s, x[i], x[i + 1]);
+        s = sl_xor3(s, x[i], x[i + 1]);
+    }
+    if (N % 2 == 0) {
+        carry[c] = s & x[N - 1];
+        s ^= x[N - 1];
+    }
+    return s;
+}
+
+// 3D: next state from up to D neighbours' words; LIFE: B5/S45, else a sum
+// over the counts the rule maps to "alive".
+template <int D, bool LIFE>
+__device__ __forceinline__ uint32_t slice_rule3(const SliceArgs &a, const uint32_t *n, uint32_t alive)
+{
+    constexpr int N1 = D / 2, N2 = N1 / 2, N3 = N2 / 2;   // carries of each weight (sl_reduce of n leaves n / 2)
+    uint32_t c1[N1], c2[N2], c3[N3], c4[1];
+    const uint32_t t0 = sl_reduce<D>(n, c1), t1 = sl_reduce<N1>(c1, c2), t2 = sl_reduce<N2>(c2, c3), t3 = sl_reduce<N3>(c3, c4);
+    static_assert(N3 / 2 == 1, "five planes");
+    const uint32_t t4 = c4[0];
+    if (LIFE) return t2 & ~t1 & ~t3 & ~t4 & (t0 | alive);
+    uint32_t r = 0u;
+    for (uint32_t m = a.birth | a.survive; m; m &= m - 1u) {
+        const int v = __ffs((int)m) - 1;
+        const uint32_t eq = ((v & 1) ? t0 : ~t0) & ((v & 2) ? t1 : ~t1) & ((v & 4) ? t2 : ~t2) & ((v & 8) ? t3 : ~t3) &
+                            ((v & 16) ? t4 : ~t4);
+        r |= eq & (((a.survive >> v) & 1u ? alive : 0u) | ((a.birth >> v) & 1u ? ~alive : 0u));
+    }
+    return r;
+}
 
 // Next state of 32 cells from their neighbours' words n[0..D-1] (absent ones
 // zero): bit-sliced count, then the rule.
@@ -228,11 +270,12 @@ __device__ __forceinline__ void slice_bytes_to_string(const SliceArgs &a, const 
 // The same for blocks that walk the groups: every thread copies the 16-byte
 // units it will convert into its own slots of shared memory, two batches
 // ahead and across group boundaries, and waits for its own copies only.
+template <int BLK>
 struct SliceRing {
     uint8_t *slot;       // this thread's first slot of batch buffer 0
     int64_t g;           // the batch to be copied next: its group, first unit, the group's units
     int first, whole, buf;
-    static constexpr int kUnits = kSliceBatch * kSliceBlock;   // per batch
+    static constexpr int kUnits = kSliceBatch * BLK;   // per batch
     __device__ __forceinline__ int units(const SliceArgs &a, const uint8_t *in, int64_t gq) const
     {
         if (gq >= a.NG || ((uintptr_t)in & 15)) return 0;
@@ -246,9 +289,9 @@ struct SliceRing {
             const uint32_t dst = smem_addr(slot) + 16 * kUnits * b;
 #pragma unroll
             for (int k = 0; k < kSliceBatch; ++k)
-                if (kSliceBlock * k < n)
-                    asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(dst + 16 * kSliceBlock * k),
-                                 "l"(src + 16 * kSliceBlock * k)
+                if (BLK * k < n)
+                    asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(dst + 16 * BLK * k),
+                                 "l"(src + 16 * BLK * k)
                                  : "memory");
         }
         asm volatile("cp.async.commit_group;" ::: "memory");
@@ -279,12 +322,12 @@ struct SliceRing {
             const int left = n - f - (int)threadIdx.x;
 #pragma unroll
             for (int k = 0; k < kSliceBatch; ++k)
-                if (kSliceBlock * k < left)
-                    slice_put16(a, B, f + (int)threadIdx.x + kSliceBlock * k, slice_bits16(p[kSliceBlock * k]));
+                if (BLK * k < left)
+                    slice_put16(a, B, f + (int)threadIdx.x + BLK * k, slice_bits16(p[BLK * k]));
             issue(a, in, buf);
         }
         const int bytes = (int)min((int64_t)32, a.NT - 32 * gc) * a.KL;
-        slice_odd_units(a, in + 32 * gc * a.KL, bytes, n, B, threadIdx.x, kSliceBlock);
+        slice_odd_units(a, in + 32 * gc * a.KL, bytes, n, B, threadIdx.x, BLK);
     }
 };
 
@@ -304,15 +347,16 @@ __device__ __forceinline__ uint32_t slice_string_chunk(const SliceArgs &a, const
 // takes 32 cells of 32 tiles at a time through the transposition.  Bound by
 // issue slots and the latency of its loads (carpet r = 10, 1.07e9 cells:
 // 0.20 ms, 5.9 TB/s read and written).
-__global__ void __launch_bounds__(kSliceBlock, 5)
+template <int BLK>
+__global__ void __launch_bounds__(BLK, BLK == kSliceBlock ? 5 : 2)
 slice_pack_kernel(SliceArgs a, const uint8_t *__restrict__ in, uint32_t *__restrict__ bits)
 {
     extern __shared__ __align__(16) uint32_t smem[];
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = blockDim.x >> 5;
     const Transpose32 tr(lane);
-    SliceRing ring;
+    SliceRing<BLK> ring;
     ring.start(a, in, smem);
-    uint32_t *N = smem + 8 * kSliceBatch * kSliceBlock;   // the packed words
+    uint32_t *N = smem + 8 * kSliceBatch * BLK;   // the packed words
     uint32_t *B = N + a.KLp;
     for (int64_t g = blockIdx.x; g < a.NG; g += gridDim.x) {
         const int nt = (int)min((int64_t)32, a.NT - 32 * g);
@@ -335,7 +379,7 @@ slice_pack_kernel(SliceArgs a, const uint8_t *__restrict__ in, uint32_t *__restr
 // Tile 32 g + lane's neighbour for halo word j, and the export word it sends.
 __device__ __forceinline__ int32_t slice_nbr(const SliceArgs &a, int64_t g, uint32_t job, int lane)
 {
-    return __ldg(a.nbr + (g * 8 + (job >> 8)) * 32 + lane);
+    return __ldg(a.nbr + (g * a.ND + (job >> 8)) * 32 + lane);
 }
 __device__ __forceinline__ uint32_t slice_import(const SliceArgs &a, const uint32_t *ex, int32_t Q, uint32_t job)
 {
@@ -427,33 +471,67 @@ __device__ __forceinline__ void slice_string_to_bytes(const SliceArgs &a, const 
     }
 }
 
+// A cell's row of the neighbour table: byte offsets of its neighbours' words,
+// two per word; columns of 8, 8 and 4 (D = 20) or 8, 8, 8 and 2 (D = 26)
+// neighbours, each contiguous over the cells.
+template <int D>
+struct SliceRow {
+    uint32_t r[(D + 1) / 2];
+    __device__ __forceinline__ void load(const SliceArgs &a, int i)
+    {
+        const uint4 v = __ldg(a.tab + i);
+        r[0] = v.x;
+        r[1] = v.y;
+        if constexpr (D > 4) r[2] = v.z;
+        if constexpr (D > 6) r[3] = v.w;
+        if constexpr (D > 8) {
+            const uint4 u = __ldg(a.tab + a.KLp + i);
+            r[4] = u.x; r[5] = u.y; r[6] = u.z; r[7] = u.w;
+            if constexpr (D == 20) {
+                const uint2 x = __ldg(reinterpret_cast<const uint2 *>(a.tab + 2 * a.KLp) + i);
+                r[8] = x.x; r[9] = x.y;
+            } else {
+                const uint4 x = __ldg(a.tab + 2 * a.KLp + i);
+                r[8] = x.x; r[9] = x.y; r[10] = x.z; r[11] = x.w;
+                r[12] = __ldg(reinterpret_cast<const uint32_t *>(a.tab + 3 * a.KLp) + i);
+            }
+        }
+    }
+};
+
 // Next state of cells 32 c .. 32 c + 31 of a group's tiles from its words A.
 template <int D, bool LIFE>
-__device__ __forceinline__ uint32_t slice_next(const SliceArgs &a, const uint4 tab, const uint32_t *A, int c, int lane)
+__device__ __forceinline__ uint32_t slice_next(const SliceArgs &a, const SliceRow<D> &row, const uint32_t *A, int c, int lane)
 {
-    const uint32_t r[4] = {tab.x, tab.y, tab.z, tab.w};
-    uint32_t n[8];
+    uint32_t n[D < 8 ? 8 : D];
 #pragma unroll
     for (int k = 0; k < D; ++k)
         n[k] = *reinterpret_cast<const uint32_t *>(reinterpret_cast<const uint8_t *>(A) +
-                                                   ((k & 1) ? r[k / 2] >> 16 : r[k / 2] & 0xffffu));
-    return slice_rule<D, LIFE>(a, n, A[32 * c + lane]);
+                                                   ((k & 1) ? row.r[k / 2] >> 16 : row.r[k / 2] & 0xffffu));
+    if constexpr (D > 8) return slice_rule3<D, LIFE>(a, n, A[32 * c + lane]);
+    else return slice_rule<D, LIFE>(a, n, A[32 * c + lane]);
 }
+
+// In 3D a group's neighbour table (Menger: 8000 cells x 40 bytes) comes from
+// L2 chunk by chunk; latency and issue slots bound it.  Menger r = 7 (1.28e9
+// cells): one generation with packing 1.61 -> 0.72 ms, further ones 0.69 ->
+// 0.31 ms each; r = 6 (250 groups, one or two per SM) 39 -> 20.4 us.
 
 // `gens` generations of a packed state, blocks walking the groups; between
 // generations the launch's blocks meet at a grid barrier (a cooperative
 // launch when there is more than one block).  BYTES: one generation whose
 // results leave as bytes.
 template <int D, bool LIFE, bool BYTES>
-__global__ void __launch_bounds__(kSliceBlock, LIFE ? 5 : 4)
+__global__ void __launch_bounds__(D > 8 ? kSliceBlock3 : kSliceBlock, D > 8 ? 2 : (LIFE ? 5 : 4))
 slice_step_kernel(SliceArgs a, const uint32_t *src, uint32_t *dst, uint8_t *__restrict__ out, int gens)
 {
     extern __shared__ __align__(16) uint32_t smem[];
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, nw = blockDim.x >> 5;
     const Transpose32 tr(lane);
-    uint32_t *N = smem + 2 * a.AW;   // the new words; BYTES: the results' bit strings
+    constexpr bool kAhead = D <= 8;   // two arrays, the next group's words loaded ahead (3D: no room, two blocks per SM instead)
+    uint32_t *N = smem + (kAhead ? 2 : 1) * a.AW;   // the new words; BYTES: the results' bit strings
     uint32_t *R = N;
-    if (tid < 64) smem[(tid >> 5) * a.AW + a.A_zero + lane] = 0u;   // the words of absent neighbours
+    if (tid < (kAhead ? 64 : 32)) smem[(tid >> 5) * a.AW + a.A_zero + lane] = 0u;   // the words of absent neighbours
     uint32_t job[kSliceAhead];
 #pragma unroll
     for (int i = 0; i < kSliceAhead; ++i) job[i] = warp + i * nw < a.NJ ? __ldg(a.jobs + warp + i * nw) : 0u;
@@ -466,12 +544,13 @@ slice_step_kernel(SliceArgs a, const uint32_t *src, uint32_t *dst, uint8_t *__re
             for (int i = 0; i < kSliceAhead; ++i)
                 e[i] = warp + i * nw < a.NJ ? slice_import(a, src + a.ex, slice_nbr(a, blockIdx.x, job[i], lane), job[i]) : 0u;
         }
-        for (int64_t g = blockIdx.x; g < a.NG; g += gridDim.x, buf ^= 1) {
+        for (int64_t g = blockIdx.x; g < a.NG; g += gridDim.x, buf ^= kAhead ? 1u : 0u) {
             uint32_t *A = smem + buf * a.AW;
             const int64_t gn = g + gridDim.x;
 #pragma unroll
             for (int i = 0; i < kSliceAhead; ++i)
                 if (warp + i * nw < a.NJ) A[a.KLp + 32 * (warp + i * nw) + lane] = tr(e[i]);
+#pragma unroll 4
             for (int j = warp + kSliceAhead * nw; j < a.NJ; j += nw) {
                 const uint32_t jb = __ldg(a.jobs + j);
                 A[a.KLp + 32 * j + lane] = tr(slice_import(a, src + a.ex, slice_nbr(a, g, jb, lane), jb));
@@ -480,14 +559,16 @@ slice_step_kernel(SliceArgs a, const uint32_t *src, uint32_t *dst, uint8_t *__re
             __syncthreads();
             int32_t Q[kSliceAhead];
             if (gn < a.NG) {
-                slice_load(a, smem + (buf ^ 1) * a.AW, src + gn * a.KLp);
+                if (kAhead) slice_load(a, smem + (buf ^ 1) * a.AW, src + gn * a.KLp);
 #pragma unroll
                 for (int i = 0; i < kSliceAhead; ++i) Q[i] = warp + i * nw < a.NJ ? slice_nbr(a, gn, job[i], lane) : -1;
             }
             uint32_t *dg = BYTES ? nullptr : dst + g * a.KLp;
 #pragma unroll 2
             for (int c = warp; c < a.NC; c += nw) {
-                const uint32_t w = slice_next<D, LIFE>(a, __ldg(a.tab + 32 * c + lane), A, c, lane);
+                SliceRow<D> row;
+                row.load(a, 32 * c + lane);
+                const uint32_t w = slice_next<D, LIFE>(a, row, A, c, lane);
                 if (BYTES) {
                     R[lane * a.RP + c] = tr(w);
                 } else {
@@ -500,6 +581,7 @@ slice_step_kernel(SliceArgs a, const uint32_t *src, uint32_t *dst, uint8_t *__re
                 for (int i = 0; i < kSliceAhead; ++i) e[i] = slice_import(a, src + a.ex, Q[i], job[i]);
             }
             __syncthreads();
+            if (!kAhead && gn < a.NG) slice_load(a, smem, src + gn * a.KLp);   // (this group's words have been read)
             if (BYTES) {
                 slice_string_to_bytes(a, R, out + 32 * g * a.KL, (int)min((int64_t)32, a.NT - 32 * g), tid, blockDim.x);
             } else {
@@ -544,7 +626,7 @@ slice_single_kernel(SliceArgs a, const uint8_t *__restrict__ in, uint8_t *__rest
     extern __shared__ __align__(16) uint32_t smem[];
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, nw = blockDim.x >> 5;
     const Transpose32 tr(lane);
-    SliceRing ring;
+    SliceRing<kSliceBlock> ring;
     ring.start(a, in, smem);
     uint32_t *A = smem + 8 * kSliceBatch * kSliceBlock, *B = A + a.AW;
     if (tid < 32) A[a.A_zero + tid] = 0u;   // the words of absent neighbours
@@ -575,8 +657,11 @@ slice_single_kernel(SliceArgs a, const uint8_t *__restrict__ in, uint8_t *__rest
         for (int c = warp; c < a.NC; c += nw) A[32 * c + lane] = slice_string_chunk(a, tr, B, c, nt, lane);
         __syncthreads();
 #pragma unroll 2
-        for (int c = warp; c < a.NC; c += nw)
-            B[lane * a.RP + c] = tr(slice_next<D, LIFE>(a, __ldg(a.tab + 32 * c + lane), A, c, lane));
+        for (int c = warp; c < a.NC; c += nw) {
+            SliceRow<D> row;
+            row.load(a, 32 * c + lane);
+            B[lane * a.RP + c] = tr(slice_next<D, LIFE>(a, row, A, c, lane));
+        }
         __syncthreads();
         slice_string_to_bytes(a, B, out + 32 * g * a.KL, nt, tid, blockDim.x);
         __syncthreads();
@@ -744,7 +829,13 @@ slice_resident_kernel(SliceArgs a, const uint8_t *__restrict__ in, uint8_t *__re
 #pragma unroll
             for (int i = 0; i < ROUNDS; ++i)
                 if (i < now) {
-                    w[i] = slice_next<D, LIFE>(a, tab[32 * k.j + lane], A0 + k.q * a.AW, k.j, lane);
+                    const uint4 v = tab[32 * k.j + lane];
+                    SliceRow<D> row;
+                    row.r[0] = v.x;
+                    row.r[1] = v.y;
+                    if constexpr (D > 4) row.r[2] = v.z;
+                    if constexpr (D > 6) row.r[3] = v.w;
+                    w[i] = slice_next<D, LIFE>(a, row, A0 + k.q * a.AW, k.j, lane);
                     k.next();
                 }
         }
@@ -786,6 +877,7 @@ slice_resident_kernel(SliceArgs a, const uint8_t *__restrict__ in, uint8_t *__re
 
 // Neighbours of every tile, a row of 32 lanes per group and direction
 // (tiles past the last have none), from rows of 8 per tile.
+template <int DIM>
 __global__ void slice_nbr_kernel(FracDev F, int64_t NT, int64_t NG, int coarse_levels, int32_t coarse_side,
                                  const SliceGroup *__restrict__ groups, int32_t *__restrict__ out)
 {
@@ -802,12 +894,14 @@ __global__ void slice_nbr_kernel(FracDev F, int64_t NT, int64_t NG, int coarse_l
         }
         int32_t c[3] = {0, 0, 0};
         if (live) lambda64(F, (uint64_t)T, coarse_levels, c);
-        for (int d = 0; d < 8; ++d) {
-            const int q = d < 4 ? d : d + 1;
-            const int32_t x = c[0] + q % 3 - 1, y = c[1] + q / 3 - 1;
+        constexpr int ND = DIM == 3 ? 26 : 8;
+        for (int d = 0; d < ND; ++d) {
+            const int q = d < ND / 2 ? d : d + 1;
+            const int32_t x = c[0] + q % 3 - 1, y = c[1] + (q / 3) % 3 - 1, z = DIM == 3 ? c[2] + q / 9 - 1 : 0;
             int64_t v = -1;
-            if (live && x >= 0 && x < coarse_side && y >= 0 && y < coarse_side) v = nu_levels(F, x, y, 0, coarse_levels);
-            out[((i >> 5) * 8 + d) * 32 + (i & 31)] = v < 0 ? -1 : (int32_t)(base + v);
+            if (live && x >= 0 && x < coarse_side && y >= 0 && y < coarse_side && z >= 0 && z < coarse_side)
+                v = nu_levels(F, x, y, z, coarse_levels);
+            out[((i >> 5) * ND + d) * 32 + (i & 31)] = v < 0 ? -1 : (int32_t)(base + v);
         }
     }
 }
@@ -821,44 +915,51 @@ static int64_t pw(int64_t b, int e)
     return v;
 }
 
-// Neighbours of the cells of an m-level box: entry [l][d9] (d9 = (dx + 1) +
-// 3 (dy + 1)) is the neighbour's number in the box that holds it | that box's
-// direction << 24 (4: the same box), or -1 where the fractal has none.
+// Neighbours of the cells of an m-level box: entry [l][q] (q = (dx + 1) + 3
+// (dy + 1) + 9 (dz + 1), Q = 9 or 27 of them) is the neighbour's number in the
+// box that holds it | that box's direction << 24 (Q / 2: the same box), or -1
+// where the fractal has none.
 using SliceNbrs = std::vector<int32_t>;
 
 // One level more: level 0 digits move as `first` says, and where they leave
 // their block the rest moves as it does with m - 1 levels.
-static SliceNbrs slice_deepen(const SliceNbrs &first, const SliceNbrs &rest, int k)
+static SliceNbrs slice_deepen(const SliceNbrs &first, const SliceNbrs &rest, int k, int Q)
 {
-    const size_t n = rest.size() / 9;
-    SliceNbrs out(n * k * 9);
+    const size_t n = rest.size() / Q;
+    SliceNbrs out(n * k * Q);
     for (size_t r = 0; r < n; ++r)
         for (int j = 0; j < k; ++j)
-            for (int d = 0; d < 9; ++d) {
-                const int32_t a = first[(size_t)j * 9 + d];
+            for (int d = 0; d < Q; ++d) {
+                const int32_t a = first[(size_t)j * Q + d];
                 int32_t v = -1;
                 if (a >= 0) {
-                    const int32_t b = (a >> 24) == 4 ? (int32_t)r | 4 << 24 : rest[r * 9 + (a >> 24)];
+                    const int32_t b = (a >> 24) == Q / 2 ? (int32_t)r | (Q / 2) << 24 : rest[r * Q + (a >> 24)];
                     if (b >= 0) v = ((b & 0xffffff) * k + (a & 0xffffff)) | (b & ~0xffffff);
                 }
-                out[(r * k + j) * 9 + d] = v;
+                out[(r * k + j) * Q + d] = v;
             }
     return out;
 }
 
-// The neighbours in a single block of s x s digits.
+// The neighbours in a single block of s^dim digits.
 static SliceNbrs slice_first(const fractal *f)
 {
-    SliceNbrs out((size_t)f->k * 9, -1);
+    const int Q = f->dim == 3 ? 27 : 9;
+    SliceNbrs out((size_t)f->k * Q, -1);
     for (int j = 0; j < f->k; ++j)
-        for (int d = 0; d < 9; ++d) {
-            int q[2] = {f->offsets[(size_t)2 * j] + d % 3 - 1, f->offsets[(size_t)2 * j + 1] + d / 3 - 1}, b[2];
-            for (int i = 0; i < 2; ++i) {
-                b[i] = q[i] < 0 ? -1 : (q[i] >= f->s ? 1 : 0);
-                q[i] -= b[i] * f->s;
+        for (int d = 0; d < Q; ++d) {
+            const int m[3] = {d % 3 - 1, (d / 3) % 3 - 1, d / 9 - 1};
+            int t = 0, w = 1, box = 0, b3 = 1;
+            for (int i = 0; i < f->dim; ++i) {
+                int q = f->offsets[(size_t)f->dim * j + i] + m[i];
+                const int b = q < 0 ? -1 : (q >= f->s ? 1 : 0);
+                t += (q - b * f->s) * w;
+                w *= f->s;
+                box += (b + 1) * b3;
+                b3 *= 3;
             }
-            const int h = f->dev.hinv[q[0] + f->s * q[1]];
-            if (h >= 0) out[(size_t)j * 9 + d] = h | ((b[0] + 1) + 3 * (b[1] + 1)) << 24;
+            const int h = f->dev.hinv[t];
+            if (h >= 0) out[(size_t)j * Q + d] = h | box << 24;
         }
     return out;
 }
@@ -867,39 +968,43 @@ struct SliceTables {
     int KL = 0, H = 0, D = 0;
     int zero = 0;                   // the first of 32 zero words in a group's array
     SliceNbrs nb;
-    std::vector<int32_t> hidx;      // [9][KL]: word of a halo cell (by its box's direction), -1 = none
+    int Q = 9;                      // directions and the centre
+    std::vector<int32_t> hidx;      // [Q][KL]: word of a halo cell (by its box's direction), -1 = none
     std::vector<uint32_t> jobs;     // halo words: export word | direction slot << 8
     std::vector<uint16_t> xlist;    // [XW][32] cells of the export words
     std::vector<uint32_t> cells;    // halo cells: cell of the neighbouring tile, word index | direction slot << 16
     int XW() const { return (int)xlist.size() / 32; }
 };
 
-static SliceTables slice_tables(SliceNbrs &&nbrs)
+static SliceTables slice_tables(SliceNbrs &&nbrs, int Q)
 {
     SliceTables t;
+    t.Q = Q;
     t.nb = std::move(nbrs);
-    t.KL = (int)(t.nb.size() / 9);
+    t.KL = (int)(t.nb.size() / Q);
     const int KL = t.KL, KLp = (KL + 31) / 32 * 32;
-    t.hidx.assign((size_t)9 * KL, -1);
+    t.hidx.assign((size_t)Q * KL, -1);
     for (int l = 0; l < KL; ++l) {
         int n = 0;
-        for (int d = 0; d < 9; ++d) {
-            const int32_t v = d == 4 ? -1 : t.nb[(size_t)l * 9 + d];
+        for (int d = 0; d < Q; ++d) {
+            const int32_t v = d == Q / 2 ? -1 : t.nb[(size_t)l * Q + d];
             if (v < 0) continue;
             ++n;
-            if ((v >> 24) != 4) t.hidx[(size_t)(v >> 24) * KL + (v & 0xffffff)] = 0;
+            if ((v >> 24) != Q / 2) t.hidx[(size_t)(v >> 24) * KL + (v & 0xffffff)] = 0;
         }
         t.D = std::max(t.D, n);
     }
     // export words: the directions with the most border cells first, their
     // cells in runs of 32; a run whose cells all lie in an earlier word uses
     // that one (a corner cell is in its sides' words)
-    std::vector<int> cells[9];
-    int order[8] = {0, 1, 2, 3, 5, 6, 7, 8};
+    std::vector<int> cells[27];
+    std::vector<int> order;
+    for (int d = 0; d < Q; ++d)
+        if (d != Q / 2) order.push_back(d);
     for (int d : order)
         for (int l = 0; l < KL; ++l)
             if (t.hidx[(size_t)d * KL + l] >= 0) cells[d].push_back(l);
-    std::stable_sort(order, order + 8, [&](int x, int y) { return cells[x].size() > cells[y].size(); });
+    std::stable_sort(order.begin(), order.end(), [&](int x, int y) { return cells[x].size() > cells[y].size(); });
     std::vector<std::vector<int>> words;
     for (int d : order)
         for (size_t i = 0; i < cells[d].size(); i += 32) {
@@ -911,7 +1016,7 @@ static SliceTables slice_tables(SliceNbrs &&nbrs)
                 w = (int)words.size();
                 words.push_back(run);
             }
-            const uint32_t slot = (uint32_t)(d < 4 ? d : d - 1);
+            const uint32_t slot = (uint32_t)(d < Q / 2 ? d : d - 1);
             for (int l : run) {
                 const int at = KLp + 32 * (int)t.jobs.size() +
                                (int)(std::lower_bound(words[w].begin(), words[w].end(), l) - words[w].begin());
@@ -928,7 +1033,7 @@ static SliceTables slice_tables(SliceNbrs &&nbrs)
     return t;
 }
 
-// The neighbour table [KLp][8] (byte offsets): the 32 cells of a chunk are
+// The neighbour table (byte offsets): the 32 cells of a chunk are
 // added by 32 lanes, one neighbour per lane and load, and the order of a
 // cell's neighbours is free; each goes to the load that has the fewest words
 // in its bank so far (triangle: 9.4 -> 6.0 shared-memory wavefronts per chunk,
@@ -936,37 +1041,43 @@ static SliceTables slice_tables(SliceNbrs &&nbrs)
 // from the emptiest bank.
 static void slice_neighbour_table(const SliceTables &t, int D, uint16_t *tab)
 {
-    const int KLp = (t.KL + 31) / 32 * 32, all = (1 << D) - 1;
-    std::vector<uint8_t> loaded((size_t)t.zero + 32, 0);   // per word: the loads of this chunk that read it
+    const int KLp = (t.KL + 31) / 32 * 32;
+    const uint32_t all = (1u << D) - 1u;
+    // entry k of cell i: column k / 8 (columns of 8, the last of 4 or 2; see SliceRow)
+    auto at = [&](int i, int k) -> uint16_t & {
+        const int col = k / 8, width = col == (D - 1) / 8 && D > 8 ? (D == 20 ? 4 : 2) : 8;
+        return tab[(size_t)col * 8 * KLp + (size_t)i * width + k % 8];
+    };
+    std::vector<uint32_t> loaded((size_t)t.zero + 32, 0);   // per word: the loads of this chunk that read it
     for (int c = 0; c < KLp; c += 32) {
         // [bank][x]: the loads that read x words of the bank, as a bit set
-        uint8_t with[32][33] = {};
-        int v[32][8], put[32][8], n[32];
-        for (int b = 0; b < 32; ++b) with[b][0] = (uint8_t)all;
+        uint32_t with[32][33] = {};
+        int v[32][26], put[32][26], n[32];
+        for (int b = 0; b < 32; ++b) with[b][0] = all;
         for (int i = 0; i < 32; ++i) {
             n[i] = 0;
-            for (int d = 0; d < 9 && c + i < t.KL; ++d) {
-                const int32_t a = d == 4 ? -1 : t.nb[(size_t)(c + i) * 9 + d];
+            for (int d = 0; d < t.Q && c + i < t.KL; ++d) {
+                const int32_t a = d == t.Q / 2 ? -1 : t.nb[(size_t)(c + i) * t.Q + d];
                 if (a < 0) continue;
-                v[i][n[i]++] = (a >> 24) == 4 ? a & 0xffffff : t.hidx[(size_t)(a >> 24) * t.KL + (a & 0xffffff)];
+                v[i][n[i]++] = (a >> 24) == t.Q / 2 ? a & 0xffffff : t.hidx[(size_t)(a >> 24) * t.KL + (a & 0xffffff)];
             }
         }
         for (int want = D; want >= 1; --want)   // cells with the most neighbours first
             for (int i = 0; i < 32; ++i) {
                 if (n[i] != want) continue;
-                int open = all;
+                uint32_t open = all;
                 for (int e = 0; e < n[i]; ++e) {
                     const int w = v[i][e], b = w & 31;
-                    int pick = open & loaded[w];
+                    uint32_t pick = open & loaded[w];
                     if (!pick) {
                         int x = 0;
                         while (!(pick = open & with[b][x])) ++x;
-                        pick &= -pick;
-                        with[b][x] &= (uint8_t)~pick;
-                        with[b][x + 1] |= (uint8_t)pick;
-                        loaded[w] |= (uint8_t)pick;
+                        pick &= 0u - pick;
+                        with[b][x] &= ~pick;
+                        with[b][x + 1] |= pick;
+                        loaded[w] |= pick;
                     }
-                    pick &= -pick;
+                    pick &= 0u - pick;
                     open &= ~pick;
                     int k = 0;
                     while (!((pick >> k) & 1)) ++k;
@@ -985,12 +1096,12 @@ static void slice_neighbour_table(const SliceTables &t, int D, uint16_t *tab)
                     z = b;
                 }
             }
-            for (int i = 0; i < 32; ++i) tab[(size_t)(c + i) * 8 + k] = (uint16_t)(4 * (t.zero + z));
+            for (int i = 0; i < 32; ++i) at(c + i, k) = (uint16_t)(4 * (t.zero + z));
         }
         for (int k = D; k < 8; ++k)
-            for (int i = 0; i < 32; ++i) tab[(size_t)(c + i) * 8 + k] = (uint16_t)(4 * t.zero);
+            for (int i = 0; i < 32; ++i) at(c + i, k) = (uint16_t)(4 * t.zero);
         for (int i = 0; i < 32; ++i)
-            for (int e = 0; e < n[i]; ++e) tab[(size_t)(c + i) * 8 + put[i][e]] = (uint16_t)(4 * v[i][e]);
+            for (int e = 0; e < n[i]; ++e) at(c + i, put[i][e]) = (uint16_t)(4 * v[i][e]);
     }
 }
 
@@ -1017,7 +1128,9 @@ static StepFn step_fn(int D, bool life, bool bytes)
         case 4: return step_fn_d<4>(life, bytes);
         case 6: return step_fn_d<6>(life, bytes);
         case 7: return step_fn_d<7>(life, bytes);
-        default: return step_fn_d<8>(life, bytes);
+        case 8: return step_fn_d<8>(life, bytes);
+        case 20: return step_fn_d<20>(life, bytes);
+        default: return step_fn_d<26>(life, bytes);
     }
 }
 
@@ -1057,7 +1170,14 @@ static ResidentFn resident_fn(const SlicePlan &s, bool life)
     }
 }
 
-static bool slice_fractal_ok(const fractal *f) { return f->dim == 2 && !f->mixed && f->k >= 2 && f->r >= 1; }
+static bool slice_fractal_ok(const fractal *f) { return !f->mixed && f->k >= 2 && f->r >= 1; }
+
+// Whether the rule is the one the kernels have a closed form for: B3/S23, in 3D B5/S45.
+static bool slice_life(const fractal *f, uint32_t birth, uint32_t survive)
+{
+    if (f->dim == 3) return (birth & 0x7ffffffu) == 0x20u && (survive & 0x7ffffffu) == 0x30u;
+    return (birth & 0x1ffu) == 0x8u && (survive & 0x1ffu) == 0xcu;
+}
 
 // The resident kernels of the plan may use its shared memory, a block per SM.
 static cudaError_t resident_ready(const SlicePlan &s)
@@ -1099,7 +1219,8 @@ static SliceGeo slice_geo(const fractal *f, int L, const SliceTables &t)
     p.NJ = (int)t.jobs.size();
     p.XW = t.XW();
     p.H = t.H;
-    p.D = t.D <= 4 ? 4 : (t.D <= 6 ? 6 : t.D);
+    p.ND = t.Q - 1;
+    p.D = t.Q == 27 ? (t.D <= 20 ? 20 : 26) : (t.D <= 4 ? 4 : (t.D <= 6 ? 6 : t.D));
     p.NT = pw(f->k, f->r - L);
     p.NG = (p.NT + 31) / 32;
     p.AW = p.KLp + std::max(32 * p.NJ, 64) + 32;   // at least a group's bit strings
@@ -1110,13 +1231,14 @@ static SliceGeo slice_geo(const fractal *f, int L, const SliceTables &t)
 }
 static int string_words(const SliceGeo &p) { return p.BP ? 32 * p.BP : p.KLp + 1; }
 
-constexpr int kSliceMaxKL = 4096;
-constexpr int kSliceWave = 760;
+constexpr int kSliceMaxKL = 4096, kSliceMaxKL3 = 8192;
+constexpr int kSliceWave = 760, kSliceWave3 = 304;
 
 // Blocks, groups per block and threads of the resident kernel, and its
 // estimated cycles per generation; false when the state does not fit.
 static bool slice_resident_shape(const SliceGeo &p, int num_sms, bool batch, SlicePlan *s, double *cost)
 {
+    if (p.D > 8) return false;   // 3D: the neighbour table alone is larger than shared memory
     // one block where that takes no more than 8 chunks per warp, else as many as there are SMs
     for (int64_t grid : {(int64_t)1, std::min<int64_t>(num_sms, p.NG)}) {
         if (grid == 1 && batch && p.NG > 1) continue;   // (batches: no kernel for a single block's exports)
@@ -1156,17 +1278,20 @@ static int slice_levels(const fractal *f, SlicePlan *plan, SliceTables *tables)
     double cost = 0;
     const SliceNbrs first = slice_first(f);
     SliceNbrs nbrs = first;
-    for (int L = 1; L <= f->r && pw(f->k, L) <= kSliceMaxKL; ++L) {
-        if (L > 1) nbrs = slice_deepen(first, nbrs, f->k);
+    const bool d3 = f->dim == 3;
+    const int Q = d3 ? 27 : 9;
+    for (int L = 1; L <= f->r && pw(f->k, L) <= (d3 ? kSliceMaxKL3 : kSliceMaxKL); ++L) {
+        if (L > 1) nbrs = slice_deepen(first, nbrs, f->k, Q);
         if ((double)pw(f->k, f->r - L) >= 2147483648.0) continue;
-        SliceTables t = slice_tables(SliceNbrs(nbrs));
+        SliceTables t = slice_tables(SliceNbrs(nbrs), Q);
         const SliceGeo p = slice_geo(f, L, t);
         if (p.AW * 4 > 65535 || p.XW > 255) continue;
         SlicePlan s;
         double c;
         if (!slice_resident_shape(p, f->num_sms, false, &s, &c)) {
-            const int64_t waves = (p.NG + kSliceWave - 1) / kSliceWave;
-            c = (double)waves * (p.NC * 45 + 30.0 * (p.NJ + p.XW) + 400);
+            const int wave = d3 ? kSliceWave3 : kSliceWave;
+            const int64_t waves = (p.NG + wave - 1) / wave;
+            c = (double)waves * (p.NC * (d3 ? 110 : 45) + 30.0 * (p.NJ + p.XW) + 400);
         }
         if (best && plan->resident && !s.resident) continue;
         if (!best || (s.resident && !plan->resident) || c < cost) {
@@ -1191,9 +1316,9 @@ static cudaError_t slice_upload(SliceGeo &p, const SliceTables &t, SlicePlan &s,
         off += (bytes + 255) / 256 * 256;
         return at;
     };
-    const size_t o_tab = take((size_t)p.KLp * 16), o_jobs = take(t.jobs.size() * 4), o_xl = take(t.xlist.size() * 2),
+    const size_t o_tab = take((size_t)p.KLp * (p.D <= 8 ? 16 : (p.D == 20 ? 40 : 52))), o_jobs = take(t.jobs.size() * 4), o_xl = take(t.xlist.size() * 2),
                  o_cells = take(t.cells.size() * 4), o_bar = take(8), o_groups = take(groups.size() * sizeof(SliceGroup)), host = off;
-    const size_t o_nbr = take((size_t)p.NG * 256 * sizeof(int32_t)),
+    const size_t o_nbr = take((size_t)p.NG * p.ND * 32 * sizeof(int32_t)),
                  exb = s.resident ? (size_t)p.NG * p.XW * 128 : 0, o_ex0 = take(exb), o_ex1 = take(exb);
     std::vector<uint8_t> img(host, 0);
     slice_neighbour_table(t, p.D, reinterpret_cast<uint16_t *>(img.data() + o_tab));
@@ -1221,15 +1346,19 @@ static int build_slice_plan(fractal *f, cudaStream_t st)
     SlicePlan s;
     if (slice_levels(f, &s, &t) < 1) return FR_EINVAL;
     SliceGeo &p = s.geo;
-    const int ring = 32 * kSliceBatch * kSliceBlock;
+    s.block = f->dim == 3 ? kSliceBlock3 : kSliceBlock;
+    const int ring = 32 * kSliceBatch * s.block, arrays = f->dim == 3 ? 1 : 2;
     s.smem_pack = ring + 4 * (string_words(p) + p.KLp);
     s.smem_single = ring + 4 * (p.AW + std::max(string_words(p), 32 * p.RP + 1));
-    s.smem_step = 4 * (2 * p.AW + p.KLp);
-    s.smem_bytes = 4 * (2 * p.AW + 32 * p.RP + 1);
+    s.smem_step = 4 * (arrays * p.AW + p.KLp);
+    s.smem_bytes = 4 * (arrays * p.AW + 32 * p.RP + 1);
     cudaError_t e = slice_upload(p, t, s, {}, st);
     if (e == cudaSuccess) {
         const int64_t blocks = std::min<int64_t>((32 * p.NG + 255) / 256, (int64_t)f->num_sms * 16);
-        slice_nbr_kernel<<<(unsigned)blocks, 256, 0, st>>>(f->dev, p.NT, p.NG, f->r - p.L, (int32_t)pw(f->s, f->r - p.L), nullptr, p.nbr);
+        if (f->dim == 3)
+            slice_nbr_kernel<3><<<(unsigned)blocks, 256, 0, st>>>(f->dev, p.NT, p.NG, f->r - p.L, (int32_t)pw(f->s, f->r - p.L), nullptr, p.nbr);
+        else
+            slice_nbr_kernel<2><<<(unsigned)blocks, 256, 0, st>>>(f->dev, p.NT, p.NG, f->r - p.L, (int32_t)pw(f->s, f->r - p.L), nullptr, p.nbr);
         e = cudaGetLastError();
         if (e == cudaSuccess) e = cudaStreamSynchronize(st);   // the tables serve calls on any stream from here on
     }
@@ -1237,11 +1366,12 @@ static int build_slice_plan(fractal *f, cudaStream_t st)
     int per_sm = 0;
     if (s.resident && e == cudaSuccess) e = resident_ready(s);
     {
-        const int most = 100 * 1024;
+        const int most = 112 * 1024;
+        auto pack = f->dim == 3 ? slice_pack_kernel<kSliceBlock3> : slice_pack_kernel<kSliceBlock>;
         if (std::max(std::max(s.smem_pack, s.smem_single), std::max(s.smem_step, s.smem_bytes)) > most) e = cudaErrorInvalidConfiguration;
-        if (e == cudaSuccess) e = cudaFuncSetAttribute(slice_pack_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, most);
-        if (e == cudaSuccess) e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, slice_pack_kernel, kSliceBlock, s.smem_pack);
-        for (int life = 0; life < 2 && p.H <= kSliceSingleHalo && e == cudaSuccess; ++life) {
+        if (e == cudaSuccess) e = cudaFuncSetAttribute(pack, cudaFuncAttributeMaxDynamicSharedMemorySize, most);
+        if (e == cudaSuccess) e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, pack, s.block, s.smem_pack);
+        for (int life = 0; life < 2 && p.D <= 8 && p.H <= kSliceSingleHalo && e == cudaSuccess; ++life) {
             int n = 0;
             e = cudaFuncSetAttribute(single_fn(p.D, life), cudaFuncAttributeMaxDynamicSharedMemorySize, most);
             if (e == cudaSuccess)
@@ -1254,7 +1384,7 @@ static int build_slice_plan(fractal *f, cudaStream_t st)
                 StepFn fn = step_fn(p.D, life, bytes);
                 e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, most);
                 if (e == cudaSuccess)
-                    e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, fn, kSliceBlock, bytes ? s.smem_bytes : s.smem_step);
+                    e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, fn, s.block, bytes ? s.smem_bytes : s.smem_step);
                 if (e == cudaSuccess && per_sm < 1) e = cudaErrorInvalidConfiguration;
                 (bytes ? s.grid_bytes : s.grid_step)[life] = (int)std::min<int64_t>((int64_t)per_sm * f->num_sms, p.NG);
             }
@@ -1291,6 +1421,7 @@ static bool slice_one_generation_by_tiles(const fractal *f, int halo_cells)
 {
     const int preset = rows_preset_of(f);
     if (preset == 1 || f->cells < (1 << 17)) return true;
+    if (f->dim == 3) return f->cells < (1 << 22);
     if (halo_cells < 0) return false;
     if (halo_cells <= kSliceSingleHalo) return false;
     return f->cells < (preset == 0 ? 4 << 20 : 1 << 20);
@@ -1318,6 +1449,9 @@ static SliceArgs slice_args(const SliceGeo &p, uint32_t birth, uint32_t survive,
     a.AW = p.AW;
     a.A_zero = p.AW - 32;
     a.XW = p.XW;
+    a.ND = p.ND;
+    a.birth = birth & 0x7ffffffu;
+    a.survive = survive & 0x7ffffffu;
     a.ex = p.NG * p.KLp;
     a.kdiv = make_div((uint32_t)p.KL);
     a.cdiv = make_div((uint32_t)std::max(2, p.NC));
@@ -1377,7 +1511,7 @@ int try_slice_step(fractal *f, const uint8_t *in, uint8_t *out, int64_t steps, u
     }
     const SliceGeo &p = s.geo;
     const SliceArgs a = slice_args(p, birth, survive, s.bar, f->status);
-    const bool life = (birth & 0x1ffu) == 0x8u && (survive & 0x1ffu) == 0xcu;
+    const bool life = slice_life(f, birth, survive);
     if (res) {
         const int rc = launch_resident(s, a, life, in, out, steps, st);
         if (rc) return rc;
@@ -1390,7 +1524,8 @@ int try_slice_step(fractal *f, const uint8_t *in, uint8_t *out, int64_t steps, u
         *done = true;
         return FR_OK;
     }
-    slice_pack_kernel<<<s.grid_pack, kSliceBlock, s.smem_pack, st>>>(a, in, s.bits[0]);
+    if (f->dim == 3) slice_pack_kernel<kSliceBlock3><<<s.grid_pack, kSliceBlock3, s.smem_pack, st>>>(a, in, s.bits[0]);
+    else slice_pack_kernel<kSliceBlock><<<s.grid_pack, kSliceBlock, s.smem_pack, st>>>(a, in, s.bits[0]);
     FR_CUDA(cudaGetLastError());
     *done = true;
     int64_t left = steps - 1;   // generations before the one that writes bytes
@@ -1403,9 +1538,9 @@ int try_slice_step(fractal *f, const uint8_t *in, uint8_t *out, int64_t steps, u
         uint8_t *none = nullptr;
         void *args[] = {(void *)&a, &src, &dst, &none, &gens};
         if (s.grid_step[life] > 1 && gens > 1)
-            FR_CUDA(cudaLaunchCooperativeKernel((const void *)fn, dim3(s.grid_step[life]), dim3(kSliceBlock), args, s.smem_step, st));
+            FR_CUDA(cudaLaunchCooperativeKernel((const void *)fn, dim3(s.grid_step[life]), dim3(s.block), args, s.smem_step, st));
         else
-            FR_CUDA(cudaLaunchKernel((const void *)fn, dim3(s.grid_step[life]), dim3(kSliceBlock), args, s.smem_step, st));
+            FR_CUDA(cudaLaunchKernel((const void *)fn, dim3(s.grid_step[life]), dim3(s.block), args, s.smem_step, st));
         left -= gens;
         if (gens & 1) cur ^= 1;
     }
@@ -1415,7 +1550,7 @@ int try_slice_step(fractal *f, const uint8_t *in, uint8_t *out, int64_t steps, u
         uint32_t *none = nullptr;
         int one = 1;
         void *args[] = {(void *)&a, &src, &none, &out, &one};
-        FR_CUDA(cudaLaunchKernel((const void *)fb, dim3(s.grid_bytes[life]), dim3(kSliceBlock), args, s.smem_bytes, st));
+        FR_CUDA(cudaLaunchKernel((const void *)fb, dim3(s.grid_bytes[life]), dim3(s.block), args, s.smem_bytes, st));
     }
     return FR_OK;
 }
@@ -1459,7 +1594,7 @@ int run_slice_batch(const SliceBatch *b, cudaStream_t st)
 
 bool slice_batch_takes(const fractal *f, int64_t steps)
 {
-    return slice_fractal_ok(f) && steps >= 2 && steps < (1 << 30) && f->cells <= kSliceBatchCells &&
+    return f->dim == 2 && slice_fractal_ok(f) && steps >= 2 && steps < (1 << 30) && f->cells <= kSliceBatchCells &&
            ((f->tile_levels_user < 0 && f->stages_user < 0) || f->sliced_tuned);
 }
 
@@ -1492,8 +1627,8 @@ int build_slice_batch(const std::vector<SliceBatchItem> &items, uint32_t birth, 
     const SliceNbrs first = slice_first(rep);
     SliceNbrs nbrs = first;
     for (int L = 1; L <= rmax && pw(rep->k, L) <= kSliceMaxKL; ++L) {
-        if (L > 1) nbrs = slice_deepen(first, nbrs, rep->k);
-        tabs.push_back(slice_tables(SliceNbrs(nbrs)));
+        if (L > 1) nbrs = slice_deepen(first, nbrs, rep->k, 9);
+        tabs.push_back(slice_tables(SliceNbrs(nbrs), 9));
         geos.push_back(slice_geo(rep, L, tabs.back()));
     }
     const int lmax = (int)tabs.size() - 1;
@@ -1540,7 +1675,7 @@ int build_slice_batch(const std::vector<SliceBatchItem> &items, uint32_t birth, 
     if (best[rmax + 1].L == 0) return FR_EINVAL;
     SliceBatch *batch = new (std::nothrow) SliceBatch();
     if (!batch) return FR_ENOMEM;
-    const bool life = (birth & 0x1ffu) == 0x8u && (survive & 0x1ffu) == 0xcu;
+    const bool life = slice_life(rep, birth, survive);
     for (int b = rmax + 1; b > 1 && best[b].L > 0; b = best[b].L) {
         const int L = best[b].L;
         std::vector<const SliceBatchItem *> in;
@@ -1572,7 +1707,7 @@ int build_slice_batch(const std::vector<SliceBatchItem> &items, uint32_t birth, 
             if (e == cudaSuccess) e = slice_upload(p, tabs[L], l.plan, groups, st);
             if (e == cudaSuccess) {
                 const int64_t blocks = std::min<int64_t>((32 * p.NG + 255) / 256, (int64_t)rep->num_sms * 16);
-                slice_nbr_kernel<<<(unsigned)blocks, 256, 0, st>>>(rep->dev, p.NT, p.NG, 0, 1,
+                slice_nbr_kernel<2><<<(unsigned)blocks, 256, 0, st>>>(rep->dev, p.NT, p.NG, 0, 1,
                                                                    reinterpret_cast<const SliceGroup *>(l.plan.groups), p.nbr);
                 e = cudaGetLastError();
                 if (e == cudaSuccess) e = cudaStreamSynchronize(st);

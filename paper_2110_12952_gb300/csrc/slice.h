@@ -1,4 +1,4 @@
-// slice.h -- the bit-sliced step of 2D fractals (slice.cu): plan and entry
+// slice.h -- the bit-sliced step (slice.cu): plan and entry
 // points (internal; not part of the ABI).
 #pragma once
 
@@ -23,14 +23,15 @@ struct SliceGeo {
     int NC = 0;               // 32-cell chunks per tile
     int64_t NT = 0, NG = 0;   // tiles, groups of 32
     int H = 0;                // halo cells per tile
-    int D = 0;                // neighbours per cell the kernel adds (the largest degree, as 4, 6, 7 or 8)
+    int D = 0;                // neighbours per cell the kernel adds (the largest degree, as 4, 6, 7, 8, 20 or 26)
+    int ND = 8;               // directions
     int NJ = 0, XW = 0;       // halo words a tile takes, export words it gives (at most 32 cells each)
     int BP = 0, RP = 0, AW = 0;   // shared-memory geometry (SliceArgs)
     uint4 *tab = nullptr;        // per cell: byte offsets (8 x uint16) of its neighbours' words in a group's word array
     uint32_t *jobs = nullptr;    // [NJ]: export word | direction << 8
     uint16_t *xlist = nullptr;   // [XW][32]: cells of the export words
     uint2 *cells = nullptr;      // [H]: cell of the neighbouring tile, its word in a group's array | direction << 16
-    int32_t *nbr = nullptr;      // [NG][8][32]: neighbouring tile of each tile of a group by direction, -1 = none
+    int32_t *nbr = nullptr;      // [NG][ND][32]: neighbouring tile of each tile of a group by direction, -1 = none
 };
 
 struct SlicePlan {
@@ -38,6 +39,7 @@ struct SlicePlan {
     SliceGeo geo;
     bool resident = false;    // the packed state stays in shared memory: one launch for all generations
     int per_block = 0, rounds = 0, block_resident = 0, grid_resident = 0, smem_resident = 0;
+    int block = 256;          // streaming kernels: threads per block
     int smem_pack = 0, smem_step = 0, smem_bytes = 0, smem_single = 0;
     int grid_pack = 0, grid_step[2] = {0, 0}, grid_bytes[2] = {0, 0}, grid_single[2] = {0, 0};   // [1]: with the constant rule
     uint32_t *bits[2] = {nullptr, nullptr};   // packed states: NG x KLp words, then the exports, NG x XW x 32

@@ -94,3 +94,41 @@ def test_streamed_states_match_single_generations(name, r):
     g.check()
     g.close()
     tiles.close()
+
+
+@pytest.mark.parametrize("name,r,L", [("menger", 2, 0), ("menger", 3, 0), ("menger", 4, 0), ("menger", 5, 0), ("cube", 3, 0), ("corners", 6, 0)])
+def test_sliced_3d_matches_oracle(name, r, L):
+    # cells with up to 19 (Menger) and 26 (the full cube) neighbours, tiles of a few and of 8000 cells
+    from paper_2110_12952_gb300 import Fractal
+    grid = [(x, y, z) for z in range(3) for y in range(3) for x in range(3)]
+    tables = {"menger": (20, 3, W.MENGER.table()), "cube": (27, 3, np.array(grid, dtype=np.int32)),
+              "corners": (4, 2, np.array([(0, 0, 0), (1, 1, 0), (1, 0, 1), (0, 1, 1)], dtype=np.int32))}
+    k, s, tab = tables[name]
+    g, o = Fractal(k, s, r, 3, tab), oracle.Fractal(k, s, r, 3, tab)
+    x = o.init_bernoulli(r, 0.3)
+    x[::7] *= 201
+    rules = [W.MENGER_B5S45, W.rule_masks([4, 26], [0, 3, 4, 5, 18, 26])]
+    for i, (rule, steps) in enumerate(zip(rules * 2, (2, 3, 1, 5))):
+        off = (0, 3, 0, 8)[i]
+        src = torch.empty(g.cells + off, dtype=torch.uint8, device="cuda")[off:]
+        whole = torch.full((g.cells + 64,), 77, dtype=torch.uint8, device="cuda")
+        src.copy_(torch.from_numpy(x))
+        dst = whole[i:i + g.cells]
+        g.step(src, out=dst, steps=steps, rule=rule)
+        assert np.array_equal(dst.cpu().numpy(), o.step(x, rule=oracle.Rule(*rule), steps=steps)), (name, r, rule, steps)
+        assert int((whole == 77).sum()) == 64
+    g.check()
+    g.close()
+
+
+def test_sliced_menger_single_generations():
+    # large enough for the sliced step at one generation: against the tile kernels
+    from paper_2110_12952_gb300 import Fractal
+    g, tiles = Fractal.from_family(W.MENGER, 6), Fractal.from_family(W.MENGER, 6)
+    tiles.tile_levels = tiles.tile_levels
+    x = g.init_bernoulli(5, 0.4)
+    one = g.step(x, steps=1)
+    assert torch.equal(one, tiles.step(x, steps=1))
+    assert torch.equal(g.step(x, steps=3), tiles.step(tiles.step(one, steps=1), steps=1))
+    g.close()
+    tiles.close()

@@ -32,7 +32,11 @@
 
 #include <algorithm>
 #include <cmath>
+#include <list>
+#include <memory>
+#include <mutex>
 #include <new>
+#include <string>
 #include <vector>
 
 #include "handle.h"
@@ -1011,7 +1015,8 @@ static SliceTables slice_tables(SliceNbrs &&nbrs, int Q)
             const std::vector<int> run(cells[d].begin() + i, cells[d].begin() + std::min(i + 32, cells[d].size()));
             int w = -1;
             for (int x = 0; x < (int)words.size() && w < 0; ++x)
-                if (std::includes(words[x].begin(), words[x].end(), run.begin(), run.end())) w = x;
+                if (words[x].size() >= run.size() && words[x].front() <= run.front() && words[x].back() >= run.back() &&
+                    std::includes(words[x].begin(), words[x].end(), run.begin(), run.end())) w = x;
             if (w < 0) {
                 w = (int)words.size();
                 words.push_back(run);
@@ -1041,68 +1046,124 @@ static SliceTables slice_tables(SliceNbrs &&nbrs, int Q)
 // from the emptiest bank.
 static void slice_neighbour_table(const SliceTables &t, int D, uint16_t *tab)
 {
-    const int KLp = (t.KL + 31) / 32 * 32;
+    const int KLp = (t.KL + 31) / 32 * 32, Q = t.Q;
     const uint32_t all = (1u << D) - 1u;
-    // entry k of cell i: column k / 8 (columns of 8, the last of 4 or 2; see SliceRow)
-    auto at = [&](int i, int k) -> uint16_t & {
-        const int col = k / 8, width = col == (D - 1) / 8 && D > 8 ? (D == 20 ? 4 : 2) : 8;
-        return tab[(size_t)col * 8 * KLp + (size_t)i * width + k % 8];
-    };
+    // entry k of cell i is at col[k] + i * step[k]: columns of 8, the last of 4 or 2 (see SliceRow)
+    const int entries = D <= 8 ? 8 : D;
+    size_t col[26], step[26];
+    for (int k = 0; k < entries; ++k) {
+        step[k] = D > 8 && k / 8 == (D - 1) / 8 ? (D == 20 ? 4 : 2) : 8;
+        col[k] = (size_t)(k / 8) * 8 * KLp + k % 8;
+    }
     std::vector<uint32_t> loaded((size_t)t.zero + 32, 0);   // per word: the loads of this chunk that read it
     for (int c = 0; c < KLp; c += 32) {
-        // [bank][x]: the loads that read x words of the bank, as a bit set
-        uint32_t with[32][33] = {};
-        int v[32][26], put[32][26], n[32];
-        for (int b = 0; b < 32; ++b) with[b][0] = all;
+        // [bank][x]: the loads that read x words of the bank, as a bit set; per load: the banks it reads
+        uint32_t with[32][33], used[26] = {};
+        int v[32][26], put[32][26], n[32], top[32];
+        for (int b = 0; b < 32; ++b) {
+            with[b][0] = all;
+            top[b] = 0;
+        }
+        int by_count[27][32], many[27] = {};
         for (int i = 0; i < 32; ++i) {
             n[i] = 0;
-            for (int d = 0; d < t.Q && c + i < t.KL; ++d) {
-                const int32_t a = d == t.Q / 2 ? -1 : t.nb[(size_t)(c + i) * t.Q + d];
-                if (a < 0) continue;
-                v[i][n[i]++] = (a >> 24) == t.Q / 2 ? a & 0xffffff : t.hidx[(size_t)(a >> 24) * t.KL + (a & 0xffffff)];
+            if (c + i < t.KL) {
+                const int32_t *nb = &t.nb[(size_t)(c + i) * Q];
+                for (int d = 0; d < Q; ++d)
+                    if (nb[d] >= 0 && d != Q / 2)
+                        v[i][n[i]++] = (nb[d] >> 24) == Q / 2 ? nb[d] & 0xffffff
+                                                              : t.hidx[(size_t)(nb[d] >> 24) * t.KL + (nb[d] & 0xffffff)];
             }
+            by_count[n[i]][many[n[i]]++] = i;
         }
         for (int want = D; want >= 1; --want)   // cells with the most neighbours first
-            for (int i = 0; i < 32; ++i) {
-                if (n[i] != want) continue;
+            for (int m = 0; m < many[want]; ++m) {
+                const int i = by_count[want][m];
                 uint32_t open = all;
-                for (int e = 0; e < n[i]; ++e) {
+                for (int e = 0; e < want; ++e) {
                     const int w = v[i][e], b = w & 31;
                     uint32_t pick = open & loaded[w];
                     if (!pick) {
                         int x = 0;
                         while (!(pick = open & with[b][x])) ++x;
                         pick &= 0u - pick;
+                        if (x == top[b]) with[b][++top[b]] = 0u;
                         with[b][x] &= ~pick;
                         with[b][x + 1] |= pick;
                         loaded[w] |= pick;
                     }
                     pick &= 0u - pick;
                     open &= ~pick;
-                    int k = 0;
-                    while (!((pick >> k) & 1)) ++k;
-                    put[i][e] = k;
+                    put[i][e] = __builtin_ctz(pick);
+                    used[put[i][e]] |= 1u << b;
                 }
             }
-        for (int i = 0; i < 32; ++i)
-            for (int e = 0; e < n[i]; ++e) loaded[v[i][e]] = 0;
-        for (int k = 0; k < D; ++k) {
-            int z = 0, least = 33;
-            for (int b = 0; b < 32; ++b) {
-                int x = 0;
-                while (!((with[(t.zero + b) & 31][x] >> k) & 1)) ++x;
-                if (x < least) {
-                    least = x;
-                    z = b;
-                }
-            }
-            for (int i = 0; i < 32; ++i) at(c + i, k) = (uint16_t)(4 * (t.zero + z));
+        for (int k = 0; k < entries; ++k) {
+            // the zero word in a bank the load does not read, where there is one
+            const uint32_t free = k < D ? ~used[k] : ~0u;
+            const uint16_t z = (uint16_t)(4 * (t.zero + (free ? (__builtin_ctz(free) - t.zero) & 31 : 0)));
+            uint16_t *p = tab + col[k] + (size_t)c * step[k];
+            for (int i = 0; i < 32; ++i) p[i * step[k]] = z;
         }
-        for (int k = D; k < 8; ++k)
-            for (int i = 0; i < 32; ++i) at(c + i, k) = (uint16_t)(4 * t.zero);
         for (int i = 0; i < 32; ++i)
-            for (int e = 0; e < n[i]; ++e) at(c + i, put[i][e]) = (uint16_t)(4 * v[i][e]);
+            for (int e = 0; e < n[i]; ++e) {
+                tab[col[put[i][e]] + (size_t)(c + i) * step[put[i][e]]] = (uint16_t)(4 * v[i][e]);
+                loaded[v[i][e]] = 0;
+            }
     }
+}
+
+// The tables of a transition table at a tile depth, and their device layout.
+struct SliceImage {
+    SliceTables t;
+    std::once_flag once;
+    std::vector<uint16_t> tab;   // neighbour table, made when first wanted
+    size_t bytes = 0;
+    const std::vector<uint16_t> &neighbours(int D)
+    {
+        std::call_once(once, [&]() {
+            tab.resize((size_t)((t.KL + 31) / 32 * 32) * (D <= 8 ? 8 : (D == 20 ? 20 : 26)));
+            slice_neighbour_table(t, D, tab.data());
+        });
+        return tab;
+    }
+};
+
+// They depend on the transition table alone, take milliseconds to make in 3D
+// and serve every handle of that fractal at any level: the most recently used
+// ones are kept (at most kSliceImageBytes of them), and handles that are being
+// planned hold what they use themselves.
+constexpr size_t kSliceImageBytes = (size_t)32 << 20;
+static std::mutex g_image_mu;
+static std::list<std::pair<std::string, std::shared_ptr<SliceImage>>> g_images;   // the latest first
+
+static std::shared_ptr<SliceImage> slice_image(const fractal *f, int L)
+{
+    std::string key = std::to_string(f->dim) + "," + std::to_string(f->s) + "," + std::to_string(L) + "|";
+    for (int32_t v : f->offsets) key += std::to_string(v) + ",";
+    {
+        std::lock_guard<std::mutex> lk(g_image_mu);
+        for (auto it = g_images.begin(); it != g_images.end(); ++it)
+            if (it->first == key) {
+                g_images.splice(g_images.begin(), g_images, it);
+                return it->second;
+            }
+    }
+    const int Q = f->dim == 3 ? 27 : 9;
+    SliceNbrs nbrs = slice_first(f);
+    if (L > 1) nbrs = slice_deepen(nbrs, slice_image(f, L - 1)->t.nb, f->k, Q);
+    auto img = std::make_shared<SliceImage>();
+    img->t = slice_tables(std::move(nbrs), Q);
+    img->bytes = (size_t)img->t.KL * (Q * 8 + 52) + 4096;
+    std::lock_guard<std::mutex> lk(g_image_mu);
+    g_images.emplace_front(key, img);
+    size_t total = 0;
+    for (auto it = g_images.begin(); it != g_images.end();) {
+        total += it->second->bytes;
+        if (total > kSliceImageBytes && it != g_images.begin()) it = g_images.erase(it);
+        else ++it;
+    }
+    return img;
 }
 
 void free_slice_plan(SlicePlan &p)
@@ -1272,18 +1333,19 @@ static bool slice_resident_shape(const SliceGeo &p, int num_sms, bool batch, Sli
 // group of 32 tiles adds its cells' neighbours, about 45 instructions per 32
 // cells, makes and takes its halo words, about 30 each, and pays its loops
 // and barriers, about 400; kSliceWave groups run at a time).
-static int slice_levels(const fractal *f, SlicePlan *plan, SliceTables *tables)
+static int slice_levels(const fractal *f, SlicePlan *plan, std::shared_ptr<SliceImage> *image)
 {
     int best = 0;
     double cost = 0;
-    const SliceNbrs first = slice_first(f);
-    SliceNbrs nbrs = first;
     const bool d3 = f->dim == 3;
-    const int Q = d3 ? 27 : 9;
+    // 3D: the deepest tiles with a group per SM, where there are such, without a look at the others
+    int only = 0;
+    for (int L = 1; d3 && L <= f->r && pw(f->k, L) <= kSliceMaxKL3; ++L)
+        if ((double)pw(f->k, f->r - L) < 2147483648.0 && (pw(f->k, f->r - L) + 31) / 32 >= f->num_sms) only = L;
     for (int L = 1; L <= f->r && pw(f->k, L) <= (d3 ? kSliceMaxKL3 : kSliceMaxKL); ++L) {
-        if (L > 1) nbrs = slice_deepen(first, nbrs, f->k, Q);
-        if ((double)pw(f->k, f->r - L) >= 2147483648.0) continue;
-        SliceTables t = slice_tables(SliceNbrs(nbrs), Q);
+        if ((only && L != only) || (double)pw(f->k, f->r - L) >= 2147483648.0) continue;
+        const std::shared_ptr<SliceImage> img = slice_image(f, L);
+        const SliceTables &t = img->t;
         const SliceGeo p = slice_geo(f, L, t);
         if (p.AW * 4 > 65535 || p.XW > 255) continue;
         SlicePlan s;
@@ -1299,7 +1361,7 @@ static int slice_levels(const fractal *f, SlicePlan *plan, SliceTables *tables)
             cost = c;
             *plan = s;
             plan->geo = p;
-            *tables = std::move(t);
+            *image = img;
         }
     }
     return best;
@@ -1307,21 +1369,23 @@ static int slice_levels(const fractal *f, SlicePlan *plan, SliceTables *tables)
 
 // One allocation: the tables (copied from the host in one piece), the grid
 // barrier's zeros, the neighbouring tiles and the resident exports.
-static cudaError_t slice_upload(SliceGeo &p, const SliceTables &t, SlicePlan &s, const std::vector<SliceGroup> &groups,
+static cudaError_t slice_upload(SliceGeo &p, SliceImage &image, SlicePlan &s, const std::vector<SliceGroup> &groups,
                                 cudaStream_t st)
 {
+    const SliceTables &t = image.t;
+    const std::vector<uint16_t> &nb = image.neighbours(p.D);
     size_t off = 0;
     auto take = [&](size_t bytes) {
         const size_t at = off;
         off += (bytes + 255) / 256 * 256;
         return at;
     };
-    const size_t o_tab = take((size_t)p.KLp * (p.D <= 8 ? 16 : (p.D == 20 ? 40 : 52))), o_jobs = take(t.jobs.size() * 4), o_xl = take(t.xlist.size() * 2),
+    const size_t o_tab = take(nb.size() * 2), o_jobs = take(t.jobs.size() * 4), o_xl = take(t.xlist.size() * 2),
                  o_cells = take(t.cells.size() * 4), o_bar = take(8), o_groups = take(groups.size() * sizeof(SliceGroup)), host = off;
     const size_t o_nbr = take((size_t)p.NG * p.ND * 32 * sizeof(int32_t)),
                  exb = s.resident ? (size_t)p.NG * p.XW * 128 : 0, o_ex0 = take(exb), o_ex1 = take(exb);
     std::vector<uint8_t> img(host, 0);
-    slice_neighbour_table(t, p.D, reinterpret_cast<uint16_t *>(img.data() + o_tab));
+    memcpy(img.data() + o_tab, nb.data(), nb.size() * 2);
     memcpy(img.data() + o_jobs, t.jobs.data(), t.jobs.size() * 4);
     memcpy(img.data() + o_xl, t.xlist.data(), t.xlist.size() * 2);
     memcpy(img.data() + o_cells, t.cells.data(), t.cells.size() * 4);
@@ -1342,9 +1406,9 @@ static cudaError_t slice_upload(SliceGeo &p, const SliceTables &t, SlicePlan &s,
 
 static int build_slice_plan(fractal *f, cudaStream_t st)
 {
-    SliceTables t;
+    std::shared_ptr<SliceImage> img;
     SlicePlan s;
-    if (slice_levels(f, &s, &t) < 1) return FR_EINVAL;
+    if (slice_levels(f, &s, &img) < 1) return FR_EINVAL;
     SliceGeo &p = s.geo;
     s.block = f->dim == 3 ? kSliceBlock3 : kSliceBlock;
     const int ring = 32 * kSliceBatch * s.block, arrays = f->dim == 3 ? 1 : 2;
@@ -1352,7 +1416,7 @@ static int build_slice_plan(fractal *f, cudaStream_t st)
     s.smem_single = ring + 4 * (p.AW + std::max(string_words(p), 32 * p.RP + 1));
     s.smem_step = 4 * (arrays * p.AW + p.KLp);
     s.smem_bytes = 4 * (arrays * p.AW + 32 * p.RP + 1);
-    cudaError_t e = slice_upload(p, t, s, {}, st);
+    cudaError_t e = slice_upload(p, *img, s, {}, st);
     if (e == cudaSuccess) {
         const int64_t blocks = std::min<int64_t>((32 * p.NG + 255) / 256, (int64_t)f->num_sms * 16);
         if (f->dim == 3)
@@ -1622,14 +1686,11 @@ int build_slice_batch(const std::vector<SliceBatchItem> &items, uint32_t birth, 
     int rmax = 0;
     for (const auto &i : items) rmax = std::max(rmax, i.f->r);
     // tables by tile depth
-    std::vector<SliceTables> tabs(1);
+    std::vector<std::shared_ptr<SliceImage>> tabs(1);
     std::vector<SliceGeo> geos(1);
-    const SliceNbrs first = slice_first(rep);
-    SliceNbrs nbrs = first;
     for (int L = 1; L <= rmax && pw(rep->k, L) <= kSliceMaxKL; ++L) {
-        if (L > 1) nbrs = slice_deepen(first, nbrs, rep->k, 9);
-        tabs.push_back(slice_tables(SliceNbrs(nbrs), 9));
-        geos.push_back(slice_geo(rep, L, tabs.back()));
+        tabs.push_back(slice_image(rep, L));
+        geos.push_back(slice_geo(rep, L, tabs.back()->t));
     }
     const int lmax = (int)tabs.size() - 1;
     auto groups_of = [&](const SliceBatchItem &i, int L) { return (pw(rep->k, i.f->r - L) + 31) / 32; };
@@ -1704,7 +1765,7 @@ int build_slice_batch(const std::vector<SliceBatchItem> &items, uint32_t birth, 
             p.NT = 32 * p.NG;
             double c = 0;
             cudaError_t e = slice_resident_shape(p, rep->num_sms, true, &l.plan, &c) ? cudaSuccess : cudaErrorInvalidConfiguration;
-            if (e == cudaSuccess) e = slice_upload(p, tabs[L], l.plan, groups, st);
+            if (e == cudaSuccess) e = slice_upload(p, *tabs[L], l.plan, groups, st);
             if (e == cudaSuccess) {
                 const int64_t blocks = std::min<int64_t>((32 * p.NG + 255) / 256, (int64_t)rep->num_sms * 16);
                 slice_nbr_kernel<2><<<(unsigned)blocks, 256, 0, st>>>(rep->dev, p.NT, p.NG, 0, 1,

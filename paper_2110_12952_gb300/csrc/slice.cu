@@ -228,12 +228,14 @@ __device__ __forceinline__ uint32_t slice_bits16(uint4 v)
     return __funnelshift_l(v.x * 0x10204080u, x, 4);
 }
 
-// The exports of a group from its words N: lane i takes cell i of an export
-// word, lane t gets tile t's bits.
-__device__ __forceinline__ void slice_export(const SliceArgs &a, const Transpose32 &tr, const uint32_t *N, uint32_t *ex,
+// The exports of a group from its words in memory (written by this block and
+// behind a barrier; a copy in shared memory would cost a block or two per SM):
+// lane i takes cell i of an export word, lane t gets tile t's bits.
+__device__ __forceinline__ void slice_export(const SliceArgs &a, const Transpose32 &tr, const uint32_t *words, uint32_t *ex,
                                              int warp, int nw, int lane)
 {
-    for (int x = warp; x < a.XW; x += nw) ex[32 * x + lane] = tr(N[__ldg(a.xlist + 32 * x + lane)]);
+#pragma unroll 2
+    for (int x = warp; x < a.XW; x += nw) ex[32 * x + lane] = tr(words[__ldg(a.xlist + 32 * x + lane)]);
 }
 
 // Words of a group's bit string in shared memory (one to spare for the funnel shifts).
@@ -352,7 +354,7 @@ __device__ __forceinline__ uint32_t slice_string_chunk(const SliceArgs &a, const
 // issue slots and the latency of its loads (carpet r = 10, 1.07e9 cells:
 // 0.20 ms, 5.9 TB/s read and written).
 template <int BLK>
-__global__ void __launch_bounds__(BLK, BLK == kSliceBlock ? 5 : 2)
+__global__ void __launch_bounds__(BLK, BLK == kSliceBlock ? 6 : 3)
 slice_pack_kernel(SliceArgs a, const uint8_t *__restrict__ in, uint32_t *__restrict__ bits)
 {
     extern __shared__ __align__(16) uint32_t smem[];
@@ -360,8 +362,7 @@ slice_pack_kernel(SliceArgs a, const uint8_t *__restrict__ in, uint32_t *__restr
     const Transpose32 tr(lane);
     SliceRing<BLK> ring;
     ring.start(a, in, smem);
-    uint32_t *N = smem + 8 * kSliceBatch * BLK;   // the packed words
-    uint32_t *B = N + a.KLp;
+    uint32_t *B = smem + 8 * kSliceBatch * BLK;
     for (int64_t g = blockIdx.x; g < a.NG; g += gridDim.x) {
         const int nt = (int)min((int64_t)32, a.NT - 32 * g);
         ring.string(a, in, g, B);
@@ -369,12 +370,10 @@ slice_pack_kernel(SliceArgs a, const uint8_t *__restrict__ in, uint32_t *__restr
         uint32_t *dst = bits + g * a.KLp;
 #pragma unroll 2
         for (int c = warp; c < a.NC; c += nw) {
-            const uint32_t x = slice_string_chunk(a, tr, B, c, nt, lane);
-            dst[32 * c + lane] = x;
-            N[32 * c + lane] = x;
+            dst[32 * c + lane] = slice_string_chunk(a, tr, B, c, nt, lane);
         }
         __syncthreads();
-        slice_export(a, tr, N, bits + a.ex + g * a.XW * 32, warp, nw, lane);
+        slice_export(a, tr, dst, bits + a.ex + g * a.XW * 32, warp, nw, lane);
     }
 }
 
@@ -533,8 +532,7 @@ slice_step_kernel(SliceArgs a, const uint32_t *src, uint32_t *dst, uint8_t *__re
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, nw = blockDim.x >> 5;
     const Transpose32 tr(lane);
     constexpr bool kAhead = D <= 8;   // two arrays, the next group's words loaded ahead (3D: no room, two blocks per SM instead)
-    uint32_t *N = smem + (kAhead ? 2 : 1) * a.AW;   // the new words; BYTES: the results' bit strings
-    uint32_t *R = N;
+    uint32_t *R = smem + (kAhead ? 2 : 1) * a.AW;   // BYTES: the results' bit strings
     if (tid < (kAhead ? 64 : 32)) smem[(tid >> 5) * a.AW + a.A_zero + lane] = 0u;   // the words of absent neighbours
     uint32_t job[kSliceAhead];
 #pragma unroll
@@ -577,7 +575,6 @@ slice_step_kernel(SliceArgs a, const uint32_t *src, uint32_t *dst, uint8_t *__re
                     R[lane * a.RP + c] = tr(w);
                 } else {
                     dg[32 * c + lane] = w;
-                    N[32 * c + lane] = w;
                 }
             }
             if (gn < a.NG) {
@@ -589,7 +586,7 @@ slice_step_kernel(SliceArgs a, const uint32_t *src, uint32_t *dst, uint8_t *__re
             if (BYTES) {
                 slice_string_to_bytes(a, R, out + 32 * g * a.KL, (int)min((int64_t)32, a.NT - 32 * g), tid, blockDim.x);
             } else {
-                slice_export(a, tr, N, dst + a.ex + g * a.XW * 32, warp, nw, lane);
+                slice_export(a, tr, dg, dst + a.ex + g * a.XW * 32, warp, nw, lane);
             }
         }
         if (!BYTES && gen + 1 < gens) {
@@ -1412,9 +1409,9 @@ static int build_slice_plan(fractal *f, cudaStream_t st)
     SliceGeo &p = s.geo;
     s.block = f->dim == 3 ? kSliceBlock3 : kSliceBlock;
     const int ring = 32 * kSliceBatch * s.block, arrays = f->dim == 3 ? 1 : 2;
-    s.smem_pack = ring + 4 * (string_words(p) + p.KLp);
+    s.smem_pack = ring + 4 * string_words(p);
     s.smem_single = ring + 4 * (p.AW + std::max(string_words(p), 32 * p.RP + 1));
-    s.smem_step = 4 * (arrays * p.AW + p.KLp);
+    s.smem_step = 4 * arrays * p.AW;
     s.smem_bytes = 4 * (arrays * p.AW + 32 * p.RP + 1);
     cudaError_t e = slice_upload(p, *img, s, {}, st);
     if (e == cudaSuccess) {

@@ -68,6 +68,7 @@ struct LambdaTab {
     int m_last, n_last;      // the same of the last group, whose table follows (n_last = n: the same table)
     int last;                // where the last group's table starts
     int wide;                // groups before which the number may reach 2^31
+    int32_t start[kMapGroups];    // where a group's table starts
     uint32_t scale[kMapGroups];   // s^(m g)
     DivU64 div64;            // by k^m
     DivU32 div32;
@@ -100,7 +101,7 @@ __device__ __forceinline__ void lambda_lookup(const LambdaTab &L, const uint32_t
         } else {
             q = divu(L.div32, v);
         }
-        const uint32_t e = tab[v - q * (uint32_t)L.n + (g == L.groups - 1 ? L.last : 0)];
+        const uint32_t e = tab[v - q * (uint32_t)L.n + (uint32_t)L.start[g]];
         v = q;
         if (DIM == 2) {
             x += L.scale[g] * (e & 0xffffu);
@@ -156,27 +157,32 @@ __global__ void __launch_bounds__(kMapBlock) lambda_tab_kernel(FracDev F, Lambda
 // nu through tables: entry x + s^m (y + s^m z) holds the replica digits of m
 // levels as a number (base k), or -1 where some level's digits are no
 // replica.  With COMPACT it holds the compact coordinate of the m levels
-// instead (m a multiple of the dimension, so that every group starts at the
-// first axis), 16 bits per component in 2D, 10 in 3D.
+// instead, 16 bits per component in 2D, 10 in 3D, in a table for each axis
+// that a group's first level may fall on.
 struct NuTab {
     int m, groups, n;        // levels per group, groups, entries (s^(m dim))
     int m_last, n_last;      // the same of the last group, whose table follows (n_last = n: the same table)
     int last;                // where the last group's table starts
+    int phases;              // tables by the axis of a group's first level (compact coordinate)
     uint32_t sm;             // s^m
     int shift;               // log2 of s^m, or -1
     DivU32 div;              // by s^m
-    int64_t scale[kMapGroups];   // k^(m g); compact coordinate: k^(m g / dim)
+    int32_t start[kMapGroups];   // where a group's table starts
+    int64_t scale[kMapGroups];   // k^(m g); compact coordinate: k^floor(m g / dim)
 };
 
 template <int DIM, bool COMPACT>
 __device__ __forceinline__ void nu_table(const FracDev &F, const NuTab &N, uint32_t *tab)
 {
-    const int all = N.n + (N.n_last == N.n ? 0 : N.n_last);
+    const int whole = N.n * N.phases, all = whole + (N.last == 0 ? 0 : N.n_last);
     for (int i = threadIdx.x; i < all; i += blockDim.x) {
         // (the last group's digits run over s^m_last only, but are laid out
         // like the others': entries in between are never read)
-        uint32_t c[3] = {0, 0, 0}, v = (uint32_t)(i < N.n ? i : i - N.n);
-        const int m = i < N.n ? N.m : N.m_last;
+        const int part = i < whole ? i / N.n : (N.groups - 1) * N.m % DIM;
+        uint32_t c[3] = {0, 0, 0}, v = (uint32_t)(i < whole ? i - part * N.n : i - whole);
+        const int m = i < whole ? N.m : N.m_last;
+        // the group of a whole table starts at axis (m part) mod dim, the last one at its own
+        int axis = COMPACT ? (i < whole ? part * N.m % DIM : part) : 0;
         for (int a = 0; a < DIM; ++a) {
             const uint32_t q = divu(N.div, v);
             c[a] = v - q * N.sm;
@@ -194,9 +200,12 @@ __device__ __forceinline__ void nu_table(const FracDev &F, const NuTab &N, uint3
             }
             const int h = F.hinv[t];
             ok = ok && h >= 0;
-            const int axis = COMPACT ? mu % DIM : 0;
             acc[axis] += (uint32_t)h * w;
-            if (!COMPACT || axis == DIM - 1) w *= F.k;
+            if (!COMPACT) w *= F.k;
+            else if (++axis == DIM) {
+                axis = 0;
+                w *= F.k;
+            }
         }
         tab[i] = !ok ? 0xffffffffu
                      : (!COMPACT ? acc[0] : (DIM == 2 ? acc[0] | acc[1] << 16 : acc[0] | acc[1] << 10 | acc[2] << 20));
@@ -217,7 +226,7 @@ __device__ __forceinline__ void nu_lookup(const NuTab &N, const uint32_t *tab, i
 #pragma unroll
     for (int g = 0; g < kMapGroups; ++g) {
         if (g == N.groups) break;
-        uint32_t i = g == N.groups - 1 ? (uint32_t)N.last : 0u, w = 1;
+        uint32_t i = (uint32_t)N.start[g], w = 1;
 #pragma unroll
         for (int a = 0; a < DIM; ++a) {
             const uint32_t q = POW2 ? v[a] >> N.shift : divu(N.div, v[a]);
@@ -296,6 +305,7 @@ static bool lambda_tab(const fractal *f, LambdaTab *L)
     L->m_last = m_last;
     L->n_last = (int)n_last;
     L->last = n_last == n ? 0 : (int)n;
+    for (int g = 0; g < kMapGroups; ++g) L->start[g] = g == groups - 1 ? L->last : 0;
     L->wide = 0;
     for (int64_t c = f->cells - 1; c >> 31; c /= n) ++L->wide;
     uint32_t scale = 1;
@@ -308,45 +318,55 @@ static bool lambda_tab(const fractal *f, LambdaTab *L)
 static bool nu_tab(const fractal *f, bool compact, NuTab *N)
 {
     if (f->mixed || f->r < 1) return false;
-    const int unit = compact ? f->dim : 1;
-    int64_t block = 1, sm1 = 1, k1 = 1;   // entries, side and members of `unit` levels
-    for (int i = 0; i < unit; ++i) {
-        sm1 *= f->s;
-        k1 *= f->k;
-    }
-    for (int i = 0; i < f->dim; ++i) block *= sm1;
-    if (block > kMapTable) return false;
+    const int dim = f->dim;
     // components are stored in 16 or 10 bits, nu in 31
-    const int64_t most = !compact ? (int64_t)1 << 31 : (f->dim == 2 ? 65535 : 1024);
-    const int64_t kc1 = compact ? f->k : k1;   // growth of a component per `unit` levels
-    int64_t n = block, sm = sm1, kc = kc1;
-    int m = unit;
-    if (kc > most) return false;
-    while (m < f->r && n * block <= kMapTable && kc * kc1 <= most) {
-        n *= block;
-        sm *= sm1;
-        kc *= kc1;
-        m += unit;
+    const int64_t most = !compact ? (int64_t)1 << 31 : (dim == 2 ? 65535 : 1024);
+    int64_t block = 1;
+    for (int i = 0; i < dim; ++i) block *= f->s;
+    int m = 0, phases = 1;
+    int64_t n = 1, sm = 1;
+    for (int t = 1; t <= f->r; ++t) {
+        int64_t nt = 1, st = 1, kc = 1;
+        for (int i = 0; i < t; ++i) {
+            nt *= block;
+            st *= f->s;
+            if (nt > kMapTable) break;
+        }
+        // (a group's components have at most ceil(t / dim) digits, wherever it starts: t levels alternate the axes)
+        for (int i = 0; i < (compact ? (t + dim - 1) / dim : t); ++i) kc = kc > most ? kc : kc * f->k;
+        const int ph = !compact || t % dim == 0 ? 1 : dim;   // (dim is 2 or 3: prime)
+        if (nt > kMapTable) break;
+        if (kc > most || nt * ph > kMapTable) continue;
+        m = t;
+        n = nt;
+        sm = st;
+        phases = ph;
     }
+    if (m == 0) return false;
     const int groups = (f->r + m - 1) / m, m_last = f->r - m * (groups - 1);
     // the last group's largest index + 1: its coordinates stay below s^m_last, in steps of s^m
     int64_t sl = 1, n_last = 0, row = 1;
     for (int i = 0; i < m_last; ++i) sl *= f->s;
-    for (int i = 0; i < f->dim; ++i, row *= sm) n_last += (sl - 1) * row;
+    for (int i = 0; i < dim; ++i, row *= sm) n_last += (sl - 1) * row;
     if (groups > kMapGroups) return false;
     N->m = m;
     N->groups = groups;
     N->n = (int)n;
     N->m_last = m_last;
     N->n_last = m_last == m ? (int)n : (int)n_last + 1;
-    N->last = m_last == m ? 0 : (int)n;
+    N->phases = phases;
+    N->last = m_last == m ? 0 : (int)n * phases;
     N->sm = (uint32_t)sm;
     N->shift = -1;
     if ((sm & (sm - 1)) == 0)
         for (N->shift = 0; (1ll << N->shift) < sm;) ++N->shift;
     N->div = make_div((uint32_t)sm);
-    uint64_t scale = 1;   // (past the last group it may wrap: never read)
-    for (int g = 0; g < kMapGroups; ++g, scale *= (uint64_t)kc) N->scale[g] = (int64_t)scale;
+    for (int g = 0; g < kMapGroups; ++g) N->start[g] = g == groups - 1 && N->last ? N->last : g % phases * (int)n;
+    for (int g = 0; g < kMapGroups; ++g) {   // (past the last group it may wrap: never read)
+        uint64_t scale = 1;
+        for (int i = 0; i < (compact ? m * g / dim : m * g); ++i) scale *= (uint64_t)f->k;
+        N->scale[g] = (int64_t)scale;
+    }
     return true;
 }
 

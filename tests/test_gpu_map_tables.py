@@ -71,3 +71,16 @@ def test_box_views_by_tiles(name, r):
         back = torch.full((o.cells + off,), 5, dtype=torch.uint8, device="cuda")[off:]
         assert np.array_equal(g.gather(box, out=back).cpu().numpy(), (x != 0).astype(np.uint8))
     g.close()
+
+
+@pytest.mark.parametrize("name,r", [("carpet", 9), ("full_square", 14), ("menger", 5)])
+def test_large_boxes_filled(name, r):
+    # rows shorter and longer than a block's run of 16384 cells: every cell is where gather finds it, nothing elsewhere
+    from paper_2110_12952_gb300 import Fractal
+    g = Fractal.from_family(W.FAMILIES[name], r)
+    x = torch.empty(g.cells, dtype=torch.uint8, device="cuda").bernoulli_(0.5)
+    box = torch.full((g.box_cells,), 9, dtype=torch.uint8, device="cuda")
+    g.scatter(x, out=box)
+    assert torch.equal(g.gather(box), x)
+    assert int(box.max()) == 1 and int(box.sum(dtype=torch.int64)) == int(x.sum(dtype=torch.int64))
+    g.close()

@@ -48,7 +48,7 @@ namespace fr {
 constexpr int kSliceBlock = 256;   // threads per block of the streaming kernels
 constexpr int kSliceBlock3 = 512;  // the same in 3D, where a group is larger (Menger: 8000 words and 3700 halo words)
 constexpr int kSliceAhead = 2;     // halo words per warp loaded ahead of their group
-constexpr int kSliceBatch = 2;     // 16-byte units per thread and batch copied to shared memory ahead
+constexpr int kSliceBatch = 4;     // 16-byte units per thread and batch copied to shared memory ahead
 constexpr int kSliceSmem = 220 * 1024;   // resident kernel: shared memory per block
 constexpr int64_t kSliceBatchCells = 60000000;   // batches: most cells of an instance
 constexpr int kSliceSingleHalo = 32;   // most halo cells of a tile for the single-pass kernel
@@ -274,39 +274,41 @@ __device__ __forceinline__ void slice_bytes_to_string(const SliceArgs &a, const 
 }
 
 // The same for blocks that walk the groups: every thread copies the 16-byte
-// units it will convert into its own slots of shared memory, two batches
-// ahead and across group boundaries, and waits for its own copies only.
+// units it will convert into its own slots of shared memory, a batch ahead
+// and across group boundaries, and waits for its own copies only.  A slot is
+// refilled as soon as it has been read; the addresses are worked out once per
+// batch (kSliceBatch units).
 template <int BLK>
 struct SliceRing {
-    uint8_t *slot;       // this thread's first slot of batch buffer 0
+    uint8_t *slot;       // this thread's first slot
     int64_t g;           // the batch to be copied next: its group, first unit, the group's units
-    int first, whole, buf;
+    int first, whole;
     static constexpr int kUnits = kSliceBatch * BLK;   // per batch
     __device__ __forceinline__ int units(const SliceArgs &a, const uint8_t *in, int64_t gq) const
     {
         if (gq >= a.NG || ((uintptr_t)in & 15)) return 0;
         return (int)min((int64_t)32, a.NT - 32 * gq) * a.KL / 16;
     }
-    __device__ __forceinline__ void issue(const SliceArgs &a, const uint8_t *__restrict__ in, int b)
+    // the source of this thread's units of the next batch and how many units
+    // are left from its first on; then on to the batch after it
+    __device__ __forceinline__ const uint8_t *next(const SliceArgs &a, const uint8_t *__restrict__ in, int *left)
     {
-        const int n = whole - first - (int)threadIdx.x;   // units left from this thread's first on
-        if (n > 0) {
-            const uint8_t *src = in + 32 * g * a.KL + 16 * (int64_t)(first + (int)threadIdx.x);
-            const uint32_t dst = smem_addr(slot) + 16 * kUnits * b;
-#pragma unroll
-            for (int k = 0; k < kSliceBatch; ++k)
-                if (BLK * k < n)
-                    asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(dst + 16 * BLK * k),
-                                 "l"(src + 16 * BLK * k)
-                                 : "memory");
-        }
-        asm volatile("cp.async.commit_group;" ::: "memory");
+        *left = whole - first - (int)threadIdx.x;
+        const uint8_t *src = in + 32 * g * a.KL + 16 * (int64_t)(first + (int)threadIdx.x);
         first += kUnits;
         if (first >= whole) {
             g += gridDim.x;
             first = 0;
             whole = units(a, in, g);
         }
+        return src;
+    }
+    __device__ __forceinline__ void copy(const uint8_t *src, int left, int k)
+    {
+        if (BLK * k < left)
+            asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(smem_addr(slot) + 16 * BLK * k), "l"(src + 16 * BLK * k)
+                         : "memory");
+        asm volatile("cp.async.commit_group;" ::: "memory");
     }
     __device__ __forceinline__ void start(const SliceArgs &a, const uint8_t *__restrict__ in, void *ring)
     {
@@ -314,23 +316,26 @@ struct SliceRing {
         g = blockIdx.x;
         first = 0;
         whole = units(a, in, g);
-        buf = 0;
-        issue(a, in, 0);
-        issue(a, in, 1);
+        int left;
+        const uint8_t *src = next(a, in, &left);
+#pragma unroll
+        for (int k = 0; k < kSliceBatch; ++k) copy(src, left, k);
     }
     // the bit string of group gc (the groups in the order of the walk)
     __device__ __forceinline__ void string(const SliceArgs &a, const uint8_t *__restrict__ in, int64_t gc, uint32_t *B)
     {
         const int n = units(a, in, gc);
-        for (int f = 0; f < n; f += kUnits, buf ^= 1) {
-            asm volatile("cp.async.wait_group 1;" ::: "memory");
-            const uint4 *p = reinterpret_cast<const uint4 *>(slot) + kUnits * buf;
+        for (int f = 0; f < n; f += kUnits) {
+            int ahead;
+            const uint8_t *src = next(a, in, &ahead);
+            const uint4 *p = reinterpret_cast<const uint4 *>(slot);
             const int left = n - f - (int)threadIdx.x;
 #pragma unroll
-            for (int k = 0; k < kSliceBatch; ++k)
-                if (BLK * k < left)
-                    slice_put16(a, B, f + (int)threadIdx.x + BLK * k, slice_bits16(p[BLK * k]));
-            issue(a, in, buf);
+            for (int k = 0; k < kSliceBatch; ++k) {
+                asm volatile("cp.async.wait_group %0;" ::"n"(kSliceBatch - 1) : "memory");
+                if (BLK * k < left) slice_put16(a, B, f + (int)threadIdx.x + BLK * k, slice_bits16(p[BLK * k]));
+                copy(src, ahead, k);
+            }
         }
         const int bytes = (int)min((int64_t)32, a.NT - 32 * gc) * a.KL;
         slice_odd_units(a, in + 32 * gc * a.KL, bytes, n, B, threadIdx.x, BLK);
@@ -362,7 +367,7 @@ slice_pack_kernel(SliceArgs a, const uint8_t *__restrict__ in, uint32_t *__restr
     const Transpose32 tr(lane);
     SliceRing<BLK> ring;
     ring.start(a, in, smem);
-    uint32_t *B = smem + 8 * kSliceBatch * BLK;
+    uint32_t *B = smem + 4 * kSliceBatch * BLK;
     for (int64_t g = blockIdx.x; g < a.NG; g += gridDim.x) {
         const int nt = (int)min((int64_t)32, a.NT - 32 * g);
         ring.string(a, in, g, B);
@@ -629,7 +634,7 @@ slice_single_kernel(SliceArgs a, const uint8_t *__restrict__ in, uint8_t *__rest
     const Transpose32 tr(lane);
     SliceRing<kSliceBlock> ring;
     ring.start(a, in, smem);
-    uint32_t *A = smem + 8 * kSliceBatch * kSliceBlock, *B = A + a.AW;
+    uint32_t *A = smem + 4 * kSliceBatch * kSliceBlock, *B = A + a.AW;
     if (tid < 32) A[a.A_zero + tid] = 0u;   // the words of absent neighbours
     // this warp's first halo cell of the next group, loaded ahead
     const uint2 h0 = warp < a.H ? __ldg(a.cells + warp) : make_uint2(0u, 0u);
@@ -1408,7 +1413,7 @@ static int build_slice_plan(fractal *f, cudaStream_t st)
     if (slice_levels(f, &s, &img) < 1) return FR_EINVAL;
     SliceGeo &p = s.geo;
     s.block = f->dim == 3 ? kSliceBlock3 : kSliceBlock;
-    const int ring = 32 * kSliceBatch * s.block, arrays = f->dim == 3 ? 1 : 2;
+    const int ring = 16 * kSliceBatch * s.block, arrays = f->dim == 3 ? 1 : 2;
     s.smem_pack = ring + 4 * string_words(p);
     s.smem_single = ring + 4 * (p.AW + std::max(string_words(p), 32 * p.RP + 1));
     s.smem_step = 4 * arrays * p.AW;

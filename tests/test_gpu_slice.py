@@ -48,8 +48,8 @@ def test_slice_step_matches_oracle(name, r):
 def test_slice_step_under_capture():
     # a captured call replays with new contents of the same buffers; a handle that has not run yet captures too
     fam = W.CARPET
-    for warm in (True, False):
-        g, o = pair(fam, 5)
+    for warm, r in ((True, 5), (True, 7), (False, 5)):   # one block, a cooperative launch, the tile kernels
+        g, o = pair(fam, r)
         x = torch.empty(g.cells, dtype=torch.uint8, device="cuda")
         y = torch.empty_like(x)
         z = torch.empty_like(x)

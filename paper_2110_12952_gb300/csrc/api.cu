@@ -244,6 +244,7 @@ extern "C" int fractal_destroy(fractal_t *f)
     cudaFree(f->b3_state[0]);
     cudaFree(f->b3_state[1]);
     for (uint32_t *w : f->bb_words) cudaFree(w);
+    if (f->packed_done) cudaEventDestroy(f->packed_done);
     cudaFree(f->bb_scratch);
     cudaFree(f->host_io[0]);
     cudaFree(f->host_io[1]);
@@ -337,6 +338,34 @@ static int ensure_buffer(uint8_t **buf, int64_t bytes, const char *what)
     return FR_OK;
 }
 
+// The packed buffers of a handle serve its calls one after the other,
+// whatever their streams: a call waits for the last one that used them.
+// Captured work has no place in that order: calls of several generations are
+// the caller's to keep apart there, as with the ping-pong scratch; single
+// generations use no packed buffer under capture, and others than those of
+// several generations elsewhere, so replays disturb none of them.
+bool fr::capturing(cudaStream_t st)
+{
+    cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
+    const bool on = cudaStreamIsCapturing(st, &cs) != cudaSuccess || cs != cudaStreamCaptureStatusNone;
+    if (on) cudaGetLastError();
+    return on;
+}
+
+int fr::packed_enter(fractal *f, cudaStream_t st, bool captured)
+{
+    if (captured) return FR_OK;
+    if (f->packed_done) FR_CUDA(cudaStreamWaitEvent(st, f->packed_done, 0));
+    else FR_CUDA(cudaEventCreateWithFlags(&f->packed_done, cudaEventDisableTiming));
+    return FR_OK;
+}
+
+int fr::packed_leave(fractal *f, cudaStream_t st, bool captured)
+{
+    if (!captured) FR_CUDA(cudaEventRecord(f->packed_done, st));
+    return FR_OK;
+}
+
 // Ping-pong `steps` generations so that the last one lands in `out`: step i
 // (1-based) writes `out` when steps - i is even, the scratch buffer otherwise.
 template <class Launch>
@@ -384,15 +413,16 @@ extern "C" int fractal_step(fractal_t *f, const uint8_t *in, uint8_t *out, int64
         }
         return FR_OK;
     }
-    int rc;
+    // (also where the sliced step takes the call: later calls under capture and
+    // fractal_step_noalloc need the tile kernels' tables and cannot build them)
+    int rc = ensure_step_plan(f);
+    if (rc) return rc;
     if (((f->tile_levels_user < 0 && f->stages_user < 0) || f->sliced_tuned) && !f->test_extra_tx) {
         // (a tile depth or stage count set by the caller asks for the tile kernels)
         bool done = false;
         rc = try_slice_step(f, in, out, steps, birth, survive, st, &done);
         if (rc || done) return rc;
     }
-    rc = ensure_step_plan(f);
-    if (rc) return rc;
     if (steps > 1 && bit3_plan(f)) return launch_bit3_generations(f, in, out, steps, birth, survive, st);
     if (steps > 1) {
         rc = ensure_buffer(&f->scratch, f->cells, "fractal_step: scratch allocation");
@@ -425,6 +455,7 @@ extern "C" int fractal_set_temporal_blocking(fractal_t *f, int generations, int 
             f->tb_levels_user = old_l;
             return rc;
         }
+        if (f->slice.several) keep_generation_buffers(f);
     }
     return FR_OK;
 }

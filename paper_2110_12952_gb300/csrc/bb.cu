@@ -881,15 +881,15 @@ static int run_bb_words(fractal *f, BWArgs a, const uint8_t *in, uint8_t *out, i
 {
     const int sms = f->num_sms, smem = 4 * (a.groups * a.yg * a.pitch + 2);
     const int stage = 2 * 16 * kBwUnits * kBwBlock;
-    bb_pack_kernel<<<(unsigned)std::min<int64_t>(a.ptiles, (int64_t)sms * 6), kBwBlock, stage, st>>>(a, in, f->bb_words[1] + 1);
+    int cur = steps == 1 ? 1 : 2;
+    bb_pack_kernel<<<(unsigned)std::min<int64_t>(a.ptiles, (int64_t)sms * 6), kBwBlock, stage, st>>>(a, in, f->bb_words[cur] + 1);
     FR_CUDA(cudaGetLastError());
     const int grid = (int)std::min<int64_t>(a.tiles, (int64_t)sms * 64);
-    int cur = 0;
-    for (int64_t g = 1; g < steps; ++g, cur ^= 1) {
-        launch_bb_words<DIM, false>(a, grid, 0, f->bb_words[1 + cur] + 1, f->bb_words[2 - cur] + 1, nullptr, st);
+    for (int64_t g = 1; g < steps; ++g, cur ^= 1) {   // (2 and 3 in turn)
+        launch_bb_words<DIM, false>(a, grid, 0, f->bb_words[cur] + 1, f->bb_words[cur ^ 1] + 1, nullptr, st);
         FR_CUDA(cudaGetLastError());
     }
-    launch_bb_words<DIM, true>(a, grid, smem, f->bb_words[1 + cur] + 1, nullptr, out, st);
+    launch_bb_words<DIM, true>(a, grid, smem, f->bb_words[cur] + 1, nullptr, out, st);
     FR_CUDA(cudaGetLastError());
     return FR_OK;
 }
@@ -907,14 +907,15 @@ int try_bb_packed(fractal *f, const uint8_t *in, uint8_t *out, int64_t steps, ui
     a.rows = f->dim == 3 ? (int64_t)n * n : n;
     if (a.rows >= ((int64_t)1 << 31)) return FR_OK;
     a.RP = a.RW + 1;
-    // three arrays: the cells' membership, computed once, and one or two states; a zero word before each
+    // the cells' membership, computed once, and one or two states; a zero word before each
     const size_t bytes = ((size_t)a.rows * a.RP + 1) * sizeof(uint32_t);
-    for (int i = 0; i < (steps > 1 ? 3 : 2); ++i) {
-        if (f->bb_words[i]) continue;
+    const bool captured = capturing(st);
+    // under capture a single generation leaves the packed box alone: its replays may run beside other calls
+    if (captured && steps == 1) return FR_OK;
+    for (int i = 0; i < 4; ++i) {
+        if (f->bb_words[i] || (i > 0 && (steps == 1) != (i == 1))) continue;
         // nothing is allocated under capture, and without the memory the row kernels run as before
-        cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
-        if (cudaStreamIsCapturing(st, &cs) != cudaSuccess || cs != cudaStreamCaptureStatusNone ||
-            cudaMalloc(&f->bb_words[i], bytes) != cudaSuccess) {
+        if (captured || cudaMalloc(&f->bb_words[i], bytes) != cudaSuccess) {
             cudaGetLastError();
             f->bb_words[i] = nullptr;
             return FR_OK;
@@ -927,6 +928,11 @@ int try_bb_packed(fractal *f, const uint8_t *in, uint8_t *out, int64_t steps, ui
             FR_CUDA(cudaGetLastError());
         }
         FR_CUDA(cudaStreamSynchronize(st));   // they serve calls on any stream from here on
+        if (i == 3 && !f->bb_scratch && cudaMalloc(&f->bb_scratch, f->box_cells) != cudaSuccess) {
+            // (the row kernels' scratch, for a later captured call whose buffers are not aligned)
+            cudaGetLastError();
+            f->bb_scratch = nullptr;
+        }
     }
     a.member = f->bb_words[0] + 1;
     a.pseg = (a.RW + kBwSeg - 1) / kBwSeg;
@@ -943,7 +949,9 @@ int try_bb_packed(fractal *f, const uint8_t *in, uint8_t *out, int64_t steps, ui
     a.rwdiv = make_div((uint32_t)std::max(2, a.RW));
     a.ndiv = make_div((uint32_t)n);
     *done = true;
-    return f->dim == 3 ? run_bb_words<3>(f, a, in, out, steps, st) : run_bb_words<2>(f, a, in, out, steps, st);
+    int rc = packed_enter(f, st, captured);
+    if (!rc) rc = f->dim == 3 ? run_bb_words<3>(f, a, in, out, steps, st) : run_bb_words<2>(f, a, in, out, steps, st);
+    return rc ? rc : packed_leave(f, st, captured);
 }
 
 int launch_bb_once(fractal *f, const uint8_t *in, uint8_t *out, uint32_t birth,

@@ -134,7 +134,9 @@ struct fractal {
     fr::BBPlan bb;
     uint8_t *scratch = nullptr;      // k^r bytes, ping-pong for steps > 1
     uint32_t *b3_state[2] = {nullptr, nullptr};  // bit3 plans, steps > 1: bit-packed tile states (ping-pong)
-    uint32_t *bb_words[3] = {nullptr, nullptr, nullptr};   // box steps: membership and packed boxes (ping-pong)
+    // box steps: membership, the packed box of single generations, two of calls of several
+    uint32_t *bb_words[4] = {nullptr, nullptr, nullptr, nullptr};
+    cudaEvent_t packed_done = nullptr;   // after the last work on the packed buffers (slice, bb_words)
     uint8_t *bb_scratch = nullptr;   // n^dim bytes, ping-pong for BB steps > 1
     uint8_t *host_io[2] = {nullptr, nullptr};  // device buffers of run_host
     fr::HostPipe pipe;                          // run_host's chunked pipeline
@@ -175,6 +177,11 @@ inline int64_t cells_above(const fractal *f, int L)
 }
 
 int ensure_step_plan(fractal *f);
+// Around work on the handle's packed buffers: ordered over all streams, except under capture.
+bool capturing(cudaStream_t st);
+int packed_enter(fractal *f, cudaStream_t st, bool captured);
+int packed_leave(fractal *f, cudaStream_t st, bool captured);
+void keep_generation_buffers(fractal *f);
 int rows_preset_of(const fractal *f);   // 0: the carpet, 1: the Vicsek fractal (preset offsets), -1: another
 int ensure_tb_plan(fractal *f);
 void fr_paper_aux_free(fractal *f);

@@ -1171,8 +1171,7 @@ static std::shared_ptr<SliceImage> slice_image(const fractal *f, int L)
 void free_slice_plan(SlicePlan &p)
 {
     cudaFree(p.arena);
-    cudaFree(p.bits[0]);
-    cudaFree(p.bits[1]);
+    for (uint32_t *b : p.bits) cudaFree(b);
     p = SlicePlan();
 }
 
@@ -1261,7 +1260,7 @@ static int launch_resident(const SlicePlan &s, const SliceArgs &a, bool life, co
                            cudaStream_t st)
 {
     ResidentFn fn = resident_fn(s, life);
-    uint32_t *e0 = s.ex[0], *e1 = s.ex[1];
+    uint32_t *e0 = steps == 1 ? s.ex[2] : s.ex[0], *e1 = s.ex[1];   // (one generation writes e0 alone)
     int per_block = s.per_block;
     void *args[] = {(void *)&a, &in, &out, &e0, &e1, &per_block, &steps};
     if (s.grid_resident > 1)
@@ -1383,9 +1382,10 @@ static cudaError_t slice_upload(SliceGeo &p, SliceImage &image, SlicePlan &s, co
         return at;
     };
     const size_t o_tab = take(nb.size() * 2), o_jobs = take(t.jobs.size() * 4), o_xl = take(t.xlist.size() * 2),
-                 o_cells = take(t.cells.size() * 4), o_bar = take(8), o_groups = take(groups.size() * sizeof(SliceGroup)), host = off;
+                 o_cells = take(t.cells.size() * 4), o_bar = take(16), o_groups = take(groups.size() * sizeof(SliceGroup)), host = off;
     const size_t o_nbr = take((size_t)p.NG * p.ND * 32 * sizeof(int32_t)),
-                 exb = s.resident ? (size_t)p.NG * p.XW * 128 : 0, o_ex0 = take(exb), o_ex1 = take(exb);
+                 exb = s.resident ? (size_t)p.NG * p.XW * 128 : 0, o_ex0 = take(exb), o_ex1 = take(exb),
+                 o_ex2 = take(groups.empty() ? exb : 0);
     std::vector<uint8_t> img(host, 0);
     memcpy(img.data() + o_tab, nb.data(), nb.size() * 2);
     memcpy(img.data() + o_jobs, t.jobs.data(), t.jobs.size() * 4);
@@ -1403,6 +1403,7 @@ static cudaError_t slice_upload(SliceGeo &p, SliceImage &image, SlicePlan &s, co
     s.groups = groups.empty() ? nullptr : s.arena + o_groups;
     s.ex[0] = reinterpret_cast<uint32_t *>(s.arena + o_ex0);
     s.ex[1] = reinterpret_cast<uint32_t *>(s.arena + o_ex1);
+    s.ex[2] = reinterpret_cast<uint32_t *>(s.arena + o_ex2);
     return e;
 }
 
@@ -1543,6 +1544,40 @@ static SliceArgs slice_args(const SliceGeo &p, uint32_t birth, uint32_t survive,
     return a;
 }
 
+// Bytes -> packed state, the generations but the last on packed states, the last one to bytes.
+static int run_packed(fractal *f, const SliceArgs &a, bool life, const uint8_t *in, uint8_t *out, int64_t steps, cudaStream_t st)
+{
+    const SlicePlan &s = f->slice;
+    int cur = steps == 1 ? 2 : 0;
+    if (f->dim == 3) slice_pack_kernel<kSliceBlock3><<<s.grid_pack, kSliceBlock3, s.smem_pack, st>>>(a, in, s.bits[cur]);
+    else slice_pack_kernel<kSliceBlock><<<s.grid_pack, kSliceBlock, s.smem_pack, st>>>(a, in, s.bits[cur]);
+    FR_CUDA(cudaGetLastError());
+    int64_t left = steps - 1;   // generations before the one that writes bytes
+    StepFn fn = step_fn(s.geo.D, life, false);
+    while (left > 0) {
+        int gens = (int)std::min<int64_t>(left, 1 << 20);
+        const uint32_t *src = s.bits[cur];
+        uint32_t *dst = s.bits[cur ^ 1];
+        uint8_t *none = nullptr;
+        void *args[] = {(void *)&a, &src, &dst, &none, &gens};
+        if (s.grid_step[life] > 1 && gens > 1)
+            FR_CUDA(cudaLaunchCooperativeKernel((const void *)fn, dim3(s.grid_step[life]), dim3(s.block), args, s.smem_step, st));
+        else
+            FR_CUDA(cudaLaunchKernel((const void *)fn, dim3(s.grid_step[life]), dim3(s.block), args, s.smem_step, st));
+        left -= gens;
+        if (gens & 1) cur ^= 1;
+    }
+    {
+        StepFn fb = step_fn(s.geo.D, life, true);
+        const uint32_t *src = s.bits[cur];
+        uint32_t *none = nullptr;
+        int one = 1;
+        void *args[] = {(void *)&a, &src, &none, &out, &one};
+        FR_CUDA(cudaLaunchKernel((const void *)fb, dim3(s.grid_bytes[life]), dim3(s.block), args, s.smem_bytes, st));
+    }
+    return FR_OK;
+}
+
 int try_slice_step(fractal *f, const uint8_t *in, uint8_t *out, int64_t steps, uint32_t birth, uint32_t survive,
                    cudaStream_t st, bool *done)
 {
@@ -1558,14 +1593,14 @@ int try_slice_step(fractal *f, const uint8_t *in, uint8_t *out, int64_t steps, u
         packed = !res && !(steps == 1 && s.grid_single[0] > 0);
     };
     choose();
-    if (s.state == 0 || (packed && (!s.bits[0] || (steps > 1 && !s.bits[1])))) {
-        // nothing is allocated under capture: the tile kernels run there as before
-        cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
-        if (cudaStreamIsCapturing(st, &cs) != cudaSuccess || cs != cudaStreamCaptureStatusNone) {
-            cudaGetLastError();
-            return FR_OK;
-        }
-        int rc = ensure_status(f);
+    int rc;
+    const bool captured = capturing(st);
+    // under capture nothing is allocated, and a single generation leaves the
+    // packed state alone (its replays may run beside other calls): the tile kernels run there
+    const bool ready = s.state > 0 && (!packed || (steps == 1 ? s.bits[2] != nullptr : s.bits[0] && s.bits[1]));
+    if (captured && (!ready || (steps == 1 && (res || packed)))) return FR_OK;
+    if (!ready) {
+        rc = ensure_status(f);
         if (rc) return rc;
         if (s.state == 0 && build_slice_plan(f, st) != FR_OK) {
             s.state = -1;
@@ -1573,52 +1608,21 @@ int try_slice_step(fractal *f, const uint8_t *in, uint8_t *out, int64_t steps, u
         }
         if (steps == 1 && slice_one_generation_by_tiles(f, s.geo.H)) return FR_OK;
         choose();
-        if (packed && (!slice_buffer(f, 0) || (steps > 1 && !slice_buffer(f, 1)))) return FR_OK;
+        if (packed && !(steps == 1 ? slice_buffer(f, 2) : slice_buffer(f, 0) && slice_buffer(f, 1))) return FR_OK;
     }
     const SliceGeo &p = s.geo;
-    const SliceArgs a = slice_args(p, birth, survive, s.bar, f->status);
+    const SliceArgs a = slice_args(p, birth, survive, steps == 1 ? s.bar + 2 : s.bar, f->status);
     const bool life = slice_life(f, birth, survive);
-    if (res) {
-        const int rc = launch_resident(s, a, life, in, out, steps, st);
-        if (rc) return rc;
-        *done = true;
-        return FR_OK;
-    }
-    if (!packed) {
+    *done = true;
+    s.several |= steps > 1;
+    if (!res && !packed) {
         single_fn(p.D, life)<<<s.grid_single[life], kSliceBlock, s.smem_single, st>>>(a, in, out);
         FR_CUDA(cudaGetLastError());
-        *done = true;
         return FR_OK;
     }
-    if (f->dim == 3) slice_pack_kernel<kSliceBlock3><<<s.grid_pack, kSliceBlock3, s.smem_pack, st>>>(a, in, s.bits[0]);
-    else slice_pack_kernel<kSliceBlock><<<s.grid_pack, kSliceBlock, s.smem_pack, st>>>(a, in, s.bits[0]);
-    FR_CUDA(cudaGetLastError());
-    *done = true;
-    int64_t left = steps - 1;   // generations before the one that writes bytes
-    int cur = 0;
-    StepFn fn = step_fn(p.D, life, false);
-    while (left > 0) {
-        int gens = (int)std::min<int64_t>(left, 1 << 20);
-        const uint32_t *src = s.bits[cur];
-        uint32_t *dst = s.bits[cur ^ 1];
-        uint8_t *none = nullptr;
-        void *args[] = {(void *)&a, &src, &dst, &none, &gens};
-        if (s.grid_step[life] > 1 && gens > 1)
-            FR_CUDA(cudaLaunchCooperativeKernel((const void *)fn, dim3(s.grid_step[life]), dim3(s.block), args, s.smem_step, st));
-        else
-            FR_CUDA(cudaLaunchKernel((const void *)fn, dim3(s.grid_step[life]), dim3(s.block), args, s.smem_step, st));
-        left -= gens;
-        if (gens & 1) cur ^= 1;
-    }
-    {
-        StepFn fb = step_fn(p.D, life, true);
-        const uint32_t *src = s.bits[cur];
-        uint32_t *none = nullptr;
-        int one = 1;
-        void *args[] = {(void *)&a, &src, &none, &out, &one};
-        FR_CUDA(cudaLaunchKernel((const void *)fb, dim3(s.grid_bytes[life]), dim3(s.block), args, s.smem_bytes, st));
-    }
-    return FR_OK;
+    rc = packed_enter(f, st, captured);
+    if (!rc) rc = res ? launch_resident(s, a, life, in, out, steps, st) : run_packed(f, a, life, in, out, steps, st);
+    return rc ? rc : packed_leave(f, st, captured);
 }
 
 // ---------------------------------------------------------------- batches

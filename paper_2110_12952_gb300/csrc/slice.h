@@ -35,6 +35,7 @@ struct SliceGeo {
 };
 
 struct SlicePlan {
+    bool several = false;     // a call of several generations has run
     int state = 0;            // 0: not planned yet, 1: planned, -1: not possible for this fractal
     SliceGeo geo;
     bool resident = false;    // the packed state stays in shared memory: one launch for all generations
@@ -42,11 +43,12 @@ struct SlicePlan {
     int block = 256;          // streaming kernels: threads per block
     int smem_pack = 0, smem_step = 0, smem_bytes = 0, smem_single = 0;
     int grid_pack = 0, grid_step[2] = {0, 0}, grid_bytes[2] = {0, 0}, grid_single[2] = {0, 0};   // [1]: with the constant rule
-    uint32_t *bits[2] = {nullptr, nullptr};   // packed states: NG x KLp words, then the exports, NG x XW x 32
+    // packed states (NG x KLp words, then the exports, NG x XW x 32): two of calls of several generations, one of single ones
+    uint32_t *bits[3] = {nullptr, nullptr, nullptr};
     uint8_t *arena = nullptr;                 // the tables, and:
     uint8_t *groups = nullptr;                // batches: the groups (SliceGroup)
-    uint32_t *ex[2] = {nullptr, nullptr};     // resident kernel: the exports alone
-    uint32_t *bar = nullptr;                  // grid barrier: arrivals, exits
+    uint32_t *ex[3] = {nullptr, nullptr, nullptr};   // resident kernel: the exports alone, likewise
+    uint32_t *bar = nullptr;                  // grid barriers: arrivals, exits; single generations' own behind them
 };
 
 void free_slice_plan(SlicePlan &p);

@@ -1063,6 +1063,21 @@ static int configure_bit3(StepPlan &p, int num_sms)
 // Selector nibble that yields a zero byte (sign of a byte whose msb is 0).
 static constexpr uint32_t kZeroSel = 0x8;
 
+// What the tile kernels need for calls of several generations, for handles
+// that have run such calls in the sliced step and then leave it for the tile
+// kernels: such a call may be captured next, where nothing can be allocated.
+// Without the memory the call itself reports it.
+void keep_generation_buffers(fractal *f)
+{
+    const bool b3 = bit3_plan(f);
+    if (!b3 && !f->scratch && cudaMalloc(&f->scratch, (size_t)f->cells) != cudaSuccess) f->scratch = nullptr;
+    for (int i = 0; b3 && i < 2; ++i)
+        if (!f->b3_state[i] &&
+            cudaMalloc(&f->b3_state[i], (size_t)f->plan.NT * kB3StateWords * sizeof(uint32_t)) != cudaSuccess)
+            f->b3_state[i] = nullptr;
+    cudaGetLastError();
+}
+
 int ensure_step_plan(fractal *f)
 {
     // the plan depends only on the fractal and on these two settings (the
@@ -1289,6 +1304,7 @@ int ensure_step_plan(fractal *f)
     p.built_levels = f->tile_levels_user;
     p.built_stages = f->stages_user;
     f->plan = p;
+    if (f->slice.several) keep_generation_buffers(f);
     return FR_OK;
 }
 

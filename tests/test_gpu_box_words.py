@@ -43,3 +43,23 @@ def test_long_box_rows():
     one = g.bb_step(g.bb_step(x, steps=1), steps=1)
     assert torch.equal(g.bb_step(x, steps=2), one)
     g.close()
+
+
+@pytest.mark.parametrize("name,r,steps", [("menger", 5, 1), ("menger", 5, 3), ("carpet", 6, 2)])
+def test_one_handle_on_two_streams(name, r, steps):
+    # calls of one handle on streams of their own share its packed boxes; they take turns
+    from paper_2110_12952_gb300 import Fractal
+    g = Fractal.from_family(W.FAMILIES[name], r)
+    rule = W.MENGER_B5S45 if g.dim == 3 else W.LIFE_B3S23
+    x = [torch.empty(g.box_cells, dtype=torch.uint8, device="cuda").bernoulli_(p) for p in (0.2, 0.5)]
+    want = [g.bb_step(v, steps=steps, rule=rule).clone() for v in x]
+    streams = [torch.cuda.Stream(), torch.cuda.Stream()]
+    out = [[torch.empty_like(x[0]) for _ in range(6)] for _ in range(2)]
+    torch.cuda.synchronize()
+    for i in range(6):
+        for j in range(2):
+            with torch.cuda.stream(streams[j]):
+                g.bb_step(x[j], out=out[j][i], steps=steps, rule=rule)
+    torch.cuda.synchronize()
+    assert all(torch.equal(y, want[j]) for j in range(2) for y in out[j])
+    g.close()

@@ -132,3 +132,61 @@ def test_sliced_menger_single_generations():
     assert torch.equal(g.step(x, steps=3), tiles.step(tiles.step(one, steps=1), steps=1))
     g.close()
     tiles.close()
+
+
+@pytest.mark.parametrize("name,r,steps", [("carpet", 7, 4), ("carpet", 8, 1), ("h_fractal", 8, 1), ("triangle", 16, 3), ("menger", 6, 1)])
+def test_one_handle_on_two_streams(name, r, steps):
+    # calls of one handle on streams of their own share its packed words; they take turns
+    fam = W.FAMILIES[name]
+    from paper_2110_12952_gb300 import Fractal
+    g, ref = Fractal.from_family(fam, r), Fractal.from_family(fam, r)
+    rule = W.MENGER_B5S45 if fam.dim == 3 else W.LIFE_B3S23
+    x = [g.init_bernoulli(seed, 0.4) for seed in (1, 2)]
+    want = [ref.step(v, steps=steps, rule=rule).clone() for v in x]
+    streams = [torch.cuda.Stream(), torch.cuda.Stream()]
+    out = [[torch.empty_like(x[0]) for _ in range(6)] for _ in range(2)]
+    torch.cuda.synchronize()
+    for i in range(6):
+        for j in range(2):
+            with torch.cuda.stream(streams[j]):
+                g.step(x[j], out=out[j][i], steps=steps, rule=rule)
+    torch.cuda.synchronize()
+    for j in range(2):
+        for y in out[j]:
+            assert torch.equal(y, want[j])
+    g.check()
+    g.close()
+    ref.close()
+
+
+@pytest.mark.parametrize("name,r", [("triangle", 8), ("carpet", 6), ("vicsek", 6), ("menger", 4)])
+def test_sliced_call_readies_the_handle(name, r):
+    # what a first step has always made possible: a captured call of another step count, the allocation-free step,
+    # and a captured call once the handle has been set to the tile kernels
+    fam = W.FAMILIES[name]
+    g, o = pair(fam, r)
+    rule = W.MENGER_B5S45 if fam.dim == 3 else W.LIFE_B3S23
+    v = o.init_bernoulli(7, 0.4)
+    x = torch.from_numpy(v).cuda()
+    g.step(x, steps=5, rule=rule)
+    want = {n: o.step(v, rule=oracle.Rule(*rule), steps=n) for n in (1, 3)}
+    y = torch.empty_like(x)
+    assert g._lib.fractal_step_noalloc(g._h, x.data_ptr(), y.data_ptr(), 3, rule[0], rule[1], 0) == 0
+    torch.cuda.synchronize()
+    assert np.array_equal(y.cpu().numpy(), want[3])
+    z = torch.empty_like(x)
+    for n in (1, 3, -3):
+        if n < 0:
+            g.tile_levels = 2
+            assert g.tile_levels == 2
+        torch.cuda.synchronize()
+        graph = torch.cuda.CUDAGraph()
+        with torch.cuda.graph(graph):
+            g.step(x, out=z, steps=abs(n), rule=rule)
+        z.zero_()
+        graph.replay()
+        torch.cuda.synchronize()
+        assert np.array_equal(z.cpu().numpy(), want[abs(n)]), n
+        del graph
+    g.check()
+    g.close()

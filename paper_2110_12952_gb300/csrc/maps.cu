@@ -60,6 +60,7 @@ constexpr int kMapGroups = 16;      // most groups of levels
 constexpr int kMapBlock = 512;
 constexpr int kMapBlocksPerSM = 4;
 constexpr int64_t kMapLong = 1 << 16;   // arrays from here on go through tables
+constexpr int64_t kMapBuild = 8;        // a block's points take at least this many times the digit steps of its tables
 
 // lambda through tables: entry i holds the coordinates of i over m levels
 // (16 bits each in 2D, 10 in 3D); omega's base-k^m digits pick the entries.
@@ -284,13 +285,30 @@ __global__ void __launch_bounds__(kMapBlock) nu_tab_kernel(FracDev F, NuTab N, i
     }
 }
 
-static bool lambda_tab(const fractal *f, LambdaTab *L)
+static int map_grid(const fractal *f, int64_t count)
+{
+    return (int)std::min<int64_t>((int64_t)f->num_sms * kMapBlocksPerSM, (count + kMapBlock - 1) / kMapBlock);
+}
+
+// Most entries x levels of a block's tables: building an entry costs what a
+// point of that many levels costs in the digit loops.  504,289 points of the
+// triangle at r = 11 (lambda, nu, compact coordinate in turn, one pass): digit
+// loops 48 us, largest tables at any length 81 us; by this rule 8 us a call
+// against 14.5, 12.4 and 14.4.  At 3 instead of 8 arrays of 2 and 8 million
+// points take up to 60 % longer; at 24 some of them take up to 30 % less and
+// others (Menger r = 7, compact coordinate) 30 % more.
+static int64_t map_budget(const fractal *f, int64_t count)
+{
+    return count / map_grid(f, count) * f->r / kMapBuild;
+}
+
+static bool lambda_tab(const fractal *f, int64_t count, LambdaTab *L)
 {
     if (f->mixed || f->k < 2 || f->r < 1) return false;
-    const int64_t most = f->dim == 2 ? 65536 : 1024;
+    const int64_t most = f->dim == 2 ? 65536 : 1024, budget = map_budget(f, count);
     int64_t n = f->k, sm = f->s;
     int m = 1;
-    while (m < f->r && n * f->k <= kMapTable && sm * f->s <= most) {
+    while (m < f->r && n * f->k <= kMapTable && sm * f->s <= most && n * f->k * (m + 1) <= budget) {
         n *= f->k;
         sm *= f->s;
         ++m;
@@ -315,11 +333,12 @@ static bool lambda_tab(const fractal *f, LambdaTab *L)
     return true;
 }
 
-static bool nu_tab(const fractal *f, bool compact, NuTab *N)
+static bool nu_tab(const fractal *f, bool compact, int64_t count, NuTab *N)
 {
     if (f->mixed || f->r < 1) return false;
     const int dim = f->dim;
     // components are stored in 16 or 10 bits, nu in 31
+    const int64_t budget = map_budget(f, count);
     const int64_t most = !compact ? (int64_t)1 << 31 : (dim == 2 ? 65535 : 1024);
     int64_t block = 1;
     for (int i = 0; i < dim; ++i) block *= f->s;
@@ -336,7 +355,7 @@ static bool nu_tab(const fractal *f, bool compact, NuTab *N)
         for (int i = 0; i < (compact ? (t + dim - 1) / dim : t); ++i) kc = kc > most ? kc : kc * f->k;
         const int ph = !compact || t % dim == 0 ? 1 : dim;   // (dim is 2 or 3: prime)
         if (nt > kMapTable) break;
-        if (kc > most || nt * ph > kMapTable) continue;
+        if (kc > most || nt * ph > kMapTable || (m > 0 && nt * ph * t > budget)) continue;
         m = t;
         n = nt;
         sm = st;
@@ -368,11 +387,6 @@ static bool nu_tab(const fractal *f, bool compact, NuTab *N)
         N->scale[g] = (int64_t)scale;
     }
     return true;
-}
-
-static int map_grid(const fractal *f, int64_t count)
-{
-    return (int)std::min<int64_t>((int64_t)f->num_sms * kMapBlocksPerSM, (count + kMapBlock - 1) / kMapBlock);
 }
 
 template <bool COMPACT>
@@ -646,7 +660,7 @@ extern "C" int fractal_lambda(const fractal_t *f, const int64_t *omega, int64_t 
     if (count < 0) return fail_null("fractal_lambda (count < 0)");
     if (count == 0) return FR_OK;
     LambdaTab L;
-    if (count >= kMapLong && lambda_tab(f, &L)) {
+    if (count >= kMapLong && lambda_tab(f, count, &L)) {
         const bool vec = ((uintptr_t)omega & 15) == 0 && ((uintptr_t)coords & 15) == 0;
         const int grid = map_grid(f, count);
         cudaStream_t st = (cudaStream_t)stream;
@@ -670,7 +684,7 @@ extern "C" int fractal_nu(const fractal_t *f, const int32_t *coords, int64_t cou
     if (count < 0) return fail_null("fractal_nu (count < 0)");
     if (count == 0) return FR_OK;
     NuTab N;
-    if (count >= kMapLong && nu_tab(f, false, &N)) return launch_nu_tab<false>(f, N, coords, count, omega, (cudaStream_t)stream);
+    if (count >= kMapLong && nu_tab(f, false, count, &N)) return launch_nu_tab<false>(f, N, coords, count, omega, (cudaStream_t)stream);
     nu_kernel<<<grid_for(count, 256, f->num_sms), 256, 0, (cudaStream_t)stream>>>(
         f->dev, (int32_t)f->side, coords, count, omega);
     FR_CUDA(cudaGetLastError());
@@ -684,7 +698,7 @@ extern "C" int fractal_nu2d(const fractal_t *f, const int32_t *coords, int64_t c
     if (count < 0) return fail_null("fractal_nu2d (count < 0)");
     if (count == 0) return FR_OK;
     NuTab N;
-    if (count >= kMapLong && nu_tab(f, true, &N)) return launch_nu_tab<true>(f, N, coords, count, out, (cudaStream_t)stream);
+    if (count >= kMapLong && nu_tab(f, true, count, &N)) return launch_nu_tab<true>(f, N, coords, count, out, (cudaStream_t)stream);
     nu2d_kernel<<<grid_for(count, 256, f->num_sms), 256, 0, (cudaStream_t)stream>>>(
         f->dev, (int32_t)f->side, coords, count, out);
     FR_CUDA(cudaGetLastError());

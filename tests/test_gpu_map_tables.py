@@ -47,6 +47,11 @@ def test_long_map_arrays(name, r, skew):
     n2 = torch.empty((N + skew) * fam.dim, dtype=torch.int64, device="cuda")[skew * fam.dim:].view(N, fam.dim)
     assert np.array_equal(g.nu(cb, out=nu).cpu().numpy(), o.nu(c))
     assert np.array_equal(g.nu2d(cb, out=n2).cpu().numpy(), o.nu2d(c))
+    # the same points many times over: the tables grow with the array
+    many = 200
+    for fn, x, y in ((g.lam, buf, out), (g.nu, cb, nu), (g.nu2d, cb, n2)):
+        big = fn(x.repeat(*((many,) + (1,) * (x.dim() - 1))))
+        assert bool((big.view(many, *y.shape) == y).all())
     g.close()
 
 

@@ -272,7 +272,7 @@ extern "C" int fractal_set_tile_levels(fractal_t *f, int levels)
         return fail(FR_EINVAL, "fractal_set_tile_levels: levels must be -1 or in [0, r]");
     if (levels != f->tile_levels_user && f->server_refs.load() > 0)
         return fail(FR_EBUSY, "fractal_set_tile_levels: a server still holds requests on this handle");
-    f->sliced_tuned = false;
+    f->tuned = f->sliced_tuned = false;
     if (levels != f->tile_levels_user) {
         f->tile_levels_user = levels;
         cudaDeviceSynchronize();
@@ -289,7 +289,7 @@ extern "C" int fractal_set_pipeline_stages(fractal_t *f, int stages)
         return fail(FR_EINVAL, "fractal_set_pipeline_stages: stages must be -1 or in [2, 4]");
     if (stages != f->stages_user && f->server_refs.load() > 0)
         return fail(FR_EBUSY, "fractal_set_pipeline_stages: a server still holds requests on this handle");
-    f->sliced_tuned = false;
+    f->tuned = f->sliced_tuned = false;
     if (stages != f->stages_user) {
         f->stages_user = stages;
         cudaDeviceSynchronize();
@@ -417,8 +417,7 @@ extern "C" int fractal_step(fractal_t *f, const uint8_t *in, uint8_t *out, int64
     // fractal_step_noalloc need the tile kernels' tables and cannot build them)
     int rc = ensure_step_plan(f);
     if (rc) return rc;
-    if (((f->tile_levels_user < 0 && f->stages_user < 0) || f->sliced_tuned) && !f->test_extra_tx) {
-        // (a tile depth or stage count set by the caller asks for the tile kernels)
+    if (slice_settings(f, steps) && !f->test_extra_tx) {
         bool done = false;
         rc = try_slice_step(f, in, out, steps, birth, survive, st, &done);
         if (rc || done) return rc;

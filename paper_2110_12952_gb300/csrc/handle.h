@@ -145,8 +145,9 @@ struct fractal {
     int tb_gens = 0;                 // temporal blocking: generations per pass (0 = off)
     int tb_levels_user = -1;         // its tile depth (-1 = automatic)
     fr::TbPlan tb;
-    fr::SlicePlan slice;             // the bit-sliced step of 2D fractals
-    bool sliced_tuned = false;       // the autotuner found it faster than the tile depth it set
+    fr::SlicePlan slice;             // the bit-sliced step
+    bool tuned = false;              // the tile depth and stages are the autotuner's (it times single generations) ...
+    bool sliced_tuned = false;       // ... which found the sliced step faster still
     void *paper_aux = nullptr;       // the paper's approaches (paper_kernels.cu): geometry and scratch
     // a different transition table per level (fractal_create_mixed); then
     // `offsets` holds the levels' tables one after the other
@@ -160,6 +161,14 @@ struct fractal {
 };
 
 namespace fr {
+
+// Whether the handle's settings leave the call to the sliced step's rules: a
+// tile depth or stage count set by the caller asks for the tile kernels, one
+// set by the autotuner speaks for single generations only.
+inline bool slice_settings(const fractal *f, int64_t steps)
+{
+    return (f->tile_levels_user < 0 && f->stages_user < 0) || (f->tuned && (steps > 1 || f->sliced_tuned));
+}
 
 // cells of a level-L subtree (product of the replica counts of levels
 // 0 .. L-1) and subtrees of level L (levels L .. r-1)

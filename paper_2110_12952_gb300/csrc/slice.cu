@@ -522,8 +522,9 @@ __device__ __forceinline__ uint32_t slice_next(const SliceArgs &a, const SliceRo
 
 // In 3D a group's neighbour table (Menger: 8000 cells x 40 bytes) comes from
 // L2 chunk by chunk; latency and issue slots bound it.  Menger r = 7 (1.28e9
-// cells): one generation with packing 1.61 -> 0.72 ms, further ones 0.69 ->
-// 0.31 ms each; r = 6 (250 groups, one or two per SM) 39 -> 20.4 us.
+// cells): one generation with packing 1.61 -> 0.70 ms, further ones 0.69 ->
+// 0.31 ms each; r = 6 (250 groups, one or two per SM), 50 generations 1.96 ->
+// 1.07 ms.
 
 // `gens` generations of a packed state, blocks walking the groups; between
 // generations the launch's blocks meet at a grid barrier (a cooperative
@@ -620,7 +621,7 @@ slice_step_kernel(SliceArgs a, const uint32_t *src, uint32_t *dst, uint8_t *__re
 // those cells are read as bytes from the neighbouring tiles (lane t follows
 // tile 32 g + t, a ballot makes the word), the rest as in the two-pass
 // kernels.  The bit strings of the old and of the new state share a place.
-// Issue-bound (60 % of the slots, HBM at 79 %): triangle r = 20 in 1.31 ms
+// Issue-bound (67 % of the slots, HBM at 80 %): triangle r = 20 in 1.29 ms
 // against 1.49 ms of the tap kernel and 1.45 ms of the two-pass kernels.
 // Tiles of 2187 cells: with 729 it took 1.57 ms (a group's fixed work, about
 // 1600 instructions, per fewer cells), with 6561 1.72 ms (the neighbour table
@@ -685,8 +686,9 @@ slice_single_kernel(SliceArgs a, const uint8_t *__restrict__ in, uint8_t *__rest
 // well: with so much of it in use little is left of L1.  ONE: a single block;
 // its exports stay in shared memory too.  Bound by issue slots and, for small
 // states, by the barrier and the chain of latencies around it.  Microseconds
-// per generation, byte-wise tile kernels -> here: triangle r = 8 6.1 -> 0.5,
-// r = 16 23 -> 6.3, carpet r = 9 96 -> 14, H-fractal r = 9 107 -> 8.
+// per call, byte-wise tile kernels -> here: triangle r = 8, 100 generations
+// 614 -> 52, r = 16, 50 generations 1151 -> 331, carpet r = 9, 20 generations
+// 1950 -> 328, H-fractal r = 9, 4 generations 426 -> 52.
 
 // A block's items (item j of its group q, n per group) dealt to its warps, a
 // run of `rounds` items each; past the last item a warp repeats it.
@@ -1664,8 +1666,7 @@ int run_slice_batch(const SliceBatch *b, cudaStream_t st)
 
 bool slice_batch_takes(const fractal *f, int64_t steps)
 {
-    return f->dim == 2 && slice_fractal_ok(f) && steps >= 2 && steps < (1 << 30) && f->cells <= kSliceBatchCells &&
-           ((f->tile_levels_user < 0 && f->stages_user < 0) || f->sliced_tuned);
+    return f->dim == 2 && slice_fractal_ok(f) && steps >= 2 && steps < (1 << 30) && f->cells <= kSliceBatchCells && slice_settings(f, steps);
 }
 
 // Groups that fit one launch at this tile depth (0: none), and its cycles per generation.

@@ -190,3 +190,15 @@ def test_sliced_call_readies_the_handle(name, r):
         del graph
     g.check()
     g.close()
+
+
+def test_several_generations_of_an_autotuned_handle():
+    # the autotuner's tile depth is for single generations; calls of several go by the rules of other handles
+    fam = W.FAMILIES["candy"]
+    g, o = pair(fam, 4)
+    v = o.init_bernoulli(9, 0.4)
+    x = torch.from_numpy(v).cuda()
+    g.autotune(x)
+    for n in (1, 4):
+        assert np.array_equal(g.step(x, steps=n).cpu().numpy(), o.step(v, steps=n))
+    g.close()

@@ -307,7 +307,7 @@ def run_ours(args, rank, world, dist):
         g.tile_levels = args.tile_levels
         g.pipeline_stages = args.stages
     else:
-        g.autotune(a, b)   # picks the tile depth; untimed
+        g.autotune(a, b)   # picks the tile depth or the bit-sliced step; untimed
     bufs = [a, b]
     cur = [0]
 
@@ -351,10 +351,11 @@ def run_ours(args, rank, world, dist):
     plan = g.plan_info()
     roof = {"bound": "hbm", "achieved": achieved, "peak": peak, "unit": "GB/s", "frac": achieved / peak,
             "traffic": traffic_per_launch(workload),
-            "kernel": f"step_tma_kernel<2,{plan['policy']},false> ({plan['policy_name']} policy)",
+            "kernel": "the autotuner's choice: slice_single_kernel (bit-sliced, one pass), or the tile plan's "
+                      f"step_tma_kernel<2,{plan['policy']},false> ({plan['policy_name']} policy) where that is faster",
             "algorithmic_bytes_per_launch": alg_bytes, "peak_source": peak_src,
-            "tile_levels": plan["tile_levels"], "launch": {k: plan[k] for k in
-                                                           ("block", "grid", "smem_bytes", "stages", "blocks_per_sm")}}
+            "tile_levels": plan["tile_levels"], "tile_launch": {k: plan[k] for k in
+                                                                ("block", "grid", "smem_bytes", "stages", "blocks_per_sm")}}
 
     extra = {}
     # end-to-end through the public API from pinned host buffers
@@ -669,7 +670,7 @@ def batched_compare(args, W):
            "batched_launches_in_graph": launches, "graph_launches_per_run": 1,
            "plain_ms": plain_ms, "plain_wall_s": plain_wall,
            "plain_updates_per_s": updates / (plain_ms / 1e3),
-           "plain_launches": sum(i.steps for i in mix),
+           "plain_calls": len(mix),
            "speedup_batched_vs_plain": plain_ms / best_b,
            "batched_equals_plain_on_sample": bool(same)}
     batch.close()

@@ -153,7 +153,22 @@ int fractal_init_bernoulli(const fractal_t *f, uint8_t *state_dev,
  * 4 at tile depth 3, fractal_plan_info policy 15), steps > 1 keep the state
  * bit-packed between the first and the last generation instead, in two
  * buffers of 3136 bytes per level-3 tile (k^(r-3) tiles), likewise allocated
- * on first need and kept until fractal_destroy; the result is the same. */
+ * on first need and kept until fractal_destroy; the result is the same.
+ *
+ * Unless the handle has a tile depth or stage count of its own, fractals with
+ * one transition table (r >= 1, k >= 2) may take the bit-sliced step instead,
+ * which packs the cells into bits (32 tiles to a word): calls of several
+ * generations, and single ones of larger states where it is faster.  It keeps
+ * its tables (a few MB at most for the benchmark fractals, 32 bytes per tile
+ * in 2D, 104 in 3D), and where the packed state does not stay on the chip one
+ * or two packed states of about k^r / 8 bytes and the tiles' border cells, all
+ * allocated on first need and kept until fractal_destroy; the ping-pong
+ * scratch is then not allocated.  Without that memory, and under capture
+ * before it exists, the byte-wise step above runs.  Calls of one handle on
+ * several streams take turns at the packed states; captured ones are outside
+ * that order: replays of calls of several generations must not overlap other
+ * calls of several generations of the handle (nor may they share the scratch).
+ * A single generation under capture uses no packed state. */
 int fractal_step(fractal_t *f, const uint8_t *in_dev, uint8_t *out_dev,
                  int64_t steps, uint32_t birth_mask, uint32_t survive_mask,
                  void *stream);
@@ -187,7 +202,11 @@ int fractal_step_noalloc(fractal_t *f, const uint8_t *in_dev, uint8_t *out_dev,
 /* The bounding-box approach (Sec. 4, "BB"): the same rule applied to every
  * cell of the n^dim box.  Cells off the fractal count as dead whatever their
  * byte and are written as 0.  box_in_dev / box_out_dev: n^dim bytes each,
- * not overlapping.  Scratch for steps > 1 as in fractal_step (n^dim bytes). */
+ * not overlapping.  Scratch for steps > 1 as in fractal_step (n^dim bytes).
+ * Boxes of side >= 32 in 16-byte aligned buffers are packed into bits for
+ * steps > 1, and in 3D for steps = 1 as well: the cells' membership and one
+ * or two packed boxes (n^dim / 8 bytes each), allocated on first need, with
+ * the rules on streams, capture and missing memory of fractal_step. */
 int fractal_bb_step(fractal_t *f, const uint8_t *box_in_dev, uint8_t *box_out_dev,
                     int64_t steps, uint32_t birth_mask, uint32_t survive_mask,
                     void *stream);
@@ -285,7 +304,9 @@ int fractal_plan_info(const fractal_t *f, int32_t *info, int n);
 /* Autotuner of fractal_step: times one generation from in_dev into out_dev
  * (both k^r bytes; out_dev is overwritten) for each candidate tile depth
  * (the deepest whose shared-memory layout fits, and the three below) with
- * 2, 3 and 4 pipeline stages, keeps the fastest plan for this handle and
+ * 2, 3 and 4 pipeline stages, and the bit-sliced step (which then goes before
+ * the tile plan it was compared with; calls of several generations take it
+ * by the rules of handles without an autotuned depth), keeps the fastest for this handle and
  * remembers it for every later handle of the same fractal and level on the
  * same GPU model in this process.  Waits for
  * `stream`.  *levels (if not NULL) receives the chosen depth. */
@@ -302,7 +323,10 @@ int fractal_autotune(fractal_t *f, const uint8_t *in_dev, uint8_t *out_dev,
  * fractal_step(handle, in, out, steps, rule) would, but with one kernel
  * launch per generation for all instances that share a fractal and tile
  * depth, and the whole run captured into one CUDA graph that is launched on
- * `stream` (asynchronously).  The graph is kept and replayed by later runs
+ * `stream` (asynchronously).  Instances of 2D fractals with one transition
+ * table, 2 generations or more and at most 60 million cells run bit-sliced
+ * instead, in one launch for all generations of as many instances as fit on
+ * the chip together.  The graph is kept and replayed by later runs
  * until instances are added or cleared.  Buffers stay owned by the caller and
  * must stay valid while a run is in flight; the batch owns a device arena for
  * its tables and for one k^r-byte ping-pong buffer per instance with

@@ -263,7 +263,7 @@ class Fractal:
 
     def autotune(self, state: torch.Tensor, out: torch.Tensor | None = None, rule=None,
                  stream=None) -> int:
-        """Pick the fastest tile depth on these buffers (``fractal_autotune``);
+        """Pick the fastest tile depth, or the bit-sliced step, on these buffers (``fractal_autotune``);
         ``out`` is overwritten.  Returns the chosen depth."""
         birth, survive = rule if rule is not None else self.default_rule()
         out = out if out is not None else torch.empty_like(state)

@@ -59,7 +59,8 @@ constexpr int kMapTable = 4096;     // most entries of a table
 constexpr int kMapGroups = 16;      // most groups of levels
 constexpr int kMapBlock = 512;
 constexpr int kMapBlocksPerSM = 4;
-constexpr int64_t kMapLong = 1 << 16;   // arrays from here on go through tables
+constexpr int64_t kMapLong = 20000000;  // points x levels x replicas from which arrays go through tables
+constexpr int64_t kViewLong = 1 << 16;  // cells from which the box views go by tiles
 constexpr int64_t kMapBuild = 8;        // a block's points take at least this many times the digit steps of its tables
 
 // lambda through tables: entry i holds the coordinates of i over m levels
@@ -285,6 +286,15 @@ __global__ void __launch_bounds__(kMapBlock) nu_tab_kernel(FracDev F, NuTab N, i
     }
 }
 
+// Whether tables pay for an array: the digit loops take longer with more
+// levels and, their constant loads being serialised, with more replicas.  The
+// triangle at r = 11, 504,289 points, lambda, nu and compact coordinate with a
+// cold cache: digit loops 48 us, tables 53; at r = 20 with a warm one 64 and 25.
+static bool map_long(const fractal *f, int64_t count)
+{
+    return (double)count * f->r * f->k >= (double)kMapLong;
+}
+
 static int map_grid(const fractal *f, int64_t count)
 {
     return (int)std::min<int64_t>((int64_t)f->num_sms * kMapBlocksPerSM, (count + kMapBlock - 1) / kMapBlock);
@@ -292,11 +302,10 @@ static int map_grid(const fractal *f, int64_t count)
 
 // Most entries x levels of a block's tables: building an entry costs what a
 // point of that many levels costs in the digit loops.  504,289 points of the
-// triangle at r = 11 (lambda, nu, compact coordinate in turn, one pass): digit
-// loops 48 us, largest tables at any length 81 us; by this rule 8 us a call
-// against 14.5, 12.4 and 14.4.  At 3 instead of 8 arrays of 2 and 8 million
-// points take up to 60 % longer; at 24 some of them take up to 30 % less and
-// others (Menger r = 7, compact coordinate) 30 % more.
+// triangle at r = 11, cold: largest tables at any length 81 us, by this rule
+// 53.  At 3 instead of 8 arrays of 2 and 8 million points take up to 60 %
+// longer; at 24 some take up to 30 % less and others (Menger r = 7, compact
+// coordinate) 30 % more.
 static int64_t map_budget(const fractal *f, int64_t count)
 {
     return count / map_grid(f, count) * f->r / kMapBuild;
@@ -623,7 +632,7 @@ using namespace fr;
 // where the state has as many (of 128 cells or more).
 static int box_tile_levels(const fractal *f)
 {
-    if (f->mixed || f->k < 2 || f->cells < kMapLong) return 0;
+    if (f->mixed || f->k < 2 || f->cells < kViewLong) return 0;
     int m = 0;
     int64_t kl = f->k, sm = f->s;
     for (; m < f->r && kl <= kMapTable; ++m, kl *= f->k, sm *= f->s) {
@@ -660,7 +669,7 @@ extern "C" int fractal_lambda(const fractal_t *f, const int64_t *omega, int64_t 
     if (count < 0) return fail_null("fractal_lambda (count < 0)");
     if (count == 0) return FR_OK;
     LambdaTab L;
-    if (count >= kMapLong && lambda_tab(f, count, &L)) {
+    if (map_long(f, count) && lambda_tab(f, count, &L)) {
         const bool vec = ((uintptr_t)omega & 15) == 0 && ((uintptr_t)coords & 15) == 0;
         const int grid = map_grid(f, count);
         cudaStream_t st = (cudaStream_t)stream;
@@ -684,7 +693,7 @@ extern "C" int fractal_nu(const fractal_t *f, const int32_t *coords, int64_t cou
     if (count < 0) return fail_null("fractal_nu (count < 0)");
     if (count == 0) return FR_OK;
     NuTab N;
-    if (count >= kMapLong && nu_tab(f, false, count, &N)) return launch_nu_tab<false>(f, N, coords, count, omega, (cudaStream_t)stream);
+    if (map_long(f, count) && nu_tab(f, false, count, &N)) return launch_nu_tab<false>(f, N, coords, count, omega, (cudaStream_t)stream);
     nu_kernel<<<grid_for(count, 256, f->num_sms), 256, 0, (cudaStream_t)stream>>>(
         f->dev, (int32_t)f->side, coords, count, omega);
     FR_CUDA(cudaGetLastError());
@@ -698,7 +707,7 @@ extern "C" int fractal_nu2d(const fractal_t *f, const int32_t *coords, int64_t c
     if (count < 0) return fail_null("fractal_nu2d (count < 0)");
     if (count == 0) return FR_OK;
     NuTab N;
-    if (count >= kMapLong && nu_tab(f, true, count, &N)) return launch_nu_tab<true>(f, N, coords, count, out, (cudaStream_t)stream);
+    if (map_long(f, count) && nu_tab(f, true, count, &N)) return launch_nu_tab<true>(f, N, coords, count, out, (cudaStream_t)stream);
     nu2d_kernel<<<grid_for(count, 256, f->num_sms), 256, 0, (cudaStream_t)stream>>>(
         f->dev, (int32_t)f->side, coords, count, out);
     FR_CUDA(cudaGetLastError());

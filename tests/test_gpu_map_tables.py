@@ -12,7 +12,7 @@ from paper_2110_12952_gb300 import workloads as W
 
 pytestmark = pytest.mark.gpu
 
-N = 66001   # from 2^16 points on the maps use tables
+N = 1000001   # from 2e7 points x levels x replicas on the maps use tables
 CASES = [("triangle", 1), ("triangle", 7), ("triangle", 13), ("triangle", 20), ("carpet", 3), ("carpet", 9), ("vicsek", 4),
          ("vicsek", 12), ("menger", 2), ("menger", 5), ("menger", 7), ("candy", 7), ("x_fractal", 11), ("full_square", 15),
          ("cantor_set", 19)]
@@ -48,7 +48,7 @@ def test_long_map_arrays(name, r, skew):
     assert np.array_equal(g.nu(cb, out=nu).cpu().numpy(), o.nu(c))
     assert np.array_equal(g.nu2d(cb, out=n2).cpu().numpy(), o.nu2d(c))
     # the same points many times over: the tables grow with the array
-    many = 200
+    many = 13
     for fn, x, y in ((g.lam, buf, out), (g.nu, cb, nu), (g.nu2d, cb, n2)):
         big = fn(x.repeat(*((many,) + (1,) * (x.dim() - 1))))
         assert bool((big.view(many, *y.shape) == y).all())

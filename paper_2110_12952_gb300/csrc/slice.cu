@@ -1371,9 +1371,12 @@ static int slice_levels(const fractal *f, SlicePlan *plan, std::shared_ptr<Slice
 }
 
 // One allocation: the tables (copied from the host in one piece), the grid
-// barrier's zeros, the neighbouring tiles and the resident exports.
+// barrier's zeros, the neighbouring tiles and the resident exports.  `img` is
+// that piece: the copy may read it until `st` has been waited for (a runtime
+// that reads pageable memory in place does not stage it first), so the caller
+// keeps it until then.
 static cudaError_t slice_upload(SliceGeo &p, SliceImage &image, SlicePlan &s, const std::vector<SliceGroup> &groups,
-                                cudaStream_t st)
+                                std::vector<uint8_t> &img, cudaStream_t st)
 {
     const SliceTables &t = image.t;
     const std::vector<uint16_t> &nb = image.neighbours(p.D);
@@ -1388,7 +1391,7 @@ static cudaError_t slice_upload(SliceGeo &p, SliceImage &image, SlicePlan &s, co
     const size_t o_nbr = take((size_t)p.NG * p.ND * 32 * sizeof(int32_t)),
                  exb = s.resident ? (size_t)p.NG * p.XW * 128 : 0, o_ex0 = take(exb), o_ex1 = take(exb),
                  o_ex2 = take(groups.empty() ? exb : 0);
-    std::vector<uint8_t> img(host, 0);
+    img.assign(host, 0);
     memcpy(img.data() + o_tab, nb.data(), nb.size() * 2);
     memcpy(img.data() + o_jobs, t.jobs.data(), t.jobs.size() * 4);
     memcpy(img.data() + o_xl, t.xlist.data(), t.xlist.size() * 2);
@@ -1421,7 +1424,8 @@ static int build_slice_plan(fractal *f, cudaStream_t st)
     s.smem_single = ring + 4 * (p.AW + std::max(string_words(p), 32 * p.RP + 1));
     s.smem_step = 4 * arrays * p.AW;
     s.smem_bytes = 4 * (arrays * p.AW + 32 * p.RP + 1);
-    cudaError_t e = slice_upload(p, *img, s, {}, st);
+    std::vector<uint8_t> host;
+    cudaError_t e = slice_upload(p, *img, s, {}, host, st);
     if (e == cudaSuccess) {
         const int64_t blocks = std::min<int64_t>((32 * p.NG + 255) / 256, (int64_t)f->num_sms * 16);
         if (f->dim == 3)
@@ -1429,7 +1433,8 @@ static int build_slice_plan(fractal *f, cudaStream_t st)
         else
             slice_nbr_kernel<2><<<(unsigned)blocks, 256, 0, st>>>(f->dev, p.NT, p.NG, f->r - p.L, (int32_t)pw(f->s, f->r - p.L), nullptr, p.nbr);
         e = cudaGetLastError();
-        if (e == cudaSuccess) e = cudaStreamSynchronize(st);   // the tables serve calls on any stream from here on
+        const cudaError_t landed = cudaStreamSynchronize(st);   // the tables serve calls on any stream from here on
+        if (e == cudaSuccess) e = landed;
     }
     // shared memory and grids
     int per_sm = 0;
@@ -1772,13 +1777,15 @@ int build_slice_batch(const std::vector<SliceBatchItem> &items, uint32_t birth, 
             p.NT = 32 * p.NG;
             double c = 0;
             cudaError_t e = slice_resident_shape(p, rep->num_sms, true, &l.plan, &c) ? cudaSuccess : cudaErrorInvalidConfiguration;
-            if (e == cudaSuccess) e = slice_upload(p, *tabs[L], l.plan, groups, st);
+            std::vector<uint8_t> host;
+            if (e == cudaSuccess) e = slice_upload(p, *tabs[L], l.plan, groups, host, st);
             if (e == cudaSuccess) {
                 const int64_t blocks = std::min<int64_t>((32 * p.NG + 255) / 256, (int64_t)rep->num_sms * 16);
                 slice_nbr_kernel<2><<<(unsigned)blocks, 256, 0, st>>>(rep->dev, p.NT, p.NG, 0, 1,
                                                                    reinterpret_cast<const SliceGroup *>(l.plan.groups), p.nbr);
                 e = cudaGetLastError();
-                if (e == cudaSuccess) e = cudaStreamSynchronize(st);
+                const cudaError_t landed = cudaStreamSynchronize(st);
+                if (e == cudaSuccess) e = landed;
             }
             if (e == cudaSuccess) e = resident_ready(l.plan);
             if (e != cudaSuccess) {

@@ -1,0 +1,85 @@
+"""The library's host code without a GPU: which kernels a call launches, what
+it allocates and keeps, and what it does when the runtime refuses a request.
+Each test runs in a process of its own on a stand-in for the CUDA runtime
+(fake_cudart.c), which notes the calls and runs no kernel."""
+import os
+import shutil
+import subprocess
+import sys
+
+import pytest
+
+from paper_2110_12952_gb300 import build, capi, workloads as W
+
+HERE = os.path.dirname(os.path.abspath(__file__))
+CUDA = os.path.dirname(os.path.dirname(shutil.which("nvcc") or "/usr/local/cuda/bin/nvcc"))
+
+pytestmark = pytest.mark.skipif(not os.path.exists(os.path.join(CUDA, "bin", "nvcc")) or shutil.which("gcc") is None,
+                                reason="nvcc or gcc not available")
+
+PRELUDE = """
+import ctypes, re
+from ctypes import byref, c_int, c_int32, c_int64, c_void_p
+fake = ctypes.CDLL({fake!r}, mode=ctypes.RTLD_GLOBAL)
+lib = ctypes.CDLL({lib!r})
+fake.fake_log.restype, lib.fractal_last_error.restype = ctypes.c_char_p, ctypes.c_char_p
+fake.fake_held.restype, fake.fake_limit.argtypes = ctypes.c_size_t, [ctypes.c_size_t]
+TABLES = {tables!r}
+A, B = 1 << 40, 1 << 41          # where a program's buffers might be: no kernel runs
+
+def handle(name, r):
+    k, s, dim, table = TABLES[name]
+    h = c_void_p()
+    assert lib.fractal_create(k, s, r, dim, (c_int32 * len(table))(*table), byref(h)) == 0, lib.fractal_last_error()
+    return h
+
+def step(h, steps, stream=0, rule=(8, 12), src=A, dst=B, fn="fractal_step"):
+    return getattr(lib, fn)(h, c_void_p(src), c_void_p(dst), c_int64(steps), *rule, c_void_p(stream))
+
+def log(pattern="", clear=True):
+    lines = [x for x in fake.fake_log().decode().split("\\n") if re.search(pattern, x)]
+    if clear:
+        fake.fake_clear()
+    return [x for x in lines if x]
+
+def kernels():
+    return [x.split()[1] for x in log("^launch")]
+
+def sliced(names):
+    return any("slice_" in x for x in names)
+"""
+
+
+@pytest.fixture(scope="module")
+def host(tmp_path_factory):
+    build.build()
+    d = tmp_path_factory.mktemp("fake_cudart")
+    (d / "versions").write_text("libcudart.so.13 { global: *; };\n")
+    so = str(d / "libcudart.so.13")
+    subprocess.run(["gcc", "-std=gnu11", "-O1", "-shared", "-fPIC", "-I", os.path.join(CUDA, "include"), "-Wl,-soname,libcudart.so.13",
+                    f"-Wl,--version-script={d / 'versions'}", os.path.join(HERE, "fake_cudart.c"), "-o", so], check=True)
+    tables = {n: (f.k, f.s, f.dim, [int(v) for row in f.table() for v in row]) for n, f in W.FAMILIES.items()}
+    prelude = PRELUDE.format(fake=so, lib=capi.LIB_PATH, tables=tables)
+
+    def run(body):
+        p = subprocess.run([sys.executable, "-c", prelude + body], capture_output=True, text=True, timeout=300)
+        assert p.returncode == 0, (p.returncode, p.stdout, p.stderr)
+    return run
+
+
+def test_tables_outlive_their_copy(host):
+    # a copy from pageable memory may read its source until the stream has been waited for
+    host("""
+for name, r, steps in (("triangle", 8, 5), ("carpet", 8, 1), ("carpet", 10, 3), ("menger", 6, 1)):
+    h = handle(name, r)
+    assert step(h, steps, stream=0x70) == 0
+    assert not log("source changed", clear=False), name
+    assert sliced(kernels()), name
+b = c_void_p()
+assert lib.fractal_batch_create(byref(b)) == 0
+h = handle("triangle", 9)
+assert lib.fractal_batch_add(b, h, c_void_p(A), c_void_p(B), c_int64(4), 8, 12, None) == 0
+fake.fake_clear()
+assert lib.fractal_batch_run(b, None) == 0
+assert not log("source changed", clear=False) and sliced(kernels())
+""")

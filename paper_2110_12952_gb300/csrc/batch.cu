@@ -106,6 +106,12 @@ static int build(fractal_batch *b)
         FR_CUDA(cudaEventCreateWithFlags(&b->ev_in, cudaEventDisableTiming));
         FR_CUDA(cudaEventCreateWithFlags(&b->ev_out, cudaEventDisableTiming));
     }
+    // (of the sliced instances too: fractal_step_noalloc and captured calls of
+    // their handles need the tile kernels' tables and cannot build them)
+    for (auto &in : b->insts) {
+        rc = ensure_step_plan(in.f);
+        if (rc) return rc;
+    }
     // sliced launches by fractal table and rule; where they cannot be built
     // (memory) their instances stay with the tile kernels
     std::vector<char> is_sliced(b->insts.size(), 0);
@@ -127,11 +133,6 @@ static int build(fractal_batch *b)
             b->sliced.push_back(s);
             for (int i : e.second) is_sliced[i] = 1;
         }
-    }
-    for (size_t i = 0; i < b->insts.size(); ++i) {
-        if (is_sliced[i]) continue;
-        rc = ensure_step_plan(b->insts[i].f);
-        if (rc) return rc;
     }
     std::map<std::string, int> cls_of;
     for (int i = 0; i < (int)b->insts.size(); ++i) {

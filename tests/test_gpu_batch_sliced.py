@@ -55,3 +55,32 @@ def test_uneven_sliced_batches(seed, even):
     for g, _ in handles.values():
         g.check()
         g.close()
+
+
+@pytest.mark.parametrize("name,r", [("triangle", 8), ("carpet", 5), ("h_fractal", 4)])
+def test_a_batch_readies_its_handles(name, r):
+    # what a batch run has always made possible: the allocation-free step and a captured generation of a handle whose
+    # only call so far was the batch
+    from paper_2110_12952_gb300 import Batch, Fractal
+    fam = W.FAMILIES[name]
+    g, o = Fractal.from_family(fam, r), oracle.Fractal(fam.k, fam.s, r, fam.dim, fam.table())
+    v = o.init_bernoulli(4, 0.45)
+    x = torch.from_numpy(v).cuda()
+    y, z, t = torch.empty_like(x), torch.empty_like(x), torch.empty_like(x)
+    batch = Batch()
+    batch.add(g, x, y, 4)
+    batch.run()
+    birth, survive = W.LIFE_B3S23
+    assert g._lib.fractal_step_noalloc(g._h, x.data_ptr(), z.data_ptr(), 3, birth, survive, 0) == 0
+    torch.cuda.synchronize()
+    graph = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(graph):
+        g.step(x, out=t, steps=1)
+    graph.replay()
+    torch.cuda.synchronize()
+    for got, n in ((y, 4), (z, 3), (t, 1)):
+        assert np.array_equal(got.cpu().numpy(), o.step(v, steps=n)), n
+    del graph
+    batch.close()
+    g.check()
+    g.close()

@@ -83,3 +83,18 @@ fake.fake_clear()
 assert lib.fractal_batch_run(b, None) == 0
 assert not log("source changed", clear=False) and sliced(kernels())
 """)
+
+
+def test_a_batch_readies_its_handles(host):
+    # the allocation-free step and captured generations need tables that only earlier calls can build
+    host("""
+b, h = c_void_p(), handle("triangle", 9)
+assert lib.fractal_batch_create(byref(b)) == 0
+assert lib.fractal_batch_add(b, h, c_void_p(A), c_void_p(B), c_int64(4), 8, 12, None) == 0
+assert lib.fractal_batch_run(b, None) == 0
+assert sliced(kernels())
+assert step(h, 3, fn="fractal_step_noalloc") == 0, lib.fractal_last_error()
+fake.fake_capturing(1)
+fake.fake_clear()
+assert step(h, 1) == 0 and not log("malloc", clear=False) and len(kernels()) == 1
+""")

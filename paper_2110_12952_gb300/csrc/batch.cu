@@ -215,7 +215,10 @@ static int build(fractal_batch *b)
                            cudaMemcpyHostToDevice);
         if (e != cudaSuccess) return cuda_fail(e, "fractal_batch_run: table upload");
     }
-    // capture: the sliced launches, then generation by generation one launch per class
+    // capture: the copies, then generation by generation one launch per class,
+    // then the sliced launches.  An instance of several generations may so
+    // start from what a copy writes, and write what an instance of one
+    // generation reads, as when all instances advance together.
     rc = preload_copy_kernel();
     if (rc) return rc;
     cudaGraph_t graph = nullptr;
@@ -224,12 +227,6 @@ static int build(fractal_batch *b)
     int64_t updates = 0;
     int lrc = FR_OK;
     std::string where;
-    for (const SliceBatch *s : b->sliced) {
-        if (lrc) break;
-        lrc = run_slice_batch(s, b->cap);
-        if (lrc) where = "a sliced launch";
-        launches += slice_batch_launches(s);
-    }
     for (size_t i = 0; i < b->insts.size() && !lrc; ++i)
         if (b->insts[i].steps == 0) {
             lrc = launch_copy_normalise(b->insts[i].in, b->insts[i].out, b->insts[i].f->cells,
@@ -250,6 +247,12 @@ static int build(fractal_batch *b)
                         ", mode " + std::to_string(c.rep->plan.mode) + ") generation " + std::to_string(j);
             ++launches;
         }
+    for (const SliceBatch *s : b->sliced) {
+        if (lrc) break;
+        lrc = run_slice_batch(s, b->cap);
+        if (lrc) where = "a sliced launch";
+        launches += slice_batch_launches(s);
+    }
     if (lrc) {
         const std::string msg = fractal_last_error();
         set_error(lrc, "fractal_batch_run: launch failed at " + where + " (launch " +

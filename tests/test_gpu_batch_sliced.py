@@ -84,3 +84,27 @@ def test_a_batch_readies_its_handles(name, r):
     batch.close()
     g.check()
     g.close()
+
+
+def test_copies_come_before_generations():
+    # an instance of no generations normalises its input into another instance's input; one of a single generation
+    # reads what an instance of four overwrites from its second generation on
+    from paper_2110_12952_gb300 import Batch, Fractal
+    fam = W.TRIANGLE
+    g, o = Fractal.from_family(fam, 9), oracle.Fractal(fam.k, fam.s, 9, fam.dim, fam.table())
+    v, w = o.init_bernoulli(1, 0.45), o.init_bernoulli(2, 0.45)
+    p, q = torch.from_numpy(v * 7).cuda(), torch.from_numpy(w).cuda()
+    x, y, z = torch.zeros_like(p), torch.zeros_like(p), torch.zeros_like(p)
+    batch = Batch()
+    batch.add(g, x, y, 3)     # reads the copy
+    batch.add(g, p, x, 0)     # the copy
+    batch.add(g, q, z, 1)     # reads q before ...
+    batch.add(g, p, q, 4)     # ... this instance writes it
+    batch.run()
+    torch.cuda.synchronize()
+    assert np.array_equal(x.cpu().numpy(), v)
+    assert np.array_equal(y.cpu().numpy(), o.step(v, steps=3))
+    assert np.array_equal(z.cpu().numpy(), o.step(w, steps=1))
+    assert np.array_equal(q.cpu().numpy(), o.step(v, steps=4))
+    batch.close()
+    g.close()

@@ -98,3 +98,16 @@ fake.fake_capturing(1)
 fake.fake_clear()
 assert step(h, 1) == 0 and not log("malloc", clear=False) and len(kernels()) == 1
 """)
+
+
+def test_copies_come_before_generations(host):
+    # an instance may start from what one of no generations copies, and overwrite what one of a single generation reads
+    host("""
+b, h = c_void_p(), handle("triangle", 9)
+assert lib.fractal_batch_create(byref(b)) == 0
+for n, src, dst in ((4, A, B), (0, A + (1 << 20), A), (1, B, B + (1 << 20))):
+    assert lib.fractal_batch_add(b, h, c_void_p(src), c_void_p(dst), c_int64(n), 8, 12, None) == 0
+assert lib.fractal_batch_run(b, None) == 0
+order = ["copy" if "copy_normalise" in x else "sliced" if "resident" in x else "tiles" if "step_" in x else "" for x in kernels()]
+assert [x for x in order if x] == ["copy", "tiles", "sliced"], order
+""")

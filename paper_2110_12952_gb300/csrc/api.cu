@@ -243,7 +243,7 @@ extern "C" int fractal_destroy(fractal_t *f)
     cudaFree(f->scratch);
     cudaFree(f->b3_state[0]);
     cudaFree(f->b3_state[1]);
-    for (uint32_t *w : f->bb_words) cudaFree(w);
+    for (uint32_t *w : f->box_words.mem) cudaFree(w);
     if (f->packed_done) cudaEventDestroy(f->packed_done);
     cudaFree(f->bb_scratch);
     cudaFree(f->host_io[0]);

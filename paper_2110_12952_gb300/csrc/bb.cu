@@ -881,17 +881,56 @@ static int run_bb_words(fractal *f, BWArgs a, const uint8_t *in, uint8_t *out, i
 {
     const int sms = f->num_sms, smem = 4 * (a.groups * a.yg * a.pitch + 2);
     const int stage = 2 * 16 * kBwUnits * kBwBlock;
-    int cur = steps == 1 ? 1 : 2;
-    bb_pack_kernel<<<(unsigned)std::min<int64_t>(a.ptiles, (int64_t)sms * 6), kBwBlock, stage, st>>>(a, in, f->bb_words[cur] + 1);
+    uint32_t *now = steps == 1 ? f->box_words.one : f->box_words.two[0], *next = f->box_words.two[1];
+    bb_pack_kernel<<<(unsigned)std::min<int64_t>(a.ptiles, (int64_t)sms * 6), kBwBlock, stage, st>>>(a, in, now);
     FR_CUDA(cudaGetLastError());
     const int grid = (int)std::min<int64_t>(a.tiles, (int64_t)sms * 64);
-    for (int64_t g = 1; g < steps; ++g, cur ^= 1) {   // (2 and 3 in turn)
-        launch_bb_words<DIM, false>(a, grid, 0, f->bb_words[cur] + 1, f->bb_words[cur ^ 1] + 1, nullptr, st);
+    for (int64_t g = 1; g < steps; ++g) {
+        launch_bb_words<DIM, false>(a, grid, 0, now, next, nullptr, st);
         FR_CUDA(cudaGetLastError());
+        std::swap(now, next);
     }
-    launch_bb_words<DIM, true>(a, grid, smem, f->bb_words[cur] + 1, nullptr, out, st);
+    launch_bb_words<DIM, true>(a, grid, smem, now, nullptr, out, st);
     FR_CUDA(cudaGetLastError());
     return FR_OK;
+}
+
+// Allocates and fills what calls of one generation (of several) lack.  The
+// handle learns of it only when it is filled; false, and nothing kept, where
+// the memory or one of the fills cannot be had.
+static bool box_words_build(fractal *f, const BWArgs &a, bool several, cudaStream_t st)
+{
+    BoxWords &w = f->box_words;
+    const size_t words = ((size_t)a.rows * a.RP + 1 + 63) / 64 * 64;
+    const int member = w.member ? 0 : 1, arrays = member + (several ? 2 : 1);
+    uint32_t *mem = nullptr;
+    cudaError_t e = cudaMalloc(&mem, arrays * words * sizeof(uint32_t));
+    if (e == cudaSuccess) {
+        e = cudaMemsetAsync(mem, 0, arrays * words * sizeof(uint32_t), st);
+        if (e == cudaSuccess && member) {
+            const unsigned grid = (unsigned)std::min<int64_t>((a.rows * a.RW + kBwBlock - 1) / kBwBlock, (int64_t)f->num_sms * 32);
+            if (f->dim == 3) bb_member_kernel<3><<<grid, kBwBlock, 0, st>>>(a, mem + 1);
+            else bb_member_kernel<2><<<grid, kBwBlock, 0, st>>>(a, mem + 1);
+            e = cudaGetLastError();
+        }
+        const cudaError_t filled = cudaStreamSynchronize(st);   // they serve calls on any stream from here on
+        if (e == cudaSuccess) e = filled;
+    }
+    if (e != cudaSuccess) {
+        cudaGetLastError();
+        cudaFree(mem);
+        return false;
+    }
+    w.mem[w.mem[0] ? 1 : 0] = mem;
+    if (member) w.member = mem + 1;
+    uint32_t *box = mem + member * words + 1;
+    if (several) {
+        w.two[0] = box;
+        w.two[1] = box + words;
+    } else {
+        w.one = box;
+    }
+    return true;
 }
 
 int try_bb_packed(fractal *f, const uint8_t *in, uint8_t *out, int64_t steps, uint32_t birth, uint32_t survive, cudaStream_t st,
@@ -907,34 +946,19 @@ int try_bb_packed(fractal *f, const uint8_t *in, uint8_t *out, int64_t steps, ui
     a.rows = f->dim == 3 ? (int64_t)n * n : n;
     if (a.rows >= ((int64_t)1 << 31)) return FR_OK;
     a.RP = a.RW + 1;
-    // the cells' membership, computed once, and one or two states; a zero word before each
-    const size_t bytes = ((size_t)a.rows * a.RP + 1) * sizeof(uint32_t);
     const bool captured = capturing(st);
     // under capture a single generation leaves the packed box alone: its replays may run beside other calls
     if (captured && steps == 1) return FR_OK;
-    for (int i = 0; i < 4; ++i) {
-        if (f->bb_words[i] || (i > 0 && (steps == 1) != (i == 1))) continue;
+    if (!(steps == 1 ? f->box_words.one : f->box_words.two[0])) {
         // nothing is allocated under capture, and without the memory the row kernels run as before
-        if (captured || cudaMalloc(&f->bb_words[i], bytes) != cudaSuccess) {
-            cudaGetLastError();
-            f->bb_words[i] = nullptr;
-            return FR_OK;
-        }
-        FR_CUDA(cudaMemsetAsync(f->bb_words[i], 0, bytes, st));
-        if (i == 0) {
-            const unsigned grid = (unsigned)std::min<int64_t>((a.rows * a.RW + kBwBlock - 1) / kBwBlock, (int64_t)f->num_sms * 32);
-            if (f->dim == 3) bb_member_kernel<3><<<grid, kBwBlock, 0, st>>>(a, f->bb_words[0] + 1);
-            else bb_member_kernel<2><<<grid, kBwBlock, 0, st>>>(a, f->bb_words[0] + 1);
-            FR_CUDA(cudaGetLastError());
-        }
-        FR_CUDA(cudaStreamSynchronize(st));   // they serve calls on any stream from here on
-        if (i == 3 && !f->bb_scratch && cudaMalloc(&f->bb_scratch, f->box_cells) != cudaSuccess) {
+        if (captured || !box_words_build(f, a, steps > 1, st)) return FR_OK;
+        if (steps > 1 && !f->bb_scratch && cudaMalloc(&f->bb_scratch, f->box_cells) != cudaSuccess) {
             // (the row kernels' scratch, for a later captured call whose buffers are not aligned)
             cudaGetLastError();
             f->bb_scratch = nullptr;
         }
     }
-    a.member = f->bb_words[0] + 1;
+    a.member = f->box_words.member;
     a.pseg = (a.RW + kBwSeg - 1) / kBwSeg;
     a.segw = (a.RW + a.pseg - 1) / a.pseg;
     a.prow = a.pseg == 1 ? std::max(1, 32 * kBwSeg / n) : 1;   // (at most 32 kBwSeg cells)

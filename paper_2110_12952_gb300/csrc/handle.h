@@ -88,6 +88,15 @@ struct BBPlan {
     int64_t local_words = 0, coarse_words = 0;
 };
 
+// The box as bits (bb.cu), each array behind a zero word: the cells'
+// membership, the box of single generations, the two of calls of several.
+// One allocation holds the membership and the boxes of the first kind of call,
+// another those of the other kind.
+struct BoxWords {
+    uint32_t *mem[2] = {nullptr, nullptr};
+    uint32_t *member = nullptr, *one = nullptr, *two[2] = {nullptr, nullptr};
+};
+
 // Temporal blocking (temporal.cuh): tile depth, tables and launch shape of
 // the multi-generation pass for the carpet and the Vicsek fractal.
 struct TbPlan {
@@ -134,9 +143,8 @@ struct fractal {
     fr::BBPlan bb;
     uint8_t *scratch = nullptr;      // k^r bytes, ping-pong for steps > 1
     uint32_t *b3_state[2] = {nullptr, nullptr};  // bit3 plans, steps > 1: bit-packed tile states (ping-pong)
-    // box steps: membership, the packed box of single generations, two of calls of several
-    uint32_t *bb_words[4] = {nullptr, nullptr, nullptr, nullptr};
-    cudaEvent_t packed_done = nullptr;   // after the last work on the packed buffers (slice, bb_words)
+    fr::BoxWords box_words;          // box steps: the box as bits
+    cudaEvent_t packed_done = nullptr;   // after the last work on the packed buffers (slice, box_words)
     uint8_t *bb_scratch = nullptr;   // n^dim bytes, ping-pong for BB steps > 1
     uint8_t *host_io[2] = {nullptr, nullptr};  // device buffers of run_host
     fr::HostPipe pipe;                          // run_host's chunked pipeline

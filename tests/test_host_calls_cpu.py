@@ -111,3 +111,25 @@ assert lib.fractal_batch_run(b, None) == 0
 order = ["copy" if "copy_normalise" in x else "sliced" if "resident" in x else "tiles" if "step_" in x else "" for x in kernels()]
 assert [x for x in order if x] == ["copy", "tiles", "sliced"], order
 """)
+
+
+def test_box_words_are_kept_only_when_filled(host):
+    # a call that cannot fill the packed box's arrays keeps none of them: the next call fills them
+    host("""
+for name, r, steps, rule in (("carpet", 5, 3, (8, 12)), ("menger", 4, 1, (32, 48))):
+    for call, after in (("cudaMemsetAsync", 0), ("launch", 0), ("cudaStreamSynchronize", 0), ("cudaMalloc", 0)):
+        h = handle(name, r)
+        assert step(h, 0, rule=rule, fn="fractal_bb_step") == 0        # builds the row kernels' tables
+        held = fake.fake_held()
+        fake.fake_clear()
+        fake.fake_fail(call.encode(), after)
+        step(h, steps, rule=rule, fn="fractal_bb_step")
+        assert step(h, steps, rule=rule, fn="fractal_bb_step") == 0, lib.fractal_last_error()
+        names = kernels()
+        filled = [i for i, x in enumerate(names) if "bb_member" in x]
+        assert filled and any("bb_words" in x for x in names[filled[-1]:]), (name, call, names)
+        assert not any("bb_words" in x for x in names[:filled[-1]]), (name, call, names)
+        assert step(h, 1 if steps > 1 else 2, rule=rule, fn="fractal_bb_step") == 0
+        assert lib.fractal_destroy(h) == 0
+assert fake.fake_held() == 0, fake.fake_held()
+""")

@@ -203,10 +203,11 @@ int fractal_step_noalloc(fractal_t *f, const uint8_t *in_dev, uint8_t *out_dev,
  * cell of the n^dim box.  Cells off the fractal count as dead whatever their
  * byte and are written as 0.  box_in_dev / box_out_dev: n^dim bytes each,
  * not overlapping.  Scratch for steps > 1 as in fractal_step (n^dim bytes).
- * Boxes of side >= 32 in 16-byte aligned buffers are packed into bits for
- * steps > 1, and in 3D for steps = 1 as well: the cells' membership and one
- * or two packed boxes (n^dim / 8 bytes each), allocated on first need, with
- * the rules on streams, capture and missing memory of fractal_step. */
+ * Boxes of side >= 32 are packed into bits for steps > 1, and in 3D in 16-byte
+ * aligned buffers for steps = 1 as well: the cells' membership and one or two
+ * packed boxes (n^dim / 8 bytes each, a little more where n is no multiple of
+ * 32), allocated on first need, with the rules on streams, capture and missing
+ * memory of fractal_step; the scratch of n^dim bytes is then not allocated. */
 int fractal_bb_step(fractal_t *f, const uint8_t *box_in_dev, uint8_t *box_out_dev,
                     int64_t steps, uint32_t birth_mask, uint32_t survive_mask,
                     void *stream);

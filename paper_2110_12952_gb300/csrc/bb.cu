@@ -585,7 +585,7 @@ bb_bits3_kernel(BBBitsArgs a, const uint8_t *__restrict__ in, uint8_t *__restric
 // the fractal zero: bytes are packed once, generations between the first and
 // the last go from bits to bits (an eighth of the traffic), the last writes
 // bytes.  Bytes and bits meet in shared memory: a block's rows are contiguous
-// in the box, so its bytes move as aligned 16-byte units, and rows that start
+// in the box, so its bytes move as 16-byte units, and rows that start
 // at any byte are cut out of (or put together from) bit strings by funnel
 // shifts.  In three dimensions a single generation goes this way too: every
 // byte is read and converted once, where the row kernel above converts each
@@ -665,6 +665,8 @@ struct BwTile {
 // Bytes -> bits.  The next tile's bytes are on their way to shared memory
 // while this one is converted (each thread waits for its own copies only).
 // Menger r = 6 (3.9e8 cells): 96 us, 4.5 TB/s; issue slots 60 %.
+// Boxes that are not 16-byte aligned (ALIGNED = false) are read byte by byte.
+template <bool ALIGNED>
 __global__ void __launch_bounds__(kBwBlock) bb_pack_kernel(BWArgs a, const uint8_t *__restrict__ in, uint32_t *__restrict__ bits)
 {
     extern __shared__ __align__(16) uint4 stage[];   // two tiles
@@ -673,7 +675,7 @@ __global__ void __launch_bounds__(kBwBlock) bb_pack_kernel(BWArgs a, const uint8
     const int tid = threadIdx.x;
     const int64_t whole = a.b.total / 16;   // 16-byte units that lie in the box entirely
     auto fetch = [&](int64_t t, int buf) {
-        if (t < a.ptiles) {
+        if (ALIGNED && t < a.ptiles) {
             const BwTile T(a, t);
             const uint8_t *src = in + T.f0 + 16 * tid;
             uint4 *dst = stage + buf * kBwUnits * kBwBlock + tid;
@@ -700,7 +702,17 @@ __global__ void __launch_bounds__(kBwBlock) bb_pack_kernel(BWArgs a, const uint8
         const uint4 *src = stage + buf * kBwUnits * kBwBlock + tid;
 #pragma unroll
         for (int k = 0; k < kBwUnits; ++k)
-            if (tid + kBwBlock * k < T.units) B16[tid + kBwBlock * k] = (uint16_t)bits16_of(src[kBwBlock * k]);
+            if (tid + kBwBlock * k < T.units) {
+                if (ALIGNED) {
+                    B16[tid + kBwBlock * k] = (uint16_t)bits16_of(src[kBwBlock * k]);
+                } else {
+                    const int64_t at = T.f0 + 16 * (tid + kBwBlock * k);
+                    uint32_t x = 0;
+#pragma unroll
+                    for (int j = 0; j < 16; ++j) x |= (uint32_t)(at + j < a.b.total && __ldg(in + at + j) != 0) << j;
+                    B16[tid + kBwBlock * k] = (uint16_t)x;
+                }
+            }
         __syncthreads();
         for (int i = tid; i < T.rows * T.wn; i += kBwBlock) {
             const int r = a.pseg == 1 ? (a.RW == 1 ? i : (int)divu(a.rwdiv, (uint32_t)i)) : 0, w = i - r * T.wn;
@@ -718,7 +730,7 @@ __global__ void __launch_bounds__(kBwBlock) bb_pack_kernel(BWArgs a, const uint8
 __device__ __forceinline__ void words_to_bytes(const uint32_t *R, int pitch, int rows, int len, const DivU32 &ldiv, uint8_t *__restrict__ out,
                                                int64_t f0)
 {
-    const int cells = rows * len, head = min((int)((16 - (f0 & 15)) & 15), cells);
+    const int cells = rows * len, head = min((int)((16 - ((uintptr_t)(out + f0) & 15)) & 15), cells);
     const int units = (cells - head) / 16, tail = head + 16 * units;
     uint4 *dst = reinterpret_cast<uint4 *>(out + f0 + head);
 #pragma unroll 2
@@ -845,10 +857,12 @@ __global__ void __launch_bounds__(kBwBlock) bb_words_kernel(BWArgs a, const uint
     }
 }
 
-// Whether the box's kernels can use 32-cell words (see above).
-static bool bb_words_ok(const fractal *f, const uint8_t *in, const uint8_t *out)
+// Whether the box's kernels can use 32-cell words (see above), and whether
+// its row kernels can.
+static bool bb_words_side(const fractal *f) { return f->bb.S >= 32 && f->side >= 32; }
+static bool bb_rows_ok(const fractal *f, const uint8_t *in, const uint8_t *out)
 {
-    return f->bb.S >= 32 && f->side >= 32 && ((uintptr_t)in & 15) == 0 && ((uintptr_t)out & 15) == 0;
+    return bb_words_side(f) && ((uintptr_t)in & 15) == 0 && ((uintptr_t)out & 15) == 0;
 }
 
 static void bb_bits_args(const fractal *f, uint32_t birth, uint32_t survive, BBBitsArgs &a)
@@ -880,9 +894,10 @@ template <int DIM>
 static int run_bb_words(fractal *f, BWArgs a, const uint8_t *in, uint8_t *out, int64_t steps, cudaStream_t st)
 {
     const int sms = f->num_sms, smem = 4 * (a.groups * a.yg * a.pitch + 2);
-    const int stage = 2 * 16 * kBwUnits * kBwBlock;
+    const unsigned pack_grid = (unsigned)std::min<int64_t>(a.ptiles, (int64_t)sms * 6);
     uint32_t *now = steps == 1 ? f->box_words.one : f->box_words.two[0], *next = f->box_words.two[1];
-    bb_pack_kernel<<<(unsigned)std::min<int64_t>(a.ptiles, (int64_t)sms * 6), kBwBlock, stage, st>>>(a, in, now);
+    if (((uintptr_t)in & 15) == 0) bb_pack_kernel<true><<<pack_grid, kBwBlock, 2 * 16 * kBwUnits * kBwBlock, st>>>(a, in, now);
+    else bb_pack_kernel<false><<<pack_grid, kBwBlock, 0, st>>>(a, in, now);
     FR_CUDA(cudaGetLastError());
     const int grid = (int)std::min<int64_t>(a.tiles, (int64_t)sms * 64);
     for (int64_t g = 1; g < steps; ++g) {
@@ -937,8 +952,9 @@ int try_bb_packed(fractal *f, const uint8_t *in, uint8_t *out, int64_t steps, ui
                   bool *done)
 {
     *done = false;
-    // a single 2D generation is at 93 % of the copy bandwidth in the row kernel
-    if (!bb_words_ok(f, in, out) || steps < (f->dim == 3 ? 1 : 2)) return FR_OK;
+    // a single 2D generation is at 93 % of the copy bandwidth in the row kernel; calls of several take buffers at
+    // any address, so that a captured one needs no scratch beside the packed boxes of an earlier call
+    if (!bb_words_side(f) || (steps == 1 && (f->dim == 2 || !bb_rows_ok(f, in, out)))) return FR_OK;
     BWArgs a;
     bb_bits_args(f, birth, survive, a.b);
     const int32_t n = a.b.n;
@@ -952,11 +968,6 @@ int try_bb_packed(fractal *f, const uint8_t *in, uint8_t *out, int64_t steps, ui
     if (!(steps == 1 ? f->box_words.one : f->box_words.two[0])) {
         // nothing is allocated under capture, and without the memory the row kernels run as before
         if (captured || !box_words_build(f, a, steps > 1, st)) return FR_OK;
-        if (steps > 1 && !f->bb_scratch && cudaMalloc(&f->bb_scratch, f->box_cells) != cudaSuccess) {
-            // (the row kernels' scratch, for a later captured call whose buffers are not aligned)
-            cudaGetLastError();
-            f->bb_scratch = nullptr;
-        }
     }
     a.member = f->box_words.member;
     a.pseg = (a.RW + kBwSeg - 1) / kBwSeg;
@@ -981,7 +992,7 @@ int try_bb_packed(fractal *f, const uint8_t *in, uint8_t *out, int64_t steps, ui
 int launch_bb_once(fractal *f, const uint8_t *in, uint8_t *out, uint32_t birth,
                    uint32_t survive, cudaStream_t st)
 {
-    if (bb_words_ok(f, in, out)) {
+    if (bb_rows_ok(f, in, out)) {
         BBBitsArgs a;
         bb_bits_args(f, birth, survive, a);
         // strip sx writes cells up to 992 sx + 1008 - k (k < 16), strip 0 from cell 0 on

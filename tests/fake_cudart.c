@@ -102,16 +102,16 @@ unsigned __cudaPushCallConfiguration(dim3 grid, dim3 block, size_t smem, void *s
 cudaError_t __cudaPopCallConfiguration(dim3 *grid, dim3 *block, size_t *smem, void *stream)
 { *grid = g_config.grid; *block = g_config.block; *smem = g_config.smem; *(void **)stream = g_config.stream; return cudaSuccess; }
 cudaError_t __cudaGetKernel(void **k, const void *fun) { *k = (void *)fun; return cudaSuccess; }
-static cudaError_t launch(const void *fun, dim3 grid, void *stream)
+static cudaError_t launch(const void *fun, dim3 grid, size_t smem, void *stream)
 {
     cudaError_t e = result("launch", cudaErrorLaunchFailure);
     if (e == cudaSuccess && (grid.x == 0 || grid.y == 0)) e = g_last = cudaErrorInvalidConfiguration;
-    if (e == cudaSuccess) note("launch %s on %zx\n", kernel_name(fun), (size_t)stream);
+    if (e == cudaSuccess) note("launch %s grid %u shared %zu on %zx\n", kernel_name(fun), grid.x, smem, (size_t)stream);
     return e;
 }
-cudaError_t __cudaLaunchKernel(void *k, dim3 grid, dim3 block, void **args, size_t smem, void *st) { (void)block; (void)args; (void)smem; return launch(k, grid, st); }
-cudaError_t cudaLaunchKernel(const void *f, dim3 grid, dim3 block, void **args, size_t smem, void *st) { (void)block; (void)args; (void)smem; return launch(f, grid, st); }
-cudaError_t cudaLaunchCooperativeKernel(const void *f, dim3 grid, dim3 block, void **args, size_t smem, void *st) { (void)block; (void)args; (void)smem; return launch(f, grid, st); }
+cudaError_t __cudaLaunchKernel(void *k, dim3 grid, dim3 block, void **args, size_t smem, void *st) { (void)block; (void)args; return launch(k, grid, smem, st); }
+cudaError_t cudaLaunchKernel(const void *f, dim3 grid, dim3 block, void **args, size_t smem, void *st) { (void)block; (void)args; return launch(f, grid, smem, st); }
+cudaError_t cudaLaunchCooperativeKernel(const void *f, dim3 grid, dim3 block, void **args, size_t smem, void *st) { (void)block; (void)args; return launch(f, grid, smem, st); }
 cudaError_t cudaLaunchHostFunc(void *st, void (*fn)(void *), void *arg) { (void)st; fn(arg); return cudaSuccess; }
 
 /* memory */

@@ -63,3 +63,37 @@ def test_one_handle_on_two_streams(name, r, steps):
     torch.cuda.synchronize()
     assert all(torch.equal(y, want[j]) for j in range(2) for y in out[j])
     g.close()
+
+
+@pytest.mark.parametrize("name,r", [("triangle", 5), ("triangle", 9), ("carpet", 5), ("carpet", 6), ("candy", 3), ("menger", 4)])
+@pytest.mark.parametrize("src_off,dst_off", [(1, 0), (0, 7), (15, 9), (8, 4)])
+def test_boxes_at_any_address(name, r, src_off, dst_off):
+    # several generations from and to boxes that are not 16-byte aligned, called and captured after an aligned call
+    from paper_2110_12952_gb300 import Fractal
+    fam = W.FAMILIES[name]
+    g, o = Fractal.from_family(fam, r), oracle.Fractal(fam.k, fam.s, r, fam.dim, fam.table())
+    rng = np.random.default_rng(r + src_off)
+    x = (rng.random(o.box_cells) < 0.45).astype(np.uint8) * rng.integers(1, 256, o.box_cells).astype(np.uint8)
+    rule = W.rule_masks([4], [3, 4, 5, 26]) if fam.dim == 3 else W.rule_masks([2, 8], [0, 1, 2, 3, 8])
+    whole = torch.full((o.box_cells + 64,), 77, dtype=torch.uint8, device="cuda")
+    base = torch.empty(o.box_cells + 16, dtype=torch.uint8, device="cuda")
+    src, dst = base[src_off:src_off + o.box_cells], whole[16 + dst_off:16 + dst_off + o.box_cells]
+    src.copy_(torch.from_numpy(x))
+    for captured in (False, True):
+        for steps in (2, 3):
+            whole.fill_(77)
+            if captured:
+                g.bb_step(src.clone(), steps=2, rule=rule)   # the handle's arrays
+                torch.cuda.synchronize()
+                graph = torch.cuda.CUDAGraph()
+                with torch.cuda.graph(graph):
+                    g.bb_step(src, out=dst, steps=steps, rule=rule)
+                graph.replay()
+                torch.cuda.synchronize()
+                del graph
+            else:
+                g.bb_step(src, out=dst, steps=steps, rule=rule)
+            want = o.bb_step(x, rule=oracle.Rule(*rule), steps=steps)
+            assert np.array_equal(dst.cpu().numpy(), want), (steps, captured)
+            assert int((whole == 77).sum()) == 64
+    g.close()

@@ -133,3 +133,21 @@ for name, r, steps, rule in (("carpet", 5, 3, (8, 12)), ("menger", 4, 1, (32, 48
         assert lib.fractal_destroy(h) == 0
 assert fake.fake_held() == 0, fake.fake_held()
 """)
+
+
+def test_packed_boxes_need_no_scratch(host):
+    # calls of several box generations hold packed boxes alone, and serve captured calls at any address
+    host("""
+for name, r, rule in (("carpet", 6, (8, 12)), ("menger", 4, (32, 48))):
+    h, side, dim = handle(name, r), TABLES[name][1] ** r, TABLES[name][2]
+    assert step(h, 3, rule=rule, fn="fractal_bb_step") == 0
+    sizes = [int(x.split()[1]) for x in log("^malloc")]
+    assert max(sizes) < side ** dim, (sizes, side ** dim)
+    fake.fake_capturing(1)
+    fake.fake_clear()
+    for src, dst in ((A, B), (A + 3, B), (A, B + 5), (A + 1, B + 2)):
+        assert step(h, 4, rule=rule, src=src, dst=dst, fn="fractal_bb_step") == 0, lib.fractal_last_error()
+    assert not log("malloc", clear=False) and sum("bb_words" in x for x in kernels()) == 16
+    fake.fake_capturing(0)
+    lib.fractal_destroy(h)
+""")

@@ -52,6 +52,7 @@ constexpr int kSliceBatch = 4;     // 16-byte units per thread and batch copied 
 constexpr int kSliceSmem = 220 * 1024;   // resident kernel: shared memory per block
 constexpr int64_t kSliceBatchCells = 60000000;   // batches: most cells of an instance
 constexpr int kSliceSingleHalo = 32;   // most halo cells of a tile for the single-pass kernel
+constexpr int kSliceWait = 16;      // calls by the tile kernels after a refused allocation before the next try
 constexpr int kSliceRounds = 32;   // resident kernel: most 32-cell chunks per warp
 
 // One group of a batch: its bytes, its tiles and where its instance lies
@@ -1466,7 +1467,7 @@ static int build_slice_plan(fractal *f, cudaStream_t st)
     if (e != cudaSuccess) {
         cudaGetLastError();
         free_slice_plan(s);
-        return e == cudaErrorMemoryAllocation ? FR_ENOMEM : FR_ECUDA;
+        return e == cudaErrorMemoryAllocation ? FR_ENOMEM : (e == cudaErrorInvalidConfiguration ? FR_EINVAL : FR_ECUDA);
     }
     s.state = 1;
     f->slice = s;
@@ -1607,15 +1608,25 @@ int try_slice_step(fractal *f, const uint8_t *in, uint8_t *out, int64_t steps, u
     const bool ready = s.state > 0 && (!packed || (steps == 1 ? s.bits[2] != nullptr : s.bits[0] && s.bits[1]));
     if (captured && (!ready || (steps == 1 && (res || packed)))) return FR_OK;
     if (!ready) {
+        // after a refused allocation a number of calls go to the tile kernels before the next try
+        if (s.wait > 0) {
+            --s.wait;
+            return FR_OK;
+        }
         rc = ensure_status(f);
         if (rc) return rc;
-        if (s.state == 0 && build_slice_plan(f, st) != FR_OK) {
-            s.state = -1;
-            return FR_OK;
+        if (s.state == 0) {
+            rc = build_slice_plan(f, st);
+            if (rc == FR_EINVAL) s.state = -1;
+            else if (rc) s.wait = kSliceWait;
+            if (rc) return FR_OK;
         }
         if (steps == 1 && slice_one_generation_by_tiles(f, s.geo.H)) return FR_OK;
         choose();
-        if (packed && !(steps == 1 ? slice_buffer(f, 2) : slice_buffer(f, 0) && slice_buffer(f, 1))) return FR_OK;
+        if (packed && !(steps == 1 ? slice_buffer(f, 2) : slice_buffer(f, 0) && slice_buffer(f, 1))) {
+            s.wait = kSliceWait;
+            return FR_OK;
+        }
     }
     const SliceGeo &p = s.geo;
     const SliceArgs a = slice_args(p, birth, survive, steps == 1 ? s.bar + 2 : s.bar, f->status);

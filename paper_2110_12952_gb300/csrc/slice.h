@@ -37,6 +37,7 @@ struct SliceGeo {
 struct SlicePlan {
     bool several = false;     // a call of several generations has run
     int state = 0;            // 0: not planned yet, 1: planned, -1: not possible for this fractal
+    int wait = 0;             // calls left to the tile kernels after a refused allocation
     SliceGeo geo;
     bool resident = false;    // the packed state stays in shared memory: one launch for all generations
     int per_block = 0, rounds = 0, block_resident = 0, grid_resident = 0, smem_resident = 0;

@@ -151,3 +151,22 @@ for name, r, rule in (("carpet", 6, (8, 12)), ("menger", 4, (32, 48))):
     fake.fake_capturing(0)
     lib.fractal_destroy(h)
 """)
+
+
+def test_sliced_again_when_memory_is_free_again(host):
+    # calls that find no memory for the tables or the packed states run on the tile kernels; once there is memory,
+    # one of the next calls has them
+    host("""
+for name, r, steps, room in (("carpet", 9, 4, 1 << 18), ("h_fractal", 10, 3, 1 << 18), ("h_fractal", 10, 3, 20 << 20)):
+    h = handle(name, r)
+    assert lib.fractal_get_tile_levels(h, byref(c_int())) == 0
+    fake.fake_limit(fake.fake_held() + room)
+    rc = step(h, steps)                       # (the ping-pong scratch may not fit either)
+    assert not sliced([x for x in kernels() if "step_kernel" in x or "resident" in x]) and rc in (0, -3)
+    fake.fake_limit(1 << 60)
+    fake.cudaGetLastError()
+    fake.fake_clear()
+    assert all(step(h, steps) == 0 for _ in range(20))
+    assert sliced([x for x in kernels() if "step_kernel" in x or "resident" in x]), (name, room)
+    lib.fractal_destroy(h)
+""")

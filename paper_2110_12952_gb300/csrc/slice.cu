@@ -49,6 +49,7 @@ constexpr int kSliceBlock = 256;   // threads per block of the streaming kernels
 constexpr int kSliceBlock3 = 512;  // the same in 3D, where a group is larger (Menger: 8000 words and 3700 halo words)
 constexpr int kSliceAhead = 2;     // halo words per warp loaded ahead of their group
 constexpr int kSliceBatch = 4;     // 16-byte units per thread and batch copied to shared memory ahead
+constexpr int kSliceMost = 112 * 1024;   // the other kernels': most shared memory per block
 constexpr int kSliceSmem = 220 * 1024;   // resident kernel: shared memory per block
 constexpr int64_t kSliceBatchCells = 60000000;   // batches: most cells of an instance
 constexpr int kSliceSingleHalo = 32;   // most halo cells of a tile for the single-pass kernel
@@ -1174,7 +1175,7 @@ static std::shared_ptr<SliceImage> slice_image(const fractal *f, int L)
 void free_slice_plan(SlicePlan &p)
 {
     cudaFree(p.arena);
-    for (uint32_t *b : p.bits) cudaFree(b);
+    for (uint8_t *m : p.packed) cudaFree(m);
     p = SlicePlan();
 }
 
@@ -1371,13 +1372,26 @@ static int slice_levels(const fractal *f, SlicePlan *plan, std::shared_ptr<Slice
     return best;
 }
 
+// Bytes of a packed state and its exports, and the states of one kind of call
+// (one of single generations, two of several) at `mem`.
+static size_t slice_packed_bytes(const SliceGeo &p)
+{
+    return ((size_t)p.NG * (p.KLp + 32 * p.XW) * sizeof(uint32_t) + 255) / 256 * 256;
+}
+static void slice_set_packed(SlicePlan &s, int states, uint8_t *mem)
+{
+    for (int i = 0; i < states; ++i)
+        s.bits[states == 1 ? 2 : i] = reinterpret_cast<uint32_t *>(mem + i * slice_packed_bytes(s.geo));
+}
+
 // One allocation: the tables (copied from the host in one piece), the grid
-// barrier's zeros, the neighbouring tiles and the resident exports.  `img` is
+// barrier's zeros, the neighbouring tiles, the resident exports and `packed`
+// packed states.  `img` is
 // that piece: the copy may read it until `st` has been waited for (a runtime
 // that reads pageable memory in place does not stage it first), so the caller
 // keeps it until then.
 static cudaError_t slice_upload(SliceGeo &p, SliceImage &image, SlicePlan &s, const std::vector<SliceGroup> &groups,
-                                std::vector<uint8_t> &img, cudaStream_t st)
+                                int packed, std::vector<uint8_t> &img, cudaStream_t st)
 {
     const SliceTables &t = image.t;
     const std::vector<uint16_t> &nb = image.neighbours(p.D);
@@ -1391,7 +1405,7 @@ static cudaError_t slice_upload(SliceGeo &p, SliceImage &image, SlicePlan &s, co
                  o_cells = take(t.cells.size() * 4), o_bar = take(16), o_groups = take(groups.size() * sizeof(SliceGroup)), host = off;
     const size_t o_nbr = take((size_t)p.NG * p.ND * 32 * sizeof(int32_t)),
                  exb = s.resident ? (size_t)p.NG * p.XW * 128 : 0, o_ex0 = take(exb), o_ex1 = take(exb),
-                 o_ex2 = take(groups.empty() ? exb : 0);
+                 o_ex2 = take(groups.empty() ? exb : 0), o_bits = take((size_t)packed * slice_packed_bytes(p));
     img.assign(host, 0);
     memcpy(img.data() + o_tab, nb.data(), nb.size() * 2);
     memcpy(img.data() + o_jobs, t.jobs.data(), t.jobs.size() * 4);
@@ -1410,79 +1424,90 @@ static cudaError_t slice_upload(SliceGeo &p, SliceImage &image, SlicePlan &s, co
     s.ex[0] = reinterpret_cast<uint32_t *>(s.arena + o_ex0);
     s.ex[1] = reinterpret_cast<uint32_t *>(s.arena + o_ex1);
     s.ex[2] = reinterpret_cast<uint32_t *>(s.arena + o_ex2);
+    if (packed) slice_set_packed(s, packed, s.arena + o_bits);
     return e;
 }
 
-static int build_slice_plan(fractal *f, cudaStream_t st)
+// The plan, on the host alone: the tile depth and the shared memory.
+static bool plan_slice(fractal *f)
 {
+    SlicePlan &s = f->slice;
     std::shared_ptr<SliceImage> img;
-    SlicePlan s;
-    if (slice_levels(f, &s, &img) < 1) return FR_EINVAL;
-    SliceGeo &p = s.geo;
+    if (slice_levels(f, &s, &img) < 1) return false;
+    const SliceGeo &p = s.geo;
     s.block = f->dim == 3 ? kSliceBlock3 : kSliceBlock;
     const int ring = 16 * kSliceBatch * s.block, arrays = f->dim == 3 ? 1 : 2;
     s.smem_pack = ring + 4 * string_words(p);
     s.smem_single = ring + 4 * (p.AW + std::max(string_words(p), 32 * p.RP + 1));
     s.smem_step = 4 * arrays * p.AW;
     s.smem_bytes = 4 * (arrays * p.AW + 32 * p.RP + 1);
+    return std::max(std::max(s.smem_pack, s.smem_single), std::max(s.smem_step, s.smem_bytes)) <= kSliceMost;
+}
+
+// Blocks of a kernel that fill the GPU, once its shared memory is allowed.
+template <class Fn>
+static cudaError_t slice_grid(Fn fn, int block, int smem, int num_sms, int64_t groups, int *grid)
+{
+    int per_sm = 0;
+    cudaError_t e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, kSliceMost);
+    if (e == cudaSuccess) e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, fn, block, smem);
+    if (e == cudaSuccess && per_sm < 1) e = cudaErrorInvalidConfiguration;
+    *grid = (int)std::min<int64_t>((int64_t)per_sm * num_sms, groups);
+    return e;
+}
+
+// Makes what a call still lacks: the tables, and with `packed` the packed
+// states of its kind.  The kernels of the routes that need no packed state
+// are set up with the tables (a later call may be captured), the others with
+// the first packed state.
+static int slice_prepare(fractal *f, bool packed, int64_t steps, cudaStream_t st)
+{
+    const bool tables = f->slice.state < 2;
+    SlicePlan s = f->slice;   // (the handle's changes only when everything is there)
+    SliceGeo &p = s.geo;
+    const int states = !packed ? 0 : (steps == 1 ? 1 : 2);
     std::vector<uint8_t> host;
-    cudaError_t e = slice_upload(p, *img, s, {}, host, st);
-    if (e == cudaSuccess) {
-        const int64_t blocks = std::min<int64_t>((32 * p.NG + 255) / 256, (int64_t)f->num_sms * 16);
-        if (f->dim == 3)
-            slice_nbr_kernel<3><<<(unsigned)blocks, 256, 0, st>>>(f->dev, p.NT, p.NG, f->r - p.L, (int32_t)pw(f->s, f->r - p.L), nullptr, p.nbr);
-        else
-            slice_nbr_kernel<2><<<(unsigned)blocks, 256, 0, st>>>(f->dev, p.NT, p.NG, f->r - p.L, (int32_t)pw(f->s, f->r - p.L), nullptr, p.nbr);
-        e = cudaGetLastError();
+    uint8_t *mem = nullptr;
+    cudaError_t e = cudaSuccess;
+    if (tables) {
+        e = slice_upload(p, *slice_image(f, p.L), s, {}, states, host, st);
+        mem = s.arena;
+        if (e == cudaSuccess) {
+            const unsigned blocks = (unsigned)std::min<int64_t>((32 * p.NG + 255) / 256, (int64_t)f->num_sms * 16);
+            const int levels = f->r - p.L;
+            const int32_t side = (int32_t)pw(f->s, levels);
+            if (f->dim == 3) slice_nbr_kernel<3><<<blocks, 256, 0, st>>>(f->dev, p.NT, p.NG, levels, side, nullptr, p.nbr);
+            else slice_nbr_kernel<2><<<blocks, 256, 0, st>>>(f->dev, p.NT, p.NG, levels, side, nullptr, p.nbr);
+            e = cudaGetLastError();
+        }
+        // the kernels while the tables are on their way
+        if (e == cudaSuccess && s.resident) e = resident_ready(s);
+        for (int life = 0; life < 2 && p.D <= 8 && p.H <= kSliceSingleHalo && e == cudaSuccess; ++life)
+            e = slice_grid(single_fn(p.D, life), kSliceBlock, s.smem_single, f->num_sms, p.NG, &s.grid_single[life]);
+    } else if (states) {
+        e = cudaMalloc(&mem, states * slice_packed_bytes(p));
+        if (e == cudaSuccess) slice_set_packed(s, states, s.packed[states == 1] = mem);
+    }
+    if (packed && s.grid_pack == 0 && e == cudaSuccess) {
+        auto pack = f->dim == 3 ? slice_pack_kernel<kSliceBlock3> : slice_pack_kernel<kSliceBlock>;
+        e = slice_grid(pack, s.block, s.smem_pack, f->num_sms, p.NG, &s.grid_pack);
+        for (int life = 0; life < 2 && e == cudaSuccess; ++life) {
+            e = slice_grid(step_fn(p.D, life, false), s.block, s.smem_step, f->num_sms, p.NG, &s.grid_step[life]);
+            if (e == cudaSuccess) e = slice_grid(step_fn(p.D, life, true), s.block, s.smem_bytes, f->num_sms, p.NG, &s.grid_bytes[life]);
+        }
+    }
+    if (tables && mem) {
         const cudaError_t landed = cudaStreamSynchronize(st);   // the tables serve calls on any stream from here on
         if (e == cudaSuccess) e = landed;
     }
-    // shared memory and grids
-    int per_sm = 0;
-    if (s.resident && e == cudaSuccess) e = resident_ready(s);
-    {
-        const int most = 112 * 1024;
-        auto pack = f->dim == 3 ? slice_pack_kernel<kSliceBlock3> : slice_pack_kernel<kSliceBlock>;
-        if (std::max(std::max(s.smem_pack, s.smem_single), std::max(s.smem_step, s.smem_bytes)) > most) e = cudaErrorInvalidConfiguration;
-        if (e == cudaSuccess) e = cudaFuncSetAttribute(pack, cudaFuncAttributeMaxDynamicSharedMemorySize, most);
-        if (e == cudaSuccess) e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, pack, s.block, s.smem_pack);
-        for (int life = 0; life < 2 && p.D <= 8 && p.H <= kSliceSingleHalo && e == cudaSuccess; ++life) {
-            int n = 0;
-            e = cudaFuncSetAttribute(single_fn(p.D, life), cudaFuncAttributeMaxDynamicSharedMemorySize, most);
-            if (e == cudaSuccess)
-                e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, single_fn(p.D, life), kSliceBlock, s.smem_single);
-            s.grid_single[life] = (int)std::min<int64_t>((int64_t)n * f->num_sms, p.NG);
-        }
-        s.grid_pack = (int)std::min<int64_t>((int64_t)std::max(per_sm, 1) * f->num_sms, p.NG);
-        for (int life = 0; life < 2 && e == cudaSuccess; ++life)
-            for (int bytes = 0; bytes < 2 && e == cudaSuccess; ++bytes) {
-                StepFn fn = step_fn(p.D, life, bytes);
-                e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, most);
-                if (e == cudaSuccess)
-                    e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, fn, s.block, bytes ? s.smem_bytes : s.smem_step);
-                if (e == cudaSuccess && per_sm < 1) e = cudaErrorInvalidConfiguration;
-                (bytes ? s.grid_bytes : s.grid_step)[life] = (int)std::min<int64_t>((int64_t)per_sm * f->num_sms, p.NG);
-            }
-    }
     if (e != cudaSuccess) {
         cudaGetLastError();
-        free_slice_plan(s);
+        cudaFree(mem);
         return e == cudaErrorMemoryAllocation ? FR_ENOMEM : (e == cudaErrorInvalidConfiguration ? FR_EINVAL : FR_ECUDA);
     }
-    s.state = 1;
+    s.state = 2;
     f->slice = s;
     return FR_OK;
-}
-
-// One packed-state buffer of the streaming kernels, allocated when first needed.
-static bool slice_buffer(fractal *f, int i)
-{
-    SlicePlan &s = f->slice;
-    if (s.bits[i]) return true;
-    if (cudaMalloc(&s.bits[i], (size_t)s.geo.NG * (s.geo.KLp + 32 * s.geo.XW) * sizeof(uint32_t)) == cudaSuccess) return true;
-    cudaGetLastError();
-    s.bits[i] = nullptr;
-    return false;
 }
 
 // Whether a single generation is faster in the tile kernels (one launch, no
@@ -1594,19 +1619,20 @@ int try_slice_step(fractal *f, const uint8_t *in, uint8_t *out, int64_t steps, u
     SlicePlan &s = f->slice;
     if (s.state < 0) return FR_OK;
     if (steps == 1 && slice_one_generation_by_tiles(f, s.state > 0 ? s.geo.H : -1)) return FR_OK;
-    // how the call will run: in one resident or single-pass launch, or with packed states between launches
-    bool res = false, packed = false;
-    auto choose = [&]() {
-        res = slice_use_resident(s, steps, f->num_sms);
-        packed = !res && !(steps == 1 && s.grid_single[0] > 0);
-    };
-    choose();
-    int rc;
     const bool captured = capturing(st);
+    if (s.state == 0) {
+        if (captured) return FR_OK;
+        s.state = plan_slice(f) ? 1 : -1;
+        if (s.state < 0 || (steps == 1 && slice_one_generation_by_tiles(f, s.geo.H))) return FR_OK;
+    }
+    // how the call will run: in one resident or single-pass launch, or with packed states between launches
+    const bool res = slice_use_resident(s, steps, f->num_sms);
+    const bool packed = !res && !(steps == 1 && s.geo.D <= 8 && s.geo.H <= kSliceSingleHalo);
     // under capture nothing is allocated, and a single generation leaves the
     // packed state alone (its replays may run beside other calls): the tile kernels run there
-    const bool ready = s.state > 0 && (!packed || (steps == 1 ? s.bits[2] != nullptr : s.bits[0] && s.bits[1]));
+    const bool ready = s.state > 1 && (!packed || (steps == 1 ? s.bits[2] != nullptr : s.bits[0] && s.bits[1]));
     if (captured && (!ready || (steps == 1 && (res || packed)))) return FR_OK;
+    int rc;
     if (!ready) {
         // after a refused allocation a number of calls go to the tile kernels before the next try
         if (s.wait > 0) {
@@ -1615,18 +1641,10 @@ int try_slice_step(fractal *f, const uint8_t *in, uint8_t *out, int64_t steps, u
         }
         rc = ensure_status(f);
         if (rc) return rc;
-        if (s.state == 0) {
-            rc = build_slice_plan(f, st);
-            if (rc == FR_EINVAL) s.state = -1;
-            else if (rc) s.wait = kSliceWait;
-            if (rc) return FR_OK;
-        }
-        if (steps == 1 && slice_one_generation_by_tiles(f, s.geo.H)) return FR_OK;
-        choose();
-        if (packed && !(steps == 1 ? slice_buffer(f, 2) : slice_buffer(f, 0) && slice_buffer(f, 1))) {
-            s.wait = kSliceWait;
-            return FR_OK;
-        }
+        rc = slice_prepare(f, packed, steps, st);
+        if (rc == FR_EINVAL) s.state = -1;   // (what the handle has stays until it is destroyed)
+        else if (rc) s.wait = kSliceWait;
+        if (rc) return FR_OK;
     }
     const SliceGeo &p = s.geo;
     const SliceArgs a = slice_args(p, birth, survive, steps == 1 ? s.bar + 2 : s.bar, f->status);
@@ -1789,7 +1807,7 @@ int build_slice_batch(const std::vector<SliceBatchItem> &items, uint32_t birth, 
             double c = 0;
             cudaError_t e = slice_resident_shape(p, rep->num_sms, true, &l.plan, &c) ? cudaSuccess : cudaErrorInvalidConfiguration;
             std::vector<uint8_t> host;
-            if (e == cudaSuccess) e = slice_upload(p, *tabs[L], l.plan, groups, host, st);
+            if (e == cudaSuccess) e = slice_upload(p, *tabs[L], l.plan, groups, 0, host, st);
             if (e == cudaSuccess) {
                 const int64_t blocks = std::min<int64_t>((32 * p.NG + 255) / 256, (int64_t)rep->num_sms * 16);
                 slice_nbr_kernel<2><<<(unsigned)blocks, 256, 0, st>>>(rep->dev, p.NT, p.NG, 0, 1,

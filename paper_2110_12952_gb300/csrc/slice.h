@@ -36,7 +36,7 @@ struct SliceGeo {
 
 struct SlicePlan {
     bool several = false;     // a call of several generations has run
-    int state = 0;            // 0: not planned yet, 1: planned, -1: not possible for this fractal
+    int state = 0;            // 0: not planned yet, 1: planned, 2: its tables exist, -1: not possible for this fractal
     int wait = 0;             // calls left to the tile kernels after a refused allocation
     SliceGeo geo;
     bool resident = false;    // the packed state stays in shared memory: one launch for all generations
@@ -46,7 +46,8 @@ struct SlicePlan {
     int grid_pack = 0, grid_step[2] = {0, 0}, grid_bytes[2] = {0, 0}, grid_single[2] = {0, 0};   // [1]: with the constant rule
     // packed states (NG x KLp words, then the exports, NG x XW x 32): two of calls of several generations, one of single ones
     uint32_t *bits[3] = {nullptr, nullptr, nullptr};
-    uint8_t *arena = nullptr;                 // the tables, and:
+    uint8_t *packed[2] = {nullptr, nullptr};  // those that are not in the arena: of several generations, of single ones
+    uint8_t *arena = nullptr;                 // the tables, packed states of the first kind of call that needs some, and:
     uint8_t *groups = nullptr;                // batches: the groups (SliceGroup)
     uint32_t *ex[3] = {nullptr, nullptr, nullptr};   // resident kernel: the exports alone, likewise
     uint32_t *bar = nullptr;                  // grid barriers: arrivals, exits; single generations' own behind them

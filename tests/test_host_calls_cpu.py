@@ -170,3 +170,26 @@ for name, r, steps, room in (("carpet", 9, 4, 1 << 18), ("h_fractal", 10, 3, 1 <
     assert sliced([x for x in kernels() if "step_kernel" in x or "resident" in x]), (name, room)
     lib.fractal_destroy(h)
 """)
+
+
+def test_a_first_call_builds_what_it_uses(host):
+    # calls that the tile kernels serve build no sliced tables; the others make one allocation for all they need
+    host("""
+def first(name, r, steps):
+    h = handle(name, r)
+    assert lib.fractal_get_tile_levels(h, byref(c_int())) == 0
+    fake.fake_clear()
+    assert step(h, steps) == 0
+    mallocs, syncs = log("^malloc", clear=False), log("^sync", clear=False)
+    names = kernels()
+    assert lib.fractal_destroy(h) == 0
+    return names, len(mallocs), len(syncs)
+for name, r in (("carpet", 7), ("vicsek", 8), ("h_fractal", 6), ("candy", 5)):
+    names, mallocs, syncs = first(name, r, 1)
+    assert (sliced(names), mallocs, syncs) == (False, 0, 0), (name, names, mallocs)
+for name, r, steps in (("triangle", 12, 1), ("carpet", 9, 1), ("carpet", 10, 1), ("carpet", 10, 4), ("menger", 6, 1), ("menger", 6, 3),
+                       ("triangle", 8, 9)):
+    names, mallocs, syncs = first(name, r, steps)
+    assert (sliced(names), mallocs, syncs) == (True, 1, 1), (name, names, mallocs, syncs)
+assert fake.fake_held() == 0
+""")

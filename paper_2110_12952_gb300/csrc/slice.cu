@@ -62,7 +62,7 @@ struct SliceGroup {
     const uint8_t *in;
     uint8_t *out;
     int32_t nt;                 // tiles (at most 32)
-    int32_t tile0, levels, side;   // first tile in its instance; the instance's levels above the tiles, and its side in tiles
+    int32_t tile0, levels;      // first tile in its instance, the instance's levels above the tiles
     int32_t group0;             // the instance's first group
     int32_t steps;              // generations; groups come in order of decreasing steps
 };
@@ -885,12 +885,31 @@ slice_resident_kernel(SliceArgs a, const uint8_t *__restrict__ in, uint8_t *__re
     }
 }
 
-// Neighbours of every tile, a row of 32 lanes per group and direction
-// (tiles past the last have none), from rows of 8 per tile.
+// Neighbours of every tile, a row of 32 lanes per group and direction (tiles
+// past the last have none).  A move changes the lowest digit, and goes on one
+// level up in the direction it leaves the block in; most end after a digit or
+// two, where lambda and nu would decode every level of every neighbour
+// (triangle r = 20, 1.6 million tiles: see slice_prepare).
 template <int DIM>
-__global__ void slice_nbr_kernel(FracDev F, int64_t NT, int64_t NG, int coarse_levels, int32_t coarse_side,
-                                 const SliceGroup *__restrict__ groups, int32_t *__restrict__ out)
+__global__ void __launch_bounds__(256) slice_nbr_kernel(FracDev F, int64_t NT, int64_t NG, int levels,
+                                                        const SliceGroup *__restrict__ groups, int32_t *__restrict__ out)
 {
+    constexpr int Q = DIM == 3 ? 27 : 9, ND = Q - 1;
+    extern __shared__ int16_t moved[];   // [k][Q]: a replica's neighbour | the direction left to move one level up << 8, or -1
+    for (int i = threadIdx.x; i < F.k * Q; i += blockDim.x) {
+        const int j = i / Q;
+        int d = i - j * Q, t = 0, w = 1, up = 0, w3 = 1;
+        for (int a = 0; a < DIM; ++a) {
+            const int q = F.off[j][a] + d % 3 - 1, b = q < 0 ? -1 : (q >= F.s ? 1 : 0);
+            t += (q - b * F.s) * w;
+            up += (b + 1) * w3;
+            w *= F.s;
+            w3 *= 3;
+            d /= 3;
+        }
+        moved[i] = F.hinv[t] < 0 ? (int16_t)-1 : (int16_t)(F.hinv[t] | up << 8);
+    }
+    __syncthreads();
     for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < 32 * NG; i += (int64_t)gridDim.x * blockDim.x) {
         int64_t T = i, base = 0;
         bool live = T < NT;
@@ -899,19 +918,21 @@ __global__ void slice_nbr_kernel(FracDev F, int64_t NT, int64_t NG, int coarse_l
             live = (i & 31) < s.nt;
             T = s.tile0 + (i & 31);
             base = 32 * (int64_t)s.group0;
-            coarse_levels = s.levels;
-            coarse_side = s.side;
+            levels = s.levels;
         }
-        int32_t c[3] = {0, 0, 0};
-        if (live) lambda64(F, (uint64_t)T, coarse_levels, c);
-        constexpr int ND = DIM == 3 ? 26 : 8;
         for (int d = 0; d < ND; ++d) {
-            const int q = d < ND / 2 ? d : d + 1;
-            const int32_t x = c[0] + q % 3 - 1, y = c[1] + (q / 3) % 3 - 1, z = DIM == 3 ? c[2] + q / 9 - 1 : 0;
-            int64_t v = -1;
-            if (live && x >= 0 && x < coarse_side && y >= 0 && y < coarse_side && z >= 0 && z < coarse_side)
-                v = nu_levels(F, x, y, z, coarse_levels);
-            out[((i >> 5) * ND + d) * 32 + (i & 31)] = v < 0 ? -1 : (int32_t)(base + v);
+            int dir = live ? (d < ND / 2 ? d : d + 1) : -1;
+            uint32_t rest = (uint32_t)T, below = 0, w = 1;
+            for (int l = 0; l < levels && dir >= 0 && dir != Q / 2; ++l) {
+                const uint32_t q = divu(F.kdiv, rest);
+                const int e = moved[(rest - q * (uint32_t)F.k) * Q + dir];
+                below += (uint32_t)(e & 0xff) * w;
+                w *= (uint32_t)F.k;
+                rest = q;
+                dir = e >> 8;
+            }
+            // (a move left over at the top leaves the box)
+            out[((i >> 5) * ND + d) * 32 + (i & 31)] = dir == Q / 2 ? (int32_t)(base + below + rest * w) : -1;
         }
     }
 }
@@ -1474,10 +1495,9 @@ static int slice_prepare(fractal *f, bool packed, int64_t steps, cudaStream_t st
         mem = s.arena;
         if (e == cudaSuccess) {
             const unsigned blocks = (unsigned)std::min<int64_t>((32 * p.NG + 255) / 256, (int64_t)f->num_sms * 16);
-            const int levels = f->r - p.L;
-            const int32_t side = (int32_t)pw(f->s, levels);
-            if (f->dim == 3) slice_nbr_kernel<3><<<blocks, 256, 0, st>>>(f->dev, p.NT, p.NG, levels, side, nullptr, p.nbr);
-            else slice_nbr_kernel<2><<<blocks, 256, 0, st>>>(f->dev, p.NT, p.NG, levels, side, nullptr, p.nbr);
+            const int moves = f->k * (p.ND + 1) * (int)sizeof(int16_t);
+            if (f->dim == 3) slice_nbr_kernel<3><<<blocks, 256, moves, st>>>(f->dev, p.NT, p.NG, f->r - p.L, nullptr, p.nbr);
+            else slice_nbr_kernel<2><<<blocks, 256, moves, st>>>(f->dev, p.NT, p.NG, f->r - p.L, nullptr, p.nbr);
             e = cudaGetLastError();
         }
         // the kernels while the tables are on their way
@@ -1790,10 +1810,10 @@ int build_slice_batch(const std::vector<SliceBatchItem> &items, uint32_t birth, 
             for (; i < in.size() && (i == i0 || (int64_t)groups.size() + groups_of(*in[i], L) <= best[b].cap); ++i) {
                 const SliceBatchItem &it = *in[i];
                 const int64_t NT = pw(rep->k, it.f->r - L), n = groups_of(it, L);
-                const int32_t g0 = (int32_t)groups.size(), levels = it.f->r - L, side = (int32_t)pw(rep->s, it.f->r - L);
+                const int32_t g0 = (int32_t)groups.size(), levels = it.f->r - L;
                 for (int64_t g = 0; g < n; ++g)
                     groups.push_back(SliceGroup{it.in + 32 * g * geos[L].KL, it.out + 32 * g * geos[L].KL,
-                                                (int32_t)std::min<int64_t>(32, NT - 32 * g), (int32_t)(32 * g), levels, side, g0,
+                                                (int32_t)std::min<int64_t>(32, NT - 32 * g), (int32_t)(32 * g), levels, g0,
                                                 (int32_t)it.steps});
             }
             batch->launches.emplace_back();
@@ -1810,8 +1830,8 @@ int build_slice_batch(const std::vector<SliceBatchItem> &items, uint32_t birth, 
             if (e == cudaSuccess) e = slice_upload(p, *tabs[L], l.plan, groups, 0, host, st);
             if (e == cudaSuccess) {
                 const int64_t blocks = std::min<int64_t>((32 * p.NG + 255) / 256, (int64_t)rep->num_sms * 16);
-                slice_nbr_kernel<2><<<(unsigned)blocks, 256, 0, st>>>(rep->dev, p.NT, p.NG, 0, 1,
-                                                                   reinterpret_cast<const SliceGroup *>(l.plan.groups), p.nbr);
+                slice_nbr_kernel<2><<<(unsigned)blocks, 256, rep->k * 9 * (int)sizeof(int16_t), st>>>(
+                    rep->dev, p.NT, p.NG, 0, reinterpret_cast<const SliceGroup *>(l.plan.groups), p.nbr);
                 e = cudaGetLastError();
                 const cudaError_t landed = cudaStreamSynchronize(st);
                 if (e == cudaSuccess) e = landed;

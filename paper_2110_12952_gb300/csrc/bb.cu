@@ -967,7 +967,12 @@ int try_bb_packed(fractal *f, const uint8_t *in, uint8_t *out, int64_t steps, ui
     if (captured && steps == 1) return FR_OK;
     if (!(steps == 1 ? f->box_words.one : f->box_words.two[0])) {
         // nothing is allocated under capture, and without the memory the row kernels run as before
-        if (captured || !box_words_build(f, a, steps > 1, st)) return FR_OK;
+        if (captured || f->box_words.memory.skip()) return FR_OK;
+        if (!box_words_build(f, a, steps > 1, st)) {
+            f->box_words.memory.refused();
+            return FR_OK;
+        }
+        f->box_words.memory.granted();
     }
     a.member = f->box_words.member;
     a.pseg = (a.RW + kBwSeg - 1) / kBwSeg;

@@ -95,6 +95,7 @@ struct BBPlan {
 struct BoxWords {
     uint32_t *mem[2] = {nullptr, nullptr};
     uint32_t *member = nullptr, *one = nullptr, *two[2] = {nullptr, nullptr};
+    Retry memory;
 };
 
 // Temporal blocking (temporal.cuh): tile depth, tables and launch shape of

@@ -53,7 +53,6 @@ constexpr int kSliceMost = 112 * 1024;   // the other kernels': most shared memo
 constexpr int kSliceSmem = 220 * 1024;   // resident kernel: shared memory per block
 constexpr int64_t kSliceBatchCells = 60000000;   // batches: most cells of an instance
 constexpr int kSliceSingleHalo = 32;   // most halo cells of a tile for the single-pass kernel
-constexpr int kSliceWait = 16;      // calls by the tile kernels after a refused allocation before the next try
 constexpr int kSliceRounds = 32;   // resident kernel: most 32-cell chunks per warp
 
 // One group of a batch: its bytes, its tiles and where its instance lies
@@ -1655,16 +1654,14 @@ int try_slice_step(fractal *f, const uint8_t *in, uint8_t *out, int64_t steps, u
     int rc;
     if (!ready) {
         // after a refused allocation a number of calls go to the tile kernels before the next try
-        if (s.wait > 0) {
-            --s.wait;
-            return FR_OK;
-        }
+        if (s.memory.skip()) return FR_OK;
         rc = ensure_status(f);
         if (rc) return rc;
         rc = slice_prepare(f, packed, steps, st);
         if (rc == FR_EINVAL) s.state = -1;   // (what the handle has stays until it is destroyed)
-        else if (rc) s.wait = kSliceWait;
+        else if (rc) s.memory.refused();
         if (rc) return FR_OK;
+        s.memory.granted();
     }
     const SliceGeo &p = s.geo;
     const SliceArgs a = slice_args(p, birth, survive, steps == 1 ? s.bar + 2 : s.bar, f->status);

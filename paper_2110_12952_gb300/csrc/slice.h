@@ -34,10 +34,28 @@ struct SliceGeo {
     int32_t *nbr = nullptr;      // [NG][ND][32]: neighbouring tile of each tile of a group by direction, -1 = none
 };
 
+// When to try an allocation again that was refused (which takes 5 ms): after
+// 16 calls, after twice as many at each further refusal, at most 1024.
+struct Retry {
+    int left = 0, next = 16;
+    bool skip()   // whether this call goes without
+    {
+        if (left == 0) return false;
+        --left;
+        return true;
+    }
+    void refused()
+    {
+        left = next;
+        next = next < 1024 ? 2 * next : next;
+    }
+    void granted() { next = 16; }
+};
+
 struct SlicePlan {
     bool several = false;     // a call of several generations has run
     int state = 0;            // 0: not planned yet, 1: planned, 2: its tables exist, -1: not possible for this fractal
-    int wait = 0;             // calls left to the tile kernels after a refused allocation
+    Retry memory;             // its allocations
     SliceGeo geo;
     bool resident = false;    // the packed state stays in shared memory: one launch for all generations
     int per_block = 0, rounds = 0, block_resident = 0, grid_resident = 0, smem_resident = 0;

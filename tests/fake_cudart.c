@@ -121,7 +121,10 @@ cudaError_t cudaMalloc(void **p, size_t n)
     int i = 0;
     while (i < MAX && g_blocks[i].p) ++i;
     if (e == cudaSuccess && (g_held + n > g_limit || i == MAX)) e = g_last = cudaErrorMemoryAllocation;
-    if (e != cudaSuccess) return e;
+    if (e != cudaSuccess) {
+        note("refused %zu\n", n);
+        return e;
+    }
     char *q = mmap(NULL, n ? n : 1, PROT_READ | PROT_WRITE, MAP_PRIVATE | MAP_ANONYMOUS | MAP_NORESERVE, -1, 0);
     if (q == MAP_FAILED) return g_last = cudaErrorMemoryAllocation;
     g_blocks[i].p = *p = q;

@@ -114,7 +114,7 @@ assert [x for x in order if x] == ["copy", "tiles", "sliced"], order
 
 
 def test_box_words_are_kept_only_when_filled(host):
-    # a call that cannot fill the packed box's arrays keeps none of them: the next call fills them
+    # a call that cannot fill the packed box's arrays keeps none of them: one of the next calls fills them
     host("""
 for name, r, steps, rule in (("carpet", 5, 3, (8, 12)), ("menger", 4, 1, (32, 48))):
     for call, after in (("cudaMemsetAsync", 0), ("launch", 0), ("cudaStreamSynchronize", 0), ("cudaMalloc", 0)):
@@ -124,7 +124,8 @@ for name, r, steps, rule in (("carpet", 5, 3, (8, 12)), ("menger", 4, 1, (32, 48
         fake.fake_clear()
         fake.fake_fail(call.encode(), after)
         step(h, steps, rule=rule, fn="fractal_bb_step")
-        assert step(h, steps, rule=rule, fn="fractal_bb_step") == 0, lib.fractal_last_error()
+        for _ in range(20):
+            assert step(h, steps, rule=rule, fn="fractal_bb_step") == 0, lib.fractal_last_error()
         names = kernels()
         filled = [i for i, x in enumerate(names) if "bb_member" in x]
         assert filled and any("bb_words" in x for x in names[filled[-1]:]), (name, call, names)
@@ -192,4 +193,27 @@ for name, r, steps in (("triangle", 12, 1), ("carpet", 9, 1), ("carpet", 10, 1),
     names, mallocs, syncs = first(name, r, steps)
     assert (sliced(names), mallocs, syncs) == (True, 1, 1), (name, names, mallocs, syncs)
 assert fake.fake_held() == 0
+""")
+
+
+def test_refused_allocations_are_tried_again_ever_later(host):
+    # a refused allocation takes milliseconds: calls that run on the byte-wise kernels meanwhile do not try each time
+    host("""
+for name, r, fn, size in (("carpet", 7, "fractal_bb_step", 3 ** 14), ("h_fractal", 10, "fractal_step", 7 ** 10)):
+    h = handle(name, r)
+    assert step(h, 1, fn=fn) == 0
+    # room for the byte-wise kernels' scratch alone, then for nothing more
+    fake.fake_fail(b"cudaMalloc", 0)
+    assert step(h, 3, fn=fn) == 0
+    fake.fake_limit(fake.fake_held() + 1000)
+    fake.cudaGetLastError()
+    fake.fake_clear()
+    assert all(step(h, 3, fn=fn) == 0 for _ in range(300))
+    assert 1 <= len(log("^refused")) <= 6, name
+    fake.fake_limit(1 << 60)
+    assert all(step(h, 3, fn=fn) == 0 for _ in range(600))
+    fake.fake_clear()
+    assert step(h, 3, fn=fn) == 0
+    assert any("bb_words" in x or "slice_" in x for x in kernels()), name
+    lib.fractal_destroy(h)
 """)

@@ -937,9 +937,7 @@ static int choose_levels(const fractal *f)
 
 void free_step_plan(StepPlan &p)
 {
-    cudaFree(p.pos);
-    cudaFree(p.ring);
-    cudaFree(p.nbr);
+    cudaFree(p.pos);   // (the others lie behind it)
     p = StepPlan();
 }
 
@@ -1270,17 +1268,19 @@ int ensure_step_plan(fractal *f)
 
     }
     p.nring = p.nhalo ? 0 : (int)(ring.size() / 2);
-    FR_CUDA(cudaMalloc(&p.pos, tab.size() * sizeof(uint32_t)));
-    FR_CUDA(cudaMemcpy(p.pos, tab.data(), tab.size() * sizeof(uint32_t), cudaMemcpyHostToDevice));
+    // one allocation: the table, the ring, the neighbour-tile table
+    const size_t ring_at = (tab.size() + 63) / 64 * 64, nbr_at = ring_at + (ring.size() + 63) / 64 * 64;
+    FR_CUDA(cudaMalloc(&p.pos, nbr_at * sizeof(uint32_t) + (size_t)p.NT * p.nbrw * sizeof(int32_t)));
     if (!ring.empty()) {
-        FR_CUDA(cudaMalloc(&p.ring, ring.size() * sizeof(uint32_t)));
-        FR_CUDA(cudaMemcpy(p.ring, ring.data(), ring.size() * sizeof(uint32_t), cudaMemcpyHostToDevice));
+        tab.resize(ring_at, 0u);
+        tab.insert(tab.end(), ring.begin(), ring.end());
+        p.ring = p.pos + ring_at;
     }
-    // neighbour-tile table
-    cudaError_t e = cudaMalloc(&p.nbr, (size_t)p.NT * p.nbrw * sizeof(int32_t));
+    p.nbr = reinterpret_cast<int32_t *>(p.pos + nbr_at);
+    const cudaError_t e = cudaMemcpy(p.pos, tab.data(), tab.size() * sizeof(uint32_t), cudaMemcpyHostToDevice);
     if (e != cudaSuccess) {
         free_step_plan(p);
-        return cuda_fail(e, "fractal_step: neighbour table allocation");
+        return cuda_fail(e, "fractal_step: table upload");
     }
     rc = launch_nbr_table(f, p.NT, p.coarse_levels, p.nbrw, p.nbr);
     if (rc) {

@@ -1451,16 +1451,18 @@ static cudaError_t slice_upload(SliceGeo &p, SliceImage &image, SlicePlan &s, co
 // The plan, on the host alone: the tile depth and the shared memory.
 static bool plan_slice(fractal *f)
 {
-    SlicePlan &s = f->slice;
+    SlicePlan s;
     std::shared_ptr<SliceImage> img;
     if (slice_levels(f, &s, &img) < 1) return false;
     const SliceGeo &p = s.geo;
+    s.single = f->slice.single;
     s.block = f->dim == 3 ? kSliceBlock3 : kSliceBlock;
     const int ring = 16 * kSliceBatch * s.block, arrays = f->dim == 3 ? 1 : 2;
     s.smem_pack = ring + 4 * string_words(p);
     s.smem_single = ring + 4 * (p.AW + std::max(string_words(p), 32 * p.RP + 1));
     s.smem_step = 4 * arrays * p.AW;
     s.smem_bytes = 4 * (arrays * p.AW + 32 * p.RP + 1);
+    f->slice = s;
     return std::max(std::max(s.smem_pack, s.smem_single), std::max(s.smem_step, s.smem_bytes)) <= kSliceMost;
 }
 
@@ -1647,6 +1649,15 @@ int try_slice_step(fractal *f, const uint8_t *in, uint8_t *out, int64_t steps, u
     // how the call will run: in one resident or single-pass launch, or with packed states between launches
     const bool res = slice_use_resident(s, steps, f->num_sms);
     const bool packed = !res && !(steps == 1 && s.geo.D <= 8 && s.geo.H <= kSliceSingleHalo);
+    // a handle's first single generation (of those that use packed states:
+    // they run on the tile kernels under capture in any case) does not pay for
+    // the tables, unless the state is large: first call of the H-fractal at
+    // r = 8 with them 314 us, without 212, the next ones 8 against 18; Menger
+    // r = 6 677 and 575, then 51 and 104; r = 7 1436 and 2150
+    if (steps == 1 && (res || packed) && s.state == 1 && !captured && !s.single && f->cells < (f->dim == 3 ? 1 << 27 : 1 << 30)) {
+        s.single = true;
+        return FR_OK;
+    }
     // under capture nothing is allocated, and a single generation leaves the
     // packed state alone (its replays may run beside other calls): the tile kernels run there
     const bool ready = s.state > 1 && (!packed || (steps == 1 ? s.bits[2] != nullptr : s.bits[0] && s.bits[1]));

@@ -54,6 +54,7 @@ struct Retry {
 
 struct SlicePlan {
     bool several = false;     // a call of several generations has run
+    bool single = false;      // a single generation has run on the tile kernels before the tables were built
     int state = 0;            // 0: not planned yet, 1: planned, 2: its tables exist, -1: not possible for this fractal
     Retry memory;             // its allocations
     SliceGeo geo;

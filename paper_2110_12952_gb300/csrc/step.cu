@@ -2998,6 +2998,7 @@ int autotune_step(fractal *f, const uint8_t *in, uint8_t *out, uint32_t birth, u
     bool sliced = false;
     {
         float ms = 0.f;
+        f->slice.single = true;   // (its first call is not left to the tile kernels)
         if (best >= 0 && time_calls(
                              [&]() {
                                  bool done = false;

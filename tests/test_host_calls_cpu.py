@@ -72,7 +72,7 @@ def test_tables_outlive_their_copy(host):
     host("""
 for name, r, steps in (("triangle", 8, 5), ("carpet", 8, 1), ("carpet", 10, 3), ("menger", 6, 1)):
     h = handle(name, r)
-    assert step(h, steps, stream=0x70) == 0
+    assert step(h, steps, stream=0x70) == 0 and step(h, steps, stream=0x70) == 0
     assert not log("source changed", clear=False), name
     assert sliced(kernels()), name
 b = c_void_p()
@@ -188,7 +188,7 @@ def first(name, r, steps):
 for name, r in (("carpet", 7), ("vicsek", 8), ("h_fractal", 6), ("candy", 5)):
     names, mallocs, syncs = first(name, r, 1)
     assert (sliced(names), mallocs, syncs) == (False, 0, 0), (name, names, mallocs)
-for name, r, steps in (("triangle", 12, 1), ("carpet", 9, 1), ("carpet", 10, 1), ("carpet", 10, 4), ("menger", 6, 1), ("menger", 6, 3),
+for name, r, steps in (("triangle", 12, 1), ("carpet", 10, 1), ("carpet", 10, 4), ("menger", 7, 1), ("menger", 6, 3),
                        ("triangle", 8, 9)):
     names, mallocs, syncs = first(name, r, steps)
     assert (sliced(names), mallocs, syncs) == (True, 1, 1), (name, names, mallocs, syncs)
@@ -216,4 +216,28 @@ for name, r, fn, size in (("carpet", 7, "fractal_bb_step", 3 ** 14), ("h_fractal
     assert step(h, 3, fn=fn) == 0
     assert any("bb_words" in x or "slice_" in x for x in kernels()), name
     lib.fractal_destroy(h)
+""")
+
+
+def test_a_single_call_does_not_pay_for_tables(host):
+    # a handle's first single generation runs on the tile kernels unless the state is large or needs no packed state;
+    # the second one, a call of several and the autotuner have the tables built
+    host("""
+def calls(name, r, *steps):
+    h, out = handle(name, r), []
+    for n in steps:
+        fake.fake_clear()
+        assert step(h, n) == 0
+        out.append(sliced(kernels()))
+    lib.fractal_destroy(h)
+    return out
+for name, r in (("carpet", 9), ("h_fractal", 8), ("menger", 6)):
+    assert calls(name, r, 1, 1, 1) == [False, True, True], name
+    assert calls(name, r, 1, 3) == [False, True], name
+    assert calls(name, r, 3, 1) == [True, True], name
+for name, r in (("carpet", 10), ("menger", 7), ("triangle", 14)):
+    assert calls(name, r, 1) == [True], name
+h = handle("carpet", 9)
+assert lib.fractal_autotune(h, c_void_p(A), c_void_p(B), 8, 12, None, None) == 0
+assert sliced(kernels())
 """)

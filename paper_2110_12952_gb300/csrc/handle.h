@@ -200,6 +200,7 @@ bool capturing(cudaStream_t st);
 int packed_enter(fractal *f, cudaStream_t st, bool captured);
 int packed_leave(fractal *f, cudaStream_t st, bool captured);
 void keep_generation_buffers(fractal *f);
+double short_generation_us(const fractal *f, int64_t NT);
 int rows_preset_of(const fractal *f);   // 0: the carpet, 1: the Vicsek fractal (preset offsets), -1: another
 int ensure_tb_plan(fractal *f);
 void fr_paper_aux_free(fractal *f);

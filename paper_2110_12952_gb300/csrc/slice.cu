@@ -1548,6 +1548,29 @@ static bool slice_one_generation_by_tiles(const fractal *f, int halo_cells)
     return f->cells < (preset == 0 ? 4 << 20 : 1 << 20);
 }
 
+// Whether a few generations of a small state are faster in the tile kernels,
+// a launch each, than in the sliced step's launches and grid barriers.  Per
+// call, tiles -> sliced: 2D, two generations, more than a chunk per warp: the
+// triangle r = 10 12.4 -> 13.4 us, Vicsek r = 7 12.5 -> 15.8, r = 10 18.7 ->
+// 20.1 (three generations of all of them are faster sliced).  3D: two
+// generations of Menger r = 2 11.7 -> 16.4 us, k = 4, s = 2, r = 8 two, four
+// and ten generations 12.6 -> 22.7, 24.8 -> 33.0, 61.7 -> 66.7, and the full
+// cube with s = 2, r = 6 two and six 20.6 -> 29.0, 61.7 -> 64.7.  The sliced
+// step's times there: three launches, and per generation a group's work, the
+// barrier once there are several groups, more groups than two per SM.
+static bool slice_few_generations_by_tiles(const fractal *f, const SlicePlan &s, int64_t steps)
+{
+    if (steps < 2 || steps > 64) return false;
+    const double tiles = (double)steps * short_generation_us(f, f->plan.NT);
+    if (f->dim == 2) {
+        if (steps != 2 || (s.resident && s.grid_resident == 1 && s.rounds == 1)) return false;
+        return tiles > 0.0 || (rows_preset_of(f) == 1 && f->plan.NT <= 5 * (int64_t)f->num_sms);
+    }
+    const double n = (double)steps, waves = (double)((s.geo.NG + 2 * f->num_sms - 1) / (2 * f->num_sms));
+    const double sliced = s.geo.NG == 1 ? 11.5 + 2.0 * n : (s.geo.NG <= f->num_sms ? 8.0 + 4.1 * n : 11.0 + (2.6 + 1.5 * waves) * n);
+    return tiles > 0.0 && tiles < sliced;
+}
+
 // Whether `steps` generations run in the resident kernel.  A single
 // generation of a state with many groups is faster as streaming launches.
 static bool slice_use_resident(const SlicePlan &s, int64_t steps, int num_sms)
@@ -1646,6 +1669,8 @@ int try_slice_step(fractal *f, const uint8_t *in, uint8_t *out, int64_t steps, u
         s.state = plan_slice(f) ? 1 : -1;
         if (s.state < 0 || (steps == 1 && slice_one_generation_by_tiles(f, s.geo.H))) return FR_OK;
     }
+    // (a captured call takes what exists: its handle may have no scratch for the tile kernels)
+    if (!captured && slice_few_generations_by_tiles(f, s, steps)) return FR_OK;
     // how the call will run: in one resident or single-pass launch, or with packed states between launches
     const bool res = slice_use_resident(s, steps, f->num_sms);
     const bool packed = !res && !(steps == 1 && s.geo.D <= 8 && s.geo.H <= kSliceSingleHalo);

@@ -1061,6 +1061,24 @@ static int configure_bit3(StepPlan &p, int num_sms)
 // Selector nibble that yields a zero byte (sign of a byte whose msb is 0).
 static constexpr uint32_t kZeroSel = 0x8;
 
+// About how long one generation of NT tiles takes in the tile kernels of the
+// handle's plan (us, as launches follow each other), where that is little more
+// than a launch; 0 where it is not known.  Measured: 6.2 for the tap, rows and
+// lid kernels with a tile per SM, and for groups of at most 2048 cells a tile;
+// box3 tiles of 256 / 2401 / 4096 cells 6.2 / 8.2 / 8.2, of 343 at three per
+// SM 8.2, of 4096 at four 12.3.
+double short_generation_us(const fractal *f, int64_t NT)
+{
+    const StepPlan &p = f->plan;
+    const double per_sm = (double)((NT + f->num_sms - 1) / f->num_sms);
+    switch (p.mode) {
+        case kModeTap: case kModeRows0: case kModeRows1: case kModeLid1: return per_sm <= 1 ? 6.2 : 0.0;
+        case kModeGroup3: case kModeGroup4: return p.KL <= 2048 && per_sm <= 2 ? 6.2 : 0.0;
+        case kModeBox3: return NT <= p.grid ? std::max(6.2, 4.5 + (double)p.KL / 900.0 + per_sm) : 0.0;
+        default: return 0.0;
+    }
+}
+
 // What the tile kernels need for calls of several generations, for handles
 // that have run such calls in the sliced step and then leave it for the tile
 // kernels: such a call may be captured next, where nothing can be allocated.

@@ -241,3 +241,22 @@ h = handle("carpet", 9)
 assert lib.fractal_autotune(h, c_void_p(A), c_void_p(B), 8, 12, None, None) == 0
 assert sliced(kernels())
 """)
+
+
+def test_a_few_generations_of_small_states(host):
+    # two generations (3D: a few) of small states are a launch each of the tile kernels; a captured call takes what exists
+    host("""
+def call(h, n):
+    fake.fake_clear()
+    assert step(h, n) == 0, lib.fractal_last_error()
+    return sliced(kernels())
+for name, r, most in (("triangle", 10, 2), ("triangle", 12, 2), ("vicsek", 7, 2), ("vicsek", 10, 2), ("chandelier", 9, 2), ("menger", 2, 2),
+                      ("triangle", 8, 1), ("carpet", 8, 1), ("full_square", 8, 1), ("menger", 3, 1), ("vicsek", 5, 1)):
+    h = handle(name, r)
+    assert [call(h, n) for n in (2, 3, 4, 10)] == [n > most for n in (2, 3, 4, 10)], (name, r)
+    lib.fractal_destroy(h)
+h = handle("triangle", 10)
+assert call(h, 3)
+fake.fake_capturing(1)
+assert call(h, 2) and not log("malloc")
+""")

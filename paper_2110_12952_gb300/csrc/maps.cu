@@ -60,7 +60,12 @@ constexpr int kMapGroups = 16;      // most groups of levels
 constexpr int kMapBlock = 512;
 constexpr int kMapBlocksPerSM = 4;
 constexpr int64_t kMapLong = 20000000;  // points x levels x replicas from which arrays go through tables
-constexpr int64_t kViewLong = 1 << 16;  // cells from which the box views go by tiles
+// Cells from which the box views go by tiles.  Scatter and gather, cell by
+// cell -> by tiles: 160,000 cells (Menger r = 4) 10.4 -> 11.9 and 7.4 -> 7.5 us,
+// 262,144 (carpet r = 6) 10.4 -> 12.0 and 7.1 -> 7.5, 390,625 (Vicsek r = 8)
+// 22.7 -> 24.7 and 8.4 -> 10.1, 531,441 (triangle r = 12) 16.5 -> 16.5 and 10.4
+// -> 10.4, 823,543 (H-fractal r = 7) 18.5 -> 14.5 and 14.4 -> 10.4.
+constexpr int64_t kViewLong = 1 << 19;
 constexpr int64_t kMapBuild = 8;        // a block's points take at least this many times the digit steps of its tables
 
 // lambda through tables: entry i holds the coordinates of i over m levels

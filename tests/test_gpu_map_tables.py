@@ -89,3 +89,27 @@ def test_large_boxes_filled(name, r):
     assert torch.equal(g.gather(box), x)
     assert int(box.max()) == 1 and int(box.sum(dtype=torch.int64)) == int(x.sum(dtype=torch.int64))
     g.close()
+
+
+@pytest.mark.parametrize("name,r", [("triangle", 12), ("carpet", 7), ("h_fractal", 7), ("full_square", 10), ("menger", 5), ("candy", 6)])
+def test_longer_box_views_by_tiles(name, r):
+    # states from the length on at which the views go by tiles, against the oracle, at any address
+    test_box_views_by_tiles(name, r)
+
+
+@pytest.mark.parametrize("name,r", [("triangle", 20), ("carpet", 9), ("menger", 6), ("vicsek", 12)])
+def test_largest_coordinates_are_outside(name, r):
+    # coordinates up to the type's ends, along each axis, in arrays that go through tables
+    from paper_2110_12952_gb300 import Fractal
+    fam = W.FAMILIES[name]
+    g, o = Fractal.from_family(fam, r), oracle.Fractal(fam.k, fam.s, r, fam.dim, fam.table())
+    rng = np.random.default_rng(r)
+    c = o.lam(rng.integers(0, o.cells, N, dtype=np.int64)).astype(np.int32)
+    ends = np.array([2**31 - 1, 2**31 - 2, -2**31, -1, o.side, o.side - 1, 0, 1 << 30, -(1 << 30)], dtype=np.int32)
+    for a in range(fam.dim):
+        c[a * 5000:(a + 1) * 5000 - 1000, a] = np.resize(ends, 4000)
+    c[20000:24000] = ends[rng.integers(0, len(ends), (4000, fam.dim))]
+    d = torch.from_numpy(c).cuda()
+    assert np.array_equal(g.nu(d).cpu().numpy(), o.nu(c))
+    assert np.array_equal(g.nu2d(d).cpu().numpy(), o.nu2d(c))
+    g.close()

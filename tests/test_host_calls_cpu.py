@@ -260,3 +260,14 @@ assert call(h, 3)
 fake.fake_capturing(1)
 assert call(h, 2) and not log("malloc")
 """)
+
+
+def test_short_box_views_go_cell_by_cell(host):
+    host("""
+for name, r, tiles in (("menger", 4, False), ("carpet", 6, False), ("vicsek", 8, False), ("triangle", 12, True), ("h_fractal", 7, True)):
+    h = handle(name, r)
+    fake.fake_clear()
+    assert lib.fractal_scatter_to_box(h, c_void_p(A), c_void_p(B), None) == 0
+    assert lib.fractal_gather_from_box(h, c_void_p(A), c_void_p(B), None) == 0
+    assert ["box_tiles" in x for x in kernels()] == [tiles, tiles], (name, r)
+""")

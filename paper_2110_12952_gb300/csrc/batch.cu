@@ -22,6 +22,7 @@
 #include <algorithm>
 #include <map>
 #include <new>
+#include <set>
 #include <string>
 #include <tuple>
 #include <vector>
@@ -126,6 +127,17 @@ static int build(fractal_batch *b)
             by_table[key].push_back(i);
         }
         for (auto &e : by_table) {
+            // two generations of one class whose launches are short: 5.5 us each
+            // there, about 14 in the sliced launch (three fractals with an
+            // instance each, two generations: 33 and 43 us)
+            std::set<std::string> classes;
+            int64_t most = 0, tiles = 0;
+            for (int i : e.second) {
+                classes.insert(class_key(b->insts[i].f));
+                most = std::max(most, b->insts[i].steps);
+                tiles += b->insts[i].f->plan.NT;
+            }
+            if (most == 2 && classes.size() == 1 && short_generation_us(b->insts[e.second[0]].f, tiles) > 0.0) continue;
             std::vector<SliceBatchItem> items;
             for (int i : e.second) items.push_back({b->insts[i].f, b->insts[i].in, b->insts[i].out, b->insts[i].steps});
             SliceBatch *s = nullptr;

@@ -271,3 +271,24 @@ for name, r, tiles in (("menger", 4, False), ("carpet", 6, False), ("vicsek", 8,
     assert lib.fractal_gather_from_box(h, c_void_p(A), c_void_p(B), None) == 0
     assert ["box_tiles" in x for x in kernels()] == [tiles, tiles], (name, r)
 """)
+
+
+def test_batches_of_two_short_generations(host):
+    # one class of instances and two generations: a launch of the tile kernels each; more classes or generations go sliced
+    host("""
+def run(*instances):
+    b = c_void_p()
+    assert lib.fractal_batch_create(byref(b)) == 0
+    for i, (name, r, n) in enumerate(instances):
+        assert lib.fractal_batch_add(b, handle(name, r), c_void_p(A + (i << 28)), c_void_p(B + (i << 28)), c_int64(n), 8, 12, None) == 0
+    fake.fake_clear()
+    assert lib.fractal_batch_run(b, None) == 0
+    names = [x for x in kernels() if "resident" in x or "step_" in x]
+    lib.fractal_batch_destroy(b)
+    return sliced(names), len(names)
+assert run(("triangle", 12, 2), ("triangle", 12, 2)) == (False, 2)
+assert run(("triangle", 10, 2), ("carpet", 6, 2), ("vicsek", 8, 2)) == (False, 6)
+assert run(("triangle", 12, 3), ("triangle", 12, 2))[0]
+assert run(("triangle", 12, 2), ("triangle", 4, 2), ("triangle", 5, 2))[0]
+assert run(("triangle", 16, 2))[0]
+""")

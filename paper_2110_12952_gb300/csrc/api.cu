@@ -272,7 +272,7 @@ extern "C" int fractal_set_tile_levels(fractal_t *f, int levels)
         return fail(FR_EINVAL, "fractal_set_tile_levels: levels must be -1 or in [0, r]");
     if (levels != f->tile_levels_user && f->server_refs.load() > 0)
         return fail(FR_EBUSY, "fractal_set_tile_levels: a server still holds requests on this handle");
-    f->tuned = f->sliced_tuned = false;
+    f->levels_tuned = f->sliced_tuned = false;
     if (levels != f->tile_levels_user) {
         f->tile_levels_user = levels;
         cudaDeviceSynchronize();
@@ -289,7 +289,7 @@ extern "C" int fractal_set_pipeline_stages(fractal_t *f, int stages)
         return fail(FR_EINVAL, "fractal_set_pipeline_stages: stages must be -1 or in [2, 4]");
     if (stages != f->stages_user && f->server_refs.load() > 0)
         return fail(FR_EBUSY, "fractal_set_pipeline_stages: a server still holds requests on this handle");
-    f->tuned = f->sliced_tuned = false;
+    f->stages_tuned = false;
     if (stages != f->stages_user) {
         f->stages_user = stages;
         cudaDeviceSynchronize();

@@ -155,8 +155,9 @@ struct fractal {
     int tb_levels_user = -1;         // its tile depth (-1 = automatic)
     fr::TbPlan tb;
     fr::SlicePlan slice;             // the bit-sliced step
-    bool tuned = false;              // the tile depth and stages are the autotuner's (it times single generations) ...
-    bool sliced_tuned = false;       // ... which found the sliced step faster still
+    // the tile depth (the stage count) is the autotuner's, which times single
+    // generations, and that it found the sliced step faster still
+    bool levels_tuned = false, stages_tuned = false, sliced_tuned = false;
     void *paper_aux = nullptr;       // the paper's approaches (paper_kernels.cu): geometry and scratch
     // a different transition table per level (fractal_create_mixed); then
     // `offsets` holds the levels' tables one after the other
@@ -172,11 +173,12 @@ struct fractal {
 namespace fr {
 
 // Whether the handle's settings leave the call to the sliced step's rules: a
-// tile depth or stage count set by the caller asks for the tile kernels, one
-// set by the autotuner speaks for single generations only.
+// tile depth or stage count set by the caller asks for the tile kernels, a
+// depth set by the autotuner speaks for single generations only.
 inline bool slice_settings(const fractal *f, int64_t steps)
 {
-    return (f->tile_levels_user < 0 && f->stages_user < 0) || (f->tuned && (steps > 1 || f->sliced_tuned));
+    if ((f->tile_levels_user >= 0 && !f->levels_tuned) || (f->stages_user >= 0 && !f->stages_tuned)) return false;
+    return f->tile_levels_user < 0 || steps > 1 || f->sliced_tuned;
 }
 
 // cells of a level-L subtree (product of the replica counts of levels

@@ -313,6 +313,7 @@ extern "C" int fractal_shard_attach(fractal_shard_t *p, fractal_t *f)
         return shard_fail(FR_EINVAL, "fractal_shard_attach: the handle is not the plan's fractal");
     if (f->server_refs.load() > 0)
         return shard_fail(FR_EBUSY, "fractal_shard_attach: a server still holds requests on this handle");
+    f->levels_tuned = f->sliced_tuned = false;
     if (f->tile_levels_user != p->L) {
         f->tile_levels_user = p->L;
         cudaDeviceSynchronize();

@@ -2962,7 +2962,7 @@ void apply_tuned(fractal *f)
     if (it == g_tune_cache.end()) return;
     f->tile_levels_user = it->second.levels;
     f->stages_user = it->second.stages;
-    f->tuned = true;
+    f->levels_tuned = f->stages_tuned = true;
     f->sliced_tuned = it->second.sliced;
 }
 
@@ -2976,7 +2976,7 @@ int autotune_step(fractal *f, const uint8_t *in, uint8_t *out, uint32_t birth, u
 {
     int lmax = 0;
     f->stages_user = -1;
-    f->tuned = f->sliced_tuned = false;
+    f->levels_tuned = f->stages_tuned = f->sliced_tuned = false;
     for (int L = 0; L <= f->r; ++L) {
         if (plan_layout(f, L).total > 200 * 1024) break;
         lmax = L;
@@ -3036,7 +3036,7 @@ int autotune_step(fractal *f, const uint8_t *in, uint8_t *out, uint32_t birth, u
     }
     f->tile_levels_user = best;
     f->stages_user = best_st;
-    f->tuned = true;
+    f->levels_tuned = f->stages_tuned = true;
     f->sliced_tuned = sliced;
     int rc = ensure_step_plan(f);
     if (rc) return rc;

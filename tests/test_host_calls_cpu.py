@@ -292,3 +292,26 @@ assert run(("triangle", 12, 3), ("triangle", 12, 2))[0]
 assert run(("triangle", 12, 2), ("triangle", 4, 2), ("triangle", 5, 2))[0]
 assert run(("triangle", 16, 2))[0]
 """)
+
+
+def test_settings_after_the_autotuner(host):
+    # a setting given back to the library is the library's again, whatever the autotuner had chosen; one set by the
+    # caller asks for the tile kernels
+    host("""
+def tuned():
+    h = handle("carpet", 8)
+    assert lib.fractal_autotune(h, c_void_p(A), c_void_p(B), 8, 12, None, None) == 0
+    return h
+def goes_sliced(h, n=4):
+    fake.fake_clear()
+    assert step(h, n) == 0
+    return sliced(kernels())
+assert goes_sliced(tuned()) and goes_sliced(handle("carpet", 8))
+for fn, back, own in ((lib.fractal_set_tile_levels, -1, 3), (lib.fractal_set_pipeline_stages, -1, 3)):
+    h = tuned()
+    assert fn(h, back) == 0 and goes_sliced(h)
+    assert fn(h, own) == 0 and not goes_sliced(h)
+    assert fn(h, back) == 0 and goes_sliced(h)
+h = tuned()
+assert lib.fractal_set_tile_levels(h, -1) == 0 and lib.fractal_set_pipeline_stages(h, -1) == 0 and goes_sliced(h)
+""")

@@ -158,17 +158,21 @@ int fractal_init_bernoulli(const fractal_t *f, uint8_t *state_dev,
  * Unless the handle has a tile depth or stage count of its own, fractals with
  * one transition table (r >= 1, k >= 2) may take the bit-sliced step instead,
  * which packs the cells into bits (32 tiles to a word): calls of several
- * generations, and single ones of larger states where it is faster.  It keeps
- * its tables (a few MB at most for the benchmark fractals, 32 bytes per tile
- * in 2D, 104 in 3D), and where the packed state does not stay on the chip one
- * or two packed states of about k^r / 8 bytes and the tiles' border cells, all
- * allocated on first need and kept until fractal_destroy; the ping-pong
- * scratch is then not allocated.  Without that memory, and under capture
- * before it exists, the byte-wise step above runs.  Calls of one handle on
- * several streams take turns at the packed states; captured ones are outside
- * that order: replays of calls of several generations must not overlap other
- * calls of several generations of the handle (nor may they share the scratch).
- * A single generation under capture uses no packed state. */
+ * generations, and single ones of larger states, where it is faster (the first
+ * single generation of a handle only if the state is large enough to pay for
+ * the tables at once).  It keeps its tables (a few MB at most for the benchmark
+ * fractals, 32 bytes per tile in 2D, 104 in 3D), and where the packed state
+ * does not stay on the chip one or two packed states of about k^r / 8 bytes and
+ * the tiles' border cells, all allocated on first need and kept until
+ * fractal_destroy; the ping-pong scratch is then not allocated.  Without that
+ * memory (a later call tries again), and under capture before it exists, the
+ * byte-wise step above runs.  Calls of several generations of one handle on
+ * several streams take turns at the packed states; a single generation that
+ * finds them in use by another stream runs byte-wise, without waiting.
+ * Captured calls are outside that order: replays of calls of several
+ * generations must not overlap other calls of several generations of the
+ * handle (nor may they share the scratch).  A single generation under capture
+ * uses no packed state. */
 int fractal_step(fractal_t *f, const uint8_t *in_dev, uint8_t *out_dev,
                  int64_t steps, uint32_t birth_mask, uint32_t survive_mask,
                  void *stream);

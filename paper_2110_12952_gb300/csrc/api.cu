@@ -244,7 +244,8 @@ extern "C" int fractal_destroy(fractal_t *f)
     cudaFree(f->b3_state[0]);
     cudaFree(f->b3_state[1]);
     for (uint32_t *w : f->box_words.mem) cudaFree(w);
-    if (f->packed_done) cudaEventDestroy(f->packed_done);
+    for (PackedTurn *t : {&f->step_turn[0], &f->step_turn[1], &f->box_turn[0], &f->box_turn[1]})
+        if (t->done) cudaEventDestroy(t->done);
     cudaFree(f->bb_scratch);
     cudaFree(f->host_io[0]);
     cudaFree(f->host_io[1]);
@@ -338,12 +339,14 @@ static int ensure_buffer(uint8_t **buf, int64_t bytes, const char *what)
     return FR_OK;
 }
 
-// The packed buffers of a handle serve its calls one after the other,
-// whatever their streams: a call waits for the last one that used them.
+// The packed buffers of a handle serve the calls of their kind (compact or
+// box, one or several generations) one after the other, whatever their
+// streams: a call waits for the last one that used them.  A single generation
+// does not wait for another stream: it runs on the byte-wise kernels, which
+// share nothing, while that stream's work is not done.
 // Captured work has no place in that order: calls of several generations are
 // the caller's to keep apart there, as with the ping-pong scratch; single
-// generations use no packed buffer under capture, and others than those of
-// several generations elsewhere, so replays disturb none of them.
+// generations use no packed buffer under capture, so replays disturb none.
 bool fr::capturing(cudaStream_t st)
 {
     cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
@@ -352,18 +355,32 @@ bool fr::capturing(cudaStream_t st)
     return on;
 }
 
-int fr::packed_enter(fractal *f, cudaStream_t st, bool captured)
+int fr::packed_enter(PackedTurn &t, cudaStream_t st, bool captured)
 {
     if (captured) return FR_OK;
-    if (f->packed_done) FR_CUDA(cudaStreamWaitEvent(st, f->packed_done, 0));
-    else FR_CUDA(cudaEventCreateWithFlags(&f->packed_done, cudaEventDisableTiming));
+    if (t.done) FR_CUDA(cudaStreamWaitEvent(st, t.done, 0));
+    else FR_CUDA(cudaEventCreateWithFlags(&t.done, cudaEventDisableTiming));
     return FR_OK;
 }
 
-int fr::packed_leave(fractal *f, cudaStream_t st, bool captured)
+int fr::packed_leave(PackedTurn &t, cudaStream_t st, bool captured)
 {
-    if (!captured) FR_CUDA(cudaEventRecord(f->packed_done, st));
+    if (captured) return FR_OK;
+    FR_CUDA(cudaEventRecord(t.done, st));
+    t.last = st;
     return FR_OK;
+}
+
+bool fr::packed_busy(const PackedTurn &t, cudaStream_t st)
+{
+    if (!t.done || t.last == st) return false;
+    // (a query would end a capture of this thread on some other stream, were it not for the relaxed mode)
+    cudaStreamCaptureMode mode = cudaStreamCaptureModeRelaxed;
+    cudaThreadExchangeStreamCaptureMode(&mode);
+    const bool busy = cudaEventQuery(t.done) != cudaSuccess;
+    cudaThreadExchangeStreamCaptureMode(&mode);
+    if (busy) cudaGetLastError();   // (not ready)
+    return busy;
 }
 
 // Ping-pong `steps` generations so that the last one lands in `out`: step i

@@ -965,6 +965,8 @@ int try_bb_packed(fractal *f, const uint8_t *in, uint8_t *out, int64_t steps, ui
     const bool captured = capturing(st);
     // under capture a single generation leaves the packed box alone: its replays may run beside other calls
     if (captured && steps == 1) return FR_OK;
+    PackedTurn &turn = f->box_turn[steps == 1];
+    if (steps == 1 && packed_busy(turn, st)) return FR_OK;
     if (!(steps == 1 ? f->box_words.one : f->box_words.two[0])) {
         // nothing is allocated under capture, and without the memory the row kernels run as before
         if (captured || f->box_words.memory.skip()) return FR_OK;
@@ -989,9 +991,9 @@ int try_bb_packed(fractal *f, const uint8_t *in, uint8_t *out, int64_t steps, ui
     a.rwdiv = make_div((uint32_t)std::max(2, a.RW));
     a.ndiv = make_div((uint32_t)n);
     *done = true;
-    int rc = packed_enter(f, st, captured);
+    int rc = packed_enter(turn, st, captured);
     if (!rc) rc = f->dim == 3 ? run_bb_words<3>(f, a, in, out, steps, st) : run_bb_words<2>(f, a, in, out, steps, st);
-    return rc ? rc : packed_leave(f, st, captured);
+    return rc ? rc : packed_leave(turn, st, captured);
 }
 
 int launch_bb_once(fractal *f, const uint8_t *in, uint8_t *out, uint32_t birth,

@@ -88,6 +88,12 @@ struct BBPlan {
     int64_t local_words = 0, coarse_words = 0;
 };
 
+// After the last work on a kind of packed buffers, and that work's stream.
+struct PackedTurn {
+    cudaEvent_t done = nullptr;
+    cudaStream_t last = nullptr;
+};
+
 // The box as bits (bb.cu), each array behind a zero word: the cells'
 // membership, the box of single generations, the two of calls of several.
 // One allocation holds the membership and the boxes of the first kind of call,
@@ -145,7 +151,8 @@ struct fractal {
     uint8_t *scratch = nullptr;      // k^r bytes, ping-pong for steps > 1
     uint32_t *b3_state[2] = {nullptr, nullptr};  // bit3 plans, steps > 1: bit-packed tile states (ping-pong)
     fr::BoxWords box_words;          // box steps: the box as bits
-    cudaEvent_t packed_done = nullptr;   // after the last work on the packed buffers (slice, box_words)
+    // turns at the packed buffers: [0] of calls of several generations, [1] of single ones
+    fr::PackedTurn step_turn[2], box_turn[2];
     uint8_t *bb_scratch = nullptr;   // n^dim bytes, ping-pong for BB steps > 1
     uint8_t *host_io[2] = {nullptr, nullptr};  // device buffers of run_host
     fr::HostPipe pipe;                          // run_host's chunked pipeline
@@ -197,10 +204,12 @@ inline int64_t cells_above(const fractal *f, int L)
 }
 
 int ensure_step_plan(fractal *f);
-// Around work on the handle's packed buffers: ordered over all streams, except under capture.
+// Around work on one kind of packed buffers: ordered over all streams, except
+// under capture; and whether another stream's work on them is not done yet.
 bool capturing(cudaStream_t st);
-int packed_enter(fractal *f, cudaStream_t st, bool captured);
-int packed_leave(fractal *f, cudaStream_t st, bool captured);
+int packed_enter(PackedTurn &t, cudaStream_t st, bool captured);
+int packed_leave(PackedTurn &t, cudaStream_t st, bool captured);
+bool packed_busy(const PackedTurn &t, cudaStream_t st);
 void keep_generation_buffers(fractal *f);
 double short_generation_us(const fractal *f, int64_t NT);
 int rows_preset_of(const fractal *f);   // 0: the carpet, 1: the Vicsek fractal (preset offsets), -1: another

@@ -1685,6 +1685,8 @@ int try_slice_step(fractal *f, const uint8_t *in, uint8_t *out, int64_t steps, u
     }
     // under capture nothing is allocated, and a single generation leaves the
     // packed state alone (its replays may run beside other calls): the tile kernels run there
+    PackedTurn &turn = f->step_turn[steps == 1];
+    if (steps == 1 && (res || packed) && !captured && packed_busy(turn, st)) return FR_OK;
     const bool ready = s.state > 1 && (!packed || (steps == 1 ? s.bits[2] != nullptr : s.bits[0] && s.bits[1]));
     if (captured && (!ready || (steps == 1 && (res || packed)))) return FR_OK;
     int rc;
@@ -1709,9 +1711,9 @@ int try_slice_step(fractal *f, const uint8_t *in, uint8_t *out, int64_t steps, u
         FR_CUDA(cudaGetLastError());
         return FR_OK;
     }
-    rc = packed_enter(f, st, captured);
+    rc = packed_enter(turn, st, captured);
     if (!rc) rc = res ? launch_resident(s, a, life, in, out, steps, st) : run_packed(f, a, life, in, out, steps, st);
-    return rc ? rc : packed_leave(f, st, captured);
+    return rc ? rc : packed_leave(turn, st, captured);
 }
 
 // ---------------------------------------------------------------- batches

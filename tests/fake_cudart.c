@@ -182,6 +182,7 @@ cudaError_t cudaStreamSynchronize(void *s) { const cudaError_t e = result("cudaS
 cudaError_t cudaDeviceSynchronize(void) { land_copies(); return cudaSuccess; }
 cudaError_t cudaStreamIsCapturing(void *s, int *st) { (void)s; *st = g_capturing; return cudaSuccess; }
 cudaError_t cudaStreamBeginCapture(void *s, int m) { (void)s; (void)m; return cudaSuccess; }
+cudaError_t cudaThreadExchangeStreamCaptureMode(int *m) { static int now; const int old = now; now = *m; *m = old; return cudaSuccess; }
 cudaError_t cudaStreamEndCapture(void *s, void **g) { (void)s; *g = number(); return cudaSuccess; }
 cudaError_t cudaGraphInstantiate(void **e, void *g, unsigned long long f) { (void)g; (void)f; *e = number(); return cudaSuccess; }
 cudaError_t cudaGraphLaunch(void *e, void *s) { (void)e; (void)s; return cudaSuccess; }

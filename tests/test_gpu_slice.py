@@ -202,3 +202,39 @@ def test_several_generations_of_an_autotuned_handle():
     for n in (1, 4):
         assert np.array_equal(g.step(x, steps=n).cpu().numpy(), o.step(v, steps=n))
     g.close()
+
+
+@pytest.mark.parametrize("name,r,box", [("carpet", 8, False), ("h_fractal", 8, False), ("menger", 6, False), ("menger", 5, True)])
+def test_single_generations_do_not_wait_for_another_stream(name, r, box):
+    # a single generation on one stream is done while the same handle's earlier call on another stream has not begun
+    from paper_2110_12952_gb300 import Fractal
+    fam = W.FAMILIES[name]
+    g, ref = Fractal.from_family(fam, r), Fractal.from_family(fam, r)
+    ref.tile_levels = ref.tile_levels
+    rule = W.MENGER_B5S45 if fam.dim == 3 else W.LIFE_B3S23
+    one = (lambda h, v, o: h.bb_step(v, out=o, steps=1, rule=rule)) if box else (lambda h, v, o: h.step(v, out=o, steps=1, rule=rule))
+    x = [ref.init_bernoulli(seed, 0.4) for seed in (1, 2)]
+    if box:
+        x = [ref.scatter(v) for v in x]
+    out = [torch.empty_like(v) for v in x]
+    for _ in range(3):
+        one(g, x[0], out[0])
+    a, b = torch.cuda.Stream(), torch.cuda.Stream()
+    out[0].zero_()
+    torch.cuda.synchronize()
+    with torch.cuda.stream(a):
+        torch.cuda._sleep(1_000_000_000)     # half a second
+        one(g, x[0], out[0])
+        after = torch.cuda.Event()
+        after.record()
+    with torch.cuda.stream(b):
+        one(g, x[1], out[1])
+    b.synchronize()
+    assert not after.query()
+    torch.cuda.synchronize()
+    want = [ref.gather(v) for v in x] if box else x
+    for v, y in zip(want, out):
+        assert torch.equal(ref.gather(y) if box else y, ref.step(v, steps=1, rule=rule))
+    g.check()
+    g.close()
+    ref.close()

@@ -315,3 +315,31 @@ for fn, back, own in ((lib.fractal_set_tile_levels, -1, 3), (lib.fractal_set_pip
 h = tuned()
 assert lib.fractal_set_tile_levels(h, -1) == 0 and lib.fractal_set_pipeline_stages(h, -1) == 0 and goes_sliced(h)
 """)
+
+
+def test_streams_wait_only_where_buffers_are_shared(host):
+    # one handle on two streams: single generations do not wait for the other stream, calls of several wait for calls
+    # of several alone, box calls never for compact ones
+    host("""
+def call(h, fn, n, stream):
+    fake.fake_clear()
+    assert step(h, n, stream=stream, fn=fn, rule=rule) == 0
+    waits = log("^wait", clear=False)
+    return len(waits), any("slice_" in x or "bb_words" in x for x in kernels())
+for name, r, rule in (("carpet", 10, (8, 12)), ("h_fractal", 8, (8, 12)), ("menger", 6, (32, 48))):
+    h, step1, box1 = handle(name, r), ("fractal_step", 1), ("fractal_bb_step", 1)
+    step3, box3 = ("fractal_step", 3), ("fractal_bb_step", 3)
+    calls = [step1, step3] + ([box1, box3] if name == "menger" else [box3] if name == "h_fractal" else [])
+    for c in calls:
+        for _ in range(2):
+            call(h, *c, 0x10)
+        assert call(h, *c, 0x10)[1], (name, c)
+    fake.fake_events_pending(1)
+    for c in calls:
+        waits, packed = call(h, *c, 0x20)
+        assert (waits, packed) == ((0, False) if c[1] == 1 else (1, True)), (name, c, waits, packed)
+    fake.fake_events_pending(0)
+    for c in calls:
+        assert call(h, *c, 0x20) == (1, True), (name, c)
+    lib.fractal_destroy(h)
+""")

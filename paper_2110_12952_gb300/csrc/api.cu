@@ -434,7 +434,7 @@ extern "C" int fractal_step(fractal_t *f, const uint8_t *in, uint8_t *out, int64
     // fractal_step_noalloc need the tile kernels' tables and cannot build them)
     int rc = ensure_step_plan(f);
     if (rc) return rc;
-    if (slice_settings(f, steps) && !f->test_extra_tx) {
+    if (slice_settings(f, steps)) {
         bool done = false;
         rc = try_slice_step(f, in, out, steps, birth, survive, st, &done);
         if (rc || done) return rc;

@@ -220,18 +220,20 @@ def test_single_generations_do_not_wait_for_another_stream(name, r, box):
     for _ in range(3):
         one(g, x[0], out[0])
     a, b = torch.cuda.Stream(), torch.cuda.Stream()
-    out[0].zero_()
-    torch.cuda.synchronize()
-    with torch.cuda.stream(a):
-        torch.cuda._sleep(1_000_000_000)     # half a second
-        one(g, x[0], out[0])
-        after = torch.cuda.Event()
-        after.record()
-    with torch.cuda.stream(b):
-        one(g, x[1], out[1])
-    b.synchronize()
-    assert not after.query()
-    torch.cuda.synchronize()
+    for cycles in (20_000_000, 1_000_000_000):   # (the first time loads the kernels, which may wait for the device)
+        out[0].zero_()
+        torch.cuda.synchronize()
+        with torch.cuda.stream(a):
+            torch.cuda._sleep(cycles)
+            one(g, x[0], out[0])
+            after = torch.cuda.Event()
+            after.record()
+        with torch.cuda.stream(b):
+            one(g, x[1], out[1])
+        b.synchronize()
+        early = not after.query()
+        torch.cuda.synchronize()
+    assert early
     want = [ref.gather(v) for v in x] if box else x
     for v, y in zip(want, out):
         assert torch.equal(ref.gather(y) if box else y, ref.step(v, steps=1, rule=rule))

@@ -343,3 +343,18 @@ for name, r, rule in (("carpet", 10, (8, 12)), ("h_fractal", 8, (8, 12)), ("meng
         assert call(h, *c, 0x20) == (1, True), (name, c)
     lib.fractal_destroy(h)
 """)
+
+
+def test_armed_calls_with_grid_barriers_stay_sliced(host):
+    # the failure-detection hook reaches the sliced step's grid barriers; calls without one go to the tile kernels
+    host("""
+for name, r, n, barrier in (("carpet", 8, 6, True), ("h_fractal", 10, 4, True), ("menger", 6, 5, True), ("triangle", 4, 6, False),
+                            ("carpet", 10, 1, False), ("triangle", 14, 1, False)):
+    h = handle(name, r)
+    for armed in (False, True, False):
+        assert not armed or lib.fractal_test_arm_timeout(h, 16, 256) == 0
+        fake.fake_clear()
+        assert step(h, n) == 0
+        assert sliced([x for x in kernels() if "nbr" not in x]) == (barrier or not armed), (name, armed)
+    lib.fractal_destroy(h)
+""")

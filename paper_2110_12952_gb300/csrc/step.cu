@@ -384,7 +384,7 @@ struct TapTables {
 static void host_lambda(const fractal *f, int64_t l, int L, int p[3]);
 static int64_t host_nu(const fractal *f, const int q[3], int L);
 
-static TapTables tap_tables(const fractal *f, int L)
+static TapTables make_tap_tables(const fractal *f, int L)
 {
     TapTables t;
     if (!is_triangle(f) || L < 4) return t;
@@ -554,7 +554,7 @@ struct RowsTables {
 };
 
 template <int P>
-static RowsTables rows_tables(const fractal *f, int L)
+static RowsTables make_rows_tables(const fractal *f, int L)
 {
     RowsTables t;
     constexpr int K = RowsPreset<P>::k, NB = K * K;
@@ -676,7 +676,7 @@ constexpr int kLidPreset = 1, kLidLevels = 3;
 // Tables of lid mode for tile depth L (>= kLidLevels), laid out as those of
 // rows mode with units of k^3 cells (27x27 blocks).
 template <int P, int U>
-static RowsTables lid_tables(const fractal *f, int L)
+static RowsTables make_lid_tables(const fractal *f, int L)
 {
     RowsTables t;
     constexpr int NB = LidUnit<P, U>::NB, SIDE = LidUnit<P, U>::side, NE = lu_next<P, U>();
@@ -760,6 +760,43 @@ static RowsTables lid_tables(const fractal *f, int L)
     return t;
 }
 
+// The presets' tables depend on the tile depth alone, take up to a
+// millisecond to make, and a plan looks at each depth's several times: they are
+// made once per depth (a dozen sets, 200 KB together).
+template <class T>
+struct Kept {
+    std::mutex mu;
+    std::map<int, T> of;
+    template <class Make>
+    const T &get(int L, Make make)
+    {
+        std::lock_guard<std::mutex> lk(mu);
+        auto it = of.find(L);
+        if (it == of.end()) it = of.emplace(L, make()).first;
+        return it->second;
+    }
+};
+
+static const TapTables &tap_tables(const fractal *f, int L)
+{
+    static Kept<TapTables> kept;
+    return kept.get(L, [&] { return make_tap_tables(f, L); });
+}
+
+template <int P>
+static const RowsTables &rows_tables(const fractal *f, int L)
+{
+    static Kept<RowsTables> kept;
+    return kept.get(L, [&] { return make_rows_tables<P>(f, L); });
+}
+
+template <int P, int U>
+static const RowsTables &lid_tables(const fractal *f, int L)
+{
+    static Kept<RowsTables> kept;
+    return kept.get(L, [&] { return make_lid_tables<P, U>(f, L); });
+}
+
 struct Geometry {
     int mode, G, xoff, halo;
     int64_t B, Px, Py, planes;
@@ -787,7 +824,7 @@ static Geometry plan_geometry(const fractal *f, int L)
     g.halo_bytes = 0;
     g.data_bytes = 0;
     if (grp && is_triangle(f) && L >= 4 && ipow(f->k, L - 4) <= 256) {
-        const TapTables t = tap_tables(f, L);
+        const TapTables &t = tap_tables(f, L);
         if (t.ok) {
             g.mode = kModeTap;
             g.Px = g.Py = g.planes = 0;
@@ -801,7 +838,7 @@ static Geometry plan_geometry(const fractal *f, int L)
     }
     const int rp = rows_preset_of(f);
     if (rp == kLidPreset && L >= kLidLevels && ipow(f->k, L - kLidLevels) <= 256) {
-        const RowsTables t = lid_tables<kLidPreset, kLidLevels>(f, L);
+        const RowsTables &t = lid_tables<kLidPreset, kLidLevels>(f, L);
         if (t.ok) {
             g.mode = kModeLid1;
             g.Px = g.Py = g.planes = 0;
@@ -814,7 +851,7 @@ static Geometry plan_geometry(const fractal *f, int L)
         }
     }
     if (rp >= 0 && L >= 2 && ipow(f->k, L - 2) <= 256) {
-        const RowsTables t = rp == 0 ? rows_tables<0>(f, L) : rows_tables<1>(f, L);
+        const RowsTables &t = rp == 0 ? rows_tables<0>(f, L) : rows_tables<1>(f, L);
         if (t.ok) {
             g.mode = rp == 0 ? kModeRows0 : kModeRows1;
             g.Px = g.Py = g.planes = 0;
@@ -1151,21 +1188,21 @@ int ensure_step_plan(fractal *f)
         p.b3.warp_bytes = bit3_warp_bytes(f);
         p.nstage = 0;
     } else if (p.mode == kModeTap) {
-        const TapTables t = tap_tables(f, L);
+        const TapTables &t = tap_tables(f, L);
         p.KG = 9;
         p.tapz = t.zero_off;
         p.nq = t.NQ;
         tab = t.words;
         ring = t.ring;
     } else if (p.mode == kModeLid1) {
-        const RowsTables t = lid_tables<kLidPreset, kLidLevels>(f, L);
+        const RowsTables &t = lid_tables<kLidPreset, kLidLevels>(f, L);
         p.KG = (int)ipow(f->k, kLidLevels);
         p.tapz = t.NU + t.H;
         p.nq = t.NU;
         tab = t.words;
         ring = t.ring;
     } else if (p.mode == kModeRows0 || p.mode == kModeRows1) {
-        const RowsTables t = p.mode == kModeRows0 ? rows_tables<0>(f, L) : rows_tables<1>(f, L);
+        const RowsTables &t = p.mode == kModeRows0 ? rows_tables<0>(f, L) : rows_tables<1>(f, L);
         p.KG = f->k * f->k;
         p.tapz = t.NU + t.H;
         p.nq = t.NU;

@@ -464,9 +464,10 @@ int fractal_shard_step(fractal_shard_t *p, const uint8_t *in_dev, uint8_t *out_d
  * then records the timeout, waits (bounded) for the copies it issued, and
  * returns without writing further results: that call's output is invalid and
  * the next fractal_check returns FR_ETIMEOUT.  A call that runs bit-sliced with
- * grid barriers between generations has its barriers wait for one block more
- * than there are, with the same limit and the same outcome; other bit-sliced
- * calls run byte-wise when armed.  Later launches are unaffected.
+ * grid barriers between generations has its first barrier wait for one block
+ * more than there are, for the default ~4 million tries (a second or two),
+ * with the same outcome; other bit-sliced calls run byte-wise when armed.
+ * Later launches are unaffected.
  * extra_bytes in [1, 4096], wait_tries in [1, 2^20], else FR_EINVAL. */
 int fractal_test_arm_timeout(fractal_t *f, uint32_t extra_bytes, uint32_t wait_tries);
 

@@ -59,12 +59,11 @@ def test_arm_timeout_rejects_bad_arguments(P):
     assert g._lib.fractal_test_arm_timeout(g._h, 8192, 10) == -1
 
 
-@pytest.mark.parametrize("fam,r,steps", [(W.CARPET, 8, 6), (W.TRIANGLE, 13, 9), (W.MENGER, 6, 5), (W.FAMILIES["h_fractal"], 10, 4),
-                                         (W.CARPET, 8, 1)],
+@pytest.mark.parametrize("fam,r,steps", [(W.CARPET, 8, 6), (W.MENGER, 6, 5), (W.FAMILIES["h_fractal"], 10, 4), (W.CARPET, 8, 1)],
                          ids=lambda v: getattr(v, "name", str(v)))
 def test_grid_barrier_times_out_and_recovers(P, fam, r, steps):
     # the sliced step's barriers between generations, resident and streaming (and a single generation of tile kernels):
-    # armed for an arrival that never comes, they give up, and the next call finds them reset
+    # a count that starts one short makes the first one run out (a second or two), and the next call finds it reset
     g, ref = P.Fractal.from_family(fam, r), P.Fractal.from_family(fam, r)
     ref.tile_levels = ref.tile_levels
     rule = W.default_rule(fam)
@@ -72,7 +71,7 @@ def test_grid_barrier_times_out_and_recovers(P, fam, r, steps):
     want = ref.step(x, steps=steps, rule=rule)
     y = torch.empty_like(x)
     lib = g._lib
-    for armed in (False, True, False, True, False):
+    for armed in (False, True, False):
         if armed:
             assert lib.fractal_test_arm_timeout(g._h, 16, 256) == 0
         g.step(x, out=y, steps=steps, rule=rule)

@@ -156,3 +156,77 @@ def test_bb_bits3_other_tables(P, fam, r):
     box = rng.integers(0, 3, size=g.box_cells).astype(np.uint8) * rng.integers(1, 200, size=g.box_cells).astype(np.uint8)
     got = g.bb_step(torch.from_numpy(box).cuda(), steps=2, rule=(0x6, 0x1E)).cpu().numpy()
     assert np.array_equal(got, o.bb_step(box, rule=orule((0x6, 0x1E)), steps=2))
+
+
+# An explicit tile depth keeps calls of several generations on the bit3 kernels (default handles run them bit-sliced).
+
+@pytest.mark.parametrize("fam,r", [(CORNERS8, 5), (EDGES12, 4), (MENGER_REV, 4), (W.MENGER, 3), (W.MENGER, 5),
+                                   (FOUR4, 6), (DENSE24, 4)],
+                         ids=lambda v: getattr(v, "name", str(v)))
+def test_tables_and_sizes_at_an_explicit_depth(P, fam, r):
+    g, o = pair(P, fam, r)
+    g.tile_levels = 3
+    assert g.plan_info()["policy_name"] == "bit3"
+    raw = nonbinary(o.cells, r)
+    x = torch.from_numpy(raw).cuda()
+    for rule, steps in ((W.MENGER_B5S45, 3), ((0x6, 0x1E), 2), ((0x2, 0x3), 5)):
+        assert np.array_equal(g.step(x, steps=steps, rule=rule).cpu().numpy(), o.step(raw, rule=orule(rule), steps=steps)), rule
+    g.check()
+
+
+@pytest.mark.parametrize("rule", RULES, ids=lambda r: f"B{r[0]:x}S{r[1]:x}")
+def test_rules_at_an_explicit_depth(P, rule):
+    g, o = pair(P, W.MENGER, 4)
+    g.tile_levels = 3
+    raw = nonbinary(o.cells, 12)
+    x = torch.from_numpy(raw).cuda()
+    for steps in (2, 6):
+        assert np.array_equal(g.step(x, steps=steps, rule=rule).cpu().numpy(), o.step(raw, rule=orule(rule), steps=steps)), steps
+
+
+# Under capture a single 3D box generation runs in the row kernel (other aligned calls use packed boxes).
+
+def captured_bb(g, box, rule):
+    out = torch.full_like(box, 9)
+    g.bb_step(box, out=out, steps=0)   # the tables
+    torch.cuda.synchronize()
+    graph = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(graph):
+        g.bb_step(box, out=out, steps=1, rule=rule)
+    out.fill_(9)
+    graph.replay()
+    torch.cuda.synchronize()
+    del graph
+    return out
+
+
+@pytest.mark.parametrize("fam,r", [(W.MENGER, 4), (W.MENGER, 5), (EDGES12, 5), (CORNERS8, 5), (DENSE24, 5)],
+                         ids=lambda v: getattr(v, "name", str(v)))
+@pytest.mark.parametrize("rule", [W.MENGER_B5S45, (0x6, 0x1E)], ids=lambda r: f"B{r[0]:x}S{r[1]:x}")
+def test_captured_box_generation_runs_by_rows(P, fam, r, rule):
+    g, o = pair(P, fam, r)
+    rng = np.random.default_rng(r)
+    box = rng.integers(0, 3, size=g.box_cells).astype(np.uint8) * rng.integers(1, 200, size=g.box_cells).astype(np.uint8)
+    got = captured_bb(g, torch.from_numpy(box).cuda(), rule)
+    assert np.array_equal(got.cpu().numpy(), o.bb_step(box, rule=orule(rule), steps=1))
+
+
+@pytest.mark.parametrize("rule", [W.MENGER_B5S45, (0x6, 0x1E)], ids=lambda r: f"B{r[0]:x}S{r[1]:x}")
+def test_captured_box_generation_of_two_strips(P, rule):
+    # side 1024, two strips per row, against the packed boxes (which the oracle checks at smaller sides)
+    tetra = W.Family("tetra4", 4, 2, 3, ((0, 0, 0), (1, 0, 0), (0, 1, 0), (0, 0, 1)))
+    g, _ = pair(P, tetra, 10)
+    box = torch.randint(0, 256, (g.box_cells,), dtype=torch.uint8, device="cuda")
+    assert torch.equal(captured_bb(g, box, rule), g.bb_step(box, steps=1, rule=rule))
+
+
+@pytest.mark.parametrize("fam,r", [(W.CARPET, 5), (W.CARPET, 7), (W.VICSEK, 6), (W.TRIANGLE, 10)], ids=lambda v: getattr(v, "name", str(v)))
+@pytest.mark.parametrize("rule", [(0x6, 0x1E), W.LIFE_B3S23], ids=lambda r: f"B{r[0]:x}S{r[1]:x}")
+def test_2d_box_rows_under_general_rules(P, fam, r, rule):
+    # single 2D box generations stay in the row kernel, one to three strips per row
+    g, o = pair(P, fam, r)
+    rng = np.random.default_rng(r)
+    box = rng.integers(0, 3, size=g.box_cells).astype(np.uint8) * rng.integers(1, 200, size=g.box_cells).astype(np.uint8)
+    orl = oracle.Rule([i for i in range(9) if (rule[0] >> i) & 1], [i for i in range(9) if (rule[1] >> i) & 1])
+    got = g.bb_step(torch.from_numpy(box).cuda(), steps=1, rule=rule).cpu().numpy()
+    assert np.array_equal(got, o.bb_step(box, rule=orl, steps=1))

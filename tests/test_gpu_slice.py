@@ -240,3 +240,40 @@ def test_single_generations_do_not_wait_for_another_stream(name, r, box):
     g.check()
     g.close()
     ref.close()
+
+
+GRID3 = [(x, y, z) for z in range(3) for y in range(3) for x in range(3)]
+
+
+@pytest.mark.parametrize("name,r,steps", [("triangle", 11, (1,)), ("triangle", 13, (1,)), ("triangle_mirrored", 12, (1,)), ("triangle", 18, (1, 3)),
+                                          ("carpet", 8, (1,)), ("h_fractal", 8, (1,)), ("h_fractal", 10, (2, 3)), ("full_square", 12, (1, 2)),
+                                          ("full_square", 13, (1, 3)), ("vicsek", 12, (2, 3)), ("chandelier", 13, (1, 3)), ("x_fractal", 10, (1, 4)),
+                                          ("candy", 7, (1, 2)), ("menger", 6, (1, 3)), ("cube", 5, (1, 3))])
+def test_rules_and_addresses_against_the_tile_kernels(name, r, steps):
+    # single generations (the single pass, packed and resident forms) and streamed states under rules without a closed
+    # form, from and to buffers at odd addresses, bytes other than 0 and 1: against a handle with a tile depth of its own
+    from paper_2110_12952_gb300 import Fractal
+    make = (lambda: Fractal(27, 3, r, 3, np.array(GRID3, dtype=np.int32))) if name == "cube" else (lambda: Fractal.from_family(W.FAMILIES[name], r))
+    g, tiles = make(), make()
+    tiles.tile_levels = tiles.tile_levels
+    rules = [W.rule_masks([4, 26], [0, 3, 4, 5, 18]), W.MENGER_B5S45] if g.dim == 3 else [W.rule_masks([1, 3, 8], [0, 1, 2, 5, 8]), W.LIFE_B3S23]
+    x = g.init_bernoulli(3, 0.45)
+    x[::7] *= 201
+    base = torch.empty(g.cells + 16, dtype=torch.uint8, device="cuda")
+    whole = torch.empty(g.cells + 64, dtype=torch.uint8, device="cuda")
+    for rule in rules:
+        want, done = x, 0
+        for n in steps:
+            for _ in range(n - done):
+                want = tiles.step(want, steps=1, rule=rule)
+            done = n
+            for src_off, dst_off in ((0, 0), (0, 0), (5, 0), (0, 9), (16, 16), (1, 3)):   # (a first single generation may go to the tiles)
+                src, dst = base[src_off:src_off + g.cells], whole[16 + dst_off:16 + dst_off + g.cells]
+                src.copy_(x)
+                whole.fill_(77)
+                g.step(src, out=dst, steps=n, rule=rule)
+                assert torch.equal(dst, want), (rule, n, src_off, dst_off)
+                assert int((whole[:16 + dst_off] == 77).all()) and int((whole[16 + dst_off + g.cells:] == 77).all())
+    g.check()
+    g.close()
+    tiles.close()

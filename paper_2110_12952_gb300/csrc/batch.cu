@@ -109,10 +109,13 @@ static int build(fractal_batch *b)
     }
     // (of the sliced instances too: fractal_step_noalloc and captured calls of
     // their handles need the tile kernels' tables and cannot build them)
+    rc = FR_OK;
     for (auto &in : b->insts) {
-        rc = ensure_step_plan(in.f);
-        if (rc) return rc;
+        rc = ensure_step_plan(in.f, false);
+        if (rc) break;
     }
+    FR_CUDA(cudaDeviceSynchronize());
+    if (rc) return rc;
     // sliced launches by fractal table and rule; where they cannot be built
     // (memory) their instances stay with the tile kernels
     std::vector<char> is_sliced(b->insts.size(), 0);

@@ -203,7 +203,7 @@ inline int64_t cells_above(const fractal *f, int L)
     return v;
 }
 
-int ensure_step_plan(fractal *f);
+int ensure_step_plan(fractal *f, bool wait = true);   // wait = false: the caller waits for the device
 // Around work on one kind of packed buffers: ordered over all streams, except
 // under capture; and whether another stream's work on them is not done yet.
 bool capturing(cudaStream_t st);

@@ -1004,14 +1004,15 @@ __global__ void nbr_table_kernel(FracDev F, int64_t NT, int coarse_levels, int32
     }
 }
 
-// Fills the table of the NT tiles' neighbours (coarse_levels levels above them).
-int launch_nbr_table(const fractal *f, int64_t NT, int coarse_levels, int nbrw, int32_t *table)
+// Fills the table of the NT tiles' neighbours (coarse_levels levels above them);
+// wait = false: the caller waits for the device.
+int launch_nbr_table(const fractal *f, int64_t NT, int coarse_levels, int nbrw, int32_t *table, bool wait = true)
 {
     const int64_t g = std::min<int64_t>((NT + 255) / 256, (int64_t)f->num_sms * 16);
     nbr_table_kernel<<<(int)std::max<int64_t>(g, 1), 256>>>(f->dev, NT, coarse_levels, (int32_t)ipow(f->s, coarse_levels),
                                                             nbrw, table);
     FR_CUDA(cudaGetLastError());
-    FR_CUDA(cudaDeviceSynchronize());
+    if (wait) FR_CUDA(cudaDeviceSynchronize());
     return FR_OK;
 }
 
@@ -1131,7 +1132,7 @@ void keep_generation_buffers(fractal *f)
     cudaGetLastError();
 }
 
-int ensure_step_plan(fractal *f)
+int ensure_step_plan(fractal *f, bool wait)
 {
     // the plan depends only on the fractal and on these two settings (the
     // tables behind the automatic choice are too costly to rebuild per call)
@@ -1337,7 +1338,7 @@ int ensure_step_plan(fractal *f)
         free_step_plan(p);
         return cuda_fail(e, "fractal_step: table upload");
     }
-    rc = launch_nbr_table(f, p.NT, p.coarse_levels, p.nbrw, p.nbr);
+    rc = launch_nbr_table(f, p.NT, p.coarse_levels, p.nbrw, p.nbr, wait);
     if (rc) {
         free_step_plan(p);
         return rc;

@@ -34,7 +34,7 @@ sys.path.insert(0, ROOT)
 
 METRIC = "compact cell-updates/s (Sierpinski triangle r=20, B3/S23) and % HBM roofline vs bounding box on 1 GB300"
 UNIT = "cell-updates/s"
-KERNEL_SRC = os.path.join(ROOT, "paper_2110_12952_gb300", "csrc", "step.cu")
+KERNEL_SRC = os.path.join(ROOT, "paper_2110_12952_gb300", "csrc", "slice.cu")
 TRAFFIC_FILE = os.path.join(ROOT, "profiles", "step_traffic.json")
 
 
@@ -133,7 +133,7 @@ class ClockSampler:
         try:
             self.proc = subprocess.Popen(
                 ["nvidia-smi", f"--id={self.idx}", f"--query-gpu={self.FIELDS}",
-                 "--format=csv,noheader,nounits", "-lms", "50"],
+                 "--format=csv,noheader,nounits", "-lms", "10"],
                 stdout=subprocess.PIPE, stderr=subprocess.DEVNULL, text=True)
             self.th = threading.Thread(target=self._read, daemon=True)
             self.th.start()
@@ -691,6 +691,7 @@ def temporal_compare(g, x, y, single_ms, peak):
     g.set_temporal_blocking(gens)
     times = time_steps(lambda: g.step(x, out=y, steps=gens), 10, 3)
     g.set_temporal_blocking(0)
+    default_ms = statistics.median(time_steps(lambda: g.step(x, out=y, steps=gens), 10, 3))
     ms = statistics.median(times)
     L = next(l for l in range(5, 1, -1) if l <= g.r and _tb_smem(l) <= 100 * 1024)
     tile = 8 ** L
@@ -699,6 +700,7 @@ def temporal_compare(g, x, y, single_ms, peak):
     return {"generations_per_pass": gens, "tile_levels": L, "ms_per_pass": ms,
             "updates_per_s": g.cells * gens / (ms / 1e3),
             "speedup_vs_single_generation": single_ms * gens / ms,
+            "default_ms_for_as_many_generations": default_ms,
             "hbm_bytes_per_update": bytes_per_pass / (g.cells * gens),
             "achieved_gbs": bytes_per_pass / (ms / 1e3) / 1e9, "peak_gbs": peak,
             "note": "bytes per update are (tile + halo units + tile) / (cells x generations); "
@@ -706,16 +708,16 @@ def temporal_compare(g, x, y, single_ms, peak):
 
 
 def multigen_compare(g, x, y, ms_single, gens=50):
-    """One call of `gens` generations (bit3 policy: the state stays bit-packed
-    between the first and the last generation), timed three times."""
+    """One call of `gens` generations (the state stays packed into bits between
+    the first and the last generation), timed three times."""
     import torch
     g.step(x, out=y, steps=gens)
     ts = time_steps(lambda: g.step(x, out=y, steps=gens), 3, 1)
     ms = statistics.median(ts)
     return {"generations_per_call": gens, "ms_per_call": ms, "ms_per_generation": ms / gens,
             "updates_per_s": g.cells * gens / (ms / 1e3), "speedup_vs_single_generation": ms_single / (ms / gens),
-            "note": "first generation bytes -> bit-packed tile states, the ones between states -> states, "
-                    "the last states -> bytes; per-generation bytes are not comparable with the 2 B/update roofline"}
+            "note": "bit-sliced: bytes packed into words of 32 tiles, generations on the words, the last one to bytes; "
+                    "per-generation bytes are not comparable with the 2 B/update roofline"}
 
 
 def _tb_smem(L):
@@ -747,6 +749,9 @@ def others_compare(args, W):
         x = g.init_bernoulli(inst.seed, inst.p)
         y = torch.empty_like(x)
         L = g.autotune(x, y)
+        # kernels run up to a quarter slower for some 45 ms of work after the autotuner's, and not after a pause
+        torch.cuda.synchronize()
+        time.sleep(0.5)
         small = 2 * g.cells < 4 * 129 * 2**20
         n = max(5, min(args.steps, 20))
         ct = time_steps(lambda: g.step(x, out=y, steps=1), n, 3,

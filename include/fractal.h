@@ -290,11 +290,17 @@ int fractal_set_pipeline_stages(fractal_t *f, int stages);
  * Only for the Sierpinski carpet and the Vicsek fractal with the preset
  * offset tables (FR_EINVAL otherwise).  tile_levels: -1 = the deepest tile
  * whose shared memory stays within 100 KB, else in [2, r].  generations = 0
- * turns it off.  The batch, server and no-allocation calls are unaffected. */
+ * turns it off.  The batch, server and no-allocation calls are unaffected.
+ * A handle without it runs several generations bit-sliced (see fractal_step),
+ * which is the faster way for most states: nine generations of the carpet at
+ * r = 10 take 1.46 ms so and 2.54 ms blocked, at r = 8 48 and 50 us.  Blocking
+ * pays for states of about 10^5 to 2 x 10^6 cells (carpet r = 6 34 and 19 us,
+ * Vicsek r = 8 29 and 17 us) and where the bit-sliced step has no memory. */
 int fractal_set_temporal_blocking(fractal_t *f, int generations, int tile_levels);
 
-/* Launch plan of fractal_step for this handle (built, with its
- * allocations, if it does not exist yet, as by fractal_get_tile_levels).
+/* Launch plan of the tile kernels of fractal_step for this handle (built, with
+ * its allocations, if it does not exist yet, as by fractal_get_tile_levels);
+ * calls that run bit-sliced have a plan of their own, which is not reported.
  * info[0..n-1] receives, in order: the policy (0: cell by cell, 3 or 4:
  * groups of s^G x s^G cells, 9: 2D groups of 9 cells in a shared-memory
  * box, 10: the triangle's 81-cell units with taps, 11 / 12: the carpet's /
@@ -331,7 +337,11 @@ int fractal_autotune(fractal_t *f, const uint8_t *in_dev, uint8_t *out_dev,
  * `stream` (asynchronously).  Instances of 2D fractals with one transition
  * table, 2 generations or more and at most 60 million cells run bit-sliced
  * instead, in one launch for all generations of as many instances as fit on
- * the chip together.  The graph is kept and replayed by later runs
+ * the chip together (unless a fractal's instances are of one tile depth, run
+ * two generations at most and are small: two launches are then shorter).
+ * Copies (steps = 0) come first, the bit-sliced launches last.  A run builds
+ * the tables of every instance's handle, as a first fractal_step would.  The
+ * graph is kept and replayed by later runs
  * until instances are added or cleared.  Buffers stay owned by the caller and
  * must stay valid while a run is in flight; the batch owns a device arena for
  * its tables and for one k^r-byte ping-pong buffer per instance with

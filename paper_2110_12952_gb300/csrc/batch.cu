@@ -7,7 +7,8 @@
 // Instances of 2D fractals with two generations or more go through sliced
 // launches instead (slice.cu), a few per fractal table and rule, each through
 // all of its generations with the packed states in shared memory: 256 uneven
-// instances (3.2e8 cells), 50 generations, 13.1 -> 2.7 ms.
+// instances (3.2e8 cells), 50 generations, 13.1 -> 2.7 ms.  (Two short
+// generations of one class stay here, see build.)
 //
 // A class is a set of instances whose fractals share the per-tile tables:
 // the same transition table (k, s, dim, offsets) and the same tile depth L.

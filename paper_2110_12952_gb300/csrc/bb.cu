@@ -10,9 +10,10 @@
 // starting anywhere in a local row reads as one bit field), so a cell's
 // membership costs two divisions by s^Lb = S and two bit look-ups.
 //
-// Two kernels: bit-sliced rows (bb_bits2_kernel, bb_bits3_kernel, below)
-// for boxes of side >= 32 in 16-byte aligned buffers (S >= 32 then); other
-// boxes take bb_kernel, where each CTA stages a tile of the box plus a
+// Three forms: bit-sliced rows (bb_bits2_kernel, bb_bits3_kernel, below) for
+// boxes of side >= 32 in 16-byte aligned buffers (S >= 32 then); packed words
+// (try_bb_packed) for several generations of such boxes at any address and for
+// single 3D ones; others take bb_kernel, where each CTA stages a tile of the box plus a
 // one-cell halo in shared memory, one byte per cell (bit 0 = alive member,
 // bit 1 = member), and applies the rule from there.
 #include <cuda_runtime.h>

@@ -1406,10 +1406,9 @@ static void slice_set_packed(SlicePlan &s, int states, uint8_t *mem)
 
 // One allocation: the tables (copied from the host in one piece), the grid
 // barrier's zeros, the neighbouring tiles, the resident exports and `packed`
-// packed states.  `img` is
-// that piece: the copy may read it until `st` has been waited for (a runtime
-// that reads pageable memory in place does not stage it first), so the caller
-// keeps it until then.
+// packed states.  `img` becomes the host's piece: the copy may read it until
+// `st` has been waited for (a runtime that reads pageable memory in place does
+// not stage it first), so the caller keeps it until then.
 static cudaError_t slice_upload(SliceGeo &p, SliceImage &image, SlicePlan &s, const std::vector<SliceGroup> &groups,
                                 int packed, std::vector<uint8_t> &img, cudaStream_t st)
 {
